@@ -17,7 +17,7 @@ __host__ __device__ __forceinline__ uint32_t balanced_warps(uint64_t units, uint
 
 // Work is dealt out in warp tiles of 32 consecutive groups, tile i to warp (i mod working warps):
 // every SM then gets the same number of tiles to within one, whatever the tensor size.
-constexpr uint32_t kSmallWarpBytes = kTabBytes / 2 + kBitsBytes;   // half a value table (two warps share one), bit-stream array
+constexpr uint32_t kSmallWarpBytes = kBitBytes;
 template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __restrict__ d_blocks, uint64_t n_groups,
@@ -25,47 +25,34 @@ ecco_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __rest
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const Tables tb = plan_tables(smem_u32(smem), d_meta);
-    const uint32_t nw = warps_that_fit(tb, kSmallWarpBytes, kTabBytes / 2);   // an odd warp count leaves half a table unused
-    WarpSmem ws;
-    ws.tab = tab_column<kTabHalf>(tb.warp_base, warp, lane);
-    ws.bits = tb.warp_base + tab_bytes<kTabHalf>(nw) + warp * kBitsBytes + lane * 4;
-    ws.syms = 0;
-    if (warp < nw) {
-        sts_u32(ws.bits + 16 * 128, 0u);
-        sts_u32(ws.bits + 17 * 128, 0u);
-    }
+    const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, true);
+    const uint32_t nw = decode_warps(tb, kSmallWarpBytes);
+    const uint32_t bits = tb.warp_base + warp * kSmallWarpBytes + lane * 4;
+    if (warp < nw) clear_tail_rows(bits);
     const uint64_t n_tiles = (n_groups + 31) / 32;
     // every working warp gets the same number of tiles (+-1 over the whole grid); warp ids interleave over
     // the CTAs, so every SM keeps the same number busy
     const uint64_t tile_stride = balanced_warps(n_tiles, gridDim.x * nw);
     uint64_t tile = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x;
     if (warp >= nw || tile >= tile_stride) tile = n_tiles;               // this warp sits the launch out (after the table barrier)
-    Block blk;
-    // lanes past the end of the tensor decode the last group again and store nothing
-    if (tile < n_tiles) ldg_block(blk, d_blocks + min(tile * 32 + lane, n_groups - 1) * kBlockBytes);
-    issue_tables(tb, d_meta);
-    if (!wait_tables(tb)) return;
+    issue_decode_tables(tb, d_meta);
+    if (!finish_decode_tables(tb)) return;
     const float T = tb.T;
 
     for (; tile < n_tiles; tile += tile_stride) {
         const uint64_t g = tile * 32 + lane;
-        const bool store = g < n_groups;
-        const GroupHeader h = open_group<kTabHalf>(blk, tb, ws, T);
-        const uint64_t tn = tile + tile_stride;
-        if (tn < n_tiles)                                  // next block in flight while this one decodes
-            ldg_block(blk, d_blocks + min(tn * 32 + lane, n_groups - 1) * kBlockBytes);
+        const bool store = g < n_groups;                   // lanes past the end of the tensor decode the last group again and store nothing
+        Block blk;
+        ldg_block(blk, d_blocks + min(g, n_groups - 1) * kBlockBytes);
+        LaneGroup lg = open_block(blk, bits, tb, T);
         uint16_t* out = d_out + min(g, n_groups - 1) * kGroup;
-        uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        const uint32_t end = decode_symbols<true, 16, kBlockBits, 0, kTabHalf>(h, ws, tb.pairs, [&](int n, uint32_t v, uint32_t, bool, uint32_t) {
-            const int slot = (n & 15) >> 1;
-            if (n & 1) r[slot] |= v << 16; else r[slot] = v;
-            if ((n & 15) == 15 && store) stg_v8(out + (n - 15), r);
+        const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, const uint32_t (&v)[4], uint32_t) {
+            if (store) *reinterpret_cast<uint4*>(out + i * 8) = make_uint4(v[0], v[1], v[2], v[3]);
         });
-        if (end && store) {
-            const int n_pad = min(kMaxPads, static_cast<int>((kBlockBits - end) / kPadBits));
+        if (store) {
+            const int n_pad = pads_of(end);
             for (int j = 0; j < n_pad; ++j) {
-                const uint32_t f = read_pad(ws, j);
+                const uint32_t f = pad_field(bits, j);
                 // same thread, same address as the vector store above: program order holds
                 out[f & 127u] = static_cast<uint16_t>(f2h_bits(fp8_to_float(f >> 7) * T));
             }
@@ -101,9 +88,9 @@ struct DecompressBatch {
     int32_t reserved[15];
     DecompressJob job[kMaxJobs];
 };
-constexpr uint32_t kTmaWarpBytes = kTabBytes / 2 + 1024 + kBitsBytes;   // half a value table (two warps share one), staging tile, bit-stream array
+constexpr uint32_t kTmaWarpBytes = 1024 + kBitBytes;                 // staging tile, bit-stream array
 
-template <int kMaxWarps, int kDecFree = 12>
+template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
 {
@@ -120,94 +107,80 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
         const DevHeader* hd = reinterpret_cast<const DevHeader*>(batch.job[t].meta);
         return make_uint2(__ldg(&hd->hash_lo), __ldg(&hd->hash_hi));
     };
-    auto tiles_of = [&](int t) { return (batch.job[t].n_groups + 31) / 32; };
+    auto tiles_of = [&](int t) { return static_cast<uint32_t>((batch.job[t].n_groups + 31) / 32); };   // at most 2^26, eight jobs 2^29
     int run = 0;
     for (int t0 = 0; t0 < batch.n; ++run) {
-        const Tables tb = plan_tables(smem_base, batch.job[t0].meta);
+        const DecodeTables tb = plan_decode_tables(smem_base, batch.job[t0].meta, true);
         int t1 = t0 + 1;
-        uint64_t run_tiles = tiles_of(t0);
+        uint32_t run_tiles = tiles_of(t0);
         for (; t1 < batch.n; ++t1) {
             const uint2 hh = hash_of(t1);
             if (hh.x != tb.hash_lo || hh.y != tb.hash_hi) break;
             run_tiles += tiles_of(t1);
         }
         if (run > 0) __syncthreads();                      // every warp is done with the previous run's tables
-        issue_tables(tb, batch.job[t0].meta, run == 0);
-        const uint32_t nw = warps_that_fit(tb, kTmaWarpBytes, kTabBytes / 2);
-        WarpSmem ws;
-        ws.tab = tab_column<kTabHalf>(tb.warp_base, warp, lane);
-        const uint32_t stage = tb.warp_base + tab_bytes<kTabHalf>(nw) + warp * 1024;     // this warp's staging tile
-        ws.bits = stage + (nw - warp) * 1024 + warp * kBitsBytes + lane * 4;
-        ws.syms = 0;
+        issue_decode_tables(tb, batch.job[t0].meta, run == 0);
+        const uint32_t tiles_base = (tb.warp_base + 1023u) & ~1023u;
+        const uint32_t nw = decode_warps(tb, kTmaWarpBytes, tiles_base - tb.warp_base);
+        const uint32_t stage = tiles_base + warp * 1024;                       // this warp's staging tile
+        const uint32_t bits = tiles_base + nw * 1024 + warp * kBitBytes + lane * 4;
         const uint32_t my_row = stage + lane * 32;
-        if (warp < nw) {
-            sts_u32(ws.bits + 16 * 128, 0u);
-            sts_u32(ws.bits + 17 * 128, 0u);
-        }
-        const uint64_t tile_stride = balanced_warps(run_tiles, gridDim.x * nw);
-        uint64_t gt = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x;       // tile in the run's tile space
+        if (warp < nw) clear_tail_rows(bits);
+        const uint32_t tile_stride = balanced_warps(run_tiles, gridDim.x * nw);
+        uint32_t gt = warp * gridDim.x + blockIdx.x;                           // tile in the run's tile space
         if (warp >= nw || gt >= tile_stride) gt = run_tiles;
-        // cursor: the job that holds tile gt, and the first tile of that job in the run's tile space
-        struct Cursor { int job; uint64_t first, tiles; };
-        Cursor cur = {t0, 0, tiles_of(t0)};
-        auto seek = [&](Cursor& c, uint64_t g) {
-            while (g >= c.first + c.tiles && c.job + 1 < t1) { c.first += c.tiles; ++c.job; c.tiles = tiles_of(c.job); }
+        // the job that holds tile gt, and the first tile of that job in the run's tile space
+        int job_at = t0;
+        uint32_t job_first = 0, job_tiles = tiles_of(t0);
+        auto seek = [&](uint32_t g) {
+            while (g >= job_first + job_tiles && job_at + 1 < t1) { job_first += job_tiles; ++job_at; job_tiles = tiles_of(job_at); }
         };
-        auto block_ptr = [&](const Cursor& c, uint64_t g) {
-            const DecompressJob& job = batch.job[c.job];
-            return job.blocks + min((g - c.first) * 32 + lane, job.n_groups - 1) * kBlockBytes;
+        auto block_ptr = [&](uint32_t g) {
+            const DecompressJob& job = batch.job[job_at];
+            return job.blocks + static_cast<uint64_t>(min((g - job_first) * 32 + lane, static_cast<uint32_t>(job.n_groups) - 1u)) * kBlockBytes;
         };
         if (run == 0) dependency_wait();                   // blocks and output: only after the previous kernel has completed
-        if (gt < run_tiles) { seek(cur, gt); prefetch_block_l2(block_ptr(cur, gt)); }
-        if (!wait_tables(tb, static_cast<uint32_t>(run & 1))) return;
-        float T = tb.T;
-        int t_of_T = t0;
+        if (gt < run_tiles) { seek(gt); prefetch_block_l2(block_ptr(gt)); }
+        if (!finish_decode_tables(tb, static_cast<uint32_t>(run & 1))) return;
 
-        for (; gt < run_tiles; gt += tile_stride) {
-            const DecompressJob& job = batch.job[cur.job];
-            if (cur.job != t_of_T) { T = __ldg(&reinterpret_cast<const DevHeader*>(job.meta)->T); t_of_T = cur.job; }
-            const uint64_t n_groups = job.n_groups;
-            const uint64_t tile = gt - cur.first;
-            const uint64_t g = tile * 32 + lane;
-            const bool store = g < n_groups;
-            uint16_t* out = job.out + min(g, n_groups - 1) * kGroup;
+        while (gt < run_tiles) {
+            const DecompressJob& job = batch.job[job_at];
+            const float T = __ldg(&reinterpret_cast<const DevHeader*>(job.meta)->T);
+            const uint32_t row0 = (gt - job_first) * 32, g = row0 + lane;
+            const bool store = g < static_cast<uint32_t>(job.n_groups);
+            uint16_t* out = job.out + static_cast<uint64_t>(g) * kGroup;
             const CUtensorMap* out_map = &job.map;
-            const int row0 = static_cast<int>(tile * 32);
             // The block is fetched when its turn comes, after a prefetch into L2 one tile earlier: holding the next
             // block in sixteen registers through a whole group would cost four of the 32 warps.
             Block blk;
-            ldg_block(blk, block_ptr(cur, gt));
-            const GroupHeader h = open_group<kTabHalf>(blk, tb, ws, T);
-            const uint64_t gn = gt + tile_stride;
-            if (gn < run_tiles) { seek(cur, gn); prefetch_block_l2(block_ptr(cur, gn)); }
-            uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            auto stage_rows = [&]() {
-                if (lane == 0) bulk_wait_read0();              // the engine has read the previous tile
-                __syncwarp();
-                sts_v4(my_row + swz, r[0], r[1], r[2], r[3]);
-                sts_v4(my_row + (swz ^ 16u), r[4], r[5], r[6], r[7]);
-            };
-            auto send_tile = [&](int chunk) {
+            ldg_block(blk, block_ptr(gt));
+            LaneGroup lg = open_block(blk, bits, tb, T);
+            gt += tile_stride;
+            if (gt < run_tiles) { seek(gt); prefetch_block_l2(block_ptr(gt)); }
+            auto send_tile = [&](int x) {
                 fence_async_smem();                            // generic-proxy writes -> visible to the engine
                 __syncwarp();
-                if (lane == 0) { tma_store_2d(out_map, stage, chunk * 16, row0); bulk_commit(); }
+                if (lane == 0) { tma_store_2d(out_map, stage, x, static_cast<int>(row0)); bulk_commit(); }
             };
-            const uint32_t end = decode_symbols<true, 16, kBlockBits, kDecFree, kTabHalf>(h, ws, tb.pairs, [&](int n, uint32_t v, uint32_t, bool, uint32_t) {
-                const int slot = (n & 15) >> 1;
-                if (n & 1) r[slot] = __byte_perm(r[slot], v, 0x5410); else r[slot] = v;
-                if ((n & 15) == 15 && n != 127) { stage_rows(); send_tile(n >> 4); }
+            const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, const uint32_t (&v)[4], uint32_t) {
+                if (!(i & 1)) {
+                    if (lane == 0) bulk_wait_read0();          // the engine has read the previous tile
+                    __syncwarp();
+                    sts_v4(my_row + swz, v[0], v[1], v[2], v[3]);
+                } else {
+                    sts_v4(my_row + (swz ^ 16u), v[0], v[1], v[2], v[3]);
+                    if (i != 15) send_tile(i * 8 - 8);
+                }
             });
-            stage_rows();                                      // values 112..127
-            const int n_pad = end ? min(kMaxPads, static_cast<int>((kBlockBits - end) / kPadBits)) : 0;
-            if (__any_sync(0xffffffffu, n_pad > 0)) {
+            const int n_pad = pads_of(end);
+            const int n_max = __reduce_max_sync(0xffffffffu, n_pad);
+            if (n_max > 0) {
                 if (lane == 0) bulk_wait_all();                // tiles 0..6 of this group are in memory
                 __syncwarp();
-                const int n_max = __reduce_max_sync(0xffffffffu, n_pad);
-#pragma unroll
-                for (int j = 0; j < kMaxPads; ++j) {           // ascending: a later pad overrides an earlier one
-                    if (j >= n_max) break;
+#pragma unroll 1
+                for (int j = 0; j < n_max; ++j) {              // ascending: a later pad overrides an earlier one
                     if (j < n_pad) {
-                        const uint32_t f = read_pad(ws, j);
+                        const uint32_t f = pad_field(bits, j);
                         const uint32_t loc = f & 127u;
                         const unsigned short val = static_cast<unsigned short>(f2h_bits(fp8_to_float(f >> 7) * T));
                         if (loc >= 112u) {
@@ -219,7 +192,7 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
                     }
                 }
             }
-            send_tile(7);
+            send_tile(112);
         }
         if (lane == 0) bulk_wait_all();                    // the staging tile may move with the next run's layout
         t0 = t1;

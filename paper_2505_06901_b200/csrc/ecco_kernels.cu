@@ -6,7 +6,8 @@
 // groups, not inside a group.  The lanes of a warp advance symbol by symbol in lock step, which
 // keeps every per-symbol index (output position, activation element) uniform across the warp.
 //
-// Shared memory per CTA (sizes from the image's header, see ecco_device_core.cuh):
+// Shared memory per CTA (sizes from the image's header, see ecco_device_core.cuh; ecco_decompress keeps the values in
+// registers, see ecco_decode_core.cuh):
 //   tables   pattern[64][16] fp16 | ID_KP table [4096] u16 | codebook records [256] x 16 B | shape tables
 //            [n_shapes][256] u8 | pair tables, brought in by three bulk copies (cp.async.bulk + mbarrier)
 //   per warp tab[16][32]  u32   per-lane dequantised centroids in rank order (the rank of the abs-max symbol
@@ -22,6 +23,7 @@
 //
 // Layout of the sources (one translation unit; the .cuh files are included here and nowhere else):
 //   ecco_device_core.cuh            shared-memory layout, PTX helpers, table staging, the per-group decoder
+//   ecco_decode_core.cuh            the group decoder with the value table in registers
 //   ecco_decompress_kernels.cuh     ecco_decompress (tile-store and small-tensor kernels), ecco_var_decompress
 //   ecco_fused_scalar_kernels.cuh   fused GEMV / attention scores, one or two dot products per group
 //   ecco_fused_mma_kernels.cuh      the same for three to eight dot products, on the tensor cores
@@ -31,6 +33,7 @@
 //   ecco_launch.cuh                 device query, overlapped launches, work plans
 //   this file                       the C ABI: argument checks and launches
 #include "ecco_device_core.cuh"
+#include "ecco_decode_core.cuh"
 #include "ecco_decompress_kernels.cuh"
 #include "ecco_fused_scalar_kernels.cuh"
 #include "ecco_attn_values_kernels.cuh"

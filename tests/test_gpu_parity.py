@@ -80,6 +80,17 @@ def check_fused(got, ref, refabs, label="fused"):
 
 
 # ------------------------------------------------------------------ decompress
+@pytest.mark.parametrize("e", [-32, -16, -15, 0, 7, 8, 16])
+def test_decompress_every_scale_byte_at_the_edges_of_the_packed_product(B, eo, e):
+    """The values of a group are packed fp16 products for 2^-15 <= T <= 2^7 and fp32 products outside: both sides of both
+    edges, every scale byte (the two NaN codes among them), skewed codes so that all ranks, escapes and ends occur."""
+    meta = make_meta(eo, skew_lens, e=e, seed=9)
+    rb = np.random.Generator(np.random.PCG64(200 + e)).integers(0, 256, size=(1024, 64), dtype=np.uint8)
+    rb[:, 0] = np.arange(1024) & 255
+    got, want = gpu_decompress(B, lib_meta_from_oracle(B, meta), rb), eo.decode(meta, rb)
+    assert_bit_exact(got, want)
+
+
 @pytest.mark.parametrize("n_groups", [0, 1, 31, 32, 33, 1000, 1023, 1025, 2048])
 def test_decompress_matches_oracle_ragged_sizes(B, eo, cfg1_small, n_groups):
     lm = lib_meta_from_oracle(B, cfg1_small["meta"])
