@@ -204,33 +204,36 @@ __device__ __forceinline__ uint32_t lds_pair(uint32_t addr)
 }
 __device__ __forceinline__ bool warp_any(bool x) { return __any_sync(0xffffffffu, x); }
 
-// Decodes the 128 symbols of the lane's group, eight per step (Sec. 4.2, Huffman decode), and hands every step's values to
-// sink(step, v, ranks): v = eight fp16 values in four words, ranks = their ranks as nibbles.  A codeword that would cross
-// the end bit ends the group: its value and all later ones are zero (clipped).  Returns the end bit if all 128 fitted,
-// else 0.  Must be called by all 32 lanes of the warp.
+// keeps the first n_ok of eight values and zeroes the rest
+__device__ __forceinline__ void cut_values(uint32_t (&v)[4], int n_ok)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t keep;                                     // shl: amounts above 31 give zero
+        asm("shl.b32 %0, -1, %1;" : "=r"(keep) : "r"(max(16 * n_ok - 32 * k, 0)));
+        v[k] &= ~keep;
+    }
+}
+
+// Decodes the 128 symbols of the lane's group, eight per step (Sec. 4.2, Huffman decode), and hands every step's ranks (nibbles,
+// first symbol lowest) to sink(step, ranks, cutting, n_ok).  A codeword that would cross the end bit ends the group: that and
+// all later positions are clipped.  cutting (uniform over the warp) says that some lane may have clipped positions in this step, n_ok how
+// many of the lane's eight are there (8 if not cutting).  Returns the end bit if all 128 fitted, else 0; *n_valid = number of positions that
+// fitted.  Must be called by all 32 lanes of the warp.
 // kLastRow / kEndBit: last data row of the lane's staged stream (two more rows follow, which read as zero) and the bit at which
 // the stream ends.  kFreeSteps: that many leading steps carry no end test; the caller guarantees that the stream cannot end in them.
 // pairs = false (uniform): one symbol per lookup through the shape table, in every step.
 template <uint32_t kLastRow, uint32_t kEndBit, int kFreeSteps, class Sink>
-__device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink)
+__device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink, int* n_valid = nullptr)
 {
-    bool alive = true;
+    int fit = kGroup;
     // second symbol of an escape entry: its codeword starts 1 + (length of the first) bits into win
     auto resolve = [&](uint32_t e, uint32_t win) {
         const uint32_t b = lds_u8(g.blut ^ ((win >> (1u + (e & 15u))) & 0xffu));
         return (e & 0x078fu) + (b >> 4) + ((b & 15u) << 11);
     };
-    // zeroes the values from number n_ok on
-    auto cut = [](uint32_t (&v)[4], int n_ok) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            uint32_t keep;                                 // shl: amounts above 31 give zero
-            asm("shl.b32 %0, -1, %1;" : "=r"(keep) : "r"(max(16 * n_ok - 32 * k, 0)));
-            v[k] &= ~keep;
-        }
-    };
     // one step symbol by symbol, with the end test
-    auto single_step = [&](uint32_t (&v)[4]) {
+    auto single_step = [&](int i) {
         uint32_t q = g.p + 1u, ranks = 0;
         int n_ok = 0;
 #pragma unroll
@@ -243,15 +246,13 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
                 const uint32_t e = lds_u8(g.blut ^ ((win >> acc) & 0xffu));
                 acc += e >> 4;
                 ranks |= (e & 15u) << (16 * h + 4 * j);
-                alive = alive && q + acc <= kEndBit;
-                n_ok += alive ? 1 : 0;
+                n_ok += q + acc <= kEndBit ? 1 : 0;        // positions only grow: once over the end, always over it
             }
             q += acc;
         }
         g.p = q - 1u;
-        map_ranks(g, ranks, v);
-        cut(v, n_ok);
-        return ranks;
+        if (n_ok < 8) fit = min(fit, 8 * i + n_ok);
+        sink(i, ranks, true, n_ok);
     };
     auto step = [&](int i, auto tested) {
         constexpr bool kTest = decltype(tested)::value;
@@ -292,22 +293,22 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
         const uint32_t n = (n01 + e2 + e3) & 0x7fu;
         // low halves of two entries side by side (a multiply-add: the integer pipe is the busier one), ranks to bytes 0 and 2
         const uint32_t ranks = prmt((e1 * 0x10000u + e0) >> 7, (e3 * 0x10000u + e2) >> 7, 0x6420u);
-        uint32_t v[4];
-        map_ranks(g, ranks, v);
+        bool cutting = false;
+        int n_ok = 8;
         if (kTest && warp_any(g.p + n >= kEndBit)) {
             // some lane's stream ends in this step: how many of its codewords end by then
+            cutting = true;
             const int room = static_cast<int>(kEndBit - 1u) - static_cast<int>(g.p);
             const int c0 = e0 & 31u, c1 = n01 & 63u, c2 = (n01 + e2) & 63u, c3 = n;
             const int start = c0 > room ? 0 : c1 > room ? c0 : c2 > room ? c1 : c2;       // of the first pair that does not fit
             const uint32_t q = g.p + 1u + start, r = bits + min(q >> 5, kLastRow) * 128;
             const int first = lds_u8(g.blut ^ (__funnelshift_r(lds_u32(r), lds_u32(r + 128), q) & 0xffu)) >> 4;
-            int n_ok = (start + first <= room ? 1 : 0) + (c0 <= room ? 2 : 0) + (c1 <= room ? 2 : 0) + (c2 <= room ? 2 : 0);
+            n_ok = (start + first <= room ? 1 : 0) + (c0 <= room ? 2 : 0) + (c1 <= room ? 2 : 0) + (c2 <= room ? 2 : 0);
             if (c3 <= room) n_ok = 8;
-            alive = c3 <= room;
-            cut(v, n_ok);
+            else fit = min(fit, 8 * i + n_ok);
         }
         g.p += n;
-        sink(i, v, ranks);
+        sink(i, ranks, cutting, n_ok);
     };
     if (pairs) {
 #pragma unroll 1
@@ -316,13 +317,10 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
         for (int i = kFreeSteps; i < 16; i += 2) { step(i, cuda::std::true_type{}); step(i + 1, cuda::std::true_type{}); }
     } else {
 #pragma unroll 1
-        for (int i = 0; i < 16; ++i) {
-            uint32_t v[4];
-            const uint32_t ranks = single_step(v);
-            sink(i, v, ranks);
-        }
+        for (int i = 0; i < 16; ++i) single_step(i);
     }
-    return alive ? g.p + 1u : 0u;
+    if (n_valid) *n_valid = fit;
+    return fit == kGroup ? g.p + 1u : 0u;
 }
 constexpr int kBlockFreeSteps = 6;     // the indices of a block start at bit 22 at the latest: 6 steps end by bit 22 + 6 * 64 = 406
 

@@ -46,7 +46,10 @@ ecco_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __rest
         ldg_block(blk, d_blocks + min(g, n_groups - 1) * kBlockBytes);
         LaneGroup lg = open_block(blk, bits, tb, T);
         uint16_t* out = d_out + min(g, n_groups - 1) * kGroup;
-        const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, const uint32_t (&v)[4], uint32_t) {
+        const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
+            uint32_t v[4];
+            map_ranks(lg, ranks, v);
+            if (cutting) cut_values(v, n_ok);
             if (store) *reinterpret_cast<uint4*>(out + i * 8) = make_uint4(v[0], v[1], v[2], v[3]);
         });
         if (store) {
@@ -162,7 +165,10 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
                 __syncwarp();
                 if (lane == 0) { tma_store_2d(out_map, stage, x, static_cast<int>(row0)); bulk_commit(); }
             };
-            const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, const uint32_t (&v)[4], uint32_t) {
+            const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
+                uint32_t v[4];
+                map_ranks(lg, ranks, v);
+                if (cutting) cut_values(v, n_ok);
                 if (!(i & 1)) {
                     if (lane == 0) bulk_wait_read0();          // the engine has read the previous tile
                     __syncwarp();

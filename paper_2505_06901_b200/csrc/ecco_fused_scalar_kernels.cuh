@@ -4,94 +4,74 @@
 
 namespace {
 
-// The fused kernels decode one symbol per lookup (shape tables only) and leave the pair tables out of shared memory:
-// measured on the 7B-shaped matrices and the cfg-3 K cache, the room the pair tables take (fewer resident warps) costs
-// them as much as two-symbol lookups save, and on KV caches, whose codebooks spread over three dozen code shapes,
-// escapes make the pair path the slower one.
-constexpr bool kFusedPairs = false;
-
 // ---------------------------------------------------------------------------------------------
 // K2/K3: fused consumers.  kV = number of dot products per group (batch rows of x, or query
-// heads per KV head).  The vector slice xs[128][kV] fp32 lives in shared memory; every lane reads
-// the same element at the same time (one broadcast wavefront), 16 bytes per load, so a slice
-// element costs 1/4 (kV = 1) to 2 (kV = 8) loads per symbol.
+// heads per KV head).  The vector slice [kV][128] fp16 lives in shared memory; every lane reads the same eight
+// elements at the same time (one broadcast wavefront per eight symbols and vector) and adds the products with the
+// mixed-precision multiply-add (fp16 x fp16 + fp32, one rounding): no operand is ever converted.
+// Bound by the decode.  Two symbols per lookup and values in registers against one symbol per lookup and a value table in
+// shared memory: the seven products of a 7B-shaped layer at batch 1 193.0 -> 166.0 us, a 4096 x 4096 matrix alone 20.3 -> 18.0 us.
 // ---------------------------------------------------------------------------------------------
-template <int kV>
-struct Accum {
-    float a[kV];
-    float4 cache;                       // the current 16 bytes of the slice (kV <= 2)
-    __device__ __forceinline__ void clear()
-    {
-#pragma unroll
-        for (int v = 0; v < kV; ++v) a[v] = 0.0f;
-    }
-    static __device__ __forceinline__ float4 lds_f4(uint32_t addr)
-    {
-        float4 x;
-        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(addr));
-        return x;
-    }
-    // value w of position n (n is a compile-time constant after unrolling); xs = shared address of xs[0][0]
-    __device__ __forceinline__ void fma(int n, float w, uint32_t xs)
-    {
-        if constexpr (kV == 1) {
-            if ((n & 3) == 0) cache = lds_f4(xs + n * 4);
-            const float x = (n & 3) == 0 ? cache.x : (n & 3) == 1 ? cache.y : (n & 3) == 2 ? cache.z : cache.w;
-            a[0] = fmaf(w, x, a[0]);
-        } else if constexpr (kV == 2) {
-            if ((n & 1) == 0) cache = lds_f4(xs + n * 8);
-            a[0] = fmaf(w, (n & 1) ? cache.z : cache.x, a[0]);
-            a[1] = fmaf(w, (n & 1) ? cache.w : cache.y, a[1]);
-        } else {
-#pragma unroll
-            for (int q = 0; q < kV / 4; ++q) {
-                const float4 x = lds_f4(xs + n * (kV * 4) + q * 16);
-                a[q * 4 + 0] = fmaf(w, x.x, a[q * 4 + 0]);
-                a[q * 4 + 1] = fmaf(w, x.y, a[q * 4 + 1]);
-                a[q * 4 + 2] = fmaf(w, x.z, a[q * 4 + 2]);
-                a[q * 4 + 3] = fmaf(w, x.w, a[q * 4 + 3]);
-            }
-        }
-    }
-    // out-of-order correction at a run-time position (outlier fix-up)
-    __device__ __forceinline__ void fma_at(uint32_t loc, float w, uint32_t xs)
-    {
-#pragma unroll
-        for (int v = 0; v < kV; ++v) {
-            float x;
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(xs + (loc * kV + v) * 4));
-            a[v] = fmaf(w, x, a[v]);
-        }
-    }
-};
+// Shared memory of a warp that keeps the decoded ranks of its groups: [27][32] words.  Rows 8..23 are the block's words, rows
+// 24..26 stay zero; the ranks of step i go to row i.  By then the stream has been read past that row: step i leaves the position
+// at bit 11 + 16 (i + 1) at least (eleven header bits, two bits per symbol), so the next window, which starts one bit early, starts in
+// row 8 + (26 + 16 i) / 32 > i or later, and the outlier fields (bits 272 and up) sit in rows 16 and up.
+constexpr uint32_t kRankRows = 8;
+constexpr uint32_t kRankedBytes = (kRankRows + kBitRows) * 128;      // 3456
 
-// decode one group and accumulate its kV dot products against xs (shared address of xs[0][0])
-template <int kV>
-__device__ __forceinline__ void fused_group(const Block& blk, const Tables& tb, const WarpSmem& ws, float T,
-                                            uint32_t xs, Accum<kV>& acc)
+// acc += w . x over the two fp16 numbers of each word
+__device__ __forceinline__ void fma_half2(float& acc, uint32_t w, uint32_t x)
 {
-    const GroupHeader h = open_group<kTabFloat>(blk, tb, ws, T);
-    RankPacker rk;
-    const uint32_t end = decode_symbols<true, 16, kBlockBits, kFusedFree>(h, ws, tb.pairs, [&](int n, uint32_t v, uint32_t, bool, uint32_t pair) {
-        acc.fma(n, __uint_as_float(v), xs);
-        rk.put(n, pair, ws.syms);
+    asm("{\n\t.reg .f16 a, b, c, d;\n\tmov.b32 {a, b}, %1;\n\tmov.b32 {c, d}, %2;\n\t"
+        "fma.rn.f32.f16 %0, a, c, %0;\n\tfma.rn.f32.f16 %0, b, d, %0;\n\t}"
+        : "+f"(acc)
+        : "r"(w), "r"(x));
+}
+// the value of one rank of the lane's group
+__device__ __forceinline__ float rank_value(const LaneGroup& g, uint32_t rank)
+{
+    const uint32_t s = rank & 7u, k = (rank >> 1) & 4u;
+    const uint32_t lo = prmt(prmt(g.vlo[0], g.vlo[1], s), prmt(g.vlo[2], g.vlo[3], s), k);
+    const uint32_t hi = prmt(prmt(g.vhi[0], g.vhi[1], s), prmt(g.vhi[2], g.vhi[3], s), k);
+    return __half2float(__ushort_as_half(static_cast<unsigned short>(prmt(lo, hi, 0x0040u))));
+}
+
+// decode one group and accumulate its kV dot products against the slice at shared address xs; two partial sums per product
+template <int kV>
+__device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, float (&acc)[kV][2])
+{
+    LaneGroup g = open_block(blk, bits, tb, T);
+    const uint32_t ranks_at = bits - kRankRows * 128;
+    const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(g, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
+        uint32_t v[4];
+        map_ranks(g, ranks, v);
+        if (cutting) cut_values(v, n_ok);
+        sts_u32(ranks_at + i * 128, ranks);
+#pragma unroll
+        for (int b = 0; b < kV; ++b) {
+            uint32_t x[4];
+            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(xs + b * (kGroup * 2) + i * 16));
+            fma_half2(acc[b][0], v[0], x[0]);
+            fma_half2(acc[b][1], v[1], x[1]);
+            fma_half2(acc[b][0], v[2], x[2]);
+            fma_half2(acc[b][1], v[3], x[3]);
+        }
     });
-    if (end) {
-        // outliers replace the mapped value at their location: add (outlier - mapped) * x
-        const int n_pad = min(kMaxPads, static_cast<int>((kBlockBits - end) / kPadBits));
-        uint64_t seen_lo = 0, seen_hi = 0;                  // 128-bit "already replaced" mask
-        for (int j = n_pad - 1; j >= 0; --j) {             // the last pad wins on a duplicate location
-            const uint32_t f = read_pad(ws, j);
-            const uint32_t loc = f & 127u;
-            const uint64_t bit = 1ull << (loc & 63u);
-            const bool upper = loc >= 64u;
-            if ((upper ? seen_hi : seen_lo) & bit) continue;
-            if (upper) seen_hi |= bit; else seen_lo |= bit;
-            const uint32_t word = lds_u32(ws.syms + (loc >> 3) * 128);
-            const uint32_t rank = (word >> ((loc & 7u) * 4)) & 15u;
-            const float mapped = __uint_as_float(lds_u32(ws.tab + rank * 128));
-            const float outlier = __half2float(__float2half_rn(fp8_to_float(f >> 7) * T));
-            acc.fma_at(loc, outlier - mapped, xs);
+    // outliers replace the mapped value at their location: add (outlier - mapped) * x
+    uint64_t seen_lo = 0, seen_hi = 0;                     // 128-bit "already replaced" mask
+    for (int j = pads_of(end) - 1; j >= 0; --j) {          // the last pad wins on a duplicate location
+        const uint32_t f = pad_field(bits, j);
+        const uint32_t loc = f & 127u;
+        const uint64_t bit = 1ull << (loc & 63u);
+        const bool upper = loc >= 64u;
+        if ((upper ? seen_hi : seen_lo) & bit) continue;
+        if (upper) seen_hi |= bit; else seen_lo |= bit;
+        const float mapped = rank_value(g, (lds_u32(ranks_at + (loc >> 3) * 128) >> ((loc & 7u) * 4)) & 15u);
+        const float outlier = __half2float(__float2half_rn(fp8_to_float(f >> 7) * T));
+#pragma unroll
+        for (int b = 0; b < kV; ++b) {
+            const float x = __half2float(__ushort_as_half(static_cast<unsigned short>(lds_u16(xs + b * (kGroup * 2) + loc * 2))));
+            acc[b][0] = fmaf(outlier - mapped, x, acc[b][0]);
         }
     }
 }
@@ -104,22 +84,6 @@ __host__ __device__ __forceinline__ int unit_owner(int64_t U, int G, int64_t u)
     while (c + 1 < G && unit_begin(U, G, c + 1) <= u) ++c;
     while (c > 0 && unit_begin(U, G, c) > u) --c;
     return c;
-}
-
-// per-warp arrays of the scalar fused kernels: value table (fp32), bit-stream array, decoded ranks
-constexpr uint32_t kFusedWarpBytes = kTabBytes + kBitsBytes + kSymsBytes;
-__device__ __forceinline__ WarpSmem fused_warp_smem(const Tables& tb, uint32_t nw)
-{
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    WarpSmem ws;
-    ws.tab = tab_column<kTabFloat>(tb.warp_base, warp, lane);
-    ws.bits = tb.warp_base + nw * kTabBytes + warp * (kBitsBytes + kSymsBytes) + lane * 4;
-    ws.syms = ws.bits + kBitsBytes;
-    if (warp < nw) {
-        sts_u32(ws.bits + 16 * 128, 0u);
-        sts_u32(ws.bits + 17 * 128, 0u);
-    }
-    return ws;
 }
 
 // One call of the fused GEMV may cover several matrices (ecco_gemv_batch): the units of all of them form one unit
@@ -142,7 +106,8 @@ struct GemvBatch {
     GemvJob job[kMaxGemvJobs];
 };
 // true (uniformly over the grid) if every matrix of the call carries the tables of the first
-__device__ __forceinline__ bool same_tables(const GemvBatch& batch, const Tables& tb)
+template <class TablesOf>
+__device__ __forceinline__ bool same_tables(const GemvBatch& batch, const TablesOf& tb)
 {
     bool same = true;
     for (int t = 1; t < batch.n; ++t) {
@@ -180,7 +145,9 @@ __device__ __forceinline__ const uint8_t* gemv_block_ptr(const GemvBatch& batch,
     return jb.blocks + (static_cast<uint64_t>(row) * jb.kblocks + p.kb) * kBlockBytes;
 }
 
-// K2 for one or two rows of x: the slice is small enough (512 B or 1 KB) for every warp to keep
+__host__ __device__ constexpr uint32_t scalar_warp_bytes(int v) { return v * kGroup * 2 + kRankedBytes; }
+
+// K2 for one or two rows of x: the slice is small enough (256 B a row) for every warp to keep
 // its own, so warps never meet at a barrier.  A work unit is (32 consecutive rows, one k-block),
 // numbered matrix by matrix, row-tile major; every working warp owns a contiguous run of units and keeps its
 // rows' partial sums in registers along k.  When a row tile is shared by several warps each writes its
@@ -193,14 +160,14 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict__ d_partial, unsigned int* __restrict__ d_tickets)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    constexpr uint32_t kXsBytes = kGroup * kV * 4;
     release_dependents();
     const uint8_t* d_meta = batch.job[0].meta;
-    const Tables tb = plan_tables(smem_u32(smem), d_meta, kFusedPairs);
-    const int nw = static_cast<int>(warps_that_fit(tb, kFusedWarpBytes + kXsBytes));
-    const WarpSmem ws = fused_warp_smem(tb, nw);
+    const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, true);
+    const int nw = static_cast<int>(decode_warps(tb, scalar_warp_bytes(kV)));
     const int lane = static_cast<int>(threadIdx.x & 31u), warp = static_cast<int>(threadIdx.x >> 5);
-    const uint32_t xs = tb.warp_base + nw * kFusedWarpBytes + warp * kXsBytes;   // this warp's slice
+    const uint32_t xs = tb.warp_base + warp * scalar_warp_bytes(kV);             // this warp's slice [kV][128] fp16
+    const uint32_t bits = xs + kV * kGroup * 2 + kRankRows * 128 + lane * 4;
+    if (warp < nw) clear_tail_rows(bits);
 
     // W working warps (chosen so that they all get the same number of units, and never more than there are
     // units); warp ids interleave over the CTAs; the other warps idle
@@ -208,18 +175,22 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     const int64_t U = batch.units;
     const int W = static_cast<int>(balanced_warps(static_cast<uint64_t>(U), gridDim.x * static_cast<uint32_t>(nw)));
     const int64_t u0 = wg < W ? unit_begin(U, W, wg) : 0, u1 = wg < W ? unit_begin(U, W, wg + 1) : 0;
-    issue_tables(tb, d_meta);
+    issue_decode_tables(tb, d_meta);
     if (!same_tables(batch, tb)) {                         // images are host-written: readable before the wait
-        wait_tables(tb);                                   // the table copies into this CTA's shared memory must land first
+        bounded_wait(tb.base, 0, kWaitLimit);              // the table copies into this CTA's shared memory must land first
         return;
     }
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     GemvPos pos = {0, 0, 0};
     if (u0 < u1) { pos = gemv_pos_of(batch, u0); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
-    if (!wait_tables(tb)) return;
+    if (!finish_decode_tables(tb)) return;
 
-    Accum<kV> acc;
-    acc.clear();
+    float acc[kV][2];                                      // two partial sums, added when the row tile is left
+    auto clear_acc = [&]() {
+#pragma unroll
+        for (int b = 0; b < kV; ++b) acc[b][0] = acc[b][1] = 0.0f;
+    };
+    clear_acc();
     auto flush = [&](int jf, int tile) {
         const GemvJob& jb = batch.job[jf];
         const int n_out = jb.n_out, kblocks = jb.kblocks, gtile = jb.tile_first + tile;
@@ -232,13 +203,13 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
         if (w_lo == w_hi) {
             if (row_ok) {
 #pragma unroll
-                for (int b = 0; b < kV; ++b) d_y[static_cast<size_t>(b) * n_out + row] = acc.a[b];
+                for (int b = 0; b < kV; ++b) d_y[static_cast<size_t>(b) * n_out + row] = acc[b][0] + acc[b][1];
             }
             return;
         }
         float* mine = d_partial + static_cast<size_t>(wg + gtile) * kV * 32;
 #pragma unroll
-        for (int b = 0; b < kV; ++b) mine[b * 32 + lane] = acc.a[b];
+        for (int b = 0; b < kV; ++b) mine[b * 32 + lane] = acc[b][0] + acc[b][1];
         __threadfence();
         __syncwarp();
         unsigned int t = 0;
@@ -292,27 +263,15 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     for (int64_t u = u0; u < u1; ++u) {
         if (pos.j != cur_j || pos.tile != cur_tile) {
             flush(cur_j, cur_tile);
-            acc.clear();
+            clear_acc();
             if (pos.j != cur_j) T = __ldg(&reinterpret_cast<const DevHeader*>(batch.job[pos.j].meta)->T);
             cur_j = pos.j;
             cur_tile = pos.tile;
         }
-        // this warp's slice: lane l converts x[b][kb*128 + 4l .. 4l+3] to fp32, layout xs[i][b]
+        // this warp's slice: lane l holds x[b][kb*128 + 4l .. 4l+3]
         __syncwarp();
-        {
-            float v[kV][4];
 #pragma unroll
-            for (int b = 0; b < kV; ++b) {
-                const __half2 h0 = *reinterpret_cast<const __half2*>(&xraw[b].x), h1 = *reinterpret_cast<const __half2*>(&xraw[b].y);
-                v[b][0] = __low2float(h0); v[b][1] = __high2float(h0); v[b][2] = __low2float(h1); v[b][3] = __high2float(h1);
-            }
-            if constexpr (kV == 1) {
-                sts_v4(xs + lane * 16, __float_as_uint(v[0][0]), __float_as_uint(v[0][1]), __float_as_uint(v[0][2]), __float_as_uint(v[0][3]));
-            } else {
-                sts_v4(xs + lane * 32, __float_as_uint(v[0][0]), __float_as_uint(v[1][0]), __float_as_uint(v[0][1]), __float_as_uint(v[1][1]));
-                sts_v4(xs + lane * 32 + 16, __float_as_uint(v[0][2]), __float_as_uint(v[1][2]), __float_as_uint(v[0][3]), __float_as_uint(v[1][3]));
-            }
-        }
+        for (int b = 0; b < kV; ++b) sts_v2(xs + b * (kGroup * 2) + lane * 8, xraw[b].x, xraw[b].y);
         __syncwarp();
         // the block is fetched when its turn comes (it was prefetched into L2 one unit earlier): holding the next
         // one in sixteen registers through a whole group costs more in resident warps than the fetch costs here
@@ -323,14 +282,14 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
             prefetch_block_l2(gemv_block_ptr(batch, pos, lane));
             load_x(pos);
         }
-        fused_group<kV>(cur, tb, ws, T, xs, acc);
+        fused_group<kV>(cur, tb, bits, T, xs, acc);
     }
     flush(cur_j, cur_tile);
 }
 
 // K3: scores[b][hq][t] = scale * q[b][hq] . K~[b][hq / q_per_kv][t] for one or two query heads per KV head.
 // Built like K2: a work unit is (one (batch, kv head) pair, 32 consecutive tokens), a lane owns one token, every
-// working warp owns a contiguous run of units and keeps its own query slice (pre-multiplied by scale, restaged
+// working warp owns a contiguous run of units and keeps its own query slice (restaged
 // when the head changes), so warps never meet at a barrier and a ragged sequence length costs at most one
 // partly filled unit per head.
 template <int kV, int kMaxWarps>
@@ -339,13 +298,13 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
                         int q_per_kv, const __half* d_q, float scale, float* __restrict__ d_scores)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    constexpr uint32_t kXsBytes = kGroup * kV * 4;
     release_dependents();
-    const Tables tb = plan_tables(smem_u32(smem), d_meta, kFusedPairs);
-    const int nw = static_cast<int>(warps_that_fit(tb, kFusedWarpBytes + kXsBytes));
-    const WarpSmem ws = fused_warp_smem(tb, nw);
+    const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, true);
+    const int nw = static_cast<int>(decode_warps(tb, scalar_warp_bytes(kV)));
     const int lane = static_cast<int>(threadIdx.x & 31u), warp = static_cast<int>(threadIdx.x >> 5);
-    const uint32_t xs = tb.warp_base + nw * kFusedWarpBytes + warp * kXsBytes;   // this warp's slice: xs[d][r]
+    const uint32_t xs = tb.warp_base + warp * scalar_warp_bytes(kV);             // this warp's slice [kV][128] fp16
+    const uint32_t bits = xs + kV * kGroup * 2 + kRankRows * 128 + lane * 4;
+    if (warp < nw) clear_tail_rows(bits);
 
     const int wg = warp < nw ? warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x) : INT_MAX;
     const int tiles = (seq + 31) / 32;
@@ -358,32 +317,23 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         return d_kblocks + (static_cast<uint64_t>(bh) * seq + min(tile * 32 + lane, seq - 1)) * kBlockBytes;
     };
     int bh = static_cast<int>(u0 / tiles), tile = static_cast<int>(u0 % tiles);
-    issue_tables(tb, d_meta);
+    issue_decode_tables(tb, d_meta);
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (u0 < u1) prefetch_block_l2(block_ptr(bh, tile));
-    if (!wait_tables(tb)) return;
+    if (!finish_decode_tables(tb)) return;
     const float T = tb.T;
 
     int cur_bh = -1;
     for (int64_t u = u0; u < u1; ++u) {
         const int t = tile * 32 + lane;
         if (bh != cur_bh) {
-            // lane l stages q[b][h*q_per_kv + r][4l .. 4l+3] * scale as fp32, layout xs[d][r]; heads beyond q_per_kv are zero
-            float v[kV][4];
+            // lane l stages q[b][h*q_per_kv + r][4l .. 4l+3]; heads beyond q_per_kv are zero
+            __syncwarp();                                  // every lane is done with the previous head's slice
 #pragma unroll
             for (int r = 0; r < kV; ++r) {
                 uint2 raw = make_uint2(0u, 0u);
                 if (r < q_per_kv) raw = __ldcg(reinterpret_cast<const uint2*>(d_q + (static_cast<size_t>(bh) * q_per_kv + r) * kGroup) + lane);
-                const __half2 h0 = *reinterpret_cast<const __half2*>(&raw.x), h1 = *reinterpret_cast<const __half2*>(&raw.y);
-                v[r][0] = scale * __low2float(h0); v[r][1] = scale * __high2float(h0);
-                v[r][2] = scale * __low2float(h1); v[r][3] = scale * __high2float(h1);
-            }
-            __syncwarp();                                  // every lane is done with the previous head's slice
-            if constexpr (kV == 1) {
-                sts_v4(xs + lane * 16, __float_as_uint(v[0][0]), __float_as_uint(v[0][1]), __float_as_uint(v[0][2]), __float_as_uint(v[0][3]));
-            } else {
-                sts_v4(xs + lane * 32, __float_as_uint(v[0][0]), __float_as_uint(v[1][0]), __float_as_uint(v[0][1]), __float_as_uint(v[1][1]));
-                sts_v4(xs + lane * 32 + 16, __float_as_uint(v[0][2]), __float_as_uint(v[1][2]), __float_as_uint(v[0][3]), __float_as_uint(v[1][3]));
+                sts_v2(xs + r * (kGroup * 2) + lane * 8, raw.x, raw.y);
             }
             __syncwarp();
             cur_bh = bh;
@@ -393,13 +343,14 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         const int out_bh = bh;
         if (++tile == tiles) { tile = 0; ++bh; }
         if (u + 1 < u1) prefetch_block_l2(block_ptr(bh, tile));
-        Accum<kV> acc;
-        acc.clear();
-        fused_group<kV>(cur, tb, ws, T, xs, acc);
+        float acc[kV][2];
+#pragma unroll
+        for (int r = 0; r < kV; ++r) acc[r][0] = acc[r][1] = 0.0f;
+        fused_group<kV>(cur, tb, bits, T, xs, acc);
         if (t < seq) {
 #pragma unroll
             for (int r = 0; r < kV; ++r)
-                if (r < q_per_kv) d_scores[(static_cast<size_t>(out_bh) * q_per_kv + r) * seq + t] = acc.a[r];
+                if (r < q_per_kv) d_scores[(static_cast<size_t>(out_bh) * q_per_kv + r) * seq + t] = scale * (acc[r][0] + acc[r][1]);
         }
     }
 }
