@@ -11,9 +11,9 @@
 //    two lookups and one end-of-stream vote per step.
 //  * The sixteen values come from a table of centroids that is already in rank order for every codebook
 //    (build_rank_tables, made once per CTA from the staged image): two 16-byte loads and eight packed multiplications.
-// Per symbol of a warp, on 1 212 416 weight groups (ncu): 15.0 instructions, 8.5 of them on the integer pipe, and 4.1
+// Per symbol of a warp, on 1 212 416 weight groups (ncu): 15.1 instructions, 8.1 of them on the integer pipe, and 4.1
 // wavefronts, against 16.8, 8.2 and 5.3 with the value table in shared memory and four symbols per step; ecco_decompress over
-// a 7B-shaped layer 135.9 -> 126.3 us, over a [16][8][32768][128] cache 405.0 -> 360.9 us.
+// a 7B-shaped layer 138.8 -> 129.9 us, over a [16][8][32768][128] cache 407.4 -> 371.0 us.
 namespace {
 
 // Shared memory of a CTA: misc words, patterns and codebook records, then the tables of the decode.  The first three fill
@@ -25,6 +25,9 @@ constexpr uint32_t kSmemPairMin = kSmemRec + kCbRecBytes;            // 7168
 constexpr uint32_t kCentBytes = kMaxPatterns * kCodebooks * 32;      // centroids in rank order, fp16 [256][16]
 constexpr uint32_t kBitRows = 19;                                    // 16 words of a block and three zero rows
 constexpr uint32_t kBitBytes = kBitRows * 128;
+// A lane whose stream has ended goes on reading rows after its own: the next warp's or, behind the last warp, this slack.  What it
+// decodes there is cut to zero, and no row lies further than 128 codewords of 8 bits behind the header: 22 + 1024 bits, rows 32..34.
+constexpr uint32_t kSlackBytes = (35 - kBitRows) * 128;              // 2048
 
 struct DecodeTables {
     uint32_t base;          // misc area (barrier word at +0)
@@ -58,7 +61,7 @@ __device__ __forceinline__ DecodeTables plan_decode_tables(uint32_t smem_base, c
 // warps of this CTA that have room for warp_bytes each (the others sit the launch out)
 __device__ __forceinline__ uint32_t decode_warps(const DecodeTables& tb, uint32_t warp_bytes, uint32_t tail_bytes = 0)
 {
-    const uint32_t used = tb.warp_base - tb.base + tail_bytes;
+    const uint32_t used = tb.warp_base - tb.base + kSlackBytes + tail_bytes;
     const uint32_t room = used < kSmemCtaBytes ? kSmemCtaBytes - used : 0u;
     return min(room / warp_bytes, blockDim.x >> 5);
 }
@@ -256,7 +259,7 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
     };
     auto step = [&](int i, auto tested) {
         constexpr bool kTest = decltype(tested)::value;
-        const uint32_t row = bits + (kTest ? min(g.p >> 5, kLastRow) : g.p >> 5) * 128;
+        const uint32_t row = bits + (g.p >> 5) * 128;      // past its end a lane reads whatever follows: see kSlackBytes
         const uint32_t w0 = lds_u32(row), w1 = lds_u32(row + 128), w2 = lds_u32(row + 256);
         const uint32_t lo = __funnelshift_r(w0, w1, g.p), hi = __funnelshift_r(w1, w2, g.p);
         // an entry's low bits are the length of its codewords; funnel shifts take their amount modulo 32
@@ -275,12 +278,12 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
             x2 = __funnelshift_rc(lo, hi, n01 & 63u);      // up to 32 bits here
         }
         uint32_t e2 = lds_pair(g.plut ^ (x2 & g.mask));
-        uint32_t x3 = x2 >> (e2 & 31u);
+        uint32_t x3 = __funnelshift_r(x2, 0u, e2);
         uint32_t e3 = lds_pair(g.plut ^ (x3 & g.mask));
         if (warp_any((e2 | e3) & 0x8000u)) {
             // long codewords: the third pair's window is fetched again, the two pairs may need 33 bits of it
             const uint32_t q = g.p + (n01 & 63u);
-            const uint32_t r2 = bits + (kTest ? min(q >> 5, kLastRow) : q >> 5) * 128;
+            const uint32_t r2 = bits + (q >> 5) * 128;
             const uint32_t y0 = lds_u32(r2), y1 = lds_u32(r2 + 128), y2 = lds_u32(r2 + 256);
             const uint32_t l2 = __funnelshift_r(y0, y1, q), h2 = __funnelshift_r(y1, y2, q);
             if (e2 & 0x8000u) {
@@ -291,8 +294,9 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
             if (e3 & 0x8000u) e3 = resolve(e3, __funnelshift_r(l2, h2, e2));
         }
         const uint32_t n = (n01 + e2 + e3) & 0x7fu;
-        // low halves of two entries side by side (a multiply-add: the integer pipe is the busier one), ranks to bytes 0 and 2
-        const uint32_t ranks = prmt((e1 * 0x10000u + e0) >> 7, (e3 * 0x10000u + e2) >> 7, 0x6420u);
+        // two entries side by side and doubled (multiply-adds: the integer pipe is the busier one): ranks in bytes 1 and 3
+        const uint32_t e01 = e1 * 0x10000u + e0, e23 = e3 * 0x10000u + e2;
+        const uint32_t ranks = prmt(e01 * 2u, e23 * 2u, 0x7531u);
         bool cutting = false;
         int n_ok = 8;
         if (kTest && warp_any(g.p + n >= kEndBit)) {
