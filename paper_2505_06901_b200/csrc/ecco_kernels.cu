@@ -135,8 +135,7 @@ static int launch_decompress_small(const DeviceInfo& di, const void* d_meta, con
     auto kernel = ecco_decompress_kernel<kDecompressWarps>;
     int rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
-    const uint64_t cta_tiles = (n_groups + kDecompressWarps * 32 - 1) / (kDecompressWarps * 32);   // one tile per warp
-    const unsigned grid = static_cast<unsigned>(cta_tiles < static_cast<uint64_t>(di.sms) ? cta_tiles : di.sms);
+    const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>((n_groups + 31) / 32), di.sms));
     kernel<<<grid, kDecompressWarps * 32, kSmemCtaBytes, stream>>>(static_cast<const uint8_t*>(d_meta), d_blocks, n_groups,
                                                                    static_cast<uint16_t*>(d_out));
     return check_launch();
@@ -151,8 +150,7 @@ static int launch_decompress_batch(const DeviceInfo& di, DecompressBatch& batch,
     if (rc) return rc;
     uint64_t tiles = 0;
     for (int t = 0; t < batch.n; ++t) tiles += (batch.job[t].n_groups + 31) / 32;
-    const uint64_t ctas = (tiles + kDecompressTmaWarps - 1) / kDecompressTmaWarps;
-    const unsigned grid = static_cast<unsigned>(ctas < static_cast<uint64_t>(di.sms) ? ctas : di.sms);
+    const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>(tiles), di.sms));
     return launch_overlapped(kernel, grid, static_cast<unsigned>(kDecompressTmaWarps * 32), kSmemCtaBytes, stream, batch);
 }
 
@@ -235,8 +233,7 @@ extern "C" int ecco_var_decompress(const void* d_meta, const uint8_t* d_stream, 
     static thread_local bool configured[64] = {};
     rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
-    const uint64_t cta_tiles = (n_groups + kVarWarps * 32 - 1) / (kVarWarps * 32);
-    const unsigned grid = static_cast<unsigned>(cta_tiles < static_cast<uint64_t>(di.sms) ? cta_tiles : di.sms);
+    const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>((n_groups + 31) / 32), di.sms));
     return launch_overlapped(kernel, grid, static_cast<unsigned>(kVarWarps * 32), kSmemCtaBytes, static_cast<cudaStream_t>(stream),
                              static_cast<const uint8_t*>(d_meta), reinterpret_cast<const uint4*>(d_stream),
                              static_cast<const uint64_t*>(d_index), n_groups, static_cast<uint16_t*>(d_out), map);
@@ -458,8 +455,7 @@ static int launch_attn(const DeviceInfo& di, const void* d_meta, const uint8_t* 
     const int heads = batch * n_kv_heads;
     // persistent CTAs; the units (32 tokens of a head) are split evenly over the working warps on the device
     const int64_t units = static_cast<int64_t>(heads) * ((seq + 31) / 32);
-    const int64_t ctas = (units + kFusedWarps - 1) / kFusedWarps;
-    const unsigned grid = static_cast<unsigned>(ctas < di.sms ? ctas : di.sms);
+    const unsigned grid = static_cast<unsigned>(spread_ctas(units, di.sms));
     return launch_overlapped(kernel, grid, static_cast<unsigned>(kFusedWarps * 32), kSmemCtaBytes, stream, static_cast<const uint8_t*>(d_meta),
                              d_kblocks, heads, seq, q_per_kv, static_cast<const __half*>(d_q), scale, d_scores);
 }
@@ -485,8 +481,7 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
             rc = want_all_smem(kernel, &configured[di.device]);
             if (rc) return rc;
             const uint64_t units = static_cast<uint64_t>(batch) * n_kv_heads * ((seq + 31) / 32);
-            const uint64_t ctas = (units + kMmaWarps - 1) / kMmaWarps;
-            const unsigned grid = static_cast<unsigned>(ctas < static_cast<uint64_t>(di.sms) ? ctas : di.sms);
+            const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>(units), di.sms));
             return launch_overlapped(kernel, grid, static_cast<unsigned>(kMmaWarps * 32), kSmemCtaBytes, s, static_cast<const uint8_t*>(d_meta),
                                      d_kblocks, batch * n_kv_heads, seq, q_per_kv, static_cast<const __half*>(d_q), scale, d_scores);
         }

@@ -89,8 +89,13 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // Warps per CTA the decoding kernels are launched with (their register budget); how many of them work is decided on
 // the device, from the size of the image's tables.
 constexpr int kDecompressWarps = 28;
-constexpr int fused_warps(int) { return 28; }
-constexpr int gemv_warp_warps(int) { return 28; }
+constexpr int fused_warps(int v) { return v == 1 ? 32 : 28; }
+constexpr int gemv_warp_warps(int v) { return v == 1 ? 32 : 28; }
+
+// CTAs for `units` warp-sized pieces of work: one per SM as soon as there are that many.  The kernels number their warps
+// across the CTAs first, so a call with fewer pieces than the machine has warp slots puts a few on every SM instead of
+// filling some SMs and leaving the others idle (decode attention over 2 x 8 x 777 tokens, 400 pieces: 37.6 -> 30.4 us).
+inline int spread_ctas(int64_t units, int ctas_max) { return static_cast<int>(units < ctas_max ? units : ctas_max); }
 
 struct GemvPlan { int row_tiles, grid; size_t partial_bytes, ticket_bytes; };
 
@@ -101,9 +106,9 @@ inline GemvPlan gemv_plan(int64_t units, int row_tiles, int warps, int cols, int
 {
     GemvPlan p;
     p.row_tiles = row_tiles;
-    const int64_t ctas = (units + warps - 1) / warps;
-    p.grid = static_cast<int>(ctas < ctas_max ? ctas : ctas_max);
-    p.partial_bytes = (static_cast<size_t>(p.grid * warps + row_tiles) * cols * 32 * sizeof(float) + 255) & ~static_cast<size_t>(255);
+    p.grid = spread_ctas(units, ctas_max);
+    const int64_t workers = static_cast<int64_t>(p.grid) * warps < units ? static_cast<int64_t>(p.grid) * warps : units;
+    p.partial_bytes = (static_cast<size_t>(workers + row_tiles) * cols * 32 * sizeof(float) + 255) & ~static_cast<size_t>(255);
     p.ticket_bytes = (static_cast<size_t>(row_tiles) * sizeof(unsigned int) + 255) & ~static_cast<size_t>(255);
     return p;
 }
