@@ -594,6 +594,9 @@ extern "C" int ecco_act_compress(const void* d_x_fp16, uint64_t n_groups, uint8_
 }
 
 
+// calls of at least this many groups: eight lanes per group and tables in shared memory (see the kernel)
+constexpr uint64_t kKvManyGroups = 16384;
+
 extern "C" int ecco_kv_compress(const void* d_meta, const void* d_x_fp16, uint64_t n_groups, uint8_t* d_blocks, void* stream)
 {
     if (n_groups == 0) return ECCO_OK;
@@ -603,9 +606,20 @@ extern "C" int ecco_kv_compress(const void* d_meta, const void* d_x_fp16, uint64
     DeviceInfo di;
     int rc = device_info(&di);
     if (rc) return rc;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (n_groups >= kKvManyGroups) {
+        static thread_local bool configured[64] = {};
+        if (!configured[di.device]) {
+            rc = set_smem(ecco_kv_compress_many_kernel, sizeof(KvManySmem));
+            if (rc) return rc;
+            configured[di.device] = true;
+        }
+        return launch_overlapped(ecco_kv_compress_many_kernel, static_cast<unsigned>(spread_ctas(static_cast<int64_t>((n_groups + 3) / 4), di.sms)),
+                                 static_cast<unsigned>(kKvManyWarps * 32), sizeof(KvManySmem), s, static_cast<const uint8_t*>(d_meta),
+                                 static_cast<const __half*>(d_x_fp16), n_groups, d_blocks);
+    }
     const uint64_t ctas = (n_groups + kKvWarps - 1) / kKvWarps;
     const uint64_t cap = static_cast<uint64_t>(di.sms) * 8;
     return launch_overlapped(ecco_kv_compress_kernel, static_cast<unsigned>(ctas < cap ? ctas : cap), static_cast<unsigned>(kKvWarps * 32), 0,
-                             static_cast<cudaStream_t>(stream), static_cast<const uint8_t*>(d_meta), static_cast<const __half*>(d_x_fp16),
-                             n_groups, d_blocks);
+                             s, static_cast<const uint8_t*>(d_meta), static_cast<const __half*>(d_x_fp16), n_groups, d_blocks);
 }

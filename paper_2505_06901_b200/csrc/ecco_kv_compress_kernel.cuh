@@ -219,4 +219,319 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The same encoder for many groups: eight lanes per group, sixteen values per lane, four groups per warp, so that what is
+// done once per group or once per reduction costs a quarter of the instructions.  Decisions are those of the kernel above;
+// what makes them cheap:
+//  * min / max of the normalised values = normalised min / max (division by the scale is monotone): packed fp16 extremes,
+//    two divisions per group.
+//  * the pattern with the least fp32 fitness wins unless another comes within 2^-20 of it; only then are the fp64 scores formed.
+//  * nearest centroid = number of midpoints below the value.  A table per pattern says for 256 cells of [-1, 1) how many
+//    midpoints lie below the cell and how many inside, so a value is compared with one midpoint or none; the value is x times the
+//    scale's reciprocal, and where that comes within 2^-21 of a midpoint the exact division and fp64 distances decide.
+//  * the four codebooks' lengths are bytes of one word, summed together.
+//  * a lane joins its sixteen codewords into one string of at most 128 bits in registers and ORs five words into the block.
+// Bound by the issue slots (74 % busy, ncu): 349 warp instructions per group against 735 of the kernel above; two calls of
+// 131 072 groups take 109.7 us against 218.5.  Making the tables costs a call 3 us, which is what the smaller instruction count
+// saves at about 16 000 groups (two calls of 8192: 26.5 against 19.5 us, of 16 384: 30.6 against 31.3): fewer go to the kernel above.
+// ---------------------------------------------------------------------------------------------
+constexpr int kKvManyWarps = 32;
+constexpr int kKvCells = 256;
+constexpr float kCellWidth = 1.0f / 127.5f;
+struct KvManySmem {
+    uint8_t cell[kMaxPatterns * kKvCells];                 // midpoints below the cell, | 0x80 if it holds several; rows of 256 bytes
+    uint16_t pat[kMaxPatterns * 16];
+    uint16_t enc[kMaxPatterns * kCodebooks * kSymbols];    // length | codeword in stream order << 8
+    uint16_t kp[kMaxPatterns];
+    uint32_t len4[kMaxPatterns * kSymbols];                // code lengths of a symbol in the four codebooks, one per byte
+    float mid[kMaxPatterns * 16];                          // midpoints of neighbouring centroids (14 per pattern)
+    float2 ends[kMaxPatterns];                             // first and last centroid
+    uint4 x[kKvManyWarps][64];                             // the warp's four groups, fp16 [4][128]
+    uint32_t blk[kKvManyWarps][64];                        // their blocks
+};
+
+__device__ __forceinline__ uint32_t kv_key(uint32_t half, int pos) { return ((half & 0x7fffu) << 7) | static_cast<uint32_t>(127 - pos); }
+
+__global__ void __launch_bounds__(kKvManyWarps * 32, 1)
+ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* __restrict__ d_x, uint64_t n_groups, uint8_t* __restrict__ d_blocks)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    KvManySmem& sm = *reinterpret_cast<KvManySmem*>(smem);
+    const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5, sub = lane & 7, grp = lane >> 3;
+    constexpr unsigned full = 0xffffffffu;
+    release_dependents();
+    const DevHeader* hdr = reinterpret_cast<const DevHeader*>(d_meta);
+    const int S = min(max(__ldg(&hdr->S), 1), kMaxPatterns);
+    const float T = __ldg(&hdr->T), invT = 1.0f / T;     // both exact powers of two
+    // tables: from the image, which is host-written and may be read before the wait on the previous kernel
+    for (int i = tid; i < static_cast<int>(kPatternBytes / 16); i += kKvManyWarps * 32) reinterpret_cast<uint4*>(sm.pat)[i] = __ldg(reinterpret_cast<const uint4*>(d_meta + kOffPattern) + i);
+    for (int i = tid; i < static_cast<int>(kEncCbBytes / 16); i += kKvManyWarps * 32) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(d_meta + kOffEncCb) + i);   // bytes of every entry swapped
+        reinterpret_cast<uint4*>(sm.enc)[i] = make_uint4(prmt(v.x, 0, 0x2301u), prmt(v.y, 0, 0x2301u), prmt(v.z, 0, 0x2301u), prmt(v.w, 0, 0x2301u));
+    }
+    for (int i = tid; i < static_cast<int>(kEncKpBytes / 16); i += kKvManyWarps * 32) reinterpret_cast<uint4*>(sm.kp)[i] = __ldg(reinterpret_cast<const uint4*>(d_meta + kOffEncKp) + i);
+    __syncthreads();
+    auto centroid = [&](int k, int j) { return __half2float(__ushort_as_half(sm.pat[k * 16 + j])); };
+    for (int i = tid; i < kMaxPatterns * kSymbols; i += kKvManyWarps * 32) {
+        const int k = i >> 4, s = i & 15;
+        uint32_t v = 0;
+#pragma unroll
+        for (int h = 0; h < kCodebooks; ++h) v |= static_cast<uint32_t>(sm.enc[(k * kCodebooks + h) * kSymbols + s] & 0xffu) << (8 * h);
+        // a centroid equal to the one before it never wins: its symbol stands for the first of them
+        int f = s;
+        while (f > 0 && f < kCentroids && centroid(k, f - 1) == centroid(k, f)) --f;
+        if (f != s) {
+            v = 0;
+#pragma unroll
+            for (int h = 0; h < kCodebooks; ++h) {
+                const uint16_t e = sm.enc[(k * kCodebooks + h) * kSymbols + f];
+                v |= static_cast<uint32_t>(e & 0xffu) << (8 * h);
+                sm.enc[(k * kCodebooks + h) * kSymbols + s] = e;
+            }
+        }
+        sm.len4[i] = v;
+        sm.mid[i] = s < kCentroids - 1 ? 0.5f * (centroid(k, s) + centroid(k, s + 1)) : INFINITY;
+        if (s == 0) sm.ends[k] = make_float2(centroid(k, 0), centroid(k, kCentroids - 1));
+    }
+    __syncthreads();
+    // cell c holds the values with |127.5 (u + 1) - c| <= 1/2 and a little more on both sides (the edge cells all that is beyond);
+    // a thread fills sixteen cells of a row, advancing through the ascending midpoints
+    for (int i = tid; i < kMaxPatterns * kKvCells / 16; i += kKvManyWarps * 32) {
+        const float* const m = sm.mid + (i / (kKvCells / 16)) * 16;
+        int c = (i % (kKvCells / 16)) * 16, below = 0, upto = 0;
+        uint32_t out[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < 16; ++q, ++c) {
+            if (c > 0) while (below < kCentroids - 1 && m[below] < (static_cast<float>(c) - 0.51f) * kCellWidth - 1.0f) ++below;
+            while (upto < kCentroids - 1 && (c == kKvCells - 1 || m[upto] <= (static_cast<float>(c) + 0.51f) * kCellWidth - 1.0f)) ++upto;
+            out[q >> 2] |= static_cast<uint32_t>(below | (upto - below > 1 ? 0x80 : 0)) << (8 * (q & 3));
+        }
+        reinterpret_cast<uint4*>(sm.cell)[i] = make_uint4(out[0], out[1], out[2], out[3]);
+    }
+    __syncthreads();
+    dependency_wait();                                     // x and the blocks: after the previous kernel of the stream
+
+    auto fp8 = [&](float v) { return static_cast<uint32_t>(__nv_cvt_float_to_fp8(v * invT, __NV_SATFINITE, __NV_E4M3)); };
+    uint16_t* const xs = reinterpret_cast<uint16_t*>(sm.x[warp]) + grp * kGroup;          // this group's values
+    uint32_t* const blk = sm.blk[warp] + grp * 16;
+    const uint64_t n_units = (n_groups + 3) / 4;
+    for (uint64_t unit = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x; unit < n_units; unit += static_cast<uint64_t>(gridDim.x) * kKvManyWarps) {
+        const uint64_t g = min(unit * 4 + grp, n_groups - 1);            // past the end: the last group again, not stored
+        uint32_t h[8];                                     // x is 16-byte aligned: two loads
+        {
+            const uint4* const src = reinterpret_cast<const uint4*>(d_x + g * kGroup + sub * 16);
+            const uint4 a = __ldcg(src), b = __ldcg(src + 1);
+            h[0] = a.x; h[1] = a.y; h[2] = a.z; h[3] = a.w; h[4] = b.x; h[5] = b.y; h[6] = b.z; h[7] = b.w;
+        }
+        uint4* const mine = reinterpret_cast<uint4*>(xs) + sub * 2;
+        mine[0] = make_uint4(h[0], h[1], h[2], h[3]);
+        mine[1] = make_uint4(h[4], h[5], h[6], h[7]);
+        blk[sub * 2] = 0;
+        blk[sub * 2 + 1] = 0;
+        auto group_max = [&](uint32_t v) {
+            v = max(v, __shfl_xor_sync(full, v, 1));
+            v = max(v, __shfl_xor_sync(full, v, 2));
+            return max(v, __shfl_xor_sync(full, v, 4));
+        };
+        // sorter: abs-max, first index on ties (key: |x|, then low index first)
+        uint32_t best = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) best = max(best, max(kv_key(h[i], sub * 16 + 2 * i), kv_key(h[i] >> 16, sub * 16 + 2 * i + 1)));
+        best = group_max(best);
+        const int pstar = 127 - static_cast<int>(best & 127u);
+        __syncwarp();
+        const float xp = __half2float(__ushort_as_half(xs[pstar]));
+        __syncwarp();
+        if (sub == 0) xs[pstar] = 0x7e00u;                 // NaN: out of the extremes and, at the end, the largest key
+        __syncwarp();
+        {
+            const uint4 a = mine[0], b = mine[1];
+            h[0] = a.x; h[1] = a.y; h[2] = a.z; h[3] = a.w; h[4] = b.x; h[5] = b.y; h[6] = b.z; h[7] = b.w;
+        }
+        const uint32_t qs = fp8(xp);
+        const float scale = fabsf(fp8_to_float(qs) * T);
+        // extremes of the rest: (min, -max) in one packed number; a lane whose sixteen values are fine gives no NaN
+        auto as_h2 = [](uint32_t v) { return *reinterpret_cast<const __half2*>(&v); };
+        __half2 mn = as_h2(h[0]), mx = as_h2(h[0]);
+#pragma unroll
+        for (int i = 1; i < 8; ++i) { mn = __hmin2(mn, as_h2(h[i])); mx = __hmax2(mx, as_h2(h[i])); }
+        __half2 ext = __halves2half2(__hmin(__low2half(mn), __high2half(mn)), __hneg(__hmax(__low2half(mx), __high2half(mx))));
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) ext = __hmin2(ext, __shfl_xor_sync(full, ext, o));
+        const float lo = scale == 0.0f ? 0.0f : __fdiv_rn(__low2float(ext), scale), hi = scale == 0.0f ? 0.0f : __fdiv_rn(-__high2float(ext), scale);
+        // pattern selector: min/max fitness, eight patterns per lane
+        float low = INFINITY, sc[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int k = sub + 8 * r;
+            const float2 e = sm.ends[k];
+            const float a = e.x - lo, b = e.y - hi;
+            sc[r] = k < S ? a * a + b * b : INFINITY;
+            low = fminf(low, sc[r]);
+        }
+        low = fminf(low, __shfl_xor_sync(full, low, 1));
+        low = fminf(low, __shfl_xor_sync(full, low, 2));
+        low = fminf(low, __shfl_xor_sync(full, low, 4));
+        uint32_t cand = 0;                                 // patterns of this lane that may be the best
+        const float limit = fmaf(low, 1.00000095367431640625f, 1e-30f);      // 1 + 2^-20
+#pragma unroll
+        for (int r = 0; r < 8; ++r) cand |= (sc[r] <= limit && sub + 8 * r < S ? 1u : 0u) << r;
+        int kp;
+        {
+            const uint32_t with = (__ballot_sync(full, cand != 0) >> (grp * 8)) & 0xffu;
+            const bool clear = __popc(with) == 1 && (__popc(cand) <= 1);
+            if (__all_sync(full, clear)) {
+                kp = __shfl_sync(full, sub + 8 * (__ffs(cand) - 1), grp * 8 + __ffs(with) - 1);
+            } else {                                       // fp64 scores of the candidates; a non-negative double orders like its bits
+                uint64_t sb = ~0ull;
+                uint32_t id = kMaxPatterns - 1;
+                for (uint32_t c = cand; c; c &= c - 1u) {
+                    const int k = sub + 8 * (__ffs(c) - 1);
+                    const float2 e = sm.ends[k];
+                    const double a = static_cast<double>(e.x) - static_cast<double>(lo), b = static_cast<double>(e.y) - static_cast<double>(hi);
+                    const uint64_t v = static_cast<uint64_t>(__double_as_longlong(__dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b))));
+                    if (v < sb) { sb = v; id = static_cast<uint32_t>(k); }
+                }
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    const uint64_t v = __shfl_xor_sync(full, sb, o);
+                    const uint32_t k = __shfl_xor_sync(full, id, o);
+                    if (v < sb || (v == sb && k < id)) { sb = v; id = k; }
+                }
+                kp = static_cast<int>(id);
+            }
+        }
+        // value mappers
+        const float inv = scale == 0.0f ? 0.0f : __fdiv_rn(1.0f, scale);
+        const uint32_t cells = smem_u32(sm.cell) + kp * kKvCells, mids = smem_u32(sm.mid) + kp * 64, lens = smem_u32(sm.len4) + kp * 64;
+        auto cell_of = [&](float u) {                      // NaN: cell 0
+            const uint32_t at = __float_as_uint(fmaf(__saturatef(fmaf(u, 0.5f, 0.5f)), 255.0f, 12582912.0f)) & (kKvCells - 1);
+            uint32_t e;
+            asm("ld.shared.u8 %0, [%1];" : "=r"(e) : "r"(cells | at));
+            return e;
+        };
+        auto shared_float = [](uint32_t a) { float v; asm("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a)); return v; };
+        auto shared_word = [](uint32_t a) { uint32_t v; asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a)); return v; };
+        constexpr float kBand = 4.76837158203125e-7f;      // 2^-21: more than x * (1 / scale) is off by for values up to 1.5
+        uint32_t syms[2] = {0, 0}, l4 = 0, flags = 0;      // nibbles of values 0..7 and 8..15, the first one highest
+        bool near = lo < -1.5f || hi > 1.5f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const float u = (j & 1 ? __high2float(as_h2(h[j >> 1])) : __low2float(as_h2(h[j >> 1]))) * inv;
+            const uint32_t e = cell_of(u);
+            flags |= e;
+            uint32_t s = e & 15u;
+            const float d = u - shared_float(mids + s * 4);   // without a midpoint in the cell this is the next one above: no step
+            near = near || fabsf(d) <= kBand;
+            if (d > 0.0f) ++s;
+            syms[j >> 3] = syms[j >> 3] * 16u + s;
+            l4 += shared_word(lens + s * 4);
+        }
+        if (warp_any(near || (flags & 0x80u))) {
+            // the values in question as defined: exact quotient, fp64 distances, ties to the first centroid
+            for (int j = 0; j < 16; ++j) {
+                const float x = __half2float(__ushort_as_half(xs[sub * 16 + j]));
+                const uint32_t e = cell_of(x * inv);
+                if (!(fabsf(x) <= 65504.0f)) continue;     // the abs-max itself
+                if (!(e & 0x80u) && fabsf(x * inv) <= 1.5f && !(fabsf(x * inv - shared_float(mids + (e & 15u) * 4)) <= kBand)) continue;
+                const float u = scale == 0.0f ? 0.0f : __fdiv_rn(x, scale);
+                int below = 0;
+                for (int i = 0; i < kCentroids; ++i) below += centroid(kp, i) <= u;
+                const int a = max(below - 1, 0), b = min(below, kCentroids - 1);
+                const double da = static_cast<double>(u) - static_cast<double>(centroid(kp, a)), db = static_cast<double>(u) - static_cast<double>(centroid(kp, b));
+                const uint32_t s = static_cast<uint32_t>(__dmul_rn(db, db) < __dmul_rn(da, da) ? b : a), sh = 28u - 4u * (j & 7);
+                uint32_t& w = j < 8 ? syms[0] : syms[1];
+                l4 += sm.len4[kp * 16 + s] - sm.len4[kp * 16 + ((w >> sh) & 15u)];
+                w = (w & ~(15u << sh)) | (s << sh);
+            }
+        }
+        if ((pstar >> 4) == sub) {                         // the NaN has counted as symbol 0
+            l4 += sm.len4[kp * 16 + 15] - sm.len4[kp * 16];
+            const uint32_t w = 15u << (28u - 4u * (pstar & 7));
+            if (pstar & 8) syms[1] |= w; else syms[0] |= w;
+        }
+        // four encoders: total length per codebook, the shortest wins (ties to the lower id)
+        uint32_t t02 = l4 & 0x00ff00ffu, t13 = (l4 >> 8) & 0x00ff00ffu;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) { t02 += __shfl_xor_sync(full, t02, o); t13 += __shfl_xor_sync(full, t13, o); }
+        const uint32_t tot[4] = {t02 & 0xffffu, t13 & 0xffffu, t02 >> 16, t13 >> 16};
+        int hf = 0;
+        uint32_t shortest = tot[0];
+#pragma unroll
+        for (int hh = 1; hh < 4; ++hh)
+            if (tot[hh] < shortest) { shortest = tot[hh]; hf = hh; }
+        // the lane's sixteen codewords as one bit string
+        const uint16_t* const enc = sm.enc + (kp * kCodebooks + hf) * kSymbols;
+        uint64_t half_bits[2];
+        uint32_t half_len[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            uint32_t bits4[2], len4[2];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                uint32_t e[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) e[j] = enc[(syms[q] >> (28 - 4 * (p * 4 + j))) & 15u];
+                // an entry's low five bits are its length: it is the shift of what follows
+                const uint32_t b01 = (e[0] >> 8) | __funnelshift_l(0u, e[1] >> 8, e[0]), b23 = (e[2] >> 8) | __funnelshift_l(0u, e[3] >> 8, e[2]);
+                const uint32_t l01 = (e[0] + e[1]) & 0xffu;
+                bits4[p] = b01 | __funnelshift_l(0u, b23, l01);
+                len4[p] = l01 + ((e[2] + e[3]) & 0xffu);
+            }
+            half_bits[q] = static_cast<uint64_t>(bits4[0]) | (static_cast<uint64_t>(bits4[1]) << len4[0]);
+            half_len[q] = len4[0] + len4[1];
+        }
+        // at most 64 bits each: the second string begins at half_len[0]
+        uint64_t s0 = half_bits[0], s1 = 0;
+        if (half_len[0] < 64) { s0 |= half_bits[1] << half_len[0]; s1 = half_len[0] ? half_bits[1] >> (64 - half_len[0]) : 0; }
+        else s1 = half_bits[1];
+        const uint32_t lane_bits = half_len[0] + half_len[1];
+        uint32_t incl = lane_bits;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(full, incl, o, 8);
+            if (sub >= o) incl += v;
+        }
+        const uint32_t kpe = sm.kp[kp], kp_len = kpe >> 12;
+        const uint32_t end_bit = kHeaderBits + kp_len + shortest;
+        const uint32_t pos = kHeaderBits + kp_len + incl - lane_bits, off = pos & 31u, w0 = pos >> 5;
+        // pack / clip: what lies past bit 512 is dropped, so the first codeword that crosses it is truncated
+        if (sub == 0) atomicOr(&blk[0], qs | (static_cast<uint32_t>(hf) << 8) | ((kpe & 0xfffu) << kHeaderBits));
+        {
+            const uint32_t q[4] = {static_cast<uint32_t>(s0), static_cast<uint32_t>(s0 >> 32), static_cast<uint32_t>(s1), static_cast<uint32_t>(s1 >> 32)};
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const uint32_t v = __funnelshift_l(i ? q[i - 1] : 0u, i < 4 ? q[i] : 0u, off);
+                if (w0 + i < 16u) atomicOr(&blk[w0 + i], v);
+            }
+        }
+        // outliers: the next-largest |x| (ties: lower index), as many 15-bit slots as fit, at most 16
+        const int n_pad = end_bit <= static_cast<uint32_t>(kBlockBits) ? min(kMaxPads, static_cast<int>((kBlockBits - end_bit) / kPadBits)) : 0;
+        const int n_max = __reduce_max_sync(full, n_pad);
+        if (n_max > 0) {
+            uint32_t key[16];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { key[2 * i] = kv_key(h[i], sub * 16 + 2 * i); key[2 * i + 1] = kv_key(h[i] >> 16, sub * 16 + 2 * i + 1); }
+            // keys are distinct and below 2^23: seen from `top` (mod 2^32) the largest smaller key is the largest number
+            uint32_t top = kv_key(0x7e00u, pstar);         // the abs-max itself (its NaN) is out
+            for (int p = 0; p < n_max; ++p) {
+                uint32_t next = 0;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) next = max(next, key[i] - top);
+                top += group_max(next);
+                if (p < n_pad && sub == 0) {
+                    const uint32_t loc = 127u - (top & 127u);
+                    const uint32_t field = loc | (fp8(__half2float(__ushort_as_half(xs[loc]))) << 7);
+                    const uint32_t bp = kBlockBits - kPadBits * (p + 1), w = bp >> 5, o = bp & 31u;
+                    atomicOr(&blk[w], field << o);
+                    if (o + kPadBits > 32u) atomicOr(&blk[w + 1], field >> (32u - o));
+                }
+            }
+        }
+        __syncwarp();
+        if (unit * 4 + grp < n_groups) reinterpret_cast<uint2*>(d_blocks + g * kBlockBytes)[sub] = make_uint2(blk[sub * 2], blk[sub * 2 + 1]);
+        __syncwarp();
+    }
+}
+
 }  // namespace

@@ -820,6 +820,45 @@ def test_kv_compress_edge_groups_and_s16(B, eo, kv_small, synth):
     assert_blocks_equal(gpu_kv_compress(B, lib_meta_from_oracle(B, skew), xs), want)
 
 
+@pytest.mark.parametrize("kind,n_groups", [("calibrated", 16383), ("calibrated", 16384), ("s16", 16385), ("equal centroids", 16386),
+                                           ("dense centroids", 16387), ("wide centroids", 16384), ("skewed codes", 16385)])
+def test_kv_compress_of_many_groups_matches_the_host_encoder(B, eo, kv_small, synth, kind, n_groups):
+    """Calls on both sides of the size from which eight lanes share a group, ragged in the last four groups, on groups that
+    decide at the edges: values at midpoints of centroids, ties, zeros, one value only, saturating and subnormal scales,
+    patterns with equal centroids, with several midpoints per table cell and with centroids far outside [-1, 1]."""
+    rng = np.random.Generator(np.random.PCG64(n_groups))
+    if kind == "calibrated":
+        om = kv_small["meta"]
+    elif kind == "s16":
+        om = eo.calibrate(synth.kv_cache(1, 4, 512, 2003, 3003), S=16, H=4, seed=3, select=eo.SELECT_MINMAX)
+    else:
+        om = make_meta(eo, skew_lens, S=7, e=-3, seed=5)
+        for k in range(om.S):
+            p = np.sort(rng.uniform(-1, 1, 15))
+            if kind == "equal centroids":
+                p[3:6], p[9] = p[3], p[10]
+            elif kind == "dense centroids":
+                p[2:12] = p[2] + np.arange(10) * 0.0007
+            elif kind == "wide centroids":
+                p *= 4.0
+            for j, c in enumerate(np.sort(p.astype(np.float16)).view(np.uint16)):
+                om.pattern[k][j] = int(c)
+    lm = lib_meta_from_oracle(B, om)
+    pat = om.patterns()[: om.S].astype(np.float64)
+    x = synth.kv_cache(1, 4, (n_groups + 3) // 4, 41, 42).reshape(-1, 128)[:n_groups].copy()
+    for g in range(0, n_groups, 11):                       # values at (or next to) midpoints of a pattern, abs-max a power of two
+        p = pat[g % om.S]
+        mids = 0.5 * (p[1:] + p[:-1])
+        x[g] = (rng.choice(mids, 128) * 4.0).astype(np.float16)
+        x[g, rng.integers(128)] = 4.0
+    x[1], x[2], x[3], x[5] = 0, 0.5, 2.0 ** -24, np.where(np.arange(128) % 2 == 0, 60000.0, -60000.0)
+    x[6] = (rng.standard_normal(128) * 3000).clip(-60000, 60000).astype(np.float16)
+    x[7] = (rng.standard_normal(128) * 1e-6).astype(np.float16)
+    x[8, :] = rng.choice(np.array([-2.0, 0.0, 2.0], dtype=np.float16), 128)
+    want, _ = B.ecco_encode_host(lm, x, B.SELECT_MINMAX | B.KEEP_EXPONENT)
+    assert_blocks_equal(gpu_kv_compress(B, lm, x), want)
+
+
 def test_kv_compress_full_size_round_trip(B, eo, W, synth):
     """cfg 3 K cache: GPU-compressed blocks equal the host encoder's, and decompress to the same fp16."""
     (t,) = W.config3(which=("K",), keep_source=True)
