@@ -249,11 +249,21 @@ def _ptr(t) -> int:
     return t.data_ptr()
 
 
-def _stream(stream) -> int:
-    if stream is None:
-        import torch
+# The current device's current stream without building a torch.cuda.Stream for it: the object takes 3.3 us of host time per
+# call, about half of what a small call costs altogether.
+_current_raw_stream = None
 
-        return torch.cuda.current_stream().cuda_stream
+
+def _stream(stream) -> int:
+    global _current_raw_stream
+    if stream is None:
+        if _current_raw_stream is None:
+            import torch
+
+            torch.cuda.init()
+            raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+            _current_raw_stream = lambda: raw(device())  # noqa: E731
+        return _current_raw_stream()
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 

@@ -79,6 +79,19 @@ def check_fused(got, ref, refabs, label="fused"):
     assert plain <= TOL, (label, plain)
 
 
+def test_calls_without_a_stream_go_to_the_current_one(B):
+    """On the default stream, inside a stream context, after it and from another thread (whose current stream is its own)."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    side = torch.cuda.Stream()
+    assert B._stream(None) == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(side):
+        assert B._stream(None) == side.cuda_stream
+        with ThreadPoolExecutor(1) as ex:
+            assert ex.submit(lambda: B._stream(None) == torch.cuda.current_stream().cuda_stream).result()
+    assert B._stream(None) == torch.cuda.current_stream().cuda_stream
+
+
 # ------------------------------------------------------------------ decompress
 @pytest.mark.parametrize("e", [-32, -16, -15, 0, 7, 8, 16])
 def test_decompress_every_scale_byte_at_the_edges_of_the_packed_product(B, eo, e):
