@@ -30,9 +30,8 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
     __shared__ __align__(16) uint16_t kp_s[kMaxPatterns];
     __shared__ uint32_t blk_s[kKvWarps][16];
     const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
-    dependency_wait();                                     // the previous kernel of the stream has completed
     release_dependents();
-    {
+    {                                                      // the image is host-written: read before the wait on the previous kernel
         const uint4* src_p = reinterpret_cast<const uint4*>(d_meta + kOffPattern);
         for (int i = tid; i < static_cast<int>(kPatternBytes / 16); i += kKvWarps * 32) reinterpret_cast<uint4*>(pat_s)[i] = src_p[i];
         const uint4* src_e = reinterpret_cast<const uint4*>(d_meta + kOffEncCb);
@@ -40,6 +39,7 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
         const uint4* src_k = reinterpret_cast<const uint4*>(d_meta + kOffEncKp);
         for (int i = tid; i < static_cast<int>(kEncKpBytes / 16); i += kKvWarps * 32) reinterpret_cast<uint4*>(kp_s)[i] = src_k[i];
     }
+    dependency_wait();                                     // x and the blocks: after the previous kernel of the stream
     __syncthreads();
     const DevHeader* hdr = reinterpret_cast<const DevHeader*>(d_meta);
     const int S = hdr->S;
