@@ -573,9 +573,8 @@ extern "C" int ecco_act_decompress(const uint8_t* d_blocks, uint64_t n_groups, v
     int rc = device_info(&di);
     if (rc) return rc;
     const uint64_t n_chunks = n_groups * 4;
-    ecco_act_decompress_kernel<<<act_grid(n_chunks, di), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        reinterpret_cast<const uint4*>(d_blocks), n_chunks, static_cast<uint4*>(d_out_fp16));
-    return check_launch();
+    return launch_overlapped(ecco_act_decompress_kernel, static_cast<unsigned>(act_grid(n_chunks, di)), static_cast<unsigned>(kActThreads), 0,
+                             static_cast<cudaStream_t>(stream), reinterpret_cast<const uint4*>(d_blocks), n_chunks, static_cast<uint4*>(d_out_fp16));
 }
 
 extern "C" int ecco_act_compress(const void* d_x_fp16, uint64_t n_groups, uint8_t* d_blocks, void* stream)
@@ -588,9 +587,8 @@ extern "C" int ecco_act_compress(const void* d_x_fp16, uint64_t n_groups, uint8_
     int rc = device_info(&di);
     if (rc) return rc;
     const uint64_t n_chunks = n_groups * 4;
-    ecco_act_compress_kernel<<<act_grid(n_chunks, di), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint4*>(d_x_fp16), n_chunks, reinterpret_cast<uint4*>(d_blocks));
-    return check_launch();
+    return launch_overlapped(ecco_act_compress_kernel, static_cast<unsigned>(act_grid(n_chunks, di)), static_cast<unsigned>(kActThreads), 0,
+                             static_cast<cudaStream_t>(stream), static_cast<const uint4*>(d_x_fp16), n_chunks, reinterpret_cast<uint4*>(d_blocks));
 }
 
 
