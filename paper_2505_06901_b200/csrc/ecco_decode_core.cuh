@@ -7,13 +7,14 @@
 //  * Sixteen dequantised values per lane are 32 bytes.  They stay in eight registers as two byte planes (low bytes and
 //    high bytes in rank order) and eight ranks are turned into eight fp16 values by byte permutes (map_ranks): no value
 //    table in shared memory, hence one wavefront per symbol and 1-2 KB per warp less than a table lookup per value.
-//  * Eight symbols per step from one 64-bit window: three words per refill, four pair-table lookups, one escape vote per
-//    two lookups and one end-of-stream vote per step.
+//  * Eight symbols per step from one 64-bit window: three words per refill, four pair-table lookups, one escape branch per
+//    two lookups and one end-of-stream vote per step.  The escapes are plain branches: a warp vote in front of them costs more
+//    instructions per step than the branch saves (layer of 7B shape 128.5 -> 123.2 us, batch-1 products 161.7 -> 152.4 us).
 //  * The sixteen values come from a table of centroids that is already in rank order for every codebook
 //    (build_rank_tables, made once per CTA from the staged image): two 16-byte loads and eight packed multiplications.
-// Per symbol of a warp, on 1 212 416 weight groups (ncu): 15.1 instructions, 8.1 of them on the integer pipe, and 4.1
-// wavefronts, against 16.8, 8.2 and 5.3 with the value table in shared memory and four symbols per step; ecco_decompress over
-// a 7B-shaped layer 138.8 -> 129.9 us, over a [16][8][32768][128] cache 407.4 -> 371.0 us.
+// Against the decoder with the value table in shared memory and four symbols per step (16.8 instructions, 8.2 of them on the
+// integer pipe, and 5.3 wavefronts per symbol of a warp on weights, ncu): ecco_decompress over a 7B-shaped layer 137.5 -> 122.3 us,
+// over a [16][8][32768][128] cache 407.4 -> 351.8 us.
 namespace {
 
 // Shared memory of a CTA: misc words, patterns and codebook records, then the tables of the decode.  The first three fill
@@ -267,7 +268,7 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
         uint32_t x1 = __funnelshift_r(lo, hi, e0);
         uint32_t e1 = lds_pair(g.plut ^ (x1 & g.mask));
         uint32_t n01 = e0 + e1, x2 = __funnelshift_r(lo, hi, n01);
-        if (warp_any((e0 | e1) & 0x8000u)) {
+        if ((e0 | e1) & 0x8000u) {
             if (e0 & 0x8000u) {
                 e0 = resolve(e0, lo);
                 x1 = __funnelshift_r(lo, hi, e0);
@@ -280,7 +281,7 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
         uint32_t e2 = lds_pair(g.plut ^ (x2 & g.mask));
         uint32_t x3 = __funnelshift_r(x2, 0u, e2);
         uint32_t e3 = lds_pair(g.plut ^ (x3 & g.mask));
-        if (warp_any((e2 | e3) & 0x8000u)) {
+        if ((e2 | e3) & 0x8000u) {
             // long codewords: the third pair's window is fetched again, the two pairs may need 33 bits of it
             const uint32_t q = g.p + (n01 & 63u);
             const uint32_t r2 = bits + (q >> 5) * 128;
@@ -335,5 +336,47 @@ __device__ __forceinline__ uint32_t pad_field(uint32_t bits, int j)
     return __funnelshift_r(lds_u32(row), lds_u32(row + 128), pos) & 0x7fffu;
 }
 __device__ __forceinline__ int pads_of(uint32_t end) { return end ? min(kMaxPads, static_cast<int>((kBlockBits - end) / kPadBits)) : 0; }
+
+// The outliers of a warp's 32 groups, one per lane.  The groups of a cache have 37 of them together, but one of them usually has
+// eight, so lanes that walk their own lists leave most of the warp idle; here the lists are joined and every lane takes one
+// outlier, 32 at a time (scores of an [8][32][4096][128] cache with the values' kernel behind them 257.4 -> 250.5 us).  On weights, 16
+// together and two or three at most, walking is the cheaper way (batch-1 products of a layer 162.7 against 164.7 us).  A round ends with a whole group,
+// so that outliers of one group at the same place (which only a corrupt block has) meet in one round and the last one wins.
+//   list     shared address of 64 bytes of scratch
+//   take(slot, owner, field, valid)  called by lane `slot` for an outlier of lane owner's group; not valid: overridden by another
+//   done(first, count)        called by all lanes after a round: slots first .. first + count - 1 were this lane's (count 0: none)
+template <class Take, class Done>
+__device__ __forceinline__ void deal_outliers(uint32_t bits, uint32_t list, int n_pad, Take&& take, Done&& done)
+{
+    constexpr uint32_t kFull = 0xffffffffu;
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t upto = n_pad;                                 // outliers of this lane and those before it
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(kFull, upto, o);
+        if (lane >= static_cast<uint32_t>(o)) upto += v;
+    }
+    const uint32_t total = __shfl_sync(kFull, upto, 31), from = upto - n_pad;
+    for (uint32_t base = 0; base < total;) {               // at least 17 of the rest fit into a round
+        const bool mine = from >= base && upto <= base + 32u;
+        const uint32_t next = __reduce_max_sync(kFull, mine ? upto : 0u);
+        if (mine)
+            for (int j = 0; j < n_pad; ++j) sts_u16(list + (from - base + j) * 2, (lane << 4) | j);
+        __syncwarp();
+        uint32_t owner = 0, field = 0, key = 0x10000u | lane;
+        if (lane < next - base) {
+            const uint32_t w = lds_u16(list + lane * 2);
+            owner = w >> 4;
+            field = pad_field(bits + (owner - lane) * 4, w & 15u);
+            key = (owner << 7) | (field & 127u);
+        }
+        const uint32_t same = __match_any_sync(kFull, key);
+        if (lane < next - base) take(lane, owner, field, ((same >> lane) >> 1) == 0u);
+        __syncwarp();
+        done(from - base, mine ? n_pad : 0);
+        __syncwarp();
+        base = next;
+    }
+}
 
 }  // namespace

@@ -159,12 +159,12 @@ __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// OCP E4M3 byte -> fp32, arithmetically (the all-ones exponent/mantissa code reads as 480)
+// OCP E4M3 byte -> fp32, exactly (the all-ones exponent/mantissa code reads as 480): exponent and mantissa lie as in an fp32 number
+// whose exponent is 120 too small; the subnormals come out right because fp32 has subnormals, too
 __device__ __forceinline__ float fp8_to_float(uint32_t b)
 {
-    uint32_t ex = (b >> 3) & 15u, man = b & 7u;
-    float mag = ex ? __uint_as_float(((ex + 120u) << 23) | (man << 20)) : static_cast<float>(man) * 0.001953125f;
-    return (b & 0x80u) ? -mag : mag;
+    const float mag = __uint_as_float((b & 0x7fu) << 20) * 1.329227995784916e36f;        // 2^120
+    return __uint_as_float(__float_as_uint(mag) | ((b & 0x80u) << 24));
 }
 __device__ __forceinline__ uint32_t f2h_bits(float f) { return static_cast<uint32_t>(__half_as_ushort(__float2half_rn(f))); }
 

@@ -10,10 +10,10 @@ namespace {
 // elements at the same time (one broadcast wavefront per eight symbols and vector) and adds the products with the
 // mixed-precision multiply-add (fp16 x fp16 + fp32, one rounding): no operand is ever converted.
 // Bound by the decode.  Two symbols per lookup and values in registers against one symbol per lookup and a value table in
-// shared memory: the seven products of a 7B-shaped layer at batch 1 193.0 -> 166.0 us, a 4096 x 4096 matrix alone 20.3 -> 18.0 us.
+// shared memory: the seven products of a 7B-shaped layer at batch 1 193.5 -> 149.2 us, a 4096 x 4096 matrix alone 20.4 -> 17.0 us.
 // ---------------------------------------------------------------------------------------------
 // Shared memory of a warp that keeps the decoded ranks of its groups: [27][32] words.  Rows 8..23 are the block's words, rows
-// 24..26 stay zero; the ranks of step i go to row i.  By then the stream has been read past that row: step i leaves the position
+// 24..26 are scratch; the ranks of step i go to row i.  By then the stream has been read past that row: step i leaves the position
 // at bit 11 + 16 (i + 1) at least (eleven header bits, two bits per symbol), so the next window, which starts one bit early, starts in
 // row 8 + (26 + 16 i) / 32 > i or later, and the outlier fields (bits 272 and up) sit in rows 16 and up.
 constexpr uint32_t kRankRows = 8;
@@ -27,6 +27,17 @@ __device__ __forceinline__ void fma_half2(float& acc, uint32_t w, uint32_t x)
         : "+f"(acc)
         : "r"(w), "r"(x));
 }
+// the value of one rank of the group that begins with stream word hdr (see open_lane_group), for a lane that has not opened it
+__device__ __forceinline__ float value_of(uint32_t hdr, uint32_t rank, const DecodeTables& tb, float T)
+{
+    const uint32_t kpe = lds_u16(tb.kp + ((hdr >> (kHeaderBits - 1)) & 0x1ffeu));
+    const uint32_t cb = (kpe & 0xffu) * kCodebooks + ((hdr >> 8) & 3u);
+    const uint32_t top = lds_u32(tb.base + kSmemRec + cb * 16 + 12);
+    const float c = __half2float(__ushort_as_half(static_cast<unsigned short>(lds_u16(cent_row(tb, cb) ^ (rank * 2)))));
+    const float v = __half2float(__float2half_rn(c * (fp8_to_float(hdr & 0x7fu) * T)));
+    return rank == top && (hdr & 0x80u) ? -v : v;
+}
+
 // the value of one rank of the lane's group
 __device__ __forceinline__ float rank_value(const LaneGroup& g, uint32_t rank)
 {
@@ -36,11 +47,13 @@ __device__ __forceinline__ float rank_value(const LaneGroup& g, uint32_t rank)
     return __half2float(__ushort_as_half(static_cast<unsigned short>(prmt(lo, hi, 0x0040u))));
 }
 
+// kDeal: deal_outliers (caches) or every lane its own (weights)
 // decode one group and accumulate its kV dot products against the slice at shared address xs; two partial sums per product
-template <int kV>
+template <int kV, bool kDeal>
 __device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, float (&acc)[kV][2])
 {
     LaneGroup g = open_block(blk, bits, tb, T);
+    if (kDeal) sts_u32(bits + 18 * 128, blk.w[0]);                    // the ranks will lie over the block's first words
     const uint32_t ranks_at = bits - kRankRows * 128;
     const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(g, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
         uint32_t v[4];
@@ -57,22 +70,46 @@ __device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables
             fma_half2(acc[b][1], v[3], x[3]);
         }
     });
-    // outliers replace the mapped value at their location: add (outlier - mapped) * x
-    uint64_t seen_lo = 0, seen_hi = 0;                     // 128-bit "already replaced" mask
-    for (int j = pads_of(end) - 1; j >= 0; --j) {          // the last pad wins on a duplicate location
-        const uint32_t f = pad_field(bits, j);
-        const uint32_t loc = f & 127u;
-        const uint64_t bit = 1ull << (loc & 63u);
-        const bool upper = loc >= 64u;
-        if ((upper ? seen_hi : seen_lo) & bit) continue;
-        if (upper) seen_hi |= bit; else seen_lo |= bit;
-        const float mapped = rank_value(g, (lds_u32(ranks_at + (loc >> 3) * 128) >> ((loc & 7u) * 4)) & 15u);
-        const float outlier = __half2float(__float2half_rn(fp8_to_float(f >> 7) * T));
+    // outliers replace the mapped value at their location: add (outlier - mapped) * x.  Rows 24 and 25 behind the block hold the
+    // list and the products.
+    const int n_pad = pads_of(end);
+    if (!kDeal) {
+        uint32_t seen = 0;                                 // location mod 32 of the outliers so far
+        for (int j = n_pad - 1; j >= 0; --j) {             // the last pad wins on a duplicate location (only corrupt blocks have one)
+            const uint32_t f = pad_field(bits, j);
+            const uint32_t loc = f & 127u, bit = 1u << (loc & 31u);
+            if (seen & bit) {
+                bool replaced = false;
+                for (int k = j + 1; k < n_pad; ++k) replaced = replaced || (pad_field(bits, k) & 127u) == loc;
+                if (replaced) continue;
+            }
+            seen |= bit;
+            const float mapped = rank_value(g, (lds_u32(ranks_at + (loc >> 3) * 128) >> ((loc & 7u) * 4)) & 15u);
+            const float outlier = __half2float(__float2half_rn(fp8_to_float(f >> 7) * T));
 #pragma unroll
-        for (int b = 0; b < kV; ++b) {
-            const float x = __half2float(__ushort_as_half(static_cast<unsigned short>(lds_u16(xs + b * (kGroup * 2) + loc * 2))));
-            acc[b][0] = fmaf(outlier - mapped, x, acc[b][0]);
+            for (int b = 0; b < kV; ++b) {
+                const float x = __half2float(__ushort_as_half(static_cast<unsigned short>(lds_u16(xs + b * (kGroup * 2) + loc * 2))));
+                acc[b][0] = fmaf(outlier - mapped, x, acc[b][0]);
+            }
         }
+    } else if (warp_any(n_pad > 0)) {
+        const uint32_t lane4 = (threadIdx.x & 31u) * 4, bits0 = bits - lane4, list = bits0 + 16 * 128;
+        deal_outliers(bits, list, n_pad, [&](uint32_t slot, uint32_t owner, uint32_t f, bool valid) {
+            const uint32_t loc = f & 127u;
+            const uint32_t rank = (lds_u32(ranks_at - lane4 + owner * 4 + (loc >> 3) * 128) >> ((loc & 7u) * 4)) & 15u;
+            const float mapped = value_of(lds_u32(bits0 + 18 * 128 + owner * 4), rank, tb, T);
+            const float outlier = __half2float(__float2half_rn(fp8_to_float(f >> 7) * T));
+#pragma unroll
+            for (int b = 0; b < kV; ++b) {
+                const float x = __half2float(__ushort_as_half(static_cast<unsigned short>(lds_u16(xs + b * (kGroup * 2) + loc * 2))));
+                const float p = valid ? (outlier - mapped) * x : 0.0f;
+                sts_u32(list + (b ? 0 : 128) + slot * 4, __float_as_uint(p));     // the list has been read
+            }
+        }, [&](uint32_t first, int count) {
+            for (int j = 0; j < count; ++j)
+#pragma unroll
+                for (int b = 0; b < kV; ++b) acc[b][0] += __uint_as_float(lds_u32(list + (b ? 0 : 128) + (first + j) * 4));
+        });
     }
 }
 
@@ -282,7 +319,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
             prefetch_block_l2(gemv_block_ptr(batch, pos, lane));
             load_x(pos);
         }
-        fused_group<kV>(cur, tb, bits, T, xs, acc);
+        fused_group<kV, false>(cur, tb, bits, T, xs, acc);
     }
     flush(cur_j, cur_tile);
 }
@@ -346,7 +383,7 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         float acc[kV][2];
 #pragma unroll
         for (int r = 0; r < kV; ++r) acc[r][0] = acc[r][1] = 0.0f;
-        fused_group<kV>(cur, tb, bits, T, xs, acc);
+        fused_group<kV, true>(cur, tb, bits, T, xs, acc);
         if (t < seq) {
 #pragma unroll
             for (int r = 0; r < kV; ++r)

@@ -448,6 +448,39 @@ def test_attn_scores_match_oracle(B, eo, kv_small, synth, batch, heads, seq, qpk
     check_fused(d_s.cpu().numpy().astype(np.float64), ref, refabs, f"scores q{qpk}")
 
 
+@pytest.mark.parametrize("seq", [1, 31, 32, 33, 200])
+def test_many_outliers_and_repeated_locations(B, eo, synth, seq):
+    """Groups of short codewords with random bits where the outlier fields sit: up to 480 outliers per warp (several rounds of
+    dealing them out), locations that occur twice (the later field wins), next to groups with few outliers and with none."""
+    rng = np.random.Generator(np.random.PCG64(900 + seq))
+    meta = make_meta(eo, skew_lens, seed=3)
+    heads, n = 3, 3 * seq
+    x = (rng.standard_normal((n, 128)) * 0.01).astype(np.float16)
+    x[:, 0] = 1.0                                          # everything else near zero: two-bit codewords
+    few = rng.random(n) < 0.3
+    x[few] = (rng.standard_t(3, size=(int(few.sum()), 128)) * 0.05).astype(np.float16)
+    blocks, st = eo.encode(meta, x, eo.SELECT_MSE)
+    _, _, info = eo.decode_block(meta, blocks[int(np.argmin(few))])
+    assert st.padded_groups > 0 and (few.all() or info.n_pad >= 15)
+    many = np.array([eo.decode_block(meta, b)[2].n_pad >= 15 for b in blocks])
+    blocks[np.ix_(many, range(36, 64))] = rng.integers(0, 256, size=(int(many.sum()), 28), dtype=np.uint8)
+    lm = lib_meta_from_oracle(B, meta)
+    assert_bit_exact(gpu_decompress(B, lm, blocks), eo.decode(meta, blocks))
+    d_meta, d_blocks = B.meta_to_device(lm), dev(blocks)
+    for qpk in (1, 2, 3, 8):
+        q = synth.queries(1, heads * qpk, 60 + qpk)
+        d_s = torch.full((1, heads * qpk, seq), float("nan"), dtype=torch.float32, device="cuda")
+        B.ecco_attn_scores(d_meta, d_blocks, 1, heads, seq, qpk, dev(q), 0.5, d_s)
+        torch.cuda.synchronize()
+        ref, refabs = eo.attn_scores(meta, blocks, 1, heads, seq, qpk, q, 0.5)
+        check_fused(d_s.cpu().numpy().astype(np.float64), ref, refabs, f"scores q{qpk} outliers")
+    for batch in (1, 2, 3):
+        a = synth.activations(batch, 128, seq)
+        got, _ = gpu_gemv(B, lm, blocks, n, 128, a, batch)
+        ref, refabs = eo.gemv(meta, blocks, n, 128, a, batch)
+        check_fused(got, ref, refabs, f"gemv b{batch} outliers")
+
+
 # ------------------------------------------------------------------ full-size configurations
 def host_threads():
     import os
