@@ -189,16 +189,16 @@ int ecco_gemv_batch(const ecco_gemv_item* items, int32_t n_items, int32_t batch,
  * of ECCO_STATIC_WORKSPACE_BYTES inside the library's device image (every GPU that loads the
  * library carries it until the process exits) instead of a caller buffer.  The call allocates
  * nothing.  A shape whose plan needs more scratch than that is refused with ECCO_ERR_WORKSPACE
- * before anything is launched.  For scale, on a 148-SM part: batch 8 on an 11008 x 4096 matrix needs 3.38 MB, batch 1
- * or 2 on the same matrix 0.6 / 1.1 MB, batch 8 on 28672 x 8192 3.96 MB; a matrix with more than about 36 000 output
+ * before anything is launched.  For scale, on a 148-SM part: batch 8 on an 11008 x 4096 matrix needs 3.39 MB, batch 1
+ * or 2 on the same matrix 0.65 / 1.2 MB, batch 8 on 28672 x 8192 3.96 MB; a matrix with more than about 65 000 output
  * rows at batch 3..8 does not fit and is refused.
  * The first call on each device looks up the array's device address (with that device current);
  * make that first call outside any stream capture.  All calls on a device share the one array:
- * it still holds the previous call's values when the next call starts (each call clears the part
- * that must start from zero), and two calls whose kernels overlap on the GPU -- different streams,
+ * it still holds the previous call's values when the next call starts (which does not matter to that
+ * call), and two calls whose kernels overlap on the GPU -- different streams,
  * no dependency between them -- race on it and give undefined results.  Serialise them, or use
  * ecco_gemv with separate workspaces. */
-#define ECCO_STATIC_WORKSPACE_BYTES (4u << 20)
+#define ECCO_STATIC_WORKSPACE_BYTES (5056u << 10)
 int ecco_gemv_static_ws(const void* d_meta, const uint8_t* d_blocks, int32_t n_out, int32_t k, const void* d_x_fp16,
                         int32_t batch, float* d_y, void* stream);
 

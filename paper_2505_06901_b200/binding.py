@@ -334,7 +334,7 @@ def ecco_gemv_batch(items, batch: int, d_workspace, workspace_bytes: int, stream
                                  workspace_bytes, _stream(stream)), "ecco_gemv_batch")
 
 
-STATIC_WORKSPACE_BYTES = 4 << 20
+STATIC_WORKSPACE_BYTES = 5056 << 10
 
 
 def ecco_gemv_static_ws(d_meta, d_blocks, n_out: int, k: int, d_x_fp16, batch: int, d_y, stream=None) -> None:

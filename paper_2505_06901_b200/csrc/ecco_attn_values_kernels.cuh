@@ -14,68 +14,11 @@ namespace {
 // (V tile)^T [16 dims x 32 tokens] x P^T [32 tokens x 8 heads] with mma.m16n8k16, fp32 accumulators
 // (4 registers per 16 dims, 32 for the 128 dims).  p is split into an fp16 head and an fp16 remainder
 // (two MMAs) so that its rounding does not show.  The result does not depend on scheduling.
+//
+// The softmax is formed on the way: p is taken relative to the largest score that the warp has seen of the row, and sums
+// and accumulators are rescaled when a larger one comes, so the scores are read once and no kernel has to go before this one
+// (a statistics kernel in front cost 25 us on a cache of 128 rows x 8 heads x 32768 scores and 4 us on the shortest rows).
 // ---------------------------------------------------------------------------------------------
-// Row maximum and reciprocal of the row's sum of exponentials, one CTA per row.  One pass: every thread keeps a running
-// (maximum, sum of exp(x - maximum)) over its elements, rescaling the sum when the maximum grows; the pairs are then
-// merged over the warp and over the warps in a fixed order.
-__device__ __forceinline__ void softmax_merge(float& m, float& s, float m2, float s2)
-{
-    const float mn = fmaxf(m, m2);
-    // an empty side has maximum -inf and sum 0: its factor is exp(-inf) = 0 unless both are empty (avoid -inf - -inf)
-    const float f1 = m == mn ? 1.0f : expf(m - mn), f2 = m2 == mn ? 1.0f : expf(m2 - mn);
-    s = s * f1 + s2 * f2;
-    m = mn;
-}
-__global__ void __launch_bounds__(256)
-ecco_softmax_stats_kernel(const float* d_scores, int rows, int seq, float2* d_stats, unsigned int* d_tickets, int n_tickets)
-{
-    __shared__ float2 part[8];
-    const int row = static_cast<int>(blockIdx.x), tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
-    release_dependents();
-    dependency_wait();                                     // the scores may come from the previous kernel of the stream
-    // also clears the ticket words of the call's workspace (the previous kernel, which may have used them, is complete)
-    for (int i = row * 256 + tid; i < n_tickets; i += static_cast<int>(gridDim.x) * 256) d_tickets[i] = 0u;
-    if (row >= rows) return;
-    const float* s = d_scores + static_cast<size_t>(row) * seq;
-    float mx = -INFINITY, sum = 0.0f;
-    auto take = [&](float x) {
-        if (x > mx) { sum = sum * expf(mx - x) + 1.0f; mx = x; }      // exp(-inf) = 0 on the first element
-        else if (x != -INFINITY) sum += expf(x - mx);                  // a masked score (-inf) adds nothing, also before any finite one
-    };
-    // the scores may come from the previous kernel: coherent loads; 16-byte loads where the row allows it
-    if ((reinterpret_cast<uintptr_t>(s) & 15u) == 0) {
-        const float4* s4 = reinterpret_cast<const float4*>(s);
-        const int n4 = seq / 4;
-        int i = tid;
-        for (; i + 3 * 256 < n4; i += 4 * 256) {           // four loads in flight per thread
-            const float4 a = __ldcg(s4 + i), b = __ldcg(s4 + i + 256), c = __ldcg(s4 + i + 512), d = __ldcg(s4 + i + 768);
-            take(a.x); take(a.y); take(a.z); take(a.w);
-            take(b.x); take(b.y); take(b.z); take(b.w);
-            take(c.x); take(c.y); take(c.z); take(c.w);
-            take(d.x); take(d.y); take(d.z); take(d.w);
-        }
-        for (; i < n4; i += 256) {
-            const float4 v = __ldcg(s4 + i);
-            take(v.x); take(v.y); take(v.z); take(v.w);
-        }
-        for (int t = (seq & ~3) + tid; t < seq; t += 256) take(__ldcg(s + t));
-    } else {
-        for (int t = tid; t < seq; t += 256) take(__ldcg(s + t));
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, mx, o), s2 = __shfl_xor_sync(0xffffffffu, sum, o);
-        softmax_merge(mx, sum, m2, s2);
-    }
-    if (lane == 0) part[warp] = make_float2(mx, sum);
-    __syncthreads();
-    if (tid == 0) {
-        float m = part[0].x, t = part[0].y;
-        for (int w = 1; w < 8; ++w) softmax_merge(m, t, part[w].x, part[w].y);
-        d_stats[row] = make_float2(m, 1.0f / t);
-    }
-}
-
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&a)[4], uint32_t addr)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -94,26 +37,31 @@ constexpr uint32_t kAvValueBytes = 7 * 1024;
 constexpr uint32_t kAvWarpBytes = kTabBytes / 2 + kAvValueBytes + kBitsBytes;   // half a value table (two warps share one), tiles, bit stream
 constexpr uint32_t kAvSlots = 8;                                            // reduction slots: see flush
 
-constexpr float kProbScale = 32768.0f, kProbUnscale = 1.0f / 32768.0f;      // powers of two: exact
+constexpr float kProbScale = 32768.0f;                                      // a power of two: exact
+constexpr int kPieceFloats = kGroup * 8 + 16;              // sums of [128 dims][8 heads], 8 sums of weights, 8 maxima
+
+// factor that takes sums relative to maximum m to maximum m_new >= m; an empty side has m = -inf and sums of zero
+__device__ __forceinline__ float rescale(float m, float m_new) { return m == m_new ? 1.0f : __expf(m - m_new); }
 
 template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __restrict__ d_vblocks, int heads, int seq,
-                        int q_per_kv, const float* d_scores, const float2* d_stats,
-                        float* __restrict__ d_out, float* __restrict__ d_partial, unsigned int* __restrict__ d_tickets)
+                        int q_per_kv, const float* d_scores, float* __restrict__ d_out, float* __restrict__ d_partial,
+                        Ticket* d_tickets, Ticket tag)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const int tid = static_cast<int>(threadIdx.x), n_threads = static_cast<int>(blockDim.x);
     release_dependents();
     const Tables tb = plan_tables(smem_u32(smem), d_meta, false);   // one symbol per lookup: see the scalar fused kernels
-    constexpr uint32_t kSlotFloats = kGroup * 8;
+    constexpr uint32_t kFull = 0xffffffffu, kSlotFloats = kGroup * 8 + 8;       // sums, sums of weights
     const uint32_t nw = warps_that_fit(tb, kAvWarpBytes, kTabBytes / 2 + kAvSlots * kSlotFloats * sizeof(float));
     const int kTokens = static_cast<int>(nw) * 32;         // tokens per unit: one per thread of the working warps
     const bool working = warp < nw;
     // small CTA-wide words in the misc area at the start of shared memory (the barrier word is its first)
     unsigned int& ticket = *reinterpret_cast<unsigned int*>(smem + 32);
-    float2* stats_s = reinterpret_cast<float2*>(smem + 64);
+    float* max_s = reinterpret_cast<float*>(smem + 64);    // [warps][8 heads]
+    static_assert(64 + kMaxWarps * 8 * 4 <= kMiscBytes, "maxima fit the misc area");
     WarpSmem ws;
     ws.tab = tab_column<kTabHalf>(tb.warp_base, warp, lane);
     const uint32_t per_warp = tb.warp_base + tab_bytes<kTabHalf>(nw);
@@ -140,13 +88,22 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         return d_vblocks + (static_cast<uint64_t>(bh) * seq + t) * kBlockBytes;
     };
     issue_tables(tb, d_meta);
-    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (u0 < u1 && working) prefetch_block_l2(block_ptr(u0));
     if (!wait_tables(tb)) return;
+    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     const float T = tb.T;
+    if (tid == 0) {                                        // thread 0 takes the tickets: of the heads at the ends of this CTA's units
+        Ticket* const ends[2] = {d_tickets + u0 / chunks, d_tickets + (u1 - 1) / chunks};
+        const Ticket seen[2] = {look_at_ticket(ends[0]), look_at_ticket(ends[1])};
+        claim_ticket(ends[0], seen[0], tag);
+        if (ends[1] != ends[0]) claim_ticket(ends[1], seen[1], tag);
+    }
 
     float acc[8][4];                                       // [16-dim chunk][mma accumulator]
+    float m = -INFINITY, l = 0.0f;                         // of head lane / 4: maximum so far, this lane's part of the sum of weights
     auto clear_acc = [&]() {
+        m = -INFINITY;
+        l = 0.0f;
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
@@ -154,11 +111,27 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     };
     clear_acc();
 
-    // all tokens of head bh seen by this CTA are in acc: reduce over the warps in a fixed order (in rounds of
+    // scales acc and l from maximum m to maximum `to` (per head lane / 4; accumulator column j & 1 is head (lane % 4) * 2 + (j & 1))
+    auto rescale_to = [&](float to) {
+        const float f = rescale(m, to);
+        const float f0 = __shfl_sync(kFull, f, (lane & 3u) * 8), f1 = __shfl_sync(kFull, f, (lane & 3u) * 8 + 4);
+        l *= f;
+#pragma unroll
+        for (int ch = 0; ch < 8; ++ch) { acc[ch][0] *= f0; acc[ch][1] *= f1; acc[ch][2] *= f0; acc[ch][3] *= f1; }
+        m = to;
+    };
+    // All tokens of head bh seen by this CTA are in acc.  The warps agree on the maxima and reduce in a fixed order (in rounds of
     // kAvSlots warps: warp w adds its sums to slot w mod kAvSlots, the first round by plain stores; then the slots are
-    // added in slot order), then either store (this CTA owns the whole head) or hand a partial to the slot-and-ticket
-    // reduction
+    // added in slot order); then either store (this CTA owns the whole head) or hand a piece to the slot-and-ticket reduction.
     auto flush = [&](int bh) {
+        if (working && (lane & 3u) == 0) max_s[warp * 8 + (lane >> 2)] = m;
+        __syncthreads();
+        auto top_of = [&](uint32_t head) {
+            float top = max_s[head];
+            for (uint32_t w = 1; w < nw; ++w) top = fmaxf(top, max_s[w * 8 + head]);
+            return top;
+        };
+        if (working) rescale_to(top_of(lane >> 2));
         for (uint32_t first = 0; first < nw; first += kAvSlots) {
             if (warp >= first && warp < first + kAvSlots && warp < nw) {
                 float* slot = out_s + (warp - first) * kSlotFloats;
@@ -168,40 +141,55 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
                     for (int j = 0; j < 4; ++j) {
                         const int dim = ch * 16 + static_cast<int>(lane >> 2) + (j >= 2 ? 8 : 0);
                         const int head = static_cast<int>(lane & 3u) * 2 + (j & 1);
-                        const float v = acc[ch][j] * kProbUnscale;
+                        const float v = acc[ch][j];
                         slot[dim * 8 + head] = first ? slot[dim * 8 + head] + v : v;
                     }
+                float s = l + __shfl_xor_sync(kFull, l, 1);
+                s += __shfl_xor_sync(kFull, s, 2);
+                if ((lane & 3u) == 0) {
+                    float* at = slot + kGroup * 8 + (lane >> 2);
+                    *at = first ? *at + s : s;
+                }
             }
             __syncthreads();
         }
         const uint32_t used = min(nw, kAvSlots);
-        for (int i = tid; i < static_cast<int>(kSlotFloats); i += n_threads) {   // thread i keeps element i from here on
+        for (int i = tid; i < static_cast<int>(kSlotFloats); i += n_threads) {
             float sum = out_s[i];
             for (uint32_t sl = 1; sl < used; ++sl) sum += out_s[sl * kSlotFloats + i];
             out_s[i] = sum;
         }
+        __syncthreads();
         const int c_lo = unit_owner(U, G, static_cast<int64_t>(bh) * chunks);
         const int c_hi = unit_owner(U, G, static_cast<int64_t>(bh + 1) * chunks - 1);
+        auto store = [&](int i, float v, float weights) {
+            if ((i & 7) < q_per_kv) d_out[(static_cast<size_t>(bh) * q_per_kv + (i & 7)) * kGroup + (i >> 3)] = v / weights;
+        };
         if (c_lo == c_hi) {
-            for (int i = tid; i < kGroup * 8; i += n_threads) {
-                const int dim = i >> 3, r = i & 7;
-                if (r < q_per_kv) d_out[(static_cast<size_t>(bh) * q_per_kv + r) * kGroup + dim] = out_s[i];
-            }
+            for (int i = tid; i < kGroup * 8; i += n_threads) store(i, out_s[i], out_s[kGroup * 8 + (i & 7)]);
         } else {
-            float* mine = d_partial + static_cast<size_t>(c + bh) * (kGroup * 8);
-            for (int i = tid; i < kGroup * 8; i += n_threads) mine[i] = out_s[i];
+            float* mine = d_partial + static_cast<size_t>(c + bh) * kPieceFloats;
+            for (int i = tid; i < kPieceFloats; i += n_threads) mine[i] = i < kGroup * 8 + 8 ? out_s[i] : top_of(i & 7);
             __threadfence();
             __syncthreads();
-            if (tid == 0) ticket = atomicAdd(&d_tickets[bh], 1u);
+            if (tid == 0) ticket = take_ticket(&d_tickets[bh]);
             __syncthreads();
             if (ticket == static_cast<unsigned int>(c_hi - c_lo)) {
                 __threadfence();
+                const float* piece = d_partial + static_cast<size_t>(c_lo + bh) * kPieceFloats;
+                const int n = c_hi - c_lo + 1;
                 for (int i = tid; i < kGroup * 8; i += n_threads) {
-                    const int dim = i >> 3, r = i & 7;
-                    if (r >= q_per_kv) continue;
-                    float sum = 0.0f;
-                    for (int cc = c_lo; cc <= c_hi; ++cc) sum += __ldcg(d_partial + static_cast<size_t>(cc + bh) * (kGroup * 8) + i);
-                    d_out[(static_cast<size_t>(bh) * q_per_kv + r) * kGroup + dim] = sum;
+                    const float* pw = piece + kGroup * 8 + (i & 7);
+                    float top = -INFINITY, v = 0.0f, weights = 0.0f;
+#pragma unroll 4
+                    for (int k = 0; k < n; ++k) top = fmaxf(top, __ldcg(pw + 8 + static_cast<size_t>(k) * kPieceFloats));
+#pragma unroll 4
+                    for (int k = 0; k < n; ++k) {
+                        const float f = rescale(__ldcg(pw + 8 + static_cast<size_t>(k) * kPieceFloats), top);
+                        v += f * __ldcg(piece + i + static_cast<size_t>(k) * kPieceFloats);
+                        weights += f * __ldcg(pw + static_cast<size_t>(k) * kPieceFloats);
+                    }
+                    store(i, v, weights);
                 }
                 if (tid == 0) d_tickets[bh] = 0;
             }
@@ -216,8 +204,6 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         const bool valid = tile_base + static_cast<int>(lane) < seq;
         if (bh != cur_bh) {
             if (cur_bh >= 0) { flush(cur_bh); clear_acc(); }
-            if (tid < 8) stats_s[tid] = tid < q_per_kv ? __ldcg(d_stats + static_cast<size_t>(bh) * q_per_kv + tid) : make_float2(0.0f, 0.0f);
-            __syncthreads();
             cur_bh = bh;
         }
         if (!working) continue;                            // warps without room for their arrays only help with the reductions
@@ -225,19 +211,26 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         uint32_t p_hi[4], p_lo[4];
         {
             const int r = static_cast<int>(lane >> 2);
-            const float2 st = stats_s[r];
-            // Probabilities enter the tensor cores as fp16 pairs (value + remainder).  Taken as they are, everything
-            // below 6e-5 would sit in fp16's subnormal range (one part in a thousand at p = 3e-5, the typical weight of
-            // a token in a 32768-token row); scaled by 2^15 they keep 22 bits down to 2e-12, and p <= 1 cannot
-            // overflow.  The sums are scaled back when they leave the accumulators (kProbUnscale in flush).
-            const float to_p = st.y * kProbScale;
             const float* srow = d_scores + (static_cast<size_t>(bh) * q_per_kv + min(r, q_per_kv - 1)) * seq;
+            float s[8], top = m;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int tk = tile_base + static_cast<int>(lane & 3u) * 2 + 8 * (j >> 1) + (j & 1);
+                s[j] = r < q_per_kv && tk < seq ? __ldcg(srow + tk) : -INFINITY;
+                top = fmaxf(top, s[j]);
+            }
+            top = fmaxf(top, __shfl_xor_sync(kFull, top, 1));
+            top = fmaxf(top, __shfl_xor_sync(kFull, top, 2));
+            if (__any_sync(kFull, top > m)) rescale_to(top);                   // rare once a few tiles have passed
+            // Probabilities enter the tensor cores as fp16 pairs (value + remainder).  Taken as they are, everything
+            // below 6e-5 would sit in fp16's subnormal range (one part in a thousand at p = 3e-5); scaled by 2^15 they keep
+            // 22 bits down to 2e-12, and exp(s - max) <= 1 cannot overflow.  The sum of weights carries the same factor.
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int tk = tile_base + static_cast<int>(lane & 3u) * 2 + 8 * j;
-                float p0 = 0.0f, p1 = 0.0f;
-                if (r < q_per_kv && tk < seq) p0 = __expf(__ldcg(srow + tk) - st.x) * to_p;
-                if (r < q_per_kv && tk + 1 < seq) p1 = __expf(__ldcg(srow + tk + 1) - st.x) * to_p;
+                // a masked score (-inf) has weight zero, also before any finite one
+                const float p0 = s[2 * j] == -INFINITY ? 0.0f : __expf(s[2 * j] - m) * kProbScale;
+                const float p1 = s[2 * j + 1] == -INFINITY ? 0.0f : __expf(s[2 * j + 1] - m) * kProbScale;
+                l += p0 + p1;
                 const __half h0 = __float2half_rn(p0), h1 = __float2half_rn(p1);
                 const __half l0 = __float2half_rn(p0 - __half2float(h0)), l1 = __float2half_rn(p1 - __half2float(h1));
                 p_hi[j] = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);

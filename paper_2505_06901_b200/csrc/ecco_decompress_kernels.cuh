@@ -142,9 +142,9 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
             const DecompressJob& job = batch.job[job_at];
             return job.blocks + static_cast<uint64_t>(min((g - job_first) * 32 + lane, static_cast<uint32_t>(job.n_groups) - 1u)) * kBlockBytes;
         };
-        if (run == 0) dependency_wait();                   // blocks and output: only after the previous kernel has completed
         if (gt < run_tiles) { seek(gt); prefetch_block_l2(block_ptr(gt)); }
         if (!finish_decode_tables(tb, static_cast<uint32_t>(run & 1))) return;
+        if (run == 0) dependency_wait();                   // blocks and output: only after the previous kernel has completed
 
         while (gt < run_tiles) {
             const DecompressJob& job = batch.job[job_at];

@@ -9,11 +9,13 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <chrono>
 #include <climits>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <random>
 
 #include "../../include/ecco.h"
 #include "ecco_format.h"
@@ -244,7 +246,8 @@ __device__ __forceinline__ bool wait_tables(const Tables& tb, uint32_t parity = 
 // Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may become resident
 // while the previous kernel in the stream is still draining.  dependency_wait() returns once that kernel has
 // completed and its writes are visible (at once if there is no such overlap); every kernel executes it before
-// its first access to global memory other than the metadata image, so stream order is what it is without the
+// its first access to global memory other than the metadata image (a prefetch into L2, where every write arrives, is no
+// access), so stream order is what it is without the
 // attribute and only launch, table fetch and prologue overlap.  The image is the exception because no kernel writes
 // it: it reaches the device by a copy, which is a stream operation of its own (a kernel behind a copy starts after
 // it), and a kernel can start early only behind one that releases its dependents, i.e. one of this file.

@@ -114,7 +114,7 @@ __device__ __forceinline__ void load_vfrag(uint32_t (&vfrag)[16], const __half* 
 template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float* __restrict__ d_partial,
-                     unsigned int* __restrict__ d_tickets)
+                     Ticket* d_tickets, Ticket tag)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int lane = static_cast<int>(threadIdx.x & 31u), warp = static_cast<int>(threadIdx.x >> 5);
@@ -134,10 +134,10 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
         wait_tables(tb);                                   // the table copies into this CTA's shared memory must land first
         return;
     }
-    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     GemvPos pos = {0, 0, 0};
     if (u0 < u1) { pos = gemv_pos_of(batch, u0); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
     if (!wait_tables(tb)) return;
+    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (u0 >= u1) return;
 
     float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
@@ -159,7 +159,7 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
             __threadfence();
             __syncwarp();
             unsigned int t = 0;
-            if (lane == 0) t = atomicAdd(&d_tickets[gtile], 1u);
+            if (lane == 0) t = take_ticket(&d_tickets[gtile * kTicketStride]);
             t = __shfl_sync(0xffffffffu, t, 0);
             if (t != static_cast<unsigned int>(w_hi - w_lo)) return;
             __threadfence();
@@ -177,9 +177,11 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
                 }
                 if (row < n_out && b < n_cols) d_y[static_cast<size_t>(b) * n_out + row] = sum;
             }
-        if (w_lo != w_hi && lane == 0) d_tickets[gtile] = 0;
+        if (w_lo != w_hi && lane == 0) d_tickets[gtile * kTicketStride] = 0;
     };
 
+    Ticket* const my_ticket[2] = {d_tickets + gemv_tile_of(batch, pos) * kTicketStride, d_tickets + gemv_tile_of(batch, gemv_pos_of(batch, u1 - 1)) * kTicketStride};
+    const Ticket seen[2] = {look_at_ticket(my_ticket[0]), look_at_ticket(my_ticket[1])};
     int cur_j = pos.j, cur_tile = pos.tile;
     float T = __ldg(&reinterpret_cast<const DevHeader*>(batch.job[pos.j].meta)->T);
     for (int64_t u = u0; u < u1; ++u) {
@@ -197,6 +199,10 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
         }
         Block cur;                                         // fetched now, prefetched into L2 one unit earlier (see the scalar kernels)
         ldg_block(cur, gemv_block_ptr(batch, pos, lane));
+        if (u == u0 && lane == 0) {                        // lane 0 is the one that takes
+            claim_ticket(my_ticket[0], seen[0], tag);
+            if (my_ticket[1] != my_ticket[0]) claim_ticket(my_ticket[1], seen[1], tag);
+        }
         const __half* xk = jb.x + pos.kb * kGroup;
         const size_t k = static_cast<size_t>(jb.kblocks) * kGroup;
         if (u + 1 < u1) { pos = gemv_pos_next(batch, pos); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
@@ -230,9 +236,9 @@ ecco_attn_scores_mma_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* _
     };
     int nbh = static_cast<int>(u0 / tiles), ntile = static_cast<int>(u0 % tiles);     // advanced by one per unit
     issue_tables(tb, d_meta);
-    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (u0 < u1) prefetch_block_l2(block_ptr(nbh, ntile));
     if (!wait_tables(tb)) return;
+    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     const float T = tb.T;
 
     uint32_t vfrag[16];

@@ -123,6 +123,22 @@ __host__ __device__ __forceinline__ int unit_owner(int64_t U, int G, int64_t u)
     return c;
 }
 
+// Ticket words of a workspace.  They need no clearing before the call, which would be a launch of its own (2 us of a small call's
+// 10): a word counts from zero once it carries the call's tag, 48 bits that the host draws at random once and advances for every
+// call (stale contents carry it with probability 2^-48).  Everyone who will take a ticket first claims the word, early, while its
+// block is on the way: if the word does not carry the tag, an exchange against what was seen installs it, and it fails exactly
+// when another has done so.  Taking is then one addition.  (Counting up by exchanges alone serialises the arrivals: 39 us instead of
+// 17 for a 4096 x 4096 product.)  The last to arrive clears the word, so a captured call that is replayed with its tag finds none of
+// its own counts.
+using Ticket = unsigned long long;
+constexpr int kTicketStride = 4;                           // words from one ticket to the next: each in a sector of its own
+__device__ __forceinline__ Ticket look_at_ticket(const Ticket* word) { return *reinterpret_cast<const volatile Ticket*>(word); }
+__device__ __forceinline__ void claim_ticket(Ticket* word, Ticket seen, Ticket tag)
+{
+    if ((seen >> 16) != tag) atomicCAS(word, seen, tag << 16);
+}
+__device__ __forceinline__ unsigned int take_ticket(Ticket* word) { return static_cast<unsigned int>(atomicAdd(word, 1ull) & 0xffffu); }
+
 // One call of the fused GEMV may cover several matrices (ecco_gemv_batch): the units of all of them form one unit
 // space, dealt out to the working warps as one, so that a group of small matrices pays one launch, one table fetch and
 // one tail.  All matrices of a call share the decode tables (equal table hash; only the exponent differs).
@@ -175,6 +191,8 @@ __device__ __forceinline__ GemvPos gemv_pos_next(const GemvBatch& batch, GemvPos
     }
     return p;
 }
+// place of a row tile in the call's tile space (tickets and slots)
+__device__ __forceinline__ int gemv_tile_of(const GemvBatch& batch, const GemvPos& p) { return batch.job[p.j].tile_first + p.tile; }
 __device__ __forceinline__ const uint8_t* gemv_block_ptr(const GemvBatch& batch, const GemvPos& p, int lane)
 {
     const GemvJob& jb = batch.job[p.j];
@@ -194,7 +212,7 @@ __host__ __device__ constexpr uint32_t scalar_warp_bytes(int v) { return v * kGr
 // one ticket per 32-row tile.
 template <int kV, int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
-ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict__ d_partial, unsigned int* __restrict__ d_tickets)
+ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict__ d_partial, Ticket* d_tickets, Ticket tag)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     release_dependents();
@@ -217,10 +235,10 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
         bounded_wait(tb.base, 0, kWaitLimit);              // the table copies into this CTA's shared memory must land first
         return;
     }
-    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     GemvPos pos = {0, 0, 0};
     if (u0 < u1) { pos = gemv_pos_of(batch, u0); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
     if (!finish_decode_tables(tb)) return;
+    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
 
     float acc[kV][2];                                      // two partial sums, added when the row tile is left
     auto clear_acc = [&]() {
@@ -250,7 +268,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
         __threadfence();
         __syncwarp();
         unsigned int t = 0;
-        if (lane == 0) t = atomicAdd(&d_tickets[gtile], 1u);
+        if (lane == 0) t = take_ticket(&d_tickets[gtile * kTicketStride]);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t == static_cast<unsigned int>(w_hi - w_lo)) {  // last of the warps that share this tile
             __threadfence();
@@ -280,7 +298,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
                     d_y[static_cast<size_t>(b) * n_out + row] = sum;
                 }
             }
-            if (lane == 0) d_tickets[gtile] = 0;
+            if (lane == 0) d_tickets[gtile * kTicketStride] = 0;
         }
     };
 
@@ -295,6 +313,8 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     };
     if (u0 >= u1) return;
     load_x(pos);
+    Ticket* const my_ticket[2] = {d_tickets + gemv_tile_of(batch, pos) * kTicketStride, d_tickets + gemv_tile_of(batch, gemv_pos_of(batch, u1 - 1)) * kTicketStride};
+    const Ticket seen[2] = {look_at_ticket(my_ticket[0]), look_at_ticket(my_ticket[1])};
     int cur_j = pos.j, cur_tile = pos.tile;
     float T = __ldg(&reinterpret_cast<const DevHeader*>(batch.job[pos.j].meta)->T);
     for (int64_t u = u0; u < u1; ++u) {
@@ -314,6 +334,10 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
         // one in sixteen registers through a whole group costs more in resident warps than the fetch costs here
         Block cur;
         ldg_block(cur, gemv_block_ptr(batch, pos, lane));
+        if (u == u0 && lane == 0) {                        // lane 0 is the one that takes
+            claim_ticket(my_ticket[0], seen[0], tag);
+            if (my_ticket[1] != my_ticket[0]) claim_ticket(my_ticket[1], seen[1], tag);
+        }
         if (u + 1 < u1) {
             pos = gemv_pos_next(batch, pos);
             prefetch_block_l2(gemv_block_ptr(batch, pos, lane));
@@ -355,9 +379,9 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     };
     int bh = static_cast<int>(u0 / tiles), tile = static_cast<int>(u0 % tiles);
     issue_decode_tables(tb, d_meta);
-    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (u0 < u1) prefetch_block_l2(block_ptr(bh, tile));
     if (!finish_decode_tables(tb)) return;
+    dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     const float T = tb.T;
 
     int cur_bh = -1;

@@ -284,11 +284,9 @@ static int launch_gemv_mma_call(const DeviceInfo& di, const GemvCall& c, int bat
     if (!d_ws || !aligned16(d_ws)) return d_ws ? ECCO_ERR_ALIGNMENT : ECCO_ERR_WORKSPACE;
     if (ws_bytes < p.partial_bytes + p.ticket_bytes) return ECCO_ERR_WORKSPACE;
     float* partial = static_cast<float*>(d_ws);
-    unsigned int* tickets = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(d_ws) + p.partial_bytes);
-    rc = zero_tickets(tickets, p.ticket_bytes, stream);
-    if (rc) return rc;
+    Ticket* tickets = reinterpret_cast<Ticket*>(static_cast<uint8_t*>(d_ws) + p.partial_bytes);
     return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(kMmaWarps * 32), kSmemCtaBytes, stream, c.b, batch,
-                             partial, tickets);
+                             partial, tickets, next_ticket_tag());
 }
 static int launch_gemv_mma(const DeviceInfo& di, const void* d_meta, const uint8_t* d_blocks, int n_out, int kblocks,
                            const void* d_x, int batch, float* d_y, void* d_ws, size_t ws_bytes, cudaStream_t stream)
@@ -312,11 +310,9 @@ static int launch_gemv_warp_call(const DeviceInfo& di, const GemvCall& c, void* 
     if (!d_ws || !aligned16(d_ws)) return d_ws ? ECCO_ERR_ALIGNMENT : ECCO_ERR_WORKSPACE;
     if (ws_bytes < p.partial_bytes + p.ticket_bytes) return ECCO_ERR_WORKSPACE;
     float* partial = static_cast<float*>(d_ws);
-    unsigned int* tickets = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(d_ws) + p.partial_bytes);
-    rc = zero_tickets(tickets, p.ticket_bytes, stream);
-    if (rc) return rc;
+    Ticket* tickets = reinterpret_cast<Ticket*>(static_cast<uint8_t*>(d_ws) + p.partial_bytes);
     return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(kFusedWarps * 32), kSmemCtaBytes, stream, c.b,
-                             partial, tickets);
+                             partial, tickets, next_ticket_tag());
 }
 template <int kV>
 static int launch_gemv_warp(const DeviceInfo& di, const void* d_meta, const uint8_t* d_blocks, int n_out, int kblocks,
@@ -496,34 +492,29 @@ namespace {
 // measured no faster on 32768-token rows (602.8 against 600.6 us) and slower on 4096-token rows, whose last unit
 // they leave half empty (99.1 against 89.3 us).
 constexpr int kAvWarps = 16;
-inline int av_warps(int) { return kAvWarps; }
-struct AvPlan { int grid, warps; size_t stats_bytes, partial_bytes, ticket_bytes; };
-AvPlan av_plan(int batch, int n_kv_heads, int seq, int q_per_kv, int ctas_max)
+struct AvPlan { int grid; size_t partial_bytes, ticket_bytes; };
+AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
 {
     AvPlan p;
-    p.warps = av_warps(seq);
     const int heads = batch * n_kv_heads;
-    // at most this many units (fewer when all p.warps warps find room); the device splits what there is evenly
-    const int64_t units = static_cast<int64_t>(heads) * ((seq + 31) / 32);
-    p.grid = static_cast<int>(units < ctas_max ? units : ctas_max);
+    // at most this many units (fewer when all warps find room); the device splits what there is evenly
+    p.grid = spread_ctas(static_cast<int64_t>(heads) * ((seq + 31) / 32), ctas_max);
     auto up = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
-    p.stats_bytes = up(static_cast<size_t>(heads) * q_per_kv * sizeof(float2));
-    p.partial_bytes = up(static_cast<size_t>(p.grid + heads) * kGroup * 8 * sizeof(float));
-    p.ticket_bytes = up(static_cast<size_t>(heads) * sizeof(unsigned int));
+    p.partial_bytes = up(static_cast<size_t>(p.grid + heads) * kPieceFloats * sizeof(float));
+    p.ticket_bytes = up(static_cast<size_t>(heads) * sizeof(Ticket));
     return p;
 }
 
 template <int kWarps>
 int launch_attn_values(const DeviceInfo& di, const AvPlan& p, const void* d_meta, const uint8_t* d_vblocks, int heads, int seq,
-                       int q_per_kv, const float* d_scores, float2* stats, float* d_out, float* partial, unsigned int* tickets,
-                       cudaStream_t s)
+                       int q_per_kv, const float* d_scores, float* d_out, float* partial, Ticket* tickets, cudaStream_t s)
 {
     auto kernel = ecco_attn_values_kernel<kWarps>;
     static thread_local bool configured[64] = {};
     const int rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
     return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(kWarps * 32), kSmemCtaBytes, s,
-                             static_cast<const uint8_t*>(d_meta), d_vblocks, heads, seq, q_per_kv, d_scores, stats, d_out, partial, tickets);
+                             static_cast<const uint8_t*>(d_meta), d_vblocks, heads, seq, q_per_kv, d_scores, d_out, partial, tickets, next_ticket_tag());
 }
 }  // namespace
 
@@ -531,8 +522,8 @@ extern "C" size_t ecco_attn_values_workspace_bytes(int32_t batch, int32_t n_kv_h
 {
     if (batch <= 0 || n_kv_heads <= 0 || seq <= 0 || q_per_kv < 1 || q_per_kv > 8) return 0;
     if (static_cast<int64_t>(batch) * n_kv_heads > (1 << 24)) return 0;
-    const AvPlan p = av_plan(batch, n_kv_heads, seq, q_per_kv, 256);
-    return p.stats_bytes + p.partial_bytes + p.ticket_bytes;
+    const AvPlan p = av_plan(batch, n_kv_heads, seq, 256);
+    return p.partial_bytes + p.ticket_bytes;
 }
 
 extern "C" int ecco_attn_values(const void* d_meta, const uint8_t* d_vblocks, int32_t batch, int32_t n_kv_heads, int32_t seq,
@@ -547,19 +538,14 @@ extern "C" int ecco_attn_values(const void* d_meta, const uint8_t* d_vblocks, in
     DeviceInfo di;
     int rc = device_info(&di);
     if (rc) return rc;
-    const AvPlan p = av_plan(batch, n_kv_heads, seq, q_per_kv, di.sms < 256 ? di.sms : 256);
+    const AvPlan p = av_plan(batch, n_kv_heads, seq, di.sms < 256 ? di.sms : 256);
     if (!d_workspace || !aligned16(d_workspace)) return d_workspace ? ECCO_ERR_ALIGNMENT : ECCO_ERR_WORKSPACE;
-    if (workspace_bytes < p.stats_bytes + p.partial_bytes + p.ticket_bytes) return ECCO_ERR_WORKSPACE;
+    if (workspace_bytes < p.partial_bytes + p.ticket_bytes) return ECCO_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* wsb = static_cast<uint8_t*>(d_workspace);
-    float2* stats = reinterpret_cast<float2*>(wsb);
-    float* partial = reinterpret_cast<float*>(wsb + p.stats_bytes);
-    unsigned int* tickets = reinterpret_cast<unsigned int*>(wsb + p.stats_bytes + p.partial_bytes);
-    const int heads = batch * n_kv_heads, rows = heads * q_per_kv;
-    rc = launch_overlapped(ecco_softmax_stats_kernel, static_cast<unsigned>(rows), 256u, 0, s, d_scores, rows, seq, stats, tickets,
-                           static_cast<int>(p.ticket_bytes / sizeof(unsigned int)));
-    if (rc) return rc;
-    return launch_attn_values<kAvWarps>(di, p, d_meta, d_vblocks, heads, seq, q_per_kv, d_scores, stats, d_out, partial, tickets, s);
+    float* partial = reinterpret_cast<float*>(wsb);
+    Ticket* tickets = reinterpret_cast<Ticket*>(wsb + p.partial_bytes);
+    return launch_attn_values<kAvWarps>(di, p, d_meta, d_vblocks, batch * n_kv_heads, seq, q_per_kv, d_scores, d_out, partial, tickets, s);
 }
 
 

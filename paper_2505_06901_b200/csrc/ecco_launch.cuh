@@ -51,21 +51,17 @@ int launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, 
     return check_launch();
 }
 
-// Zeroes the ticket words of a workspace.  A kernel rather than a memset so that it can sit in a chain of
-// overlapped launches: it lets its successor start at once and clears only after its predecessor (which may
-// still be using the same workspace) has completed.
-__global__ void ecco_zero_words_kernel(unsigned int* __restrict__ p, size_t n)
+// the tag of a call's ticket words (see take_ticket): 48 bits, never zero, another one for every call of the process
+inline Ticket next_ticket_tag()
 {
-    release_dependents();
-    dependency_wait();
-    for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * blockDim.x) p[i] = 0u;
-}
-inline int zero_tickets(unsigned int* tickets, size_t bytes, cudaStream_t stream)
-{
-    const size_t n = bytes / sizeof(unsigned int);
-    if (n == 0) return ECCO_OK;
-    const unsigned grid = static_cast<unsigned>(n < 8192 ? (n + 255) / 256 : 32);
-    return launch_overlapped(ecco_zero_words_kernel, grid, 256u, 0, stream, tickets, n);
+    static std::atomic<uint64_t> next{[] {
+        std::random_device rd;
+        return (static_cast<uint64_t>(rd()) << 32 | rd()) ^ static_cast<uint64_t>(std::chrono::steady_clock::now().time_since_epoch().count());
+    }()};
+    for (;;) {
+        const Ticket tag = next.fetch_add(1, std::memory_order_relaxed) & ((1ull << 48) - 1);
+        if (tag) return tag;
+    }
 }
 
 template <class K>
@@ -109,7 +105,7 @@ inline GemvPlan gemv_plan(int64_t units, int row_tiles, int warps, int cols, int
     p.grid = spread_ctas(units, ctas_max);
     const int64_t workers = static_cast<int64_t>(p.grid) * warps < units ? static_cast<int64_t>(p.grid) * warps : units;
     p.partial_bytes = (static_cast<size_t>(workers + row_tiles) * cols * 32 * sizeof(float) + 255) & ~static_cast<size_t>(255);
-    p.ticket_bytes = (static_cast<size_t>(row_tiles) * sizeof(unsigned int) + 255) & ~static_cast<size_t>(255);
+    p.ticket_bytes = (static_cast<size_t>(row_tiles) * kTicketStride * sizeof(Ticket) + 255) & ~static_cast<size_t>(255);
     return p;
 }
 

@@ -430,6 +430,29 @@ def test_gemv_workspace_errors(B, cfg1_small, synth):
     assert ei.value.code == B.ERR_WORKSPACE
 
 
+@pytest.mark.parametrize("n_out,k,batch", [(32, 128, 1), (40, 8192, 1), (4096, 1024, 2), (96, 16384, 3), (513, 4096, 8)])
+def test_gemv_does_not_care_what_the_workspace_holds(B, eo, cfg1_small, synth, n_out, k, batch):
+    """Row tiles of one warp, of a few and of a hundred: the same bits from a workspace of zeros, of ones, of random words and of
+    what earlier calls left in it (an odd number of calls later, and after a call of another shape)."""
+    lm = lib_meta_from_oracle(B, cfg1_small["meta"])
+    n = n_out * (k // 128)
+    blocks = np.tile(cfg1_small["blocks"], (-(-n // 2048), 1))[:n]
+    d_meta, d_blocks, d_x = B.meta_to_device(lm), dev(blocks), dev(synth.activations(batch, k, 5))
+    wsb = max(B.ecco_gemv_workspace_bytes(n_out, k, batch), B.ecco_gemv_workspace_bytes(64, 256, batch))
+    first = None
+    for fill in (0, 0xFF, None, "left", "left", "other"):
+        if fill == "other":
+            B.ecco_gemv(d_meta, d_blocks, 32, 128, d_x, batch, torch.empty((batch, 32), device="cuda"), ws, wsb)
+        elif fill != "left":
+            ws = torch.randint(0, 256, (wsb,), dtype=torch.uint8, device="cuda") if fill is None else torch.full((wsb,), fill, dtype=torch.uint8, device="cuda")
+        y = torch.full((batch, n_out), float("nan"), dtype=torch.float32, device="cuda")
+        B.ecco_gemv(d_meta, d_blocks, n_out, k, d_x, batch, y, ws, wsb)
+        first = y if first is None else first
+        assert torch.equal(y, first), fill
+    ref, refabs = eo.gemv(cfg1_small["meta"], blocks[: n], n_out, k, synth.activations(batch, k, 5), batch)
+    check_fused(first.cpu().numpy().astype(np.float64), ref, refabs, f"gemv b{batch} workspaces")
+
+
 # ------------------------------------------------------------------ fused attention scores
 @pytest.mark.parametrize("batch,heads,seq,qpk", [(2, 4, 256, 1), (2, 4, 256, 2), (2, 4, 256, 8), (1, 3, 77, 4), (1, 1, 1, 1),
                                                  (2, 2, 513, 3)])
@@ -787,6 +810,32 @@ def test_attn_values_keeps_small_probabilities(B, eo, kv_small, synth, qpk):
     assert np.abs(ref[0, 0]).max() < 1e-6 and np.abs(got[0, 0]).max() > 0      # the small sums are really there
     if qpk > 1:
         assert np.all(err[0, 1] <= 2e-5 * refabs[0, 1])    # evenly spread weights: far inside the bound
+
+
+@pytest.mark.parametrize("seq", [33, 700, 3000])
+def test_attn_values_with_rising_scores_and_any_workspace(B, eo, kv_small, seq):
+    """Scores that grow along the row (every tile raises the running maximum), fall, or hold their largest value in the last token, over
+    heads split between several blocks; the same bits whatever the workspace held."""
+    meta, heads, qpk = kv_small["meta"], 3, 4
+    rng = np.random.Generator(np.random.PCG64(seq))
+    n = heads * seq
+    blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
+    s = (rng.standard_normal((1, heads * qpk, seq)) * 2).astype(np.float32)
+    s[0, 0::4] += np.linspace(-60, 60, seq, dtype=np.float32)
+    s[0, 1::4] += np.linspace(60, -60, seq, dtype=np.float32)
+    s[0, 2::4, -1] = 80.0
+    d_meta, d_blocks, d_s = B.meta_to_device(lib_meta_from_oracle(B, meta)), dev(blocks), dev(s)
+    wsb = B.ecco_attn_values_workspace_bytes(1, heads, seq, qpk)
+    first = None
+    for fill in (0, 0xFF, 0x3C, "left"):
+        if fill != "left":
+            ws = torch.full((wsb,), fill, dtype=torch.uint8, device="cuda")
+        out = torch.full((1, heads * qpk, 128), float("nan"), dtype=torch.float32, device="cuda")
+        B.ecco_attn_values(d_meta, d_blocks, 1, heads, seq, qpk, d_s, out, ws, wsb)
+        first = out if first is None else first
+        assert torch.equal(out, first), fill
+    ref, refabs = eo.attn_values(meta, blocks, 1, heads, seq, qpk, s)
+    check_fused(first.cpu().numpy().astype(np.float64), ref, refabs, "values rising")
 
 
 @pytest.mark.parametrize("seq", [301, 4100])
