@@ -151,7 +151,7 @@ static int launch_decompress_batch(const DeviceInfo& di, DecompressBatch& batch,
     uint64_t tiles = 0;
     for (int t = 0; t < batch.n; ++t) tiles += (batch.job[t].n_groups + 31) / 32;
     const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>(tiles), di.sms));
-    return launch_overlapped(kernel, grid, static_cast<unsigned>(kDecompressTmaWarps * 32), kSmemCtaBytes, stream, batch);
+    return launch_overlapped(kernel, grid, spread_threads(static_cast<int64_t>(tiles), static_cast<int>(grid), kDecompressTmaWarps), kSmemCtaBytes, stream, batch);
 }
 
 // The tile-store kernel addresses output rows with the 32-bit signed coordinates of the TMA unit: tensors of 2^31 groups
@@ -234,7 +234,7 @@ extern "C" int ecco_var_decompress(const void* d_meta, const uint8_t* d_stream, 
     rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
     const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>((n_groups + 31) / 32), di.sms));
-    return launch_overlapped(kernel, grid, static_cast<unsigned>(kVarWarps * 32), kSmemCtaBytes, static_cast<cudaStream_t>(stream),
+    return launch_overlapped(kernel, grid, spread_threads(static_cast<int64_t>((n_groups + 31) / 32), static_cast<int>(grid), kVarWarps), kSmemCtaBytes, static_cast<cudaStream_t>(stream),
                              static_cast<const uint8_t*>(d_meta), reinterpret_cast<const uint4*>(d_stream),
                              static_cast<const uint64_t*>(d_index), n_groups, static_cast<uint16_t*>(d_out), map);
 }
@@ -285,7 +285,7 @@ static int launch_gemv_mma_call(const DeviceInfo& di, const GemvCall& c, int bat
     if (ws_bytes < p.partial_bytes + p.ticket_bytes) return ECCO_ERR_WORKSPACE;
     float* partial = static_cast<float*>(d_ws);
     Ticket* tickets = reinterpret_cast<Ticket*>(static_cast<uint8_t*>(d_ws) + p.partial_bytes);
-    return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(kMmaWarps * 32), kSmemCtaBytes, stream, c.b, batch,
+    return launch_overlapped(kernel, static_cast<unsigned>(p.grid), spread_threads(c.b.units, p.grid, kMmaWarps), kSmemCtaBytes, stream, c.b, batch,
                              partial, tickets, next_ticket_tag());
 }
 static int launch_gemv_mma(const DeviceInfo& di, const void* d_meta, const uint8_t* d_blocks, int n_out, int kblocks,
@@ -311,7 +311,7 @@ static int launch_gemv_warp_call(const DeviceInfo& di, const GemvCall& c, void* 
     if (ws_bytes < p.partial_bytes + p.ticket_bytes) return ECCO_ERR_WORKSPACE;
     float* partial = static_cast<float*>(d_ws);
     Ticket* tickets = reinterpret_cast<Ticket*>(static_cast<uint8_t*>(d_ws) + p.partial_bytes);
-    return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(kFusedWarps * 32), kSmemCtaBytes, stream, c.b,
+    return launch_overlapped(kernel, static_cast<unsigned>(p.grid), spread_threads(c.b.units, p.grid, kFusedWarps), kSmemCtaBytes, stream, c.b,
                              partial, tickets, next_ticket_tag());
 }
 template <int kV>
@@ -452,7 +452,7 @@ static int launch_attn(const DeviceInfo& di, const void* d_meta, const uint8_t* 
     // persistent CTAs; the units (32 tokens of a head) are split evenly over the working warps on the device
     const int64_t units = static_cast<int64_t>(heads) * ((seq + 31) / 32);
     const unsigned grid = static_cast<unsigned>(spread_ctas(units, di.sms));
-    return launch_overlapped(kernel, grid, static_cast<unsigned>(kFusedWarps * 32), kSmemCtaBytes, stream, static_cast<const uint8_t*>(d_meta),
+    return launch_overlapped(kernel, grid, spread_threads(units, static_cast<int>(grid), kFusedWarps), kSmemCtaBytes, stream, static_cast<const uint8_t*>(d_meta),
                              d_kblocks, heads, seq, q_per_kv, static_cast<const __half*>(d_q), scale, d_scores);
 }
 
@@ -478,7 +478,7 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
             if (rc) return rc;
             const uint64_t units = static_cast<uint64_t>(batch) * n_kv_heads * ((seq + 31) / 32);
             const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>(units), di.sms));
-            return launch_overlapped(kernel, grid, static_cast<unsigned>(kMmaWarps * 32), kSmemCtaBytes, s, static_cast<const uint8_t*>(d_meta),
+            return launch_overlapped(kernel, grid, spread_threads(static_cast<int64_t>(units), static_cast<int>(grid), kMmaWarps), kSmemCtaBytes, s, static_cast<const uint8_t*>(d_meta),
                                      d_kblocks, batch * n_kv_heads, seq, q_per_kv, static_cast<const __half*>(d_q), scale, d_scores);
         }
     }

@@ -93,6 +93,15 @@ constexpr int gemv_warp_warps(int v) { return v == 1 ? 32 : 28; }
 // filling some SMs and leaving the others idle (decode attention over 2 x 8 x 777 tokens, 400 pieces: 37.6 -> 30.4 us).
 inline int spread_ctas(int64_t units, int ctas_max) { return static_cast<int>(units < ctas_max ? units : ctas_max); }
 
+// Threads of such a CTA: a warp per piece it can get, but no more than the kernel is made for, and at least eight (they share the
+// work of laying out the tables).  Warps without work are not free: they take part in every barrier of the set-up.
+inline unsigned spread_threads(int64_t units, int grid, int max_warps)
+{
+    const int64_t per_cta = (units + grid - 1) / grid;
+    const int64_t warps = per_cta < 8 ? 8 : per_cta < max_warps ? per_cta : max_warps;
+    return static_cast<unsigned>((warps < max_warps ? warps : max_warps) * 32);
+}
+
 struct GemvPlan { int row_tiles, grid; size_t partial_bytes, ticket_bytes; };
 
 // plan of a fused GEMV call over `units` units in `row_tiles` 32-row tiles (all matrices of the call together):
