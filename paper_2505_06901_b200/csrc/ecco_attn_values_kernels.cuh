@@ -46,7 +46,7 @@ __device__ __forceinline__ float rescale(float m, float m_new) { return m == m_n
 template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __restrict__ d_vblocks, int heads, int seq,
-                        int q_per_kv, const float* d_scores, float* __restrict__ d_out, float* __restrict__ d_partial,
+                        int q_per_kv, int unit_warps, const float* d_scores, float* __restrict__ d_out, float* __restrict__ d_partial,
                         Ticket* d_tickets, Ticket tag)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -55,7 +55,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     release_dependents();
     const Tables tb = plan_tables(smem_u32(smem), d_meta, false);   // one symbol per lookup: see the scalar fused kernels
     constexpr uint32_t kFull = 0xffffffffu, kSlotFloats = kGroup * 8 + 8;       // sums, sums of weights
-    const uint32_t nw = warps_that_fit(tb, kAvWarpBytes, kTabBytes / 2 + kAvSlots * kSlotFloats * sizeof(float));
+    const uint32_t nw = min(warps_that_fit(tb, kAvWarpBytes, kTabBytes / 2 + kAvSlots * kSlotFloats * sizeof(float)), static_cast<uint32_t>(unit_warps));
     const int kTokens = static_cast<int>(nw) * 32;         // tokens per unit: one per thread of the working warps
     const bool working = warp < nw;
     // small CTA-wide words in the misc area at the start of shared memory (the barrier word is its first)
@@ -177,19 +177,42 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
             if (ticket == static_cast<unsigned int>(c_hi - c_lo)) {
                 __threadfence();
                 const float* piece = d_partial + static_cast<size_t>(c_lo + bh) * kPieceFloats;
-                const int n = c_hi - c_lo + 1;
-                for (int i = tid; i < kGroup * 8; i += n_threads) {
-                    const float* pw = piece + kGroup * 8 + (i & 7);
-                    float top = -INFINITY, v = 0.0f, weights = 0.0f;
-#pragma unroll 4
-                    for (int k = 0; k < n; ++k) top = fmaxf(top, __ldcg(pw + 8 + static_cast<size_t>(k) * kPieceFloats));
-#pragma unroll 4
-                    for (int k = 0; k < n; ++k) {
+                const int n = c_hi - c_lo + 1;             // at most 256
+                // factor of every piece and head, then the heads' sums of weights: warp h does head h (a CTA has eight warps at least)
+                float *fac = out_s, *weights = out_s + n * 8;
+                if (warp < 8) {
+                    const float* pw = piece + kGroup * 8 + warp;
+                    float top = -INFINITY, sum = 0.0f;
+                    for (int k = lane; k < n; k += 32) top = fmaxf(top, __ldcg(pw + 8 + static_cast<size_t>(k) * kPieceFloats));
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) top = fmaxf(top, __shfl_xor_sync(kFull, top, o));
+                    for (int k = lane; k < n; k += 32) {
                         const float f = rescale(__ldcg(pw + 8 + static_cast<size_t>(k) * kPieceFloats), top);
-                        v += f * __ldcg(piece + i + static_cast<size_t>(k) * kPieceFloats);
-                        weights += f * __ldcg(pw + static_cast<size_t>(k) * kPieceFloats);
+                        fac[k * 8 + warp] = f;
+                        sum += f * __ldcg(pw + static_cast<size_t>(k) * kPieceFloats);
                     }
-                    store(i, v, weights);
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+                    if (lane == 0) weights[warp] = sum;
+                }
+                __syncthreads();
+                for (int i = tid; i < kGroup * 2; i += n_threads) {            // four heads of a dim at a time, eight loads in flight
+                    const float4* from = reinterpret_cast<const float4*>(piece) + i;
+                    const float4* by = reinterpret_cast<const float4*>(fac) + (i & 1);
+                    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    auto add = [&](float4 f, float4 x) { v.x += f.x * x.x; v.y += f.y * x.y; v.z += f.z * x.z; v.w += f.w * x.w; };
+                    int k = 0;
+                    for (; k + 8 <= n; k += 8) {
+                        float4 x[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) x[j] = __ldcg(from + static_cast<size_t>(k + j) * (kPieceFloats / 4));
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) add(by[(k + j) * 2], x[j]);
+                    }
+                    for (; k < n; ++k) add(by[k * 2], __ldcg(from + static_cast<size_t>(k) * (kPieceFloats / 4)));
+                    const float vs[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) store(i * 4 + j, vs[j], weights[(i & 1) * 4 + j]);
                 }
                 if (tid == 0) d_tickets[bh] = 0;
             }

@@ -488,16 +488,30 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
 // ecco_attn_values
 // ---------------------------------------------------------------------------------------------
 namespace {
-// A CTA of ecco_attn_values has 16 warps (512 tokens per unit).  18 find room (10.25 KB of shared memory per warp) but
-// measured no faster on 32768-token rows (602.8 against 600.6 us) and slower on 4096-token rows, whose last unit
-// they leave half empty (99.1 against 89.3 us).
+// At most 16 warps of a CTA of ecco_attn_values decode (512 tokens per unit).  18 find room (10.25 KB of shared memory per
+// warp) but measured no faster on 32768-token rows (602.8 against 600.6 us).
 constexpr int kAvWarps = 16;
-struct AvPlan { int grid; size_t partial_bytes, ticket_bytes; };
+struct AvPlan { int grid, unit_warps; size_t partial_bytes, ticket_bytes; };
+// Warps per unit (a unit is that many 32-token tiles of one head): all SMs should be busy for the same number of turns.  A turn
+// costs about the time of six tiles' decoding however few tiles it has (6, 16 and 40 measured alike), so long rows take the
+// largest units (16 x 8 x 32768 tokens: 16 warps) and short ones are cut until every SM has some.  Against 16 warps throughout:
+// 8 x 32 x 64 tokens 27.1 -> 20.7 us, 2 x 8 x 777 17.4 -> 14.5, 1 x 1 x 32768 39.9 -> 25.5 (with the merge of a head's pieces).
+int av_unit_warps(int heads, int seq, int ctas)
+{
+    const int64_t tiles = (seq + 31) / 32;
+    int best = kAvWarps;
+    int64_t best_cost = INT64_MAX;
+    for (int w = kAvWarps; w >= 1; --w) {
+        const int64_t units = heads * ((tiles + w - 1) / w), cost = (units + ctas - 1) / ctas * (6 + w);
+        if (cost < best_cost) { best = w; best_cost = cost; }
+    }
+    return best;
+}
 AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
 {
     AvPlan p;
     const int heads = batch * n_kv_heads;
-    // at most this many units (fewer when all warps find room); the device splits what there is evenly
+    // at most this many units; the device splits what there is evenly
     p.grid = spread_ctas(static_cast<int64_t>(heads) * ((seq + 31) / 32), ctas_max);
     auto up = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
     p.partial_bytes = up(static_cast<size_t>(p.grid + heads) * kPieceFloats * sizeof(float));
@@ -508,13 +522,16 @@ AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
 template <int kWarps>
 int launch_attn_values(const DeviceInfo& di, const AvPlan& p, const void* d_meta, const uint8_t* d_vblocks, int heads, int seq,
                        int q_per_kv, const float* d_scores, float* d_out, float* partial, Ticket* tickets, cudaStream_t s)
+    p.unit_warps = av_unit_warps(heads, seq, ctas_max);
 {
     auto kernel = ecco_attn_values_kernel<kWarps>;
     static thread_local bool configured[64] = {};
     const int rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
-    return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(kWarps * 32), kSmemCtaBytes, s,
-                             static_cast<const uint8_t*>(d_meta), d_vblocks, heads, seq, q_per_kv, d_scores, d_out, partial, tickets, next_ticket_tag());
+    // at least eight warps: those beyond the unit's help with the reductions
+    const int warps = p.unit_warps < 8 ? 8 : p.unit_warps;
+    return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(warps * 32), kSmemCtaBytes, s,
+                             static_cast<const uint8_t*>(d_meta), d_vblocks, heads, seq, q_per_kv, p.unit_warps, d_scores, d_out, partial, tickets, next_ticket_tag());
 }
 }  // namespace
 

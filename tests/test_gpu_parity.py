@@ -826,6 +826,18 @@ def test_attn_values_with_rising_scores_and_any_workspace(B, eo, kv_small, seq):
     s[0, 2::4, -1] = 80.0
     d_meta, d_blocks, d_s = B.meta_to_device(lib_meta_from_oracle(B, meta)), dev(blocks), dev(s)
     wsb = B.ecco_attn_values_workspace_bytes(1, heads, seq, qpk)
+@pytest.mark.parametrize("batch,heads,seq,qpk", [(1, 1, 31, 8), (1, 1, 6000, 5), (3, 50, 65, 1), (2, 8, 777, 2), (1, 3, 40000, 1)])
+def test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk):
+    """Units of one warp to sixteen; one head in a piece per SM; more short heads than SMs."""
+    meta = kv_small["meta"]
+    n = batch * heads * seq
+    blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
+    scores = (np.random.Generator(np.random.PCG64(seq)).standard_normal((batch, heads * qpk, seq)) * 3).astype(np.float32)
+    got = gpu_attn_values(B, lib_meta_from_oracle(B, meta), blocks, batch, heads, seq, qpk, scores)
+    ref, refabs = eo.attn_values(meta, blocks, batch, heads, seq, qpk, scores)
+    check_fused(got, ref, refabs, "values unit sizes")
+
+
     first = None
     for fill in (0, 0xFF, 0x3C, "left"):
         if fill != "left":
