@@ -191,7 +191,7 @@ int ecco_gemv_batch(const ecco_gemv_item* items, int32_t n_items, int32_t batch,
  * nothing.  A shape whose plan needs more scratch than that is refused with ECCO_ERR_WORKSPACE
  * before anything is launched.  For scale, on a 148-SM part: batch 8 on an 11008 x 4096 matrix needs 3.39 MB, batch 1
  * or 2 on the same matrix 0.65 / 1.2 MB, batch 8 on 28672 x 8192 3.96 MB; a matrix with more than about 65 000 output
- * rows at batch 3..8 does not fit and is refused.
+ * rows at batch 8 does not fit and is refused.
  * The first call on each device looks up the array's device address (with that device current);
  * make that first call outside any stream capture.  All calls on a device share the one array:
  * it still holds the previous call's values when the next call starts (which does not matter to that

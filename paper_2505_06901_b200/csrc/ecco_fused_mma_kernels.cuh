@@ -1,11 +1,11 @@
-// ecco_fused_mma_kernels.cuh -- K2m / K3m: fused GEMV and attention scores for three to eight dot products per group (tensor cores)
+// ecco_fused_mma_kernels.cuh -- K2m / K3m: fused GEMV (six to eight rows) and attention scores (three to eight heads) on the tensor cores
 // Part of the one translation unit ecco_kernels.cu; included from there only.
 #pragma once
 
 namespace {
 
 // ---------------------------------------------------------------------------------------------
-// K2m / K3m: the fused consumers for 3 to 8 dot products per group (rows of x, query heads) on the
+// K2m / K3m: the fused consumers for six to eight rows of x and three to eight query heads on the
 // tensor cores.  With eight products per weight the scalar path spends four shared-memory
 // wavefronts and eight FMAs per symbol on the vector operand alone.  Here a group is decoded once,
 // values and all, into eight [32 rows][16 k] fp16 tiles of the warp (as in K5); when the end bit is
@@ -109,7 +109,7 @@ __device__ __forceinline__ void load_vfrag(uint32_t (&vfrag)[16], const __half* 
     }
 }
 
-// K2m: y[b][n] = sum_k W~[n][k] x[b][k] for 3..8 rows of x.  Units (over all matrices of the call), ownership and the
+// K2m: y[b][n] = sum_k W~[n][k] x[b][k] for six to eight rows of x.  Units (over all matrices of the call), ownership and the
 // slot-and-ticket reduction are those of the per-warp kernel (unit = 32 rows x one k-block).
 template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)

@@ -1,4 +1,4 @@
-// ecco_fused_scalar_kernels.cuh -- K2 / K3: fused GEMV and attention scores for one or two dot products per group
+// ecco_fused_scalar_kernels.cuh -- K2 / K3: fused GEMV (one to five rows of x) and attention scores (one or two heads)
 // Part of the one translation unit ecco_kernels.cu; included from there only.
 #pragma once
 
@@ -47,10 +47,15 @@ __device__ __forceinline__ float rank_value(const LaneGroup& g, uint32_t rank)
     return __half2float(__ushort_as_half(static_cast<unsigned short>(prmt(lo, hi, 0x0040u))));
 }
 
+// partial sums per product: two short chains for one or two products, one chain each for more
+__host__ __device__ constexpr int chains(int v) { return v <= 2 ? 2 : 1; }
+__device__ __forceinline__ float sum_of(const float (&a)[2]) { return a[0] + a[1]; }
+__device__ __forceinline__ float sum_of(const float (&a)[1]) { return a[0]; }
+
 // kDeal: deal_outliers (caches) or every lane its own (weights)
-// decode one group and accumulate its kV dot products against the slice at shared address xs; two partial sums per product
+// decode one group and accumulate its kV dot products against the slice at shared address xs
 template <int kV, bool kDeal>
-__device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, float (&acc)[kV][2])
+__device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, float (&acc)[kV][chains(kV)])
 {
     LaneGroup g = open_block(blk, bits, tb, T);
     if (kDeal) sts_u32(bits + 18 * 128, blk.w[0]);                    // the ranks will lie over the block's first words
@@ -64,10 +69,11 @@ __device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables
         for (int b = 0; b < kV; ++b) {
             uint32_t x[4];
             asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(xs + b * (kGroup * 2) + i * 16));
+            constexpr int kLast = chains(kV) - 1;
             fma_half2(acc[b][0], v[0], x[0]);
-            fma_half2(acc[b][1], v[1], x[1]);
+            fma_half2(acc[b][kLast], v[1], x[1]);
             fma_half2(acc[b][0], v[2], x[2]);
-            fma_half2(acc[b][1], v[3], x[3]);
+            fma_half2(acc[b][kLast], v[3], x[3]);
         }
     });
     // outliers replace the mapped value at their location: add (outlier - mapped) * x.  Rows 24 and 25 behind the block hold the
@@ -202,7 +208,7 @@ __device__ __forceinline__ const uint8_t* gemv_block_ptr(const GemvBatch& batch,
 
 __host__ __device__ constexpr uint32_t scalar_warp_bytes(int v) { return v * kGroup * 2 + kRankedBytes; }
 
-// K2 for one or two rows of x: the slice is small enough (256 B a row) for every warp to keep
+// K2 for one to five rows of x: the slice is small enough (256 B a row) for every warp to keep
 // its own, so warps never meet at a barrier.  A work unit is (32 consecutive rows, one k-block),
 // numbered matrix by matrix, row-tile major; every working warp owns a contiguous run of units and keeps its
 // rows' partial sums in registers along k.  When a row tile is shared by several warps each writes its
@@ -240,10 +246,12 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     if (!finish_decode_tables(tb)) return;
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
 
-    float acc[kV][2];                                      // two partial sums, added when the row tile is left
+    float acc[kV][chains(kV)];                             // partial sums, added when the row tile is left
     auto clear_acc = [&]() {
 #pragma unroll
-        for (int b = 0; b < kV; ++b) acc[b][0] = acc[b][1] = 0.0f;
+        for (int b = 0; b < kV; ++b)
+#pragma unroll
+            for (int i = 0; i < chains(kV); ++i) acc[b][i] = 0.0f;
     };
     clear_acc();
     auto flush = [&](int jf, int tile) {
@@ -258,13 +266,13 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
         if (w_lo == w_hi) {
             if (row_ok) {
 #pragma unroll
-                for (int b = 0; b < kV; ++b) d_y[static_cast<size_t>(b) * n_out + row] = acc[b][0] + acc[b][1];
+                for (int b = 0; b < kV; ++b) d_y[static_cast<size_t>(b) * n_out + row] = sum_of(acc[b]);
             }
             return;
         }
         float* mine = d_partial + static_cast<size_t>(wg + gtile) * kV * 32;
 #pragma unroll
-        for (int b = 0; b < kV; ++b) mine[b * 32 + lane] = acc[b][0] + acc[b][1];
+        for (int b = 0; b < kV; ++b) mine[b * 32 + lane] = sum_of(acc[b]);
         __threadfence();
         __syncwarp();
         unsigned int t = 0;
@@ -404,14 +412,16 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         const int out_bh = bh;
         if (++tile == tiles) { tile = 0; ++bh; }
         if (u + 1 < u1) prefetch_block_l2(block_ptr(bh, tile));
-        float acc[kV][2];
+        float acc[kV][chains(kV)];
 #pragma unroll
-        for (int r = 0; r < kV; ++r) acc[r][0] = acc[r][1] = 0.0f;
+        for (int r = 0; r < kV; ++r)
+#pragma unroll
+            for (int i = 0; i < chains(kV); ++i) acc[r][i] = 0.0f;
         fused_group<kV, true>(cur, tb, bits, T, xs, acc);
         if (t < seq) {
 #pragma unroll
             for (int r = 0; r < kV; ++r)
-                if (r < q_per_kv) d_scores[(static_cast<size_t>(out_bh) * q_per_kv + r) * seq + t] = scale * (acc[r][0] + acc[r][1]);
+                if (r < q_per_kv) d_scores[(static_cast<size_t>(out_bh) * q_per_kv + r) * seq + t] = scale * sum_of(acc[r]);
         }
     }
 }

@@ -25,8 +25,8 @@
 //   ecco_device_core.cuh            shared-memory layout, PTX helpers, table staging, the per-group decoder
 //   ecco_decode_core.cuh            the group decoder with the value table in registers
 //   ecco_decompress_kernels.cuh     ecco_decompress (tile-store and small-tensor kernels), ecco_var_decompress
-//   ecco_fused_scalar_kernels.cuh   fused GEMV / attention scores, one or two dot products per group
-//   ecco_fused_mma_kernels.cuh      the same for three to eight dot products, on the tensor cores
+//   ecco_fused_scalar_kernels.cuh   fused GEMV (one to five rows) / attention scores (one or two heads)
+//   ecco_fused_mma_kernels.cuh      the same for more rows and heads, on the tensor cores
 //   ecco_attn_values_kernels.cuh    softmax(scores) . V over a compressed V cache
 //   ecco_act2x_kernels.cuh          2x activation codec
 //   ecco_kv_compress_kernel.cuh     online 4x compressor
@@ -273,7 +273,7 @@ static void gemv_call_add(GemvCall* c, const void* d_meta, const uint8_t* d_bloc
     c->b.units += static_cast<int64_t>(tiles) * kblocks;
 }
 
-// three to eight rows of x: the tensor-core kernel
+// six to eight rows of x: the tensor-core kernel
 static int launch_gemv_mma_call(const DeviceInfo& di, const GemvCall& c, int batch, void* d_ws, size_t ws_bytes, cudaStream_t stream)
 {
     auto kernel = ecco_gemv_mma_kernel<kMmaWarps>;
@@ -297,7 +297,7 @@ static int launch_gemv_mma(const DeviceInfo& di, const void* d_meta, const uint8
     return launch_gemv_mma_call(di, c, batch, d_ws, ws_bytes, stream);
 }
 
-// one or two rows of x (batch == kV): the per-warp kernel
+// one to five rows of x (batch == kV): the per-warp kernel
 template <int kV>
 static int launch_gemv_warp_call(const DeviceInfo& di, const GemvCall& c, void* d_ws, size_t ws_bytes, cudaStream_t stream)
 {
@@ -338,6 +338,9 @@ extern "C" int ecco_gemv(const void* d_meta, const uint8_t* d_blocks, int32_t n_
     switch (pad_v(batch)) {
         case 1: return launch_gemv_warp<1>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, d_workspace, workspace_bytes, s);
         case 2: return launch_gemv_warp<2>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, d_workspace, workspace_bytes, s);
+        case 3: return launch_gemv_warp<3>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, d_workspace, workspace_bytes, s);
+        case 4: return launch_gemv_warp<4>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, d_workspace, workspace_bytes, s);
+        case 5: return launch_gemv_warp<5>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, d_workspace, workspace_bytes, s);
         default: return launch_gemv_mma(di, d_meta, d_blocks, n_out, kblocks, d_x, batch, d_y, d_workspace, workspace_bytes, s);
     }
 }
@@ -390,6 +393,9 @@ extern "C" int ecco_gemv_batch(const ecco_gemv_item* items, int32_t n_items, int
     switch (pad_v(batch)) {
         case 1: return launch_gemv_warp_call<1>(di, c, d_workspace, workspace_bytes, s);
         case 2: return launch_gemv_warp_call<2>(di, c, d_workspace, workspace_bytes, s);
+        case 3: return launch_gemv_warp_call<3>(di, c, d_workspace, workspace_bytes, s);
+        case 4: return launch_gemv_warp_call<4>(di, c, d_workspace, workspace_bytes, s);
+        case 5: return launch_gemv_warp_call<5>(di, c, d_workspace, workspace_bytes, s);
         default: return launch_gemv_mma_call(di, c, batch, d_workspace, workspace_bytes, s);
     }
 }
@@ -435,6 +441,9 @@ extern "C" int ecco_gemv_static_ws(const void* d_meta, const uint8_t* d_blocks, 
     switch (vpad) {
         case 1: return launch_gemv_warp<1>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, ws, ECCO_STATIC_WORKSPACE_BYTES, s);
         case 2: return launch_gemv_warp<2>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, ws, ECCO_STATIC_WORKSPACE_BYTES, s);
+        case 3: return launch_gemv_warp<3>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, ws, ECCO_STATIC_WORKSPACE_BYTES, s);
+        case 4: return launch_gemv_warp<4>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, ws, ECCO_STATIC_WORKSPACE_BYTES, s);
+        case 5: return launch_gemv_warp<5>(di, d_meta, d_blocks, n_out, kblocks, d_x, d_y, ws, ECCO_STATIC_WORKSPACE_BYTES, s);
         default: return launch_gemv_mma(di, d_meta, d_blocks, n_out, kblocks, d_x, batch, d_y, ws, ECCO_STATIC_WORKSPACE_BYTES, s);
     }
 }
@@ -513,6 +522,7 @@ AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
     const int heads = batch * n_kv_heads;
     // at most this many units; the device splits what there is evenly
     p.grid = spread_ctas(static_cast<int64_t>(heads) * ((seq + 31) / 32), ctas_max);
+    p.unit_warps = av_unit_warps(heads, seq, ctas_max);
     auto up = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
     p.partial_bytes = up(static_cast<size_t>(p.grid + heads) * kPieceFloats * sizeof(float));
     p.ticket_bytes = up(static_cast<size_t>(heads) * sizeof(Ticket));
@@ -522,7 +532,6 @@ AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
 template <int kWarps>
 int launch_attn_values(const DeviceInfo& di, const AvPlan& p, const void* d_meta, const uint8_t* d_vblocks, int heads, int seq,
                        int q_per_kv, const float* d_scores, float* d_out, float* partial, Ticket* tickets, cudaStream_t s)
-    p.unit_warps = av_unit_warps(heads, seq, ctas_max);
 {
     auto kernel = ecco_attn_values_kernel<kWarps>;
     static thread_local bool configured[64] = {};

@@ -86,7 +86,7 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // the device, from the size of the image's tables.
 constexpr int kDecompressWarps = 28;
 constexpr int fused_warps(int v) { return v == 1 ? 32 : 28; }
-constexpr int gemv_warp_warps(int v) { return v == 1 ? 32 : 28; }
+constexpr int gemv_warp_warps(int v) { return v == 1 ? 32 : v <= 3 ? 28 : v == 4 ? 26 : 22; }
 
 // CTAs for `units` warp-sized pieces of work: one per SM as soon as there are that many.  The kernels number their warps
 // across the CTAs first, so a call with fewer pieces than the machine has warp slots puts a few on every SM instead of
@@ -120,13 +120,15 @@ inline GemvPlan gemv_plan(int64_t units, int row_tiles, int warps, int cols, int
 
 constexpr int kMmaWarps = 20;      // 18 find room beside the tables of a typical image (11.25 KB of shared memory per warp)
 
-// the per-warp kernel (one or two rows of x: vpad columns) or the tensor-core kernel (3..8 rows: eight columns)
+// the per-warp kernel (one to five rows of x: vpad columns) or the tensor-core kernel (6..8 rows: eight columns)
+// Per-warp against tensor-core kernel, two 11008 x 4096 matrices in a call: 69 against 86 us at three rows, 81 against 88 at five,
+// 85 against 90 at six, 104 against 91 at eight; 4096 x 4096: 26.1 against 26.3 at five, 28.0 against 26.5 at six.
 inline GemvPlan gemv_plan_for(int64_t units, int row_tiles, int vpad, int ctas_max)
 {
-    return vpad <= 2 ? gemv_plan(units, row_tiles, gemv_warp_warps(vpad), vpad, ctas_max) : gemv_plan(units, row_tiles, kMmaWarps, 8, ctas_max);
+    return vpad <= 5 ? gemv_plan(units, row_tiles, gemv_warp_warps(vpad), vpad, ctas_max) : gemv_plan(units, row_tiles, kMmaWarps, 8, ctas_max);
 }
 
-inline int pad_v(int v) { return v <= 1 ? 1 : v <= 2 ? 2 : v <= 4 ? 4 : 8; }
+inline int pad_v(int v) { return v <= 5 ? v : 8; }
 
 
 }  // namespace

@@ -351,6 +351,20 @@ def test_gemv_handles_pads_clips_and_garbage(B, eo, cfg1_small, synth):
     check_fused(got, ref, refabs, "gemv b2 skewed code")
 
 
+@pytest.mark.parametrize("batch", [3, 4, 5, 6])
+@pytest.mark.parametrize("n_out,k", [(33, 2048), (2047, 512), (4999, 640)])
+def test_gemv_of_three_to_six_rows(B, eo, cfg1_small, synth, batch, n_out, k):
+    """Either side of the line between the per-warp and the tensor-core kernel: one tile of rows split between many warps, and
+    calls with more units than warps, with a ragged last tile."""
+    meta = cfg1_small["meta"]
+    n = n_out * k // 128
+    blocks = np.tile(cfg1_small["blocks"], (-(-n // len(cfg1_small["blocks"])), 1))[:n]
+    x = synth.activations(batch, k, 90 + batch)
+    got, _ = gpu_gemv(B, lib_meta_from_oracle(B, meta), blocks, n_out, k, x, batch)
+    ref, refabs = eo.gemv(meta, blocks, n_out, k, x, batch)
+    check_fused(got, ref, refabs, f"gemv b{batch}")
+
+
 @pytest.mark.parametrize("batch", [1, 2, 3, 8])
 def test_gemv_batch_gives_every_item_what_gemv_gives(B, eo, cfg1_small, synth, batch):
     """Several matrices in one call (shapes that differ in rows and in k, a ragged row count, a one-row matrix, a shared
@@ -812,6 +826,18 @@ def test_attn_values_keeps_small_probabilities(B, eo, kv_small, synth, qpk):
         assert np.all(err[0, 1] <= 2e-5 * refabs[0, 1])    # evenly spread weights: far inside the bound
 
 
+@pytest.mark.parametrize("batch,heads,seq,qpk", [(1, 1, 31, 8), (1, 1, 6000, 5), (3, 50, 65, 1), (2, 8, 777, 2), (1, 3, 40000, 1)])
+def test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk):
+    """Units of one warp to sixteen; one head in a piece per SM; more short heads than SMs."""
+    meta = kv_small["meta"]
+    n = batch * heads * seq
+    blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
+    scores = (np.random.Generator(np.random.PCG64(seq)).standard_normal((batch, heads * qpk, seq)) * 3).astype(np.float32)
+    got = gpu_attn_values(B, lib_meta_from_oracle(B, meta), blocks, batch, heads, seq, qpk, scores)
+    ref, refabs = eo.attn_values(meta, blocks, batch, heads, seq, qpk, scores)
+    check_fused(got, ref, refabs, "values unit sizes")
+
+
 @pytest.mark.parametrize("seq", [33, 700, 3000])
 def test_attn_values_with_rising_scores_and_any_workspace(B, eo, kv_small, seq):
     """Scores that grow along the row (every tile raises the running maximum), fall, or hold their largest value in the last token, over
@@ -826,18 +852,6 @@ def test_attn_values_with_rising_scores_and_any_workspace(B, eo, kv_small, seq):
     s[0, 2::4, -1] = 80.0
     d_meta, d_blocks, d_s = B.meta_to_device(lib_meta_from_oracle(B, meta)), dev(blocks), dev(s)
     wsb = B.ecco_attn_values_workspace_bytes(1, heads, seq, qpk)
-@pytest.mark.parametrize("batch,heads,seq,qpk", [(1, 1, 31, 8), (1, 1, 6000, 5), (3, 50, 65, 1), (2, 8, 777, 2), (1, 3, 40000, 1)])
-def test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk):
-    """Units of one warp to sixteen; one head in a piece per SM; more short heads than SMs."""
-    meta = kv_small["meta"]
-    n = batch * heads * seq
-    blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
-    scores = (np.random.Generator(np.random.PCG64(seq)).standard_normal((batch, heads * qpk, seq)) * 3).astype(np.float32)
-    got = gpu_attn_values(B, lib_meta_from_oracle(B, meta), blocks, batch, heads, seq, qpk, scores)
-    ref, refabs = eo.attn_values(meta, blocks, batch, heads, seq, qpk, scores)
-    check_fused(got, ref, refabs, "values unit sizes")
-
-
     first = None
     for fill in (0, 0xFF, 0x3C, "left"):
         if fill != "left":
