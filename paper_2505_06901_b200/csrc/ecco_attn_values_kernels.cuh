@@ -7,10 +7,8 @@ namespace {
 // ---------------------------------------------------------------------------------------------
 // K5: attention output over a compressed V cache (Eq. 3: softmax(QK^T / sqrt(d_k)) V).
 // out[b][hq][d] = sum_t p[b][hq][t] * V~[b][hq / q_per_kv][t][d] with p = softmax_t(scores).
-// A thread owns one token (one group) as in K3, but here the sum runs over tokens, i.e. across
-// lanes.  The group is decoded once, values and all, into eight [32 tokens][16 dims] fp16 tiles of the
-// warp (the swizzle of the decompress staging tile); when the end bit is known the outliers are
-// written over their positions in the tiles; then every tile is contracted on the tensor cores:
+// A lane owns one token (one group) as in K3, but here the sum runs over tokens, i.e. across lanes: the groups are
+// decoded into tiles (decode_to_tiles), then every tile is contracted on the tensor cores:
 // (V tile)^T [16 dims x 32 tokens] x P^T [32 tokens x 8 heads] with mma.m16n8k16, fp32 accumulators
 // (4 registers per 16 dims, 32 for the 128 dims).  p is split into an fp16 head and an fp16 remainder
 // (two MMAs) so that its rounding does not show.  The result does not depend on scheduling.
@@ -19,22 +17,6 @@ namespace {
 // and accumulators are rescaled when a larger one comes, so the scores are read once and no kernel has to go before this one
 // (a statistics kernel in front cost 25 us on a cache of 128 rows x 8 heads x 32768 scores and 4 us on the shortest rows).
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&a)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
-                 : "r"(addr));
-}
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// eight [32 tokens][16 dims] fp16 tiles, the last of which lies over rows 0..7 of the warp's bit-stream array (see K2m)
-constexpr uint32_t kAvValueBytes = 7 * 1024;
-constexpr uint32_t kAvWarpBytes = kTabBytes / 2 + kAvValueBytes + kBitsBytes;   // half a value table (two warps share one), tiles, bit stream
 constexpr uint32_t kAvSlots = 8;                                            // reduction slots: see flush
 
 constexpr float kProbScale = 32768.0f;                                      // a power of two: exact
@@ -53,28 +35,17 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const int tid = static_cast<int>(threadIdx.x), n_threads = static_cast<int>(blockDim.x);
     release_dependents();
-    const Tables tb = plan_tables(smem_u32(smem), d_meta, false);   // one symbol per lookup: see the scalar fused kernels
+    const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, false);       // one symbol per lookup: the tiles need the room
     constexpr uint32_t kFull = 0xffffffffu, kSlotFloats = kGroup * 8 + 8;       // sums, sums of weights
-    const uint32_t nw = min(warps_that_fit(tb, kAvWarpBytes, kTabBytes / 2 + kAvSlots * kSlotFloats * sizeof(float)), static_cast<uint32_t>(unit_warps));
+    const uint32_t nw = min(decode_warps(tb, kTiledWarpBytes), static_cast<uint32_t>(unit_warps));
     const int kTokens = static_cast<int>(nw) * 32;         // tokens per unit: one per thread of the working warps
     const bool working = warp < nw;
     // small CTA-wide words in the misc area at the start of shared memory (the barrier word is its first)
     unsigned int& ticket = *reinterpret_cast<unsigned int*>(smem + 32);
     float* max_s = reinterpret_cast<float*>(smem + 64);    // [warps][8 heads]
-    static_assert(64 + kMaxWarps * 8 * 4 <= kMiscBytes, "maxima fit the misc area");
-    WarpSmem ws;
-    ws.tab = tab_column<kTabHalf>(tb.warp_base, warp, lane);
-    const uint32_t per_warp = tb.warp_base + tab_bytes<kTabHalf>(nw);
-    const uint32_t vals = per_warp + warp * (kAvValueBytes + kBitsBytes);      // this warp's eight tiles
-    ws.bits = vals + kAvValueBytes + lane * 4;
-    ws.syms = 0;
-    if (working) {
-        sts_u32(ws.bits + 16 * 128, 0u);
-        sts_u32(ws.bits + 17 * 128, 0u);
-    }
-    const uint32_t swz = ((lane >> 2) & 1u) << 4;
-    const uint32_t my_row = vals + lane * 32;
-    float* out_s = reinterpret_cast<float*>(smem + (per_warp - tb.base) + nw * (kAvValueBytes + kBitsBytes));    // slots of [128 dims][8 heads]
+    static_assert(64 + kMaxWarps * 8 * 4 <= kMisc, "maxima fit the misc area");
+    const uint32_t tiles = tb.warp_base + warp * kTiledWarpBytes;
+    float* out_s = reinterpret_cast<float*>(smem + (tb.warp_base - tb.base));  // over the warps' arrays: slots of [128 dims][8 heads]
 
     const int chunks = (seq + kTokens - 1) / kTokens;
     const int64_t U = static_cast<int64_t>(heads) * chunks;
@@ -87,9 +58,9 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         const int bh = static_cast<int>(u / chunks), t = min(static_cast<int>(u % chunks) * kTokens + tid, seq - 1);
         return d_vblocks + (static_cast<uint64_t>(bh) * seq + t) * kBlockBytes;
     };
-    issue_tables(tb, d_meta);
+    issue_decode_tables(tb, d_meta);
     if (u0 < u1 && working) prefetch_block_l2(block_ptr(u0));
-    if (!wait_tables(tb)) return;
+    if (!finish_decode_tables(tb)) return;
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     const float T = tb.T;
     if (tid == 0) {                                        // thread 0 takes the tickets: of the heads at the ends of this CTA's units
@@ -125,7 +96,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     // added in slot order); then either store (this CTA owns the whole head) or hand a piece to the slot-and-ticket reduction.
     auto flush = [&](int bh) {
         if (working && (lane & 3u) == 0) max_s[warp * 8 + (lane >> 2)] = m;
-        __syncthreads();
+        __syncthreads();                                   // every warp is done with its tiles: the slots lie over them
         auto top_of = [&](uint32_t head) {
             float top = max_s[head];
             for (uint32_t w = 1; w < nw; ++w) top = fmaxf(top, max_s[w * 8 + head]);
@@ -269,46 +240,14 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
             if (static_cast<int>(lane) < q_per_kv && nt < seq)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(d_scores + (static_cast<size_t>(nbh) * q_per_kv + lane) * seq + nt));
         }
-        // lanes past the end of the row decode the row's last token again (zeroed below)
-        __syncwarp();                                      // the tiles of the previous token tile have been read
-        const GroupHeader h = open_group<kTabHalf>(cur, tb, ws, T);
-        uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        const uint32_t end = decode_symbols<true, 16, kBlockBits, kFusedFree, kTabHalf>(h, ws, tb.pairs, [&](int n, uint32_t v, uint32_t, bool, uint32_t) {
-            const int slot = (n & 15) >> 1;                // clipped positions arrive as +0
-            if (n & 1) r[slot] = __byte_perm(r[slot], v, 0x5410); else r[slot] = v;
-            if ((n & 15) == 15) {
-                const uint32_t row = my_row + (n >> 4) * 1024;
-                sts_v4(row + swz, r[0], r[1], r[2], r[3]);
-                sts_v4(row + (swz ^ 16u), r[4], r[5], r[6], r[7]);
-            }
-        });
-        // outliers of a complete group replace the mapped values in the tiles (ascending: a later pad overrides an earlier one)
-        const int n_pad = end ? min(kMaxPads, static_cast<int>((kBlockBits - end) / kPadBits)) : 0;
-        for (int j = 0; j < n_pad; ++j) {
-            const uint32_t f = read_pad(ws, j);
-            const uint32_t loc = f & 127u, byte = (loc & 15u) * 2;
-            asm volatile("st.shared.u16 [%0], %1;" ::"r"(my_row + (loc >> 4) * 1024 + ((byte & 16u) ^ swz) + (byte & 15u)),
-                         "h"(static_cast<unsigned short>(f2h_bits(fp8_to_float(f >> 7) * T))) : "memory");
-        }
-        if (__any_sync(0xffffffffu, !valid)) {             // a row's ragged last tile: lanes past its end hold zeros (p is
-            if (!valid) {                                  // zero there, but a decoded value need not be finite)
-#pragma unroll
-                for (int ch = 0; ch < 8; ++ch) {
-                    sts_v4(my_row + ch * 1024, 0u, 0u, 0u, 0u);
-                    sts_v4(my_row + ch * 1024 + 16, 0u, 0u, 0u, 0u);
-                }
-            }
-        }
-        __syncwarp();                                      // tiles complete
-        // per 16-dim chunk: (V tile)^T x P^T on the tensor cores
+        decode_to_tiles<false, true>(cur, tb, tiles, T, valid);                 // past the end of the row: zeros
+        // per 16-dim tile: (V tile)^T x P^T on the tensor cores
+        const uint32_t a_at = tiles + tile_byte((lane >> 4) * 8 + (lane & 7u), ((lane >> 3) & 1u) * 8);
 #pragma unroll
         for (int ch = 0; ch < 8; ++ch) {
             uint32_t a[2][4];
 #pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-                const uint32_t tok = (lane >> 4) * 8 + (lane & 7u) + 16 * ks, half = (lane >> 3) & 1u;
-                ldmatrix_x4_trans(a[ks], vals + ch * 1024 + tok * 32 + ((half ^ ((tok >> 2) & 1u)) << 4));
-            }
+            for (int ks = 0; ks < 2; ++ks) ldmatrix_x4_trans(a[ks], a_at + ch * kTileBytes + ks * 512);     // tokens + 16: the same swizzle
 #pragma unroll
             for (int ks = 0; ks < 2; ++ks) {
                 mma_16816(acc[ch], a[ks], p_hi[2 * ks], p_hi[2 * ks + 1]);

@@ -199,7 +199,13 @@ __device__ __forceinline__ void map_ranks(const LaneGroup& g, uint32_t ranks, ui
     }
 }
 
-// pair-table entry: the tables are read-only while a CTA decodes, so the compiler may move this load
+// table entries: the tables are read-only while a CTA decodes, so the compiler may move these loads
+__device__ __forceinline__ uint32_t lds_shape(uint32_t addr)
+{
+    uint32_t v;
+    asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
 __device__ __forceinline__ uint32_t lds_pair(uint32_t addr)
 {
     uint32_t v;
@@ -219,6 +225,52 @@ __device__ __forceinline__ void cut_values(uint32_t (&v)[4], int n_ok)
     }
 }
 
+// decode_group (below) symbol by symbol through the shape tables, for images without pair tables and for kernels whose arrays leave no room for
+// them: twice the lookups (3.4 wavefronts per symbol of a warp instead of 1.7).
+template <uint32_t kEndBit, int kFreeSteps, class Sink>
+__device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t bits, Sink&& sink, int* n_valid = nullptr)
+{
+    int fit = kGroup;
+    uint32_t q = g.p + 1u;
+    auto step = [&](int i, auto tested) {
+        constexpr bool kTest = decltype(tested)::value;
+        const uint32_t row = bits + (q >> 5) * 128;        // past its end a lane reads whatever follows: see kSlackBytes
+        const uint32_t w0 = lds_u32(row), w1 = lds_u32(row + 128), w2 = lds_u32(row + 256);
+        const uint32_t lo = __funnelshift_r(w0, w1, q), hi = __funnelshift_r(w1, w2, q);
+        uint32_t e[8], x = lo, n = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (j == 4) { x = __funnelshift_rc(lo, hi, n); q += n; n = 0; }    // up to 32 bits
+            e[j] = lds_shape(g.blut ^ ((x >> n) & 0xffu));
+            n += e[j] >> 4;
+        }
+        // ranks are the low nibbles: even and odd symbols side by side in bytes (multiply-adds: the integer pipe is the busier one)
+        const uint32_t ev = (e[6] * 256u + e[4]) * 65536u + (e[2] * 256u + e[0]), od = (e[7] * 256u + e[5]) * 65536u + (e[3] * 256u + e[1]);
+        const uint32_t ranks = (ev & 0x0f0f0f0fu) | ((od * 16u) & 0xf0f0f0f0u);
+        q += n;
+        bool cutting = false;
+        int n_ok = 8;
+        if (kTest && warp_any(q > kEndBit)) {
+            cutting = true;                                // some lane's stream ends in this step: how many of its codewords end by then
+            uint32_t at = q;
+#pragma unroll
+            for (int j = 7; j >= 0; --j) {
+                if (at > kEndBit) n_ok = j;                // positions only grow
+                at -= e[j] >> 4;
+            }
+            if (n_ok < 8) fit = min(fit, 8 * i + n_ok);
+        }
+        sink(i, ranks, cutting, n_ok);
+    };
+#pragma unroll 1
+    for (int i = 0; i < kFreeSteps; i += 2) { step(i, cuda::std::false_type{}); step(i + 1, cuda::std::false_type{}); }
+#pragma unroll 1
+    for (int i = kFreeSteps; i < 16; i += 2) { step(i, cuda::std::true_type{}); step(i + 1, cuda::std::true_type{}); }
+    g.p = q - 1u;
+    if (n_valid) *n_valid = fit;
+    return fit == kGroup ? q : 0u;
+}
+
 // Decodes the 128 symbols of the lane's group, eight per step (Sec. 4.2, Huffman decode), and hands every step's ranks (nibbles,
 // first symbol lowest) to sink(step, ranks, cutting, n_ok).  A codeword that would cross the end bit ends the group: that and
 // all later positions are clipped.  cutting (uniform over the warp) says that some lane may have clipped positions in this step, n_ok how
@@ -226,37 +278,16 @@ __device__ __forceinline__ void cut_values(uint32_t (&v)[4], int n_ok)
 // fitted.  Must be called by all 32 lanes of the warp.
 // kLastRow / kEndBit: last data row of the lane's staged stream (two more rows follow, which read as zero) and the bit at which
 // the stream ends.  kFreeSteps: that many leading steps carry no end test; the caller guarantees that the stream cannot end in them.
-// pairs = false (uniform): one symbol per lookup through the shape table, in every step.
+// pairs = false (uniform): decode_group_by_one.
 template <uint32_t kLastRow, uint32_t kEndBit, int kFreeSteps, class Sink>
 __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink, int* n_valid = nullptr)
 {
+    if (!pairs) return decode_group_by_one<kEndBit, kFreeSteps>(g, bits, sink, n_valid);
     int fit = kGroup;
     // second symbol of an escape entry: its codeword starts 1 + (length of the first) bits into win
     auto resolve = [&](uint32_t e, uint32_t win) {
         const uint32_t b = lds_u8(g.blut ^ ((win >> (1u + (e & 15u))) & 0xffu));
         return (e & 0x078fu) + (b >> 4) + ((b & 15u) << 11);
-    };
-    // one step symbol by symbol, with the end test
-    auto single_step = [&](int i) {
-        uint32_t q = g.p + 1u, ranks = 0;
-        int n_ok = 0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t row = bits + min(q >> 5, kLastRow) * 128;
-            const uint32_t win = __funnelshift_r(lds_u32(row), lds_u32(row + 128), q);
-            uint32_t acc = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t e = lds_u8(g.blut ^ ((win >> acc) & 0xffu));
-                acc += e >> 4;
-                ranks |= (e & 15u) << (16 * h + 4 * j);
-                n_ok += q + acc <= kEndBit ? 1 : 0;        // positions only grow: once over the end, always over it
-            }
-            q += acc;
-        }
-        g.p = q - 1u;
-        if (n_ok < 8) fit = min(fit, 8 * i + n_ok);
-        sink(i, ranks, true, n_ok);
     };
     auto step = [&](int i, auto tested) {
         constexpr bool kTest = decltype(tested)::value;
@@ -315,15 +346,10 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
         g.p += n;
         sink(i, ranks, cutting, n_ok);
     };
-    if (pairs) {
 #pragma unroll 1
-        for (int i = 0; i < kFreeSteps; i += 2) { step(i, cuda::std::false_type{}); step(i + 1, cuda::std::false_type{}); }
+    for (int i = 0; i < kFreeSteps; i += 2) { step(i, cuda::std::false_type{}); step(i + 1, cuda::std::false_type{}); }
 #pragma unroll 1
-        for (int i = kFreeSteps; i < 16; i += 2) { step(i, cuda::std::true_type{}); step(i + 1, cuda::std::true_type{}); }
-    } else {
-#pragma unroll 1
-        for (int i = 0; i < 16; ++i) single_step(i);
-    }
+    for (int i = kFreeSteps; i < 16; i += 2) { step(i, cuda::std::true_type{}); step(i + 1, cuda::std::true_type{}); }
     if (n_valid) *n_valid = fit;
     return fit == kGroup ? g.p + 1u : 0u;
 }

@@ -54,8 +54,10 @@ __device__ __forceinline__ float sum_of(const float (&a)[1]) { return a[0]; }
 
 // kDeal: deal_outliers (caches) or every lane its own (weights)
 // decode one group and accumulate its kV dot products against the slice at shared address xs
+// keep = false: the products are not wanted.  The lanes past the end of a row decode its last group again; with 23 copies of a
+// group of many outliers to deal, one warp held up a whole call (scores of 2 x 8 x 777 tokens 14.6 instead of 9.0 us).
 template <int kV, bool kDeal>
-__device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, float (&acc)[kV][chains(kV)])
+__device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, bool keep, float (&acc)[kV][chains(kV)])
 {
     LaneGroup g = open_block(blk, bits, tb, T);
     if (kDeal) sts_u32(bits + 18 * 128, blk.w[0]);                    // the ranks will lie over the block's first words
@@ -78,7 +80,7 @@ __device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables
     });
     // outliers replace the mapped value at their location: add (outlier - mapped) * x.  Rows 24 and 25 behind the block hold the
     // list and the products.
-    const int n_pad = pads_of(end);
+    const int n_pad = keep ? pads_of(end) : 0;
     if (!kDeal) {
         uint32_t seen = 0;                                 // location mod 32 of the outliers so far
         for (int j = n_pad - 1; j >= 0; --j) {             // the last pad wins on a duplicate location (only corrupt blocks have one)
@@ -165,8 +167,7 @@ struct GemvBatch {
     GemvJob job[kMaxGemvJobs];
 };
 // true (uniformly over the grid) if every matrix of the call carries the tables of the first
-template <class TablesOf>
-__device__ __forceinline__ bool same_tables(const GemvBatch& batch, const TablesOf& tb)
+__device__ __forceinline__ bool same_tables(const GemvBatch& batch, const DecodeTables& tb)
 {
     bool same = true;
     for (int t = 1; t < batch.n; ++t) {
@@ -351,7 +352,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
             prefetch_block_l2(gemv_block_ptr(batch, pos, lane));
             load_x(pos);
         }
-        fused_group<kV, false>(cur, tb, bits, T, xs, acc);
+        fused_group<kV, false>(cur, tb, bits, T, xs, true, acc);
     }
     flush(cur_j, cur_tile);
 }
@@ -417,7 +418,7 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         for (int r = 0; r < kV; ++r)
 #pragma unroll
             for (int i = 0; i < chains(kV); ++i) acc[r][i] = 0.0f;
-        fused_group<kV, true>(cur, tb, bits, T, xs, acc);
+        fused_group<kV, true>(cur, tb, bits, T, xs, t < seq, acc);
         if (t < seq) {
 #pragma unroll
             for (int r = 0; r < kV; ++r)

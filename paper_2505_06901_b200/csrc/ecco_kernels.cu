@@ -26,6 +26,7 @@
 //   ecco_decode_core.cuh            the group decoder with the value table in registers
 //   ecco_decompress_kernels.cuh     ecco_decompress (tile-store and small-tensor kernels), ecco_var_decompress
 //   ecco_fused_scalar_kernels.cuh   fused GEMV (one to five rows) / attention scores (one or two heads)
+//   ecco_group_tiles.cuh            decoded groups as fp16 tiles in shared memory
 //   ecco_fused_mma_kernels.cuh      the same for more rows and heads, on the tensor cores
 //   ecco_attn_values_kernels.cuh    softmax(scores) . V over a compressed V cache
 //   ecco_act2x_kernels.cuh          2x activation codec
@@ -36,6 +37,7 @@
 #include "ecco_decode_core.cuh"
 #include "ecco_decompress_kernels.cuh"
 #include "ecco_fused_scalar_kernels.cuh"
+#include "ecco_group_tiles.cuh"
 #include "ecco_attn_values_kernels.cuh"
 #include "ecco_fused_mma_kernels.cuh"
 #include "ecco_launch.cuh"
@@ -497,8 +499,9 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
 // ecco_attn_values
 // ---------------------------------------------------------------------------------------------
 namespace {
-// At most 16 warps of a CTA of ecco_attn_values decode (512 tokens per unit).  18 find room (10.25 KB of shared memory per
-// warp) but measured no faster on 32768-token rows (602.8 against 600.6 us).
+// At most 16 warps of a CTA of ecco_attn_values decode (512 tokens per unit).  19 find room (9.4 KB of shared memory per
+// warp), but with more than 16 the accumulators no longer fit the registers: scores and values of a [16][8][32768][128] cache 986
+// us with 16, 1011 with 17, 1000 with 18.
 constexpr int kAvWarps = 16;
 struct AvPlan { int grid, unit_warps; size_t partial_bytes, ticket_bytes; };
 // Warps per unit (a unit is that many 32-token tiles of one head): all SMs should be busy for the same number of turns.  A turn
