@@ -17,8 +17,10 @@
 // over a [16][8][32768][128] cache 407.4 -> 351.8 us.
 namespace {
 
-// Shared memory of a CTA: misc words, patterns and codebook records, then the tables of the decode.  The first three fill
-// the gap in front of the pair tables, which are aligned to the widest.
+// Shared memory of a CTA, from its 1 KB-aligned base: misc words (the barrier word first: images come and go, the barrier stays), patterns
+// and codebook records, then the tables of the decode and the arrays of as many warps as find room behind them.  The first three fill
+// the gap in front of the pair tables, which are aligned to the widest.  The sizes come from the image's header, so the kernels are
+// launched with all the shared memory an SM has and lay themselves out once they have read it.
 constexpr uint32_t kMisc = 1024;
 constexpr uint32_t kSmemPat = kMisc;                                 // [64][16] fp16
 constexpr uint32_t kSmemRec = kSmemPat + kPatternBytes;              // [256] x 16 B codebook records, see build_rank_tables
@@ -227,8 +229,9 @@ __device__ __forceinline__ void cut_values(uint32_t (&v)[4], int n_ok)
 
 // decode_group (below) symbol by symbol through the shape tables, for images without pair tables and for kernels whose arrays leave no room for
 // them: twice the lookups (3.4 wavefronts per symbol of a warp instead of 1.7).
-template <uint32_t kEndBit, int kFreeSteps, class Sink>
-__device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t bits, Sink&& sink, int* n_valid = nullptr)
+struct NoRefill {};
+template <uint32_t kEndBit, int kFreeSteps, class Sink, class Refill = NoRefill>
+__device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t bits, Sink&& sink, int* n_valid = nullptr, Refill&& refill = {})
 {
     int fit = kGroup;
     uint32_t q = g.p + 1u;
@@ -261,6 +264,11 @@ __device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t b
             if (n_ok < 8) fit = min(fit, 8 * i + n_ok);
         }
         sink(i, ranks, cutting, n_ok);
+        if constexpr (!cuda::std::is_same_v<cuda::std::remove_reference_t<Refill>, NoRefill>) {
+            uint32_t p = q - 1u;
+            refill(p);
+            q = p + 1u;
+        }
     };
 #pragma unroll 1
     for (int i = 0; i < kFreeSteps; i += 2) { step(i, cuda::std::false_type{}); step(i + 1, cuda::std::false_type{}); }
@@ -279,10 +287,11 @@ __device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t b
 // kLastRow / kEndBit: last data row of the lane's staged stream (two more rows follow, which read as zero) and the bit at which
 // the stream ends.  kFreeSteps: that many leading steps carry no end test; the caller guarantees that the stream cannot end in them.
 // pairs = false (uniform): decode_group_by_one.
-template <uint32_t kLastRow, uint32_t kEndBit, int kFreeSteps, class Sink>
-__device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink, int* n_valid = nullptr)
+// refill(p): called after every step, for a lane that holds a part of its stream only; it may move p, which is LaneGroup::p.
+template <uint32_t kLastRow, uint32_t kEndBit, int kFreeSteps, class Sink, class Refill = NoRefill>
+__device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink, int* n_valid = nullptr, Refill&& refill = {})
 {
-    if (!pairs) return decode_group_by_one<kEndBit, kFreeSteps>(g, bits, sink, n_valid);
+    if (!pairs) return decode_group_by_one<kEndBit, kFreeSteps>(g, bits, sink, n_valid, refill);
     int fit = kGroup;
     // second symbol of an escape entry: its codeword starts 1 + (length of the first) bits into win
     auto resolve = [&](uint32_t e, uint32_t win) {
@@ -345,6 +354,7 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
         }
         g.p += n;
         sink(i, ranks, cutting, n_ok);
+        if constexpr (!cuda::std::is_same_v<cuda::std::remove_reference_t<Refill>, NoRefill>) refill(g.p);
     };
 #pragma unroll 1
     for (int i = 0; i < kFreeSteps; i += 2) { step(i, cuda::std::false_type{}); step(i + 1, cuda::std::false_type{}); }

@@ -208,42 +208,41 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
 // ---------------------------------------------------------------------------------------------
 // K1v: decompress of the variable-length container (groups back to back in one bit stream, start
 // index on the side; nothing clipped, nothing padded).  Same thread-per-group decode and the same
-// TMA tile store as K1; the difference is the front end: a lane copies the 16-byte chunks that
-// cover its group (on average 5) into its column of a 40-row transposed array, masks the bits
-// that belong to the next group, and starts decoding at bit (start mod 128).
+// TMA tile store as K1; the difference is the front end: a lane copies twenty words of the stream, from the 64-bit word in which
+// its group begins, into its column of a transposed array, masks the bits that belong to the next group, and starts
+// decoding at bit (start mod 64).  Groups of weights take 503 bits, and one in ten thousand does not fit; such a lane
+// fetches again from where it has got to, in the middle of the group, and so does one that has run past its group's end
+// (a corrupt index), for zeros.  A column of 24 rows instead of the 40 that the longest group covers is what leaves
+// room for 28 warps beside the pair tables, hence one round of tiles where 19 warps would need two.  Against one symbol per lookup
+// and a value table in shared memory: 131 072 groups of weights 19.9 -> 14.8 us, of which the memory traffic is 6.5.
 // ---------------------------------------------------------------------------------------------
-constexpr uint32_t kVarRows = 40;                        // 10 chunks: 127 + 1046 bits at most, plus slack
+constexpr uint32_t kVarBits = 640;                       // of the stream at a time
+constexpr uint32_t kVarRows = kVarBits / 32 + 4;         // and four zero rows: how far a step that starts inside the data may read
 constexpr uint32_t kVarBitsBytes = kVarRows * 128;
-
-constexpr uint32_t kVarWarpBytes = kTabBytes / 2 + 1024 + kVarBitsBytes;
+constexpr uint32_t kVarWarpBytes = 1024 + kVarBitsBytes;
 
 template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_var_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint4* __restrict__ d_stream,
-                           const uint64_t* __restrict__ d_index, uint64_t n_groups, uint16_t* __restrict__ d_out,
+                           const uint64_t* __restrict__ d_index, uint64_t n_groups,
                            const __grid_constant__ CUtensorMap out_map)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
 
     release_dependents();
-    // one symbol per lookup: a warp's 40-row stream array takes 5 KB, and 28 warps beside the shape tables measured
-    // as fast as 20 beside the pair tables
-    const Tables tb = plan_tables(smem_u32(smem), d_meta, false);
-    const uint32_t nw = warps_that_fit(tb, kVarWarpBytes, kTabBytes / 2);
-    WarpSmem ws;
-    ws.tab = tab_column<kTabHalf>(tb.warp_base, warp, lane);
-    const uint32_t stage = tb.warp_base + tab_bytes<kTabHalf>(nw) + warp * 1024;
-    ws.bits = stage + (nw - warp) * 1024 + warp * kVarBitsBytes + lane * 4;
-    ws.syms = 0;
+    const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, true);
+    const uint32_t tiles_base = (tb.warp_base + 1023u) & ~1023u;
+    const uint32_t nw = decode_warps(tb, kVarWarpBytes, tiles_base - tb.warp_base);
+    const uint32_t stage = tiles_base + warp * 1024;
+    const uint32_t bits = tiles_base + nw * 1024 + warp * kVarBitsBytes + lane * 4;
     if (warp < nw)
-        for (uint32_t r = 0; r < kVarRows; ++r) sts_u32(ws.bits + r * 128, 0u);
+        for (uint32_t r = kVarBits / 32; r < kVarRows; ++r) sts_u32(bits + r * 128, 0u);
     const uint32_t swz = ((lane >> 2) & 1u) << 4;
     const uint32_t my_row = stage + lane * 32;
-    issue_tables(tb, d_meta);
+    issue_decode_tables(tb, d_meta);
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     const uint64_t total_bits = d_index[0];
-    const uint64_t stream_chunks = (total_bits + 127) >> 7;
     const uint64_t* chunk_base = d_index + 1;
     const uint32_t* off32 = reinterpret_cast<const uint32_t*>(d_index + 1 + var_chunks(n_groups));
     auto start_of = [&](uint64_t g) { return g < n_groups ? chunk_base[g >> kVarChunkShift] + off32[g] : total_bits; };
@@ -252,84 +251,91 @@ ecco_var_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint4* __re
     const uint64_t tile_stride = balanced_warps(n_tiles, gridDim.x * nw);
     uint64_t tile = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x;
     if (warp >= nw || tile >= tile_stride) tile = n_tiles;
-    uint32_t dirty_rows = 0;                               // rows of this lane's column that hold a previous group
 
     // The span of a group comes from the index and its chunks from the stream: two dependent trips to memory.
-    // Both are fetched one tile ahead, the first kVarAhead chunks into registers (an average group covers five),
-    // the rare rest when the tile is staged.
-    constexpr uint32_t kVarAhead = 6;
-    struct Span { uint64_t start, end, c0; uint32_t nc; };
+    // The span is fetched one tile ahead and its chunks are sent for, into L2.
+    struct Span { const uint2* at; uint32_t first, end; };               // first 64-bit word; bits in it before the group, and up to its end
     auto span_of = [&](uint64_t t) {
-        Span sp;
         const uint64_t g = min(t * 32 + lane, n_groups - 1);
-        sp.start = min(start_of(g), total_bits);
-        sp.end = max(min(start_of(g + 1), total_bits), sp.start);          // the group sees [start, end), zeros after
-        sp.c0 = sp.start >> 7;
-        sp.nc = static_cast<uint32_t>(min(static_cast<uint64_t>(kVarRows / 4), ((sp.end + 127) >> 7) - sp.c0));
+        const uint64_t from = min(start_of(g), total_bits);
+        const uint64_t to = max(min(start_of(g + 1), total_bits), from);   // the group sees [from, to), zeros after
+        const uint64_t w0 = from >> 6;
+        Span sp;
+        sp.at = reinterpret_cast<const uint2*>(d_stream) + w0;
+        sp.first = static_cast<uint32_t>(from & 63u);
+        sp.end = static_cast<uint32_t>(min(to - (w0 << 6), static_cast<uint64_t>(2048)));      // the longest group ends by 63 + 1046
+        // groups lie back to back: the lanes' two sectors each cover the stream but for single sectors of long groups
+        if (sp.end) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(sp.at));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(sp.at + ((sp.end - 1u) >> 7)));
+        }
         return sp;
     };
-    auto load_chunk = [&](uint64_t c) {
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (c < stream_chunks) asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(d_stream + c));
-        return v;
-    };
-    Span cur = {0, 0, 0, 0};
-    uint4 ahead[kVarAhead];
-    if (tile < n_tiles) {
-        cur = span_of(tile);
-#pragma unroll
-        for (uint32_t c = 0; c < kVarAhead; ++c) ahead[c] = c < cur.nc ? load_chunk(cur.c0 + c) : make_uint4(0, 0, 0, 0);
-    }
-
-    if (!wait_tables(tb)) return;
+    Span cur = {nullptr, 0, 0};
+    if (tile < n_tiles) cur = span_of(tile);
+    if (!finish_decode_tables(tb)) return;
     const float T = tb.T;
 
     for (; tile < n_tiles; tile += tile_stride) {
-        const uint64_t end = cur.end;
-        const uint64_t c0 = cur.c0;
-        const uint32_t nc = cur.nc;
-        const uint32_t first_bit = static_cast<uint32_t>(cur.start & 127u);
-        auto stage_chunk = [&](uint32_t c, const uint4& v) {
-            uint32_t w[4] = {v.x, v.y, v.z, v.w};
-            const uint64_t first = (c0 + c) << 7;          // stream bit of w[0] bit 0
-            if (first + 128 > end) {                       // bits of the next group read as zero
+        Span sp = cur;
+        uint32_t limit = 0;                                // a lane that starts a step behind this bit fetches first
+        auto fill = [&]() {
+            // whole 16-byte chunks are loaded: from half a chunk earlier, and half a chunk more, if the first word is a chunk's second
+            const uint32_t odd = (reinterpret_cast<uintptr_t>(sp.at) >> 3) & 1u, end = sp.end ? sp.end + odd * 64u : 0u;
+            const uint2* from = sp.at - odd;
+            const uint32_t to = bits - odd * 256u;
+            uint4 ch[kVarBits / 128 + 1];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint64_t wb = first + 32 * k;
-                    w[k] = wb >= end ? 0u : (end - wb >= 32 ? w[k] : (w[k] & ((1u << static_cast<uint32_t>(end - wb)) - 1u)));
-                }
+            for (uint32_t c = 0; c <= kVarBits / 128; ++c) {
+                ch[c] = make_uint4(0, 0, 0, 0);
+                if (c * 128 < end && (c < kVarBits / 128 || odd))
+                    asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(ch[c].x), "=r"(ch[c].y), "=r"(ch[c].z), "=r"(ch[c].w) : "l"(from + 2 * c));
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) sts_u32(ws.bits + (4 * c + k) * 128, w[k]);
+            for (uint32_t c = 0; c <= kVarBits / 128; ++c) {
+                uint32_t w[4] = {ch[c].x, ch[c].y, ch[c].z, ch[c].w};
+                if (end < c * 128 + 128) {                 // bits of the next group read as zero
+#pragma unroll
+                    for (uint32_t k = 0; k < 4; ++k) {
+                        uint32_t drop;                     // shl: amounts above 31 give zero
+                        asm("shl.b32 %0, -1, %1;" : "=r"(drop) : "r"(static_cast<uint32_t>(max(static_cast<int>(end) - static_cast<int>(c * 128 + 32 * k), 0))));
+                        w[k] &= ~drop;
+                    }
+                }
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k) {
+                    const uint32_t r = 4 * c + k;
+                    if (r < 2 ? !odd : r < kVarBits / 32 || (odd && r < kVarBits / 32 + 2)) sts_u32(to + r * 128, w[k]);
+                }
+            }
+            // a step takes 64 bits at most, from the position p + 1 on
+            limit = sp.end > kVarBits ? kVarBits - 65u : sp.end;
         };
-#pragma unroll
-        for (uint32_t c = 0; c < kVarAhead; ++c)
-            if (c < nc) stage_chunk(c, ahead[c]);
-        for (uint32_t c = kVarAhead; c < nc; ++c) stage_chunk(c, load_chunk(c0 + c));
-        const uint64_t tn = tile + tile_stride;
-        if (tn < n_tiles) {                                // the next tile's span and first chunks, in flight during this decode
-            cur = span_of(tn);
-#pragma unroll
-            for (uint32_t c = 0; c < kVarAhead; ++c) ahead[c] = c < cur.nc ? load_chunk(cur.c0 + c) : make_uint4(0, 0, 0, 0);
-        }
-        for (uint32_t r = 4 * nc; r < dirty_rows; ++r) sts_u32(ws.bits + r * 128, 0u);
-        dirty_rows = 4 * nc;
-        const uint32_t hw = first_bit >> 5;
-        const uint32_t hdr = __funnelshift_r(lds_u32(ws.bits + hw * 128), lds_u32(ws.bits + hw * 128 + 128), first_bit);
-        const GroupHeader h = open_header<kTabHalf>(hdr, first_bit, tb, ws, T);
+        fill();
+        const uint32_t first = sp.first;
+        if (tile + tile_stride < n_tiles) cur = span_of(tile + tile_stride);
+        const uint32_t hdr = __funnelshift_r(lds_u32(bits + (first >> 5) * 128), lds_u32(bits + (first >> 5) * 128 + 128), first);
+        LaneGroup lg = open_lane_group(hdr, first, tb, T);
         const int row0 = static_cast<int>(tile * 32);
-        uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        decode_symbols<true, kVarRows - 2, kVarRows * 32, 28, kTabHalf>(h, ws, tb.pairs, [&](int n, uint32_t v, uint32_t, bool, uint32_t) {
-            const int slot = (n & 15) >> 1;
-            if (n & 1) r[slot] |= v << 16; else r[slot] = v;
-            if ((n & 15) == 15) {
+        decode_group<kVarRows - 3, kVarRows * 32, 16>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool, int) {
+            uint32_t v[4];
+            map_ranks(lg, ranks, v);
+            if (!(i & 1)) {
                 if (lane == 0) bulk_wait_read0();          // the engine has read the previous tile
                 __syncwarp();
-                sts_v4(my_row + swz, r[0], r[1], r[2], r[3]);
-                sts_v4(my_row + (swz ^ 16u), r[4], r[5], r[6], r[7]);
+                sts_v4(my_row + swz, v[0], v[1], v[2], v[3]);
+            } else {
+                sts_v4(my_row + (swz ^ 16u), v[0], v[1], v[2], v[3]);
                 fence_async_smem();
                 __syncwarp();
-                if (lane == 0) { tma_store_2d(&out_map, stage, (n >> 4) * 16, row0); bulk_commit(); }
+                if (lane == 0) { tma_store_2d(&out_map, stage, i * 8 - 8, row0); bulk_commit(); }
+            }
+        }, nullptr, [&](uint32_t& p) {
+            if (p > limit) {
+                sp.at += p >> 6;
+                sp.end -= min(sp.end, p & ~63u);
+                p &= 63u;
+                fill();
             }
         });
     }

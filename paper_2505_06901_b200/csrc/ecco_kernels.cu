@@ -6,23 +6,18 @@
 // groups, not inside a group.  The lanes of a warp advance symbol by symbol in lock step, which
 // keeps every per-symbol index (output position, activation element) uniform across the warp.
 //
-// Shared memory per CTA (sizes from the image's header, see ecco_device_core.cuh; ecco_decompress keeps the values in
-// registers, see ecco_decode_core.cuh):
-//   tables   pattern[64][16] fp16 | ID_KP table [4096] u16 | codebook records [256] x 16 B | shape tables
-//            [n_shapes][256] u8 | pair tables, brought in by three bulk copies (cp.async.bulk + mbarrier)
-//   per warp tab[16][32]  u32   per-lane dequantised centroids in rank order (the rank of the abs-max symbol
-//                               holds the abs-max); fp32 in the scalar fused kernels, fp16 with two warps to an
-//                               array elsewhere
-//            bits[18][32] u32   the warp's 32 blocks, word-transposed: lane L's word w at
+// Shared memory per CTA (sizes from the image's header, see ecco_decode_core.cuh):
+//   tables   pattern[64][16] fp16 | codebook records [256] x 16 B | pair tables | ID_KP table [4096] u16 | centroids in rank order
+//            [256][16] fp16 | shape tables [n_shapes][256] u8; all but the centroids are brought in by bulk copies (cp.async.bulk + mbarrier)
+//   per warp bits[19][32] u32   the warp's 32 blocks, word-transposed: lane L's word w at
 //                               [w][L] -> bank L whatever w is (conflict-free refills);
-//                               rows 16 and 17 stay zero (stream bits past 512 read as 0)
-//            syms[16][32] u32   (scalar fused kernels) decoded ranks, 8 nibbles per word, for the
-//                               outlier fix-up
+//                               rows 16 to 18 stay zero (stream bits past 512 read as 0).  The scalar fused kernels keep the decoded
+//                               ranks over its consumed rows, for the outlier fix-up
 //            tiles              ecco_decompress: one [32 groups][16 values] fp16 staging tile for the tensor stores;
 //                               tensor-core kernels: eight of them, the whole decoded group, as MMA operands
 //
 // Layout of the sources (one translation unit; the .cuh files are included here and nowhere else):
-//   ecco_device_core.cuh            shared-memory layout, PTX helpers, table staging, the per-group decoder
+//   ecco_device_core.cuh            PTX helpers, bounded waits, overlapped launches
 //   ecco_decode_core.cuh            the group decoder with the value table in registers
 //   ecco_decompress_kernels.cuh     ecco_decompress (tile-store and small-tensor kernels), ecco_var_decompress
 //   ecco_fused_scalar_kernels.cuh   fused GEMV (one to five rows) / attention scores (one or two heads)
@@ -238,7 +233,7 @@ extern "C" int ecco_var_decompress(const void* d_meta, const uint8_t* d_stream, 
     const unsigned grid = static_cast<unsigned>(spread_ctas(static_cast<int64_t>((n_groups + 31) / 32), di.sms));
     return launch_overlapped(kernel, grid, spread_threads(static_cast<int64_t>((n_groups + 31) / 32), static_cast<int>(grid), kVarWarps), kSmemCtaBytes, static_cast<cudaStream_t>(stream),
                              static_cast<const uint8_t*>(d_meta), reinterpret_cast<const uint4*>(d_stream),
-                             static_cast<const uint64_t*>(d_index), n_groups, static_cast<uint16_t*>(d_out), map);
+                             static_cast<const uint64_t*>(d_index), n_groups, map);
 }
 
 extern "C" size_t ecco_gemv_workspace_bytes(int32_t n_out, int32_t k, int32_t batch)

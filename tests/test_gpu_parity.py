@@ -1034,6 +1034,24 @@ def test_var_decompress_is_total_on_garbage(B, eo, cfg1_small, synth):
     assert_bit_exact(got, eo.var_decode(meta, stream, np.concatenate([starts, [np.uint64(total)]]).astype(np.uint64)))
 
 
+@pytest.mark.parametrize("long_share", [0.0, 0.03, 1.0])
+def test_var_decompress_groups_longer_than_a_lane_holds(B, eo, cfg1_small, synth, long_share):
+    """A lane stages 640 bits of the stream; longer groups (values from the rare, long codewords of the ends of the range) are
+    fetched in two parts, in some lanes of a warp or in all.  Exact: decoding has one result."""
+    lm = lib_meta_from_oracle(B, cfg1_small["meta"])
+    n = 1000 + 7
+    rng = np.random.Generator(np.random.PCG64(31))
+    w = synth.weight_matrix(128, 1024, 9).reshape(-1, 128)[:n].astype(np.float32)
+    ends = rng.choice([-1.0, 1.0], (n, 128)) * rng.uniform(0.6, 1.0, (n, 128)) * np.abs(w).max(1, keepdims=True)
+    x = np.where(rng.random((n, 1)) < long_share, ends, w).astype(np.float16)
+    stream, index, total = B.ecco_var_encode_host(lm, x, B.SELECT_MSE | B.KEEP_EXPONENT)
+    offs = oracle_offsets_from_index(index, n).astype(np.int64)
+    covered = np.diff(offs) + offs[:n] % 64
+    assert (covered > 640).mean() >= 0.4 * long_share
+    got = gpu_var_decompress(B, lm, stream, index, n)
+    assert_bit_exact(got, eo.var_decode(cfg1_small["meta"], stream, oracle_offsets_from_index(index, n)))
+
+
 def test_var_decompress_config2_gate_full_size(B, eo, W, synth):
     (t,) = W.config2(names=("gate",), keep_source=True)
     stream, index, total = B.ecco_var_encode_host(t.meta, t.source, B.SELECT_MSE | B.KEEP_EXPONENT)
