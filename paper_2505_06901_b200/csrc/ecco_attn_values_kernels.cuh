@@ -28,32 +28,44 @@ __device__ __forceinline__ float rescale(float m, float m_new) { return m == m_n
 template <int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __restrict__ d_vblocks, int heads, int seq,
-                        int q_per_kv, int unit_warps, const float* d_scores, float* __restrict__ d_out, float* __restrict__ d_partial,
+                        int q_per_kv, int unit_warps, int n_teams, const float* d_scores, float* __restrict__ d_out, float* __restrict__ d_partial,
                         Ticket* d_tickets, Ticket tag)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const int tid = static_cast<int>(threadIdx.x), n_threads = static_cast<int>(blockDim.x);
     release_dependents();
     const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, false);       // one symbol per lookup: the tiles need the room
     constexpr uint32_t kFull = 0xffffffffu, kSlotFloats = kGroup * 8 + 8;       // sums, sums of weights
-    const uint32_t nw = min(decode_warps(tb, kTiledWarpBytes), static_cast<uint32_t>(unit_warps));
+    // A team of nw warps takes a head at a time.  One team: all CTAs share the units, and the CTA's other warps help with the
+    // reductions.  Several: every team has whole heads of its own and meets at a barrier of its own.
+    const uint32_t fit = decode_warps(tb, kTiledWarpBytes), nw = min(fit, static_cast<uint32_t>(unit_warps));
+    const uint32_t teams = min(static_cast<uint32_t>(n_teams), fit / nw), team = teams > 1 ? warp / nw : 0;
+    const int tid = static_cast<int>(threadIdx.x - team * nw * 32u), n_threads = static_cast<int>(teams > 1 ? nw * 32u : blockDim.x);
+    auto team_sync = [&]() {
+        if (teams == 1) __syncthreads();
+        else if (nw == 1) __syncwarp();                    // up to sixteen teams: more than there are barriers beside the CTA's
+        else asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(nw * 32u) : "memory");
+    };
     const int kTokens = static_cast<int>(nw) * 32;         // tokens per unit: one per thread of the working warps
-    const bool working = warp < nw;
+    const bool working = warp < (teams > 1 ? teams * nw : nw);
     // small CTA-wide words in the misc area at the start of shared memory (the barrier word is its first)
     unsigned int& ticket = *reinterpret_cast<unsigned int*>(smem + 32);
     float* max_s = reinterpret_cast<float*>(smem + 64);    // [warps][8 heads]
     static_assert(64 + kMaxWarps * 8 * 4 <= kMisc, "maxima fit the misc area");
     const uint32_t tiles = tb.warp_base + warp * kTiledWarpBytes;
-    float* out_s = reinterpret_cast<float*>(smem + (tb.warp_base - tb.base));  // over the warps' arrays: slots of [128 dims][8 heads]
+    // over the team's arrays: slots of [128 dims][8 heads]
+    float* out_s = reinterpret_cast<float*>(smem + (tb.warp_base - tb.base) + team * nw * kTiledWarpBytes);
+    const uint32_t first_warp = team * nw;
 
     const int chunks = (seq + kTokens - 1) / kTokens;
     const int64_t U = static_cast<int64_t>(heads) * chunks;
     // the CTAs that share a head count each other in (ticket), so every CTA of the split must own a unit: the
     // launch may bring more CTAs than there are units (the host does not know how many warps find room)
     const int G = static_cast<int>(min(static_cast<int64_t>(gridDim.x), U)), c = blockIdx.x;
-    if (c >= G) return;
-    const int64_t u0 = unit_begin(U, G, c), u1 = unit_begin(U, G, c + 1);
+    if (teams == 1 && c >= G) return;
+    const int all_teams = static_cast<int>(gridDim.x * teams), my_team = static_cast<int>(team * gridDim.x) + c;
+    const int64_t u0 = teams > 1 ? unit_begin(heads, all_teams, my_team) * chunks : unit_begin(U, G, c);
+    const int64_t u1 = teams > 1 ? unit_begin(heads, all_teams, my_team + 1) * chunks : unit_begin(U, G, c + 1);
     auto block_ptr = [&](int64_t u) {
         const int bh = static_cast<int>(u / chunks), t = min(static_cast<int>(u % chunks) * kTokens + tid, seq - 1);
         return d_vblocks + (static_cast<uint64_t>(bh) * seq + t) * kBlockBytes;
@@ -62,8 +74,9 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     if (u0 < u1 && working) prefetch_block_l2(block_ptr(u0));
     if (!finish_decode_tables(tb)) return;
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
+    if (teams > 1 && (!working || u0 >= u1)) return;
     const float T = tb.T;
-    if (tid == 0) {                                        // thread 0 takes the tickets: of the heads at the ends of this CTA's units
+    if (teams == 1 && tid == 0) {                                        // thread 0 takes the tickets: of the heads at the ends of this CTA's units
         Ticket* const ends[2] = {d_tickets + u0 / chunks, d_tickets + (u1 - 1) / chunks};
         const Ticket seen[2] = {look_at_ticket(ends[0]), look_at_ticket(ends[1])};
         claim_ticket(ends[0], seen[0], tag);
@@ -96,16 +109,17 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     // added in slot order); then either store (this CTA owns the whole head) or hand a piece to the slot-and-ticket reduction.
     auto flush = [&](int bh) {
         if (working && (lane & 3u) == 0) max_s[warp * 8 + (lane >> 2)] = m;
-        __syncthreads();                                   // every warp is done with its tiles: the slots lie over them
+        team_sync();                                   // every warp is done with its tiles: the slots lie over them
         auto top_of = [&](uint32_t head) {
-            float top = max_s[head];
-            for (uint32_t w = 1; w < nw; ++w) top = fmaxf(top, max_s[w * 8 + head]);
+            float top = max_s[first_warp * 8 + head];
+            for (uint32_t w = 1; w < nw; ++w) top = fmaxf(top, max_s[(first_warp + w) * 8 + head]);
             return top;
         };
         if (working) rescale_to(top_of(lane >> 2));
         for (uint32_t first = 0; first < nw; first += kAvSlots) {
-            if (warp >= first && warp < first + kAvSlots && warp < nw) {
-                float* slot = out_s + (warp - first) * kSlotFloats;
+            const uint32_t w = warp - first_warp;
+            if (w >= first && w < first + kAvSlots && w < nw) {
+                float* slot = out_s + (w - first) * kSlotFloats;
 #pragma unroll
                 for (int ch = 0; ch < 8; ++ch)
 #pragma unroll
@@ -122,7 +136,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
                     *at = first ? *at + s : s;
                 }
             }
-            __syncthreads();
+            team_sync();
         }
         const uint32_t used = min(nw, kAvSlots);
         for (int i = tid; i < static_cast<int>(kSlotFloats); i += n_threads) {
@@ -130,9 +144,9 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
             for (uint32_t sl = 1; sl < used; ++sl) sum += out_s[sl * kSlotFloats + i];
             out_s[i] = sum;
         }
-        __syncthreads();
-        const int c_lo = unit_owner(U, G, static_cast<int64_t>(bh) * chunks);
-        const int c_hi = unit_owner(U, G, static_cast<int64_t>(bh + 1) * chunks - 1);
+        team_sync();
+        const int c_lo = teams > 1 ? 0 : unit_owner(U, G, static_cast<int64_t>(bh) * chunks);
+        const int c_hi = teams > 1 ? 0 : unit_owner(U, G, static_cast<int64_t>(bh + 1) * chunks - 1);
         auto store = [&](int i, float v, float weights) {
             if ((i & 7) < q_per_kv) d_out[(static_cast<size_t>(bh) * q_per_kv + (i & 7)) * kGroup + (i >> 3)] = v / weights;
         };
@@ -142,9 +156,9 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
             float* mine = d_partial + static_cast<size_t>(c + bh) * kPieceFloats;
             for (int i = tid; i < kPieceFloats; i += n_threads) mine[i] = i < kGroup * 8 + 8 ? out_s[i] : top_of(i & 7);
             __threadfence();
-            __syncthreads();
+            team_sync();
             if (tid == 0) ticket = take_ticket(&d_tickets[bh]);
-            __syncthreads();
+            team_sync();
             if (ticket == static_cast<unsigned int>(c_hi - c_lo)) {
                 __threadfence();
                 const float* piece = d_partial + static_cast<size_t>(c_lo + bh) * kPieceFloats;
@@ -166,7 +180,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
                     for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
                     if (lane == 0) weights[warp] = sum;
                 }
-                __syncthreads();
+                team_sync();
                 for (int i = tid; i < kGroup * 2; i += n_threads) {            // four heads of a dim at a time, eight loads in flight
                     const float4* from = reinterpret_cast<const float4*>(piece) + i;
                     const float4* by = reinterpret_cast<const float4*>(fac) + (i & 1);
@@ -188,13 +202,13 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
                 if (tid == 0) d_tickets[bh] = 0;
             }
         }
-        __syncthreads();
+        team_sync();
     };
 
     int cur_bh = -1;
     for (int64_t u = u0; u < u1; ++u) {
         const int bh = static_cast<int>(u / chunks);
-        const int tile_base = static_cast<int>(u % chunks) * kTokens + static_cast<int>(warp) * 32;
+        const int tile_base = static_cast<int>(u % chunks) * kTokens + static_cast<int>(warp - first_warp) * 32;
         const bool valid = tile_base + static_cast<int>(lane) < seq;
         if (bh != cur_bh) {
             if (cur_bh >= 0) { flush(cur_bh); clear_acc(); }
@@ -236,7 +250,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         if (u + 1 < u1) {
             prefetch_block_l2(block_ptr(u + 1));
             // the scores of this warp's tokens in the next unit, one 128-byte line per query head: into L2 now
-            const int nbh = static_cast<int>((u + 1) / chunks), nt = static_cast<int>((u + 1) % chunks) * kTokens + static_cast<int>(warp) * 32;
+            const int nbh = static_cast<int>((u + 1) / chunks), nt = static_cast<int>((u + 1) % chunks) * kTokens + static_cast<int>(warp - first_warp) * 32;
             if (static_cast<int>(lane) < q_per_kv && nt < seq)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(d_scores + (static_cast<size_t>(nbh) * q_per_kv + lane) * seq + nt));
         }

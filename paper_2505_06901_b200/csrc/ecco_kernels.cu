@@ -498,21 +498,33 @@ namespace {
 // warp), but with more than 16 the accumulators no longer fit the registers: scores and values of a [16][8][32768][128] cache 986
 // us with 16, 1011 with 17, 1000 with 18.
 constexpr int kAvWarps = 16;
-struct AvPlan { int grid, unit_warps; size_t partial_bytes, ticket_bytes; };
-// Warps per unit (a unit is that many 32-token tiles of one head): all SMs should be busy for the same number of turns.  A turn
+struct AvPlan { int grid, unit_warps, teams; size_t partial_bytes, ticket_bytes; };
+// How a CTA's warps share the work.  A unit is unit_warps tiles (of 32 tokens) of one head.
+// One team: the units of all heads are split evenly over the CTAs, and all SMs should be busy for the same number of turns.  A turn
 // costs about the time of six tiles' decoding however few tiles it has (6, 16 and 40 measured alike), so long rows take the
 // largest units (16 x 8 x 32768 tokens: 16 warps) and short ones are cut until every SM has some.  Against 16 warps throughout:
-// 8 x 32 x 64 tokens 27.1 -> 20.7 us, 2 x 8 x 777 17.4 -> 14.5, 1 x 1 x 32768 39.9 -> 25.5 (with the merge of a head's pieces).
-int av_unit_warps(int heads, int seq, int ctas)
+// 8 x 32 x 64 tokens 27.1 -> 22.2 us, 2 x 8 x 777 17.4 -> 15.9, 1 x 1 x 32768 39.9 -> 25.5.
+// Several teams of warps, each with heads of its own, for many short rows: one team spends 5 us on every head's reduction, most of it
+// waiting, and the warps beyond the row's few tiles have nothing to do.  Against one team: 32 x 32 x 40 tokens 69.7 -> 17.6 us, 8 x 32 x 64
+// 22.2 -> 14.4, 16 x 32 x 300 48.8 -> 34.5, 32 x 8 x 700 49.9 -> 33.9; from 4 x 32 x 1500 on one team is as fast (49.2 against 50.0).
+void av_teams(AvPlan* p, int heads, int seq)
 {
-    const int64_t tiles = (seq + 31) / 32;
-    int best = kAvWarps;
-    int64_t best_cost = INT64_MAX;
+    constexpr int64_t kTurn = 6, kReduce = 10;             // a turn's fixed cost, and that of the reduction of a head, in tiles' decoding
+    const int64_t tiles = (seq + 31) / 32, ctas = p->grid;
+    int64_t best = INT64_MAX;
+    p->teams = 1;
     for (int w = kAvWarps; w >= 1; --w) {
-        const int64_t units = heads * ((tiles + w - 1) / w), cost = (units + ctas - 1) / ctas * (6 + w);
-        if (cost < best_cost) { best = w; best_cost = cost; }
+        const int64_t units = heads * ((tiles + w - 1) / w), turns = (units + ctas - 1) / ctas;
+        const int64_t cost = turns * (kTurn + w) + std::max<int64_t>(1, (heads + ctas - 1) / ctas - 1) * kReduce;
+        if (cost < best) { best = cost; p->unit_warps = w; }
     }
-    return best;
+    for (int t = 2; t <= kAvWarps; ++t) {
+        const int64_t per_team = (heads + ctas * t - 1) / (ctas * t), active = std::min<int64_t>(t, (heads + ctas - 1) / ctas);
+        for (int w = 1; w * t <= kAvWarps; ++w) {
+            const int64_t cost = per_team * ((tiles + w - 1) / w * (kTurn + w * active) + kReduce);
+            if (cost < best) { best = cost; p->unit_warps = w; p->teams = t; }
+        }
+    }
 }
 AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
 {
@@ -520,7 +532,7 @@ AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
     const int heads = batch * n_kv_heads;
     // at most this many units; the device splits what there is evenly
     p.grid = spread_ctas(static_cast<int64_t>(heads) * ((seq + 31) / 32), ctas_max);
-    p.unit_warps = av_unit_warps(heads, seq, ctas_max);
+    av_teams(&p, heads, seq);
     auto up = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
     p.partial_bytes = up(static_cast<size_t>(p.grid + heads) * kPieceFloats * sizeof(float));
     p.ticket_bytes = up(static_cast<size_t>(heads) * sizeof(Ticket));
@@ -536,9 +548,9 @@ int launch_attn_values(const DeviceInfo& di, const AvPlan& p, const void* d_meta
     const int rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
     // at least eight warps: those beyond the unit's help with the reductions
-    const int warps = p.unit_warps < 8 ? 8 : p.unit_warps;
+    const int warps = p.unit_warps * p.teams < 8 ? 8 : p.unit_warps * p.teams;
     return launch_overlapped(kernel, static_cast<unsigned>(p.grid), static_cast<unsigned>(warps * 32), kSmemCtaBytes, s,
-                             static_cast<const uint8_t*>(d_meta), d_vblocks, heads, seq, q_per_kv, p.unit_warps, d_scores, d_out, partial, tickets, next_ticket_tag());
+                             static_cast<const uint8_t*>(d_meta), d_vblocks, heads, seq, q_per_kv, p.unit_warps, p.teams, d_scores, d_out, partial, tickets, next_ticket_tag());
 }
 }  // namespace
 

@@ -838,6 +838,12 @@ def test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk)
     check_fused(got, ref, refabs, "values unit sizes")
 
 
+@pytest.mark.parametrize("batch,heads,seq,qpk", [(8, 295, 20, 4), (3, 100, 33, 8), (9, 50, 65, 2), (4, 128, 150, 3), (10, 26, 513, 8)])
+def test_attn_values_of_many_short_rows(B, eo, kv_small, batch, heads, seq, qpk):
+    """Teams of one to eight warps with heads of their own, up to sixteen teams to a CTA; rows that end inside a tile and a turn."""
+    test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk)
+
+
 @pytest.mark.parametrize("seq", [33, 700, 3000])
 def test_attn_values_with_rising_scores_and_any_workspace(B, eo, kv_small, seq):
     """Scores that grow along the row (every tile raises the running maximum), fall, or hold their largest value in the last token, over
