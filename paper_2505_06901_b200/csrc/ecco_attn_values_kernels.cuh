@@ -35,6 +35,9 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     release_dependents();
     const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, false);       // one symbol per lookup: the tiles need the room
+    // More than sixteen warps leave 96 registers to a thread: then the weights are formed behind the decode, not held through it
+    // (19 warps, [16][8][32768][128] cache, eight heads: 535 -> 526 us; 16 warps 551 -> 565).
+    constexpr bool kLate = kMaxWarps > 16;
     constexpr uint32_t kFull = 0xffffffffu, kSlotFloats = kGroup * 8 + 8;       // sums, sums of weights
     // A team of nw warps takes a head at a time.  One team: all CTAs share the units, and the CTA's other warps help with the
     // reductions.  Several: every team has whole heads of its own and meets at a barrier of its own.
@@ -66,12 +69,11 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     const int all_teams = static_cast<int>(gridDim.x * teams), my_team = static_cast<int>(team * gridDim.x) + c;
     const int64_t u0 = teams > 1 ? unit_begin(heads, all_teams, my_team) * chunks : unit_begin(U, G, c);
     const int64_t u1 = teams > 1 ? unit_begin(heads, all_teams, my_team + 1) * chunks : unit_begin(U, G, c + 1);
-    auto block_ptr = [&](int64_t u) {
-        const int bh = static_cast<int>(u / chunks), t = min(static_cast<int>(u % chunks) * kTokens + tid, seq - 1);
-        return d_vblocks + (static_cast<uint64_t>(bh) * seq + t) * kBlockBytes;
-    };
+    // (head, first token) of a unit: advanced by one unit at a time, not divided out of its number
+    int bh = static_cast<int>(u0 / chunks), token = static_cast<int>(u0 % chunks) * kTokens;
+    auto block_ptr = [&](int head, int from) { return d_vblocks + (static_cast<uint64_t>(head) * seq + min(from + tid, seq - 1)) * kBlockBytes; };
     issue_decode_tables(tb, d_meta);
-    if (u0 < u1 && working) prefetch_block_l2(block_ptr(u0));
+    if (u0 < u1 && working) prefetch_block_l2(block_ptr(bh, token));
     if (!finish_decode_tables(tb)) return;
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (teams > 1 && (!working || u0 >= u1)) return;
@@ -205,71 +207,68 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         team_sync();
     };
 
-    int cur_bh = -1;
-    for (int64_t u = u0; u < u1; ++u) {
-        const int bh = static_cast<int>(u / chunks);
-        const int tile_base = static_cast<int>(u % chunks) * kTokens + static_cast<int>(warp - first_warp) * 32;
+    for (int64_t n = u1 - u0; n > 0; --n) {
+        const int head = bh, first_token = token, tile_base = first_token + static_cast<int>(warp - first_warp) * 32;
         const bool valid = tile_base + static_cast<int>(lane) < seq;
-        if (bh != cur_bh) {
-            if (cur_bh >= 0) { flush(cur_bh); clear_acc(); }
-            cur_bh = bh;
-        }
-        if (!working) continue;                            // warps without room for their arrays only help with the reductions
-        // P^T fragments (B operand): head = lane / 4, tokens (lane % 4) * 2 + {0, 1} + 8 j
-        uint32_t p_hi[4], p_lo[4];
-        {
-            const int r = static_cast<int>(lane >> 2);
-            const float* srow = d_scores + (static_cast<size_t>(bh) * q_per_kv + min(r, q_per_kv - 1)) * seq;
-            float s[8], top = m;
+        if ((token += kTokens) >= seq) { token = 0; ++bh; }
+        if (working) {                                     // warps without room for their arrays only help with the reductions
+            uint32_t p_hi[4], p_lo[4];                     // P^T fragments (B operand): head = lane / 4, tokens (lane % 4) * 2 + {0, 1} + 8 j
+            auto weigh = [&]() {
+                const int r = static_cast<int>(lane >> 2);
+                const float* srow = d_scores + (static_cast<size_t>(head) * q_per_kv + min(r, q_per_kv - 1)) * seq;
+                float s[8], top = m;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int tk = tile_base + static_cast<int>(lane & 3u) * 2 + 8 * (j >> 1) + (j & 1);
-                s[j] = r < q_per_kv && tk < seq ? __ldcg(srow + tk) : -INFINITY;
-                top = fmaxf(top, s[j]);
+                for (int j = 0; j < 8; ++j) {
+                    const int tk = tile_base + static_cast<int>(lane & 3u) * 2 + 8 * (j >> 1) + (j & 1);
+                    s[j] = r < q_per_kv && tk < seq ? __ldcg(srow + tk) : -INFINITY;
+                    top = fmaxf(top, s[j]);
+                }
+                top = fmaxf(top, __shfl_xor_sync(kFull, top, 1));
+                top = fmaxf(top, __shfl_xor_sync(kFull, top, 2));
+                if (__any_sync(kFull, top > m)) rescale_to(top);               // rare once a few tiles have passed
+                // Probabilities enter the tensor cores as fp16 pairs (value + remainder).  Taken as they are, everything
+                // below 6e-5 would sit in fp16's subnormal range (one part in a thousand at p = 3e-5); scaled by 2^15 they keep
+                // 22 bits down to 2e-12, and exp(s - max) <= 1 cannot overflow.  The sum of weights carries the same factor.
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    // a masked score (-inf) has weight zero, also before any finite one
+                    const float p0 = s[2 * j] == -INFINITY ? 0.0f : __expf(s[2 * j] - m) * kProbScale;
+                    const float p1 = s[2 * j + 1] == -INFINITY ? 0.0f : __expf(s[2 * j + 1] - m) * kProbScale;
+                    l += p0 + p1;
+                    const __half h0 = __float2half_rn(p0), h1 = __float2half_rn(p1);
+                    const __half l0 = __float2half_rn(p0 - __half2float(h0)), l1 = __float2half_rn(p1 - __half2float(h1));
+                    p_hi[j] = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);
+                    p_lo[j] = static_cast<uint32_t>(__half_as_ushort(l0)) | (static_cast<uint32_t>(__half_as_ushort(l1)) << 16);
+                }
+            };
+            if (!kLate) weigh();
+            Block cur;                                     // fetched now, prefetched into L2 one unit earlier
+            ldg_block(cur, block_ptr(head, first_token));
+            if (n > 1) {
+                prefetch_block_l2(block_ptr(bh, token));
+                // the scores of this warp's tokens in the next unit, one 128-byte line per query head: into L2 now
+                const int nt = token + static_cast<int>(warp - first_warp) * 32;
+                if (static_cast<int>(lane) < q_per_kv && nt < seq)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(d_scores + (static_cast<size_t>(bh) * q_per_kv + lane) * seq + nt));
             }
-            top = fmaxf(top, __shfl_xor_sync(kFull, top, 1));
-            top = fmaxf(top, __shfl_xor_sync(kFull, top, 2));
-            if (__any_sync(kFull, top > m)) rescale_to(top);                   // rare once a few tiles have passed
-            // Probabilities enter the tensor cores as fp16 pairs (value + remainder).  Taken as they are, everything
-            // below 6e-5 would sit in fp16's subnormal range (one part in a thousand at p = 3e-5); scaled by 2^15 they keep
-            // 22 bits down to 2e-12, and exp(s - max) <= 1 cannot overflow.  The sum of weights carries the same factor.
+            decode_to_tiles<false, true>(cur, tb, tiles, T, valid);             // past the end of the row: zeros
+            if (kLate) weigh();
+            // per 16-dim tile: (V tile)^T x P^T on the tensor cores
+            const uint32_t a_at = tiles + tile_byte((lane >> 4) * 8 + (lane & 7u), ((lane >> 3) & 1u) * 8);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                // a masked score (-inf) has weight zero, also before any finite one
-                const float p0 = s[2 * j] == -INFINITY ? 0.0f : __expf(s[2 * j] - m) * kProbScale;
-                const float p1 = s[2 * j + 1] == -INFINITY ? 0.0f : __expf(s[2 * j + 1] - m) * kProbScale;
-                l += p0 + p1;
-                const __half h0 = __float2half_rn(p0), h1 = __float2half_rn(p1);
-                const __half l0 = __float2half_rn(p0 - __half2float(h0)), l1 = __float2half_rn(p1 - __half2float(h1));
-                p_hi[j] = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);
-                p_lo[j] = static_cast<uint32_t>(__half_as_ushort(l0)) | (static_cast<uint32_t>(__half_as_ushort(l1)) << 16);
+            for (int ch = 0; ch < 8; ++ch) {
+                uint32_t a[2][4];
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) ldmatrix_x4_trans(a[ks], a_at + ch * kTileBytes + ks * 512);     // tokens + 16: the same swizzle
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                    mma_16816(acc[ch], a[ks], p_hi[2 * ks], p_hi[2 * ks + 1]);
+                    mma_16816(acc[ch], a[ks], p_lo[2 * ks], p_lo[2 * ks + 1]);
+                }
             }
         }
-        Block cur;                                         // fetched now, prefetched into L2 one unit earlier
-        ldg_block(cur, block_ptr(u));
-        if (u + 1 < u1) {
-            prefetch_block_l2(block_ptr(u + 1));
-            // the scores of this warp's tokens in the next unit, one 128-byte line per query head: into L2 now
-            const int nbh = static_cast<int>((u + 1) / chunks), nt = static_cast<int>((u + 1) % chunks) * kTokens + static_cast<int>(warp - first_warp) * 32;
-            if (static_cast<int>(lane) < q_per_kv && nt < seq)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(d_scores + (static_cast<size_t>(nbh) * q_per_kv + lane) * seq + nt));
-        }
-        decode_to_tiles<false, true>(cur, tb, tiles, T, valid);                 // past the end of the row: zeros
-        // per 16-dim tile: (V tile)^T x P^T on the tensor cores
-        const uint32_t a_at = tiles + tile_byte((lane >> 4) * 8 + (lane & 7u), ((lane >> 3) & 1u) * 8);
-#pragma unroll
-        for (int ch = 0; ch < 8; ++ch) {
-            uint32_t a[2][4];
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) ldmatrix_x4_trans(a[ks], a_at + ch * kTileBytes + ks * 512);     // tokens + 16: the same swizzle
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-                mma_16816(acc[ch], a[ks], p_hi[2 * ks], p_hi[2 * ks + 1]);
-                mma_16816(acc[ch], a[ks], p_lo[2 * ks], p_lo[2 * ks + 1]);
-            }
-        }
+        if (n == 1 || bh != head) { flush(head); clear_acc(); }                 // the head's last unit here
     }
-    if (cur_bh >= 0) flush(cur_bh);
 }
 
 

@@ -494,10 +494,10 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
 // ecco_attn_values
 // ---------------------------------------------------------------------------------------------
 namespace {
-// At most 16 warps of a CTA of ecco_attn_values decode (512 tokens per unit).  19 find room (9.4 KB of shared memory per
-// warp), but with more than 16 the accumulators no longer fit the registers: scores and values of a [16][8][32768][128] cache 986
-// us with 16, 1011 with 17, 1000 with 18.
-constexpr int kAvWarps = 16;
+// Warps of a CTA of ecco_attn_values that decode.  19 find room (9.4 KB of shared memory per warp), but with more than 16 a thread has 96
+// registers and the kernel spills a little and takes a few percent more per tile: two kernels, and units of 17 to 19 tiles only where
+// they save turns (a [16][8][32768][128] cache, eight heads, 551 us with 16 and 526 with 19; [8][32][4096][128] 162 and 166).
+constexpr int kAvWarps = 16, kAvManyWarps = 19;
 struct AvPlan { int grid, unit_warps, teams; size_t partial_bytes, ticket_bytes; };
 // How a CTA's warps share the work.  A unit is unit_warps tiles (of 32 tokens) of one head.
 // One team: the units of all heads are split evenly over the CTAs, and all SMs should be busy for the same number of turns.  A turn
@@ -513,9 +513,10 @@ void av_teams(AvPlan* p, int heads, int seq)
     const int64_t tiles = (seq + 31) / 32, ctas = p->grid;
     int64_t best = INT64_MAX;
     p->teams = 1;
-    for (int w = kAvWarps; w >= 1; --w) {
+    for (int w = kAvManyWarps; w >= 1; --w) {
         const int64_t units = heads * ((tiles + w - 1) / w), turns = (units + ctas - 1) / ctas;
-        const int64_t cost = turns * (kTurn + w) + std::max<int64_t>(1, (heads + ctas - 1) / ctas - 1) * kReduce;
+        int64_t cost = turns * (kTurn + w) + std::max<int64_t>(1, (heads + ctas - 1) / ctas - 1) * kReduce;
+        if (w > kAvWarps) cost += cost / 32 + 1;
         if (cost < best) { best = cost; p->unit_warps = w; }
     }
     for (int t = 2; t <= kAvWarps; ++t) {
@@ -581,7 +582,8 @@ extern "C" int ecco_attn_values(const void* d_meta, const uint8_t* d_vblocks, in
     uint8_t* wsb = static_cast<uint8_t*>(d_workspace);
     float* partial = reinterpret_cast<float*>(wsb);
     Ticket* tickets = reinterpret_cast<Ticket*>(wsb + p.partial_bytes);
-    return launch_attn_values<kAvWarps>(di, p, d_meta, d_vblocks, batch * n_kv_heads, seq, q_per_kv, d_scores, d_out, partial, tickets, s);
+    auto launch = p.unit_warps > kAvWarps ? launch_attn_values<kAvManyWarps> : launch_attn_values<kAvWarps>;
+    return launch(di, p, d_meta, d_vblocks, batch * n_kv_heads, seq, q_per_kv, d_scores, d_out, partial, tickets, s);
 }
 
 

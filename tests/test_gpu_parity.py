@@ -826,9 +826,9 @@ def test_attn_values_keeps_small_probabilities(B, eo, kv_small, synth, qpk):
         assert np.all(err[0, 1] <= 2e-5 * refabs[0, 1])    # evenly spread weights: far inside the bound
 
 
-@pytest.mark.parametrize("batch,heads,seq,qpk", [(1, 1, 31, 8), (1, 1, 6000, 5), (3, 50, 65, 1), (2, 8, 777, 2), (1, 3, 40000, 1)])
+@pytest.mark.parametrize("batch,heads,seq,qpk", [(1, 1, 31, 8), (1, 1, 6000, 5), (3, 50, 65, 1), (2, 8, 777, 2), (1, 3, 40000, 1), (1, 4, 22000, 8), (2, 70, 590, 3)])
 def test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk):
-    """Units of one warp to sixteen; one head in a piece per SM; more short heads than SMs."""
+    """Units of one warp to nineteen; one head in a piece per SM; more short heads than SMs."""
     meta = kv_small["meta"]
     n = batch * heads * seq
     blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
