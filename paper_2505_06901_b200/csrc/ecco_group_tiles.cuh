@@ -58,11 +58,14 @@ __device__ __forceinline__ void decode_to_tiles(const Block& blk, const DecodeTa
         map_ranks(g, ranks, v);
         if (cutting) cut_values(v, n_ok);
         const uint32_t row = my_row + (i >> 1) * kTileBytes;
-        if (!kSpread) {
-            sts_v4(row + (i & 1 ? swz ^ 16u : swz), v[0], v[1], v[2], v[3]);
-        } else if (i & 1) {
-            sts_v4(row + swz, even[0], even[2], v[0], v[2]);
-            sts_v4(row + (swz ^ 16u), even[1], even[3], v[1], v[3]);
+        if (i & 1) {                                       // both halves now: the last tile may not be touched before symbol 127
+            if (kSpread) {
+                sts_v4(row + swz, even[0], even[2], v[0], v[2]);
+                sts_v4(row + (swz ^ 16u), even[1], even[3], v[1], v[3]);
+            } else {
+                sts_v4(row + swz, even[0], even[1], even[2], even[3]);
+                sts_v4(row + (swz ^ 16u), v[0], v[1], v[2], v[3]);
+            }
         } else {
 #pragma unroll
             for (int k = 0; k < 4; ++k) even[k] = v[k];
