@@ -67,10 +67,12 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     const int G = static_cast<int>(min(static_cast<int64_t>(gridDim.x), U)), c = blockIdx.x;
     if (teams == 1 && c >= G) return;
     const int all_teams = static_cast<int>(gridDim.x * teams), my_team = static_cast<int>(team * gridDim.x) + c;
-    const int64_t u0 = teams > 1 ? unit_begin(heads, all_teams, my_team) * chunks : unit_begin(U, G, c);
-    const int64_t u1 = teams > 1 ? unit_begin(heads, all_teams, my_team + 1) * chunks : unit_begin(U, G, c + 1);
+    const UnitSplit split(teams > 1 ? heads : U, teams > 1 ? all_teams : G);                // of heads or of units
+    const int me = teams > 1 ? my_team : c, scale = teams > 1 ? chunks : 1;
+    const int64_t u0 = split.begin(me) * scale, u1 = split.begin(me + 1) * scale;
     // (head, first token) of a unit: advanced by one unit at a time, not divided out of its number
-    int bh = static_cast<int>(u0 / chunks), token = static_cast<int>(u0 % chunks) * kTokens;
+    int bh = static_cast<int>(divide(static_cast<uint64_t>(u0), static_cast<uint64_t>(chunks)));
+    int token = static_cast<int>(u0 - static_cast<int64_t>(bh) * chunks) * kTokens;
     auto block_ptr = [&](int head, int from) { return d_vblocks + (static_cast<uint64_t>(head) * seq + min(from + tid, seq - 1)) * kBlockBytes; };
     issue_decode_tables(tb, d_meta);
     if (u0 < u1 && working) prefetch_block_l2(block_ptr(bh, token));
@@ -79,7 +81,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     if (teams > 1 && (!working || u0 >= u1)) return;
     const float T = tb.T;
     if (teams == 1 && tid == 0) {                                        // thread 0 takes the tickets: of the heads at the ends of this CTA's units
-        Ticket* const ends[2] = {d_tickets + u0 / chunks, d_tickets + (u1 - 1) / chunks};
+        Ticket* const ends[2] = {d_tickets + bh, d_tickets + divide(static_cast<uint64_t>(u1 - 1), static_cast<uint64_t>(chunks))};
         const Ticket seen[2] = {look_at_ticket(ends[0]), look_at_ticket(ends[1])};
         claim_ticket(ends[0], seen[0], tag);
         if (ends[1] != ends[0]) claim_ticket(ends[1], seen[1], tag);
@@ -147,8 +149,9 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
             out_s[i] = sum;
         }
         team_sync();
-        const int c_lo = teams > 1 ? 0 : unit_owner(U, G, static_cast<int64_t>(bh) * chunks);
-        const int c_hi = teams > 1 ? 0 : unit_owner(U, G, static_cast<int64_t>(bh + 1) * chunks - 1);
+        const UnitSplit split(U, G);                       // again: not held in registers through the decode
+        const int c_lo = teams > 1 ? 0 : split.owner(static_cast<int64_t>(bh) * chunks);
+        const int c_hi = teams > 1 ? 0 : split.owner(static_cast<int64_t>(bh + 1) * chunks - 1);
         auto store = [&](int i, float v, float weights) {
             if ((i & 7) < q_per_kv) d_out[(static_cast<size_t>(bh) * q_per_kv + (i & 7)) * kGroup + (i >> 3)] = v / weights;
         };
@@ -207,7 +210,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         team_sync();
     };
 
-    for (int64_t n = u1 - u0; n > 0; --n) {
+    for (int n = static_cast<int>(u1 - u0); n > 0; --n) {
         const int head = bh, first_token = token, tile_base = first_token + static_cast<int>(warp - first_warp) * 32;
         const bool valid = tile_base + static_cast<int>(lane) < seq;
         if ((token += kTokens) >= seq) { token = 0; ++bh; }

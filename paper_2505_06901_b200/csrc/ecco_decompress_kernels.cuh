@@ -11,8 +11,8 @@ namespace {
 __host__ __device__ __forceinline__ uint32_t balanced_warps(uint64_t units, uint32_t w_max)
 {
     if (units <= w_max) return static_cast<uint32_t>(units);
-    const uint64_t per_warp = (units + w_max - 1) / w_max;
-    return static_cast<uint32_t>((units + per_warp - 1) / per_warp);
+    const uint64_t per_warp = divide(units + w_max - 1, w_max);
+    return static_cast<uint32_t>(divide(units + per_warp - 1, per_warp));
 }
 
 // Work is dealt out in warp tiles of 32 consecutive groups, tile i to warp (i mod working warps):

@@ -33,6 +33,13 @@ std::atomic<uint64_t> g_launches{0};
 constexpr uint32_t kSmemCtaBytes = 232448;                           // 227 KB: what every decoding kernel asks for
 constexpr int kWaitLimit = 1 << 22;                                  // bounded mbarrier polling
 
+// Quotient of numbers that are rarely beyond 32 bits: a 64-bit division takes some hundred instructions, one after the other
+// (eight of them stood at the end of every split sum: see UnitSplit).
+__host__ __device__ __forceinline__ uint64_t divide(uint64_t a, uint64_t b)
+{
+    return (a | b) >> 32 ? a / b : static_cast<uint32_t>(a) / static_cast<uint32_t>(b);
+}
+
 // ---------------------------------------------------------------------------------------------
 // small PTX helpers
 // ---------------------------------------------------------------------------------------------

@@ -71,7 +71,8 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
     const int wg = warp < nw ? warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x) : INT_MAX;
     const int64_t U = batch.units;
     const int W = static_cast<int>(balanced_warps(static_cast<uint64_t>(U), gridDim.x * static_cast<uint32_t>(nw)));
-    const int64_t u0 = wg < W ? unit_begin(U, W, wg) : 0, u1 = wg < W ? unit_begin(U, W, wg + 1) : 0;
+    const UnitSplit split(U, W);
+    const int64_t u0 = wg < W ? split.begin(wg) : 0, u1 = wg < W ? split.begin(wg + 1) : 0;
     issue_decode_tables(tb, d_meta);
     if (!same_tables(batch, tb)) {                         // images are host-written: readable before the wait
         bounded_wait(tb.base, 0, kWaitLimit);              // the table copies into this CTA's shared memory must land first
@@ -90,8 +91,9 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
         const int n_out = jb.n_out, kblocks = jb.kblocks, gtile = jb.tile_first + tile;
         float* d_y = jb.y;
         const int64_t g0 = jb.unit_first + static_cast<int64_t>(tile) * kblocks;
-        const int w_lo = unit_owner(U, W, g0);
-        const int w_hi = unit_owner(U, W, g0 + kblocks - 1);
+        const UnitSplit split(U, W);                       // again: not held in registers through the decode
+        const int w_lo = split.owner(g0);
+        const int w_hi = split.owner(g0 + kblocks - 1);
         float* mine = d_partial + static_cast<size_t>(wg + gtile) * 8 * 32;
         if (w_lo != w_hi) {
 #pragma unroll
@@ -127,7 +129,8 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
     const Ticket seen[2] = {look_at_ticket(my_ticket[0]), look_at_ticket(my_ticket[1])};
     int cur_j = pos.j, cur_tile = pos.tile;
     float T = __ldg(&reinterpret_cast<const DevHeader*>(batch.job[pos.j].meta)->T);
-    for (int64_t u = u0; u < u1; ++u) {
+    const int n_units = static_cast<int>(u1 - u0);
+    for (int left = n_units; left > 0; --left) {
         const GemvJob& jb = batch.job[pos.j];
         const int tile = pos.tile;
         if (pos.j != cur_j || tile != cur_tile) {
@@ -142,13 +145,13 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
         }
         Block cur;                                         // fetched now, prefetched into L2 one unit earlier (see the scalar kernels)
         ldg_block(cur, gemv_block_ptr(batch, pos, lane));
-        if (u == u0 && lane == 0) {                        // lane 0 is the one that takes
+        if (left == n_units && lane == 0) {                        // lane 0 is the one that takes
             claim_ticket(my_ticket[0], seen[0], tag);
             if (my_ticket[1] != my_ticket[0]) claim_ticket(my_ticket[1], seen[1], tag);
         }
         const __half* xk = jb.x + pos.kb * kGroup;
         const size_t k = static_cast<size_t>(jb.kblocks) * kGroup;
-        if (u + 1 < u1) { pos = gemv_pos_next(batch, pos); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
+        if (left > 1) { pos = gemv_pos_next(batch, pos); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
         row_dot_mma<false>(cur, tb, tiles_at, T, true, [&](uint32_t (&v)[16]) { load_vfrag(v, xk, k, n_cols); }, acc);
     }
     flush(cur_j, cur_tile);
@@ -172,11 +175,12 @@ ecco_attn_scores_mma_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* _
     const int tiles = (seq + 31) / 32;
     const int64_t U = static_cast<int64_t>(heads) * tiles;
     const int W = static_cast<int>(balanced_warps(static_cast<uint64_t>(U), gridDim.x * static_cast<uint32_t>(nw)));
-    const int64_t u0 = wg < W ? unit_begin(U, W, wg) : 0, u1 = wg < W ? unit_begin(U, W, wg + 1) : 0;
+    const UnitSplit split(U, W);
+    const int64_t u0 = wg < W ? split.begin(wg) : 0, u1 = wg < W ? split.begin(wg + 1) : 0;
     auto block_ptr = [&](int bh, int tile) {
         return d_kblocks + (static_cast<uint64_t>(bh) * seq + min(tile * 32 + lane, seq - 1)) * kBlockBytes;
     };
-    int nbh = static_cast<int>(u0 / tiles), ntile = static_cast<int>(u0 % tiles);     // advanced by one per unit
+    int nbh = static_cast<int>(divide(static_cast<uint64_t>(u0), static_cast<uint64_t>(tiles))), ntile = static_cast<int>(u0 - static_cast<int64_t>(nbh) * tiles);     // advanced by one per unit
     issue_decode_tables(tb, d_meta);
     if (u0 < u1) prefetch_block_l2(block_ptr(nbh, ntile));
     if (!finish_decode_tables(tb)) return;

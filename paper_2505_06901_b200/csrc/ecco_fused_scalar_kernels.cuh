@@ -121,15 +121,24 @@ __device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables
     }
 }
 
-// Contiguous split of U work units over G CTAs: CTA c owns [unit_begin(c), unit_begin(c + 1)).
-__host__ __device__ __forceinline__ int64_t unit_begin(int64_t U, int G, int c) { return U * c / G; }
-__host__ __device__ __forceinline__ int unit_owner(int64_t U, int G, int64_t u)
-{
-    int c = static_cast<int>(u * G / U);
-    while (c + 1 < G && unit_begin(U, G, c + 1) <= u) ++c;
-    while (c > 0 && unit_begin(U, G, c) > u) --c;
-    return c;
-}
+// Contiguous split of U work units over G workers: worker c owns [begin(c), begin(c + 1)), the first U mod G of them one unit more
+// than the others.  (Boundaries at U * c / G took four 64-bit divisions to find a unit's owner, which every split sum does twice at its end.)
+struct UnitSplit {
+    int64_t per;
+    int more;                                              // workers with per + 1 units
+    __device__ __forceinline__ UnitSplit(int64_t U, int G)
+    {
+        per = static_cast<int64_t>(divide(static_cast<uint64_t>(U), static_cast<uint64_t>(G)));
+        more = static_cast<int>(U - per * G);
+    }
+    __device__ __forceinline__ int64_t begin(int c) const { return per * c + min(c, more); }
+    __device__ __forceinline__ int owner(int64_t u) const
+    {
+        const int64_t cut = (per + 1) * more;
+        return u < cut ? static_cast<int>(divide(static_cast<uint64_t>(u), static_cast<uint64_t>(per + 1)))
+                       : more + static_cast<int>(divide(static_cast<uint64_t>(u - cut), static_cast<uint64_t>(per)));
+    }
+};
 
 // Ticket words of a workspace.  They need no clearing before the call, which would be a launch of its own (2 us of a small call's
 // 10): a word counts from zero once it carries the call's tag, 48 bits that the host draws at random once and advances for every
@@ -186,8 +195,8 @@ __device__ __forceinline__ GemvPos gemv_pos_of(const GemvBatch& batch, int64_t u
     GemvPos p = {0, 0, 0};
     while (p.j + 1 < batch.n && u >= batch.job[p.j + 1].unit_first) ++p.j;
     const int64_t lu = u - batch.job[p.j].unit_first;
-    p.tile = static_cast<int>(lu / batch.job[p.j].kblocks);
-    p.kb = static_cast<int>(lu % batch.job[p.j].kblocks);
+    p.tile = static_cast<int>(divide(static_cast<uint64_t>(lu), static_cast<uint64_t>(batch.job[p.j].kblocks)));
+    p.kb = static_cast<int>(lu - static_cast<int64_t>(p.tile) * batch.job[p.j].kblocks);
     return p;
 }
 __device__ __forceinline__ GemvPos gemv_pos_next(const GemvBatch& batch, GemvPos p)
@@ -236,7 +245,8 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     const int wg = warp < nw ? warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x) : INT_MAX;
     const int64_t U = batch.units;
     const int W = static_cast<int>(balanced_warps(static_cast<uint64_t>(U), gridDim.x * static_cast<uint32_t>(nw)));
-    const int64_t u0 = wg < W ? unit_begin(U, W, wg) : 0, u1 = wg < W ? unit_begin(U, W, wg + 1) : 0;
+    const UnitSplit split(U, W);
+    const int64_t u0 = wg < W ? split.begin(wg) : 0, u1 = wg < W ? split.begin(wg + 1) : 0;
     issue_decode_tables(tb, d_meta);
     if (!same_tables(batch, tb)) {                         // images are host-written: readable before the wait
         bounded_wait(tb.base, 0, kWaitLimit);              // the table copies into this CTA's shared memory must land first
@@ -262,8 +272,9 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
         const int row = tile * 32 + lane;
         const bool row_ok = row < n_out;
         const int64_t g0 = jb.unit_first + static_cast<int64_t>(tile) * kblocks;
-        const int w_lo = unit_owner(U, W, g0);
-        const int w_hi = unit_owner(U, W, g0 + kblocks - 1);
+        const UnitSplit split(U, W);                       // again: not held in registers through the decode
+        const int w_lo = split.owner(g0);
+        const int w_hi = split.owner(g0 + kblocks - 1);
         if (w_lo == w_hi) {
             if (row_ok) {
 #pragma unroll
@@ -326,7 +337,8 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     const Ticket seen[2] = {look_at_ticket(my_ticket[0]), look_at_ticket(my_ticket[1])};
     int cur_j = pos.j, cur_tile = pos.tile;
     float T = __ldg(&reinterpret_cast<const DevHeader*>(batch.job[pos.j].meta)->T);
-    for (int64_t u = u0; u < u1; ++u) {
+    const int n_units = static_cast<int>(u1 - u0);
+    for (int left = n_units; left > 0; --left) {
         if (pos.j != cur_j || pos.tile != cur_tile) {
             flush(cur_j, cur_tile);
             clear_acc();
@@ -343,11 +355,11 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
         // one in sixteen registers through a whole group costs more in resident warps than the fetch costs here
         Block cur;
         ldg_block(cur, gemv_block_ptr(batch, pos, lane));
-        if (u == u0 && lane == 0) {                        // lane 0 is the one that takes
+        if (left == n_units && lane == 0) {                        // lane 0 is the one that takes
             claim_ticket(my_ticket[0], seen[0], tag);
             if (my_ticket[1] != my_ticket[0]) claim_ticket(my_ticket[1], seen[1], tag);
         }
-        if (u + 1 < u1) {
+        if (left > 1) {
             pos = gemv_pos_next(batch, pos);
             prefetch_block_l2(gemv_block_ptr(batch, pos, lane));
             load_x(pos);
@@ -380,13 +392,14 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     const int tiles = (seq + 31) / 32;
     const int64_t U = static_cast<int64_t>(heads) * tiles;
     const int W = static_cast<int>(balanced_warps(static_cast<uint64_t>(U), gridDim.x * static_cast<uint32_t>(nw)));
-    const int64_t u0 = wg < W ? unit_begin(U, W, wg) : 0, u1 = wg < W ? unit_begin(U, W, wg + 1) : 0;
+    const UnitSplit split(U, W);
+    const int64_t u0 = wg < W ? split.begin(wg) : 0, u1 = wg < W ? split.begin(wg + 1) : 0;
     // lanes past the end of the sequence decode its last token again and store nothing; (head, tile) of a unit is
     // advanced by one per unit instead of divided out of the unit number
     auto block_ptr = [&](int bh, int tile) {
         return d_kblocks + (static_cast<uint64_t>(bh) * seq + min(tile * 32 + lane, seq - 1)) * kBlockBytes;
     };
-    int bh = static_cast<int>(u0 / tiles), tile = static_cast<int>(u0 % tiles);
+    int bh = static_cast<int>(divide(static_cast<uint64_t>(u0), static_cast<uint64_t>(tiles))), tile = static_cast<int>(u0 - static_cast<int64_t>(bh) * tiles);
     issue_decode_tables(tb, d_meta);
     if (u0 < u1) prefetch_block_l2(block_ptr(bh, tile));
     if (!finish_decode_tables(tb)) return;
