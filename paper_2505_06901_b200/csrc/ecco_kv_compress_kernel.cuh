@@ -231,8 +231,8 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
 //    scale's reciprocal, and where that comes within 2^-21 of a midpoint the exact division and fp64 distances decide.
 //  * the four codebooks' lengths are bytes of one word, summed together.
 //  * a lane joins its sixteen codewords into one string of at most 128 bits in registers and ORs five words into the block.
-// Bound by the issue slots (74 % busy, ncu): 349 warp instructions per group against 735 of the kernel above; two calls of
-// 131 072 groups take 109.7 us against 218.5.  Making the tables costs a call 3 us, which is what the smaller instruction count
+// Bound by the issue slots (80 % busy, ncu): 310 warp instructions per group against 735 of the kernel above; two calls of
+// 131 072 groups take 106 us against 218.5.  Making the tables costs a call 3 us, which is what the smaller instruction count
 // saves at about 16 000 groups (two calls of 8192: 26.5 against 19.5 us, of 16 384: 30.6 against 31.3): fewer go to the kernel above.
 // ---------------------------------------------------------------------------------------------
 constexpr int kKvManyWarps = 32;
