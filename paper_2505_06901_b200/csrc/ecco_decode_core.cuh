@@ -110,10 +110,11 @@ __device__ __forceinline__ void build_rank_tables(const DecodeTables& tb)
     }
     __syncthreads();
 }
-// The whole CTA waits for its tables and builds the rest; false (CTA-uniform) if the bounded wait expired.
+// The whole CTA waits for its tables and builds the rest; false (CTA-uniform) if the bounded wait expired.  Then it has waited for the
+// previous kernel of the stream, too: see dependency_wait.
 __device__ __forceinline__ bool finish_decode_tables(const DecodeTables& tb, uint32_t parity = 0)
 {
-    if (!bounded_wait(tb.base, parity, kWaitLimit)) return false;
+    if (!bounded_wait(tb.base, parity, kWaitLimit)) { dependency_wait(); return false; }
     build_rank_tables(tb);
     return true;
 }

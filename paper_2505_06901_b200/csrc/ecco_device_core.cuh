@@ -175,6 +175,8 @@ __device__ __forceinline__ bool bounded_wait(uint32_t bar, uint32_t parity, int 
 // attribute and only launch, table fetch and prologue overlap.  The image is the exception because no kernel writes
 // it: it reaches the device by a copy, which is a stream operation of its own (a kernel behind a copy starts after
 // it), and a kernel can start early only behind one that releases its dependents, i.e. one of this file.
+// A grid that ends without having waited breaks the chain: the kernel behind it waits for this grid only and could start on data that
+// the one before it is still writing.  So a way out that every CTA may take leads through dependency_wait(), too.
 // release_dependents() lets the next kernel of the stream do the same with respect to this one.
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -250,6 +250,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     issue_decode_tables(tb, d_meta);
     if (!same_tables(batch, tb)) {                         // images are host-written: readable before the wait
         bounded_wait(tb.base, 0, kWaitLimit);              // the table copies into this CTA's shared memory must land first
+        dependency_wait();                                 // and the next kernel relies on this one for the previous one's completion
         return;
     }
     GemvPos pos = {0, 0, 0};

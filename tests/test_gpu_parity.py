@@ -1210,3 +1210,42 @@ def test_back_to_back_calls_keep_stream_order(B, eo, kv_small, cfg1_small, synth
     torch.cuda.synchronize()
     assert B.ecco_device_status() == 0
     assert np.array_equal(out.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("batch", [1, 8])
+def test_a_refused_call_keeps_the_stream_order_of_its_neighbours(B, eo, cfg1_small, synth, batch):
+    """A grouped product over matrices with different tables ends without doing anything, on SMs that the call before it leaves
+    free.  The call behind it must still find that call's output complete: as it does with a synchronisation in between."""
+    lm = lib_meta_from_oracle(B, cfg1_small["meta"])
+    S, e, pat, cb, kp = lm.tables()
+    cb = cb.copy()
+    cb[0, 0] = cb[0, 0][::-1]
+    d_meta, other = B.meta_to_device(lm), B.meta_to_device(B.ecco_meta_create(S, e, pat, cb, kp))
+    d_blocks, n = dev(cfg1_small["blocks"]), 2048          # 64 tiles of 32 groups: 64 SMs
+    d_x, d_y = dev(synth.activations(batch, 1024, 5)), torch.zeros((2, batch, 256), device="cuda")
+    items = [(d_meta, d_blocks, 256, 1024, d_x, d_y[0]), (other, d_blocks, 256, 1024, d_x, d_y[1])]
+    wsb = B.ecco_gemv_batch_workspace_bytes(items, batch)
+    ws, arr = torch.empty(wsb, dtype=torch.uint8, device="cuda"), B.gemv_items(items)
+    out, act = torch.zeros(n * 128, dtype=torch.float16, device="cuda"), torch.zeros((2 * n, 64), dtype=torch.uint8, device="cuda")
+    want = dev(eo.act_encode(eo.decode(cfg1_small["meta"], cfg1_small["blocks"]).reshape(-1)))
+
+    def chain(st):
+        B.ecco_decompress(d_meta, d_blocks, n, out, st)
+        B.ecco_gemv_batch(arr, batch, ws, wsb, st)
+        B.ecco_act_compress(out, 2 * n, act, st)
+
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        chain(st)
+        st.synchronize()
+        assert torch.equal(act, want) and B.ecco_device_status() == B.ERR_INVALID_ARG
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            chain(st)
+        for i in range(40):                                # eager and as a graph, whose launches follow one another at once
+            out.zero_()
+            act.zero_()
+            g.replay() if i & 1 else chain(st)
+            st.synchronize()
+            assert torch.equal(act, want), i
+    assert B.ecco_device_status() == B.ERR_INVALID_ARG and not d_y.any()
