@@ -121,7 +121,12 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
             if (hh.x != tb.hash_lo || hh.y != tb.hash_hi) break;
             run_tiles += tiles_of(t1);
         }
-        if (run > 0) __syncthreads();                      // every warp is done with the previous run's tables
+        if (run > 0) {
+            // Every warp is done with the previous run's tables.  The copies below write where ordinary stores have written (the records
+            // that build_rank_tables rewrote, warps' arrays of another layout): every thread orders its stores before them.
+            fence_async_smem();
+            __syncthreads();
+        }
         issue_decode_tables(tb, batch.job[t0].meta, run == 0);
         const uint32_t tiles_base = (tb.warp_base + 1023u) & ~1023u;
         const uint32_t nw = decode_warps(tb, kTmaWarpBytes, tiles_base - tb.warp_base);

@@ -245,6 +245,28 @@ def test_decompress_batch_matches_oracle_per_item(B, eo, cfg1_small, kv_small, s
     assert bool((canary == 7.0).all())
 
 
+@pytest.mark.parametrize("n_groups", [32, 33, 700])
+def test_decompress_batch_of_short_tensors_with_tables_of_their_own(B, eo, cfg1_small, kv_small, synth, n_groups):
+    """Eight runs in one launch, each with other tables than the one before and its arrays elsewhere: most warps
+    help with the tables of a run and have no tile in it.  Repeated, in two orders; exact: decoding has one result."""
+    shapes = np.array([[2, 2, 2, 4, 4, 4, 6, 6, 8, 8, 8, 8, 8, 8, 8, 8], [4] * 16])
+    metas = [cfg1_small["meta"], kv_small["meta"], make_meta(eo, skew_lens, S=7, seed=4), make_meta(eo, lambda k, h, r: list(r.permutation(shapes[k & 1])), S=64, seed=6)]
+    plan = []
+    for i in range(8):
+        m = metas[i % 4].copy()
+        blocks = synth.random_blocks(n_groups, 60 + i)
+        plan.append((B.meta_to_device(lib_meta_from_oracle(B, m)), dev(blocks), dev(eo.decode(m, blocks))))
+    outs = [torch.empty((n_groups, 128), dtype=torch.float16, device="cuda") for _ in plan]
+    for order in (range(8), (3, 0, 2, 1, 7, 6, 5, 4)):
+        items = B.decompress_items([(plan[i][0], plan[i][1], n_groups, outs[i]) for i in order])
+        for _ in range(20):
+            for o in outs:
+                o.fill_(7.0)
+            B.ecco_decompress_batch(items)
+            assert all(torch.equal(o.view(torch.int16), p[2].view(torch.int16)) for o, p in zip(outs, plan))
+    assert B.ecco_device_status() == 0
+
+
 def test_decompress_every_code_shape_on_random_streams(B, eo, synth):
     """All 255 admissible shapes of a 2..8-bit code on 16 symbols (every multiset of lengths with Kraft sum 1,
     dealt to the symbols at random), one per codebook, decoded from random bit streams: whatever a block's header
