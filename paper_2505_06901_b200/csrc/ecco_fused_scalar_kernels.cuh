@@ -47,17 +47,18 @@ __device__ __forceinline__ float rank_value(const LaneGroup& g, uint32_t rank)
     return __half2float(__ushort_as_half(static_cast<unsigned short>(prmt(lo, hi, 0x0040u))));
 }
 
-// partial sums per product: two short chains for one or two products, one chain each for more
-__host__ __device__ constexpr int chains(int v) { return v <= 2 ? 2 : 1; }
-__device__ __forceinline__ float sum_of(const float (&a)[2]) { return a[0] + a[1]; }
-__device__ __forceinline__ float sum_of(const float (&a)[1]) { return a[0]; }
+// Partial sums per product.  One chain over a group's 128 products is less exact than the tensor cores' shorter ones where a warp has
+// a single unit: 513 x 512 by three rows, error 2.06e-7 of the result against 1.97e-7, and 1.38e-7 with two chains.  At three to
+// five rows the second chain costs 1.5 to 4 % (two 11008 x 4096 matrices 65.7 -> 66.8, 71.5 -> 74.4 and 79.4 -> 81.0 us).
+constexpr int kChains = 2;
+__device__ __forceinline__ float sum_of(const float (&a)[kChains]) { return a[0] + a[1]; }
 
 // kDeal: deal_outliers (caches) or every lane its own (weights)
 // decode one group and accumulate its kV dot products against the slice at shared address xs
 // keep = false: the products are not wanted.  The lanes past the end of a row decode its last group again; with 23 copies of a
 // group of many outliers to deal, one warp held up a whole call (scores of 2 x 8 x 777 tokens 14.6 instead of 9.0 us).
 template <int kV, bool kDeal>
-__device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, bool keep, float (&acc)[kV][chains(kV)])
+__device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables& tb, uint32_t bits, float T, uint32_t xs, bool keep, float (&acc)[kV][kChains])
 {
     LaneGroup g = open_block(blk, bits, tb, T);
     if (kDeal) sts_u32(bits + 18 * 128, blk.w[0]);                    // the ranks will lie over the block's first words
@@ -71,11 +72,10 @@ __device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables
         for (int b = 0; b < kV; ++b) {
             uint32_t x[4];
             asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(xs + b * (kGroup * 2) + i * 16));
-            constexpr int kLast = chains(kV) - 1;
             fma_half2(acc[b][0], v[0], x[0]);
-            fma_half2(acc[b][kLast], v[1], x[1]);
+            fma_half2(acc[b][1], v[1], x[1]);
             fma_half2(acc[b][0], v[2], x[2]);
-            fma_half2(acc[b][kLast], v[3], x[3]);
+            fma_half2(acc[b][1], v[3], x[3]);
         }
     });
     // outliers replace the mapped value at their location: add (outlier - mapped) * x.  Rows 24 and 25 behind the block hold the
@@ -258,12 +258,12 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     if (!finish_decode_tables(tb)) return;
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
 
-    float acc[kV][chains(kV)];                             // partial sums, added when the row tile is left
+    float acc[kV][kChains];                             // partial sums, added when the row tile is left
     auto clear_acc = [&]() {
 #pragma unroll
         for (int b = 0; b < kV; ++b)
 #pragma unroll
-            for (int i = 0; i < chains(kV); ++i) acc[b][i] = 0.0f;
+            for (int i = 0; i < kChains; ++i) acc[b][i] = 0.0f;
     };
     clear_acc();
     auto flush = [&](int jf, int tile) {
@@ -427,11 +427,11 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         const int out_bh = bh;
         if (++tile == tiles) { tile = 0; ++bh; }
         if (u + 1 < u1) prefetch_block_l2(block_ptr(bh, tile));
-        float acc[kV][chains(kV)];
+        float acc[kV][kChains];
 #pragma unroll
         for (int r = 0; r < kV; ++r)
 #pragma unroll
-            for (int i = 0; i < chains(kV); ++i) acc[r][i] = 0.0f;
+            for (int i = 0; i < kChains; ++i) acc[r][i] = 0.0f;
         fused_group<kV, true>(cur, tb, bits, T, xs, t < seq, acc);
         if (t < seq) {
 #pragma unroll

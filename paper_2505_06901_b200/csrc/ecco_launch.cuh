@@ -121,8 +121,8 @@ inline GemvPlan gemv_plan(int64_t units, int row_tiles, int warps, int cols, int
 constexpr int kMmaWarps = 20;      // 19 find room beside the tables of a typical image (9.4 KB of shared memory per warp)
 
 // the per-warp kernel (one to five rows of x: vpad columns) or the tensor-core kernel (6..8 rows: eight columns)
-// Per-warp against tensor-core kernel, two 11008 x 4096 matrices in a call: 67 against 83 us at three rows, 80 against 83 at five,
-// 85 against 83.5 at six, 104 against 83.6 at eight; 1000 x 4096: 14.6 against 18.1 at five, 15.3 against 17.9 at six.
+// Per-warp against tensor-core kernel, two 11008 x 4096 matrices in a call: 67 against 81 us at three rows, 81 against 81 at five,
+// 85 against 81 at six, 104 against 81 at eight; 1000 x 4096: 14.2 against 18.1 at five, 15.3 against 17.9 at six.
 inline GemvPlan gemv_plan_for(int64_t units, int row_tiles, int vpad, int ctas_max)
 {
     return vpad <= 5 ? gemv_plan(units, row_tiles, gemv_warp_warps(vpad), vpad, ctas_max) : gemv_plan(units, row_tiles, kMmaWarps, 8, ctas_max);

@@ -387,6 +387,22 @@ def test_gemv_of_three_to_six_rows(B, eo, cfg1_small, synth, batch, n_out, k):
     check_fused(got, ref, refabs, f"gemv b{batch}")
 
 
+@pytest.mark.parametrize("batch", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("n_out,k", [(513, 512), (999, 4096)])
+def test_gemv_error_does_not_grow_with_the_rows_of_x(B, eo, cfg1_small, synth, batch, n_out, k):
+    """Calls of one k-block per warp, 2-norm of the error over that of the result.  An addition is off by 0.43 * 2^-24 of its result
+    (rms: half a last place is 2^-25..2^-24 of a number, its uniform error 1 / sqrt(3) of that), so a chain of n products of random
+    sign by that times sqrt(n / 2).  Two chains of 64 make a k-block's 128 products and one of k / 128 the partial sums; the limit lies
+    halfway to a single chain of 128, i.e. at 96."""
+    n = n_out * (k // 128)
+    blocks = np.tile(cfg1_small["blocks"], (-(-n // 2048), 1))[:n]
+    x = synth.activations(batch, k, 7)
+    got, _ = gpu_gemv(B, lib_meta_from_oracle(B, cfg1_small["meta"]), blocks, n_out, k, x, batch)
+    ref, _ = eo.gemv(cfg1_small["meta"], blocks, n_out, k, x, batch)
+    rel = float(np.linalg.norm(got - ref) / np.linalg.norm(ref))
+    assert rel <= 0.43 * 2.0 ** -24 * np.sqrt((96 + k // 128) / 2), rel
+
+
 @pytest.mark.parametrize("batch", [1, 2, 3, 8])
 def test_gemv_batch_gives_every_item_what_gemv_gives(B, eo, cfg1_small, synth, batch):
     """Several matrices in one call (shapes that differ in rows and in k, a ragged row count, a one-row matrix, a shared
