@@ -882,6 +882,23 @@ def test_attn_values_of_many_short_rows(B, eo, kv_small, batch, heads, seq, qpk)
     test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk)
 
 
+@pytest.mark.parametrize("batch,heads,seq,qpk", [(16, 32, 300, 2), (4, 32, 1500, 1)])
+def test_attn_values_error_does_not_grow_with_the_tiles_of_a_warp(B, eo, kv_small, batch, heads, seq, qpk):
+    """2-norm of the error over that of the result, rows of which a warp takes several tiles.  An addition is off by 0.43 * 2^-24 of its
+    result (rms), a chain of n terms of random sign by that times sqrt(n / 2): 47 tiles one after the other make 1.2e-7.  A weight
+    is off by a last place or two (2^-24..2^-22), at random over some hundred tokens that count: 1e-7.  Together 1.6e-7; sums
+    that grow inside the tensor cores, which cut off, are off by 2.5e-7 here.  Limit 2e-7."""
+    n = batch * heads * seq
+    blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
+    scores = np.random.Generator(np.random.PCG64(seq)).standard_normal((batch, heads * qpk, seq)).astype(np.float32)
+    got = gpu_attn_values(B, lib_meta_from_oracle(B, kv_small["meta"]), blocks, batch, heads, seq, qpk, scores)
+    dec = np.tile(eo.decode(kv_small["meta"], kv_small["blocks"]), (-(-n // 2048), 1))[:n].astype(np.float64).reshape(batch * heads, seq, 128)
+    p = np.exp(scores.astype(np.float64).reshape(batch * heads, qpk, seq))
+    ref = np.matmul(p / p.sum(axis=-1, keepdims=True), dec).reshape(got.shape)
+    rel = float(np.linalg.norm(got - ref) / np.linalg.norm(ref))
+    assert rel <= 2e-7, rel
+
+
 @pytest.mark.parametrize("seq", [33, 700, 3000])
 def test_attn_values_with_rising_scores_and_any_workspace(B, eo, kv_small, seq):
     """Scores that grow along the row (every tile raises the running maximum), fall, or hold their largest value in the last token, over
