@@ -281,6 +281,15 @@ uint64_t ecco_kernel_launch_count(void);
  * no copy will deliver -- nothing is in flight and nothing can hang --, polls it a few hundred times, gives up and
  * returns normally.  Afterwards ecco_device_status() reports ECCO_ERR_DEVICE_TIMEOUT once. */
 int ecco_test_wait_timeout(void* stream);
+/* Test aid for what such a time-out leaves behind where blocks count each other in: ecco_gemv_batch (one row of x, or six to
+ * eight) and ecco_attn_values (shapes of at most 16 warps to a unit, others ECCO_ERR_INVALID_ARG) in which every second CTA of
+ * the launch gives up when its tables have arrived, as if they had not.  Outputs are undefined; ecco_device_status() then
+ * reports ECCO_ERR_DEVICE_TIMEOUT once. */
+int ecco_test_gemv_give_up(const ecco_gemv_item* items, int32_t n_items, int32_t batch, void* d_workspace,
+                           size_t workspace_bytes, void* stream);
+int ecco_test_attn_values_give_up(const void* d_meta, const uint8_t* d_vblocks, int32_t batch, int32_t n_kv_heads, int32_t seq,
+                                  int32_t q_per_kv, const float* d_scores, float* d_out, void* d_workspace, size_t workspace_bytes,
+                                  void* stream);
 
 #ifdef __cplusplus
 }

@@ -36,7 +36,7 @@ EXPORTS = [
     "ecco_gemv", "ecco_gemv_batch_workspace_bytes", "ecco_gemv_batch", "ecco_gemv_static_ws", "ecco_attn_scores", "ecco_act_compress", "ecco_act_decompress",
     "ecco_attn_values_workspace_bytes", "ecco_attn_values", "ecco_kv_compress",
     "ecco_var_stream_bytes_bound", "ecco_var_index_bytes", "ecco_var_encode_host", "ecco_var_decompress", "ecco_error_string", "ecco_last_cuda_error", "ecco_device_status",
-    "ecco_kernel_launch_count", "ecco_test_wait_timeout",
+    "ecco_kernel_launch_count", "ecco_test_wait_timeout", "ecco_test_gemv_give_up", "ecco_test_attn_values_give_up",
 ]
 
 
@@ -124,6 +124,8 @@ def lib():
         L.ecco_device_status.restype = C.c_int
         L.ecco_kernel_launch_count.restype = u64
         L.ecco_test_wait_timeout.argtypes = [vp]
+        L.ecco_test_gemv_give_up.argtypes = L.ecco_gemv_batch.argtypes
+        L.ecco_test_attn_values_give_up.argtypes = L.ecco_attn_values.argtypes
         _lib = L
     return _lib
 
@@ -396,3 +398,16 @@ def ecco_kernel_launch_count() -> int:
 def ecco_test_wait_timeout(stream=None) -> None:
     """Test aid: one small kernel whose bounded wait runs out (see include/ecco.h)."""
     _check(lib().ecco_test_wait_timeout(_stream(stream)), "ecco_test_wait_timeout")
+
+
+def ecco_test_gemv_give_up(items, batch: int, d_workspace, workspace_bytes: int, stream=None) -> None:
+    """Test aid: ecco_gemv_batch in which every second CTA gives up (see include/ecco.h)."""
+    arr = items if isinstance(items, C.Array) else gemv_items(items)
+    _check(lib().ecco_test_gemv_give_up(arr, arr.n_items, batch, _ptr(d_workspace), workspace_bytes, _stream(stream)), "ecco_test_gemv_give_up")
+
+
+def ecco_test_attn_values_give_up(d_meta, d_vblocks, batch: int, n_kv_heads: int, seq: int, q_per_kv: int, d_scores, d_out, d_workspace,
+                                  workspace_bytes: int, stream=None) -> None:
+    """Test aid: ecco_attn_values in which every second CTA gives up (see include/ecco.h)."""
+    _check(lib().ecco_test_attn_values_give_up(_ptr(d_meta), _ptr(d_vblocks), batch, n_kv_heads, seq, q_per_kv, _ptr(d_scores), _ptr(d_out),
+                                               _ptr(d_workspace), workspace_bytes, _stream(stream)), "ecco_test_attn_values_give_up")

@@ -25,7 +25,7 @@ constexpr int kPieceFloats = kGroup * 8 + 16;              // sums of [128 dims]
 // factor that takes sums relative to maximum m to maximum m_new >= m; an empty side has m = -inf and sums of zero
 __device__ __forceinline__ float rescale(float m, float m_new) { return m == m_new ? 1.0f : __expf(m - m_new); }
 
-template <int kMaxWarps>
+template <int kMaxWarps, bool kGiveUp>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __restrict__ d_vblocks, int heads, int seq,
                         int q_per_kv, int unit_warps, int n_teams, const float* d_scores, float* __restrict__ d_out, float* __restrict__ d_partial,
@@ -76,7 +76,16 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     auto block_ptr = [&](int head, int from) { return d_vblocks + (static_cast<uint64_t>(head) * seq + min(from + tid, seq - 1)) * kBlockBytes; };
     issue_decode_tables(tb, d_meta);
     if (u0 < u1 && working) prefetch_block_l2(block_ptr(bh, token));
-    if (!finish_decode_tables(tb)) return;
+    if (!finish_decode_tables<kGiveUp>(tb)) {
+        if (teams == 1 && tid == 0) {                      // passes the tickets of the heads it shares: at most the first and the last
+            const int ends[2] = {bh, static_cast<int>(divide(static_cast<uint64_t>(u1 - 1), static_cast<uint64_t>(chunks)))};
+            for (int i = 0; i < 2; ++i) {
+                const int last = split.owner(static_cast<int64_t>(ends[i] + 1) * chunks - 1) - split.owner(static_cast<int64_t>(ends[i]) * chunks);
+                if (last && (i == 0 || ends[1] != ends[0])) pass_ticket(d_tickets + ends[i], last, tag);
+            }
+        }
+        return;
+    }
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (teams > 1 && (!working || u0 >= u1)) return;
     const float T = tb.T;

@@ -112,9 +112,16 @@ __device__ __forceinline__ void build_rank_tables(const DecodeTables& tb)
 }
 // The whole CTA waits for its tables and builds the rest; false (CTA-uniform) if the bounded wait expired.  Then it has waited for the
 // previous kernel of the stream, too: see dependency_wait.
+// kGiveUp (tests): every second CTA does as if it had expired; its copies have landed.
+template <bool kGiveUp = false>
 __device__ __forceinline__ bool finish_decode_tables(const DecodeTables& tb, uint32_t parity = 0)
 {
-    if (!bounded_wait(tb.base, parity, kWaitLimit)) { dependency_wait(); return false; }
+    bool there = bounded_wait(tb.base, parity, kWaitLimit);
+    if (kGiveUp && (blockIdx.x & 1u)) {
+        there = false;
+        if (threadIdx.x == 0) atomicExch(&g_device_status, ECCO_ERR_DEVICE_TIMEOUT);
+    }
+    if (!there) { dependency_wait(); return false; }
     build_rank_tables(tb);
     return true;
 }

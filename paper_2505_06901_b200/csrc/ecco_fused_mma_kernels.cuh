@@ -55,7 +55,7 @@ __device__ __forceinline__ void load_vfrag(uint32_t (&vfrag)[16], const __half* 
 
 // K2m: y[b][n] = sum_k W~[n][k] x[b][k] for six to eight rows of x.  Units (over all matrices of the call), ownership and the
 // slot-and-ticket reduction are those of the per-warp kernel (unit = 32 rows x one k-block).
-template <int kMaxWarps>
+template <int kMaxWarps, bool kGiveUp>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float* __restrict__ d_partial,
                      Ticket* d_tickets, Ticket tag)
@@ -81,7 +81,7 @@ ecco_gemv_mma_kernel(const __grid_constant__ GemvBatch batch, int n_cols, float*
     }
     GemvPos pos = {0, 0, 0};
     if (u0 < u1) { pos = gemv_pos_of(batch, u0); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
-    if (!finish_decode_tables(tb)) return;
+    if (!finish_decode_tables<kGiveUp>(tb)) { pass_gemv_tickets(batch, split, u0, u1, d_tickets, tag); return; }
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
     if (u0 >= u1) return;
 

@@ -146,7 +146,8 @@ struct UnitSplit {
 // block is on the way: if the word does not carry the tag, an exchange against what was seen installs it, and it fails exactly
 // when another has done so.  Taking is then one addition.  (Counting up by exchanges alone serialises the arrivals: 39 us instead of
 // 17 for a 4096 x 4096 product.)  The last to arrive clears the word, so a captured call that is replayed with its tag finds none of
-// its own counts.
+// its own counts.  For that everyone has to arrive: a CTA whose table fetch timed out passes its tickets (and its call's output is
+// undefined, but the next replay's is not).
 using Ticket = unsigned long long;
 constexpr int kTicketStride = 4;                           // words from one ticket to the next: each in a sector of its own
 __device__ __forceinline__ Ticket look_at_ticket(const Ticket* word) { return *reinterpret_cast<const volatile Ticket*>(word); }
@@ -155,6 +156,12 @@ __device__ __forceinline__ void claim_ticket(Ticket* word, Ticket seen, Ticket t
     if ((seen >> 16) != tag) atomicCAS(word, seen, tag << 16);
 }
 __device__ __forceinline__ unsigned int take_ticket(Ticket* word) { return static_cast<unsigned int>(atomicAdd(word, 1ull) & 0xffffu); }
+// takes a ticket for nothing; the last of them has number `last`
+__device__ __forceinline__ void pass_ticket(Ticket* word, int last, Ticket tag)
+{
+    claim_ticket(word, look_at_ticket(word), tag);
+    if (take_ticket(word) == static_cast<unsigned int>(last)) *word = 0;
+}
 
 // One call of the fused GEMV may cover several matrices (ecco_gemv_batch): the units of all of them form one unit
 // space, dealt out to the working warps as one, so that a group of small matrices pays one launch, one table fetch and
@@ -216,6 +223,21 @@ __device__ __forceinline__ const uint8_t* gemv_block_ptr(const GemvBatch& batch,
     return jb.blocks + (static_cast<uint64_t>(row) * jb.kblocks + p.kb) * kBlockBytes;
 }
 
+// A warp that gives up units u0 .. u1 - 1 passes the tickets of the row tiles it shares: at most the first and the last.
+__device__ __forceinline__ void pass_gemv_tickets(const GemvBatch& batch, const UnitSplit& split, int64_t u0, int64_t u1, Ticket* d_tickets, Ticket tag)
+{
+    if (u0 >= u1 || (threadIdx.x & 31u)) return;
+    int done = -1;
+    for (int end = 0; end < 2; ++end) {
+        const GemvPos pos = gemv_pos_of(batch, end ? u1 - 1 : u0);
+        const GemvJob& jb = batch.job[pos.j];
+        const int64_t g0 = jb.unit_first + static_cast<int64_t>(pos.tile) * jb.kblocks;
+        const int gtile = gemv_tile_of(batch, pos), last = split.owner(g0 + jb.kblocks - 1) - split.owner(g0);
+        if (last && gtile != done) pass_ticket(d_tickets + gtile * kTicketStride, last, tag);
+        done = gtile;
+    }
+}
+
 __host__ __device__ constexpr uint32_t scalar_warp_bytes(int v) { return v * kGroup * 2 + kRankedBytes; }
 
 // K2 for one to five rows of x: the slice is small enough (256 B a row) for every warp to keep
@@ -226,7 +248,7 @@ __host__ __device__ constexpr uint32_t scalar_warp_bytes(int v) { return v * kGr
 // staircase of (warp, tile) pairs) and the last to arrive (ticket counter) adds the slots in warp
 // order: the result does not depend on scheduling.  Workspace: partial[slot][kV][32] floats, then
 // one ticket per 32-row tile.
-template <int kV, int kMaxWarps>
+template <int kV, int kMaxWarps, bool kGiveUp>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict__ d_partial, Ticket* d_tickets, Ticket tag)
 {
@@ -255,7 +277,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     }
     GemvPos pos = {0, 0, 0};
     if (u0 < u1) { pos = gemv_pos_of(batch, u0); prefetch_block_l2(gemv_block_ptr(batch, pos, lane)); }
-    if (!finish_decode_tables(tb)) return;
+    if (!finish_decode_tables<kGiveUp>(tb)) { pass_gemv_tickets(batch, split, u0, u1, d_tickets, tag); return; }
     dependency_wait();                                     // everything but the host-written tables: after the previous kernel of the stream
 
     float acc[kV][kChains];                             // partial sums, added when the row tile is left

@@ -271,9 +271,10 @@ static void gemv_call_add(GemvCall* c, const void* d_meta, const uint8_t* d_bloc
 }
 
 // six to eight rows of x: the tensor-core kernel
+template <bool kGiveUp = false>
 static int launch_gemv_mma_call(const DeviceInfo& di, const GemvCall& c, int batch, void* d_ws, size_t ws_bytes, cudaStream_t stream)
 {
-    auto kernel = ecco_gemv_mma_kernel<kMmaWarps>;
+    auto kernel = ecco_gemv_mma_kernel<kMmaWarps, kGiveUp>;
     static thread_local bool configured[64] = {};
     int rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
@@ -295,11 +296,11 @@ static int launch_gemv_mma(const DeviceInfo& di, const void* d_meta, const uint8
 }
 
 // one to five rows of x (batch == kV): the per-warp kernel
-template <int kV>
+template <int kV, bool kGiveUp = false>
 static int launch_gemv_warp_call(const DeviceInfo& di, const GemvCall& c, void* d_ws, size_t ws_bytes, cudaStream_t stream)
 {
     constexpr int kFusedWarps = gemv_warp_warps(kV);
-    auto kernel = ecco_gemv_warp_kernel<kV, kFusedWarps>;
+    auto kernel = ecco_gemv_warp_kernel<kV, kFusedWarps, kGiveUp>;
     static thread_local bool configured[64] = {};
     int rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
@@ -395,6 +396,22 @@ extern "C" int ecco_gemv_batch(const ecco_gemv_item* items, int32_t n_items, int
         case 5: return launch_gemv_warp_call<5>(di, c, d_workspace, workspace_bytes, s);
         default: return launch_gemv_mma_call(di, c, batch, d_workspace, workspace_bytes, s);
     }
+}
+
+extern "C" int ecco_test_gemv_give_up(const ecco_gemv_item* items, int32_t n_items, int32_t batch, void* d_workspace,
+                                      size_t workspace_bytes, void* stream)
+{
+    int rc = check_gemv_items(items, n_items, batch);
+    if (rc) return rc;
+    if (batch > 1 && pad_v(batch) < 8) return ECCO_ERR_INVALID_ARG;
+    DeviceInfo di;
+    rc = device_info(&di);
+    if (rc) return rc;
+    GemvCall c;
+    gemv_call_from_items(&c, items, n_items);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return batch == 1 ? launch_gemv_warp_call<1, true>(di, c, d_workspace, workspace_bytes, s)
+                      : launch_gemv_mma_call<true>(di, c, batch, d_workspace, workspace_bytes, s);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -540,11 +557,11 @@ AvPlan av_plan(int batch, int n_kv_heads, int seq, int ctas_max)
     return p;
 }
 
-template <int kWarps>
+template <int kWarps, bool kGiveUp = false>
 int launch_attn_values(const DeviceInfo& di, const AvPlan& p, const void* d_meta, const uint8_t* d_vblocks, int heads, int seq,
                        int q_per_kv, const float* d_scores, float* d_out, float* partial, Ticket* tickets, cudaStream_t s)
 {
-    auto kernel = ecco_attn_values_kernel<kWarps>;
+    auto kernel = ecco_attn_values_kernel<kWarps, kGiveUp>;
     static thread_local bool configured[64] = {};
     const int rc = want_all_smem(kernel, &configured[di.device]);
     if (rc) return rc;
@@ -563,9 +580,10 @@ extern "C" size_t ecco_attn_values_workspace_bytes(int32_t batch, int32_t n_kv_h
     return p.partial_bytes + p.ticket_bytes;
 }
 
-extern "C" int ecco_attn_values(const void* d_meta, const uint8_t* d_vblocks, int32_t batch, int32_t n_kv_heads, int32_t seq,
-                                int32_t q_per_kv, const float* d_scores, float* d_out, void* d_workspace, size_t workspace_bytes,
-                                void* stream)
+template <bool kGiveUp>
+static int attn_values(const void* d_meta, const uint8_t* d_vblocks, int32_t batch, int32_t n_kv_heads, int32_t seq,
+                       int32_t q_per_kv, const float* d_scores, float* d_out, void* d_workspace, size_t workspace_bytes,
+                       void* stream)
 {
     if (batch == 0 || n_kv_heads == 0) return (batch < 0 || n_kv_heads < 0) ? ECCO_ERR_INVALID_ARG : ECCO_OK;
     if (!d_meta || !d_vblocks || !d_scores || !d_out) return ECCO_ERR_INVALID_ARG;
@@ -578,12 +596,27 @@ extern "C" int ecco_attn_values(const void* d_meta, const uint8_t* d_vblocks, in
     const AvPlan p = av_plan(batch, n_kv_heads, seq, di.sms < 256 ? di.sms : 256);
     if (!d_workspace || !aligned16(d_workspace)) return d_workspace ? ECCO_ERR_ALIGNMENT : ECCO_ERR_WORKSPACE;
     if (workspace_bytes < p.partial_bytes + p.ticket_bytes) return ECCO_ERR_WORKSPACE;
+    if (kGiveUp && p.unit_warps > kAvWarps) return ECCO_ERR_INVALID_ARG;       // no kernel for it
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* wsb = static_cast<uint8_t*>(d_workspace);
     float* partial = reinterpret_cast<float*>(wsb);
     Ticket* tickets = reinterpret_cast<Ticket*>(wsb + p.partial_bytes);
-    auto launch = p.unit_warps > kAvWarps ? launch_attn_values<kAvManyWarps> : launch_attn_values<kAvWarps>;
+    auto launch = p.unit_warps > kAvWarps ? launch_attn_values<kAvManyWarps> : launch_attn_values<kAvWarps, kGiveUp>;
     return launch(di, p, d_meta, d_vblocks, batch * n_kv_heads, seq, q_per_kv, d_scores, d_out, partial, tickets, s);
+}
+
+extern "C" int ecco_attn_values(const void* d_meta, const uint8_t* d_vblocks, int32_t batch, int32_t n_kv_heads, int32_t seq,
+                                int32_t q_per_kv, const float* d_scores, float* d_out, void* d_workspace, size_t workspace_bytes,
+                                void* stream)
+{
+    return attn_values<false>(d_meta, d_vblocks, batch, n_kv_heads, seq, q_per_kv, d_scores, d_out, d_workspace, workspace_bytes, stream);
+}
+
+extern "C" int ecco_test_attn_values_give_up(const void* d_meta, const uint8_t* d_vblocks, int32_t batch, int32_t n_kv_heads, int32_t seq,
+                                             int32_t q_per_kv, const float* d_scores, float* d_out, void* d_workspace, size_t workspace_bytes,
+                                             void* stream)
+{
+    return attn_values<true>(d_meta, d_vblocks, batch, n_kv_heads, seq, q_per_kv, d_scores, d_out, d_workspace, workspace_bytes, stream);
 }
 
 

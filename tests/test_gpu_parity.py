@@ -505,6 +505,58 @@ def test_gemv_does_not_care_what_the_workspace_holds(B, eo, cfg1_small, synth, n
     check_fused(first.cpu().numpy().astype(np.float64), ref, refabs, f"gemv b{batch} workspaces")
 
 
+def counts_left(ws, partial_floats, stride, n):
+    """The counts in the ticket words of a workspace: the low 16 bits of n 64-bit words, `stride` words apart, behind the partial sums."""
+    at = -(-partial_floats * 4 // 256) * 256
+    return ws[at: at + 8 * stride * n].cpu().numpy().view(np.uint64)[::stride] & np.uint64(0xFFFF)
+
+
+@pytest.mark.parametrize("batch", [1, 8])
+@pytest.mark.parametrize("n_out,k", [(40, 4096), (96, 640), (32, 8192)])
+def test_gemv_blocks_that_give_up_leave_no_count(B, cfg1_small, synth, batch, n_out, k):
+    """A CTA whose table fetch times out passes the tickets of the row tiles it shares: a word left with a count would be wrong at
+    every replay of a captured call.  At most 64 units, so every unit has a CTA and a slot of its own."""
+    n = n_out * (k // 128)
+    tiles = -(-n_out // 32)
+    units = tiles * (k // 128)
+    blocks = np.tile(cfg1_small["blocks"], (-(-n // 2048), 1))[:n]
+    y = torch.empty((batch, n_out), device="cuda")
+    items = [(B.meta_to_device(lib_meta_from_oracle(B, cfg1_small["meta"])), dev(blocks), n_out, k, dev(synth.activations(batch, k, 3)), y)]
+    wsb = B.ecco_gemv_batch_workspace_bytes(items, batch)
+    ws = torch.zeros(wsb, dtype=torch.uint8, device="cuda")
+    B.ecco_gemv_batch(items, batch, ws, wsb)
+    want = y.clone()
+    for _ in range(3):
+        B.ecco_test_gemv_give_up(items, batch, ws, wsb)
+        torch.cuda.synchronize()
+        assert B.ecco_device_status() == B.ERR_DEVICE_TIMEOUT
+        words = ws.view(torch.int64)
+        assert bool((words != 0).any())
+        assert not counts_left(ws, (units + tiles) * (1 if batch == 1 else 8) * 32, 4, tiles).any()
+        B.ecco_gemv_batch(items, batch, ws, wsb)
+        assert torch.equal(y, want) and B.ecco_device_status() == 0
+
+
+def test_attn_values_blocks_that_give_up_leave_no_count(B, kv_small):
+    """The same for the heads that CTAs share: two rows of 20 tiles, one tile to a CTA."""
+    heads, seq, qpk = 2, 640, 4
+    blocks = kv_small["blocks"][: heads * seq]
+    scores = np.random.Generator(np.random.PCG64(1)).standard_normal((1, heads * qpk, seq)).astype(np.float32)
+    out = torch.empty((1, heads * qpk, 128), device="cuda")
+    wsb = B.ecco_attn_values_workspace_bytes(1, heads, seq, qpk)
+    ws = torch.zeros(wsb, dtype=torch.uint8, device="cuda")
+    args = (B.meta_to_device(lib_meta_from_oracle(B, kv_small["meta"])), dev(blocks), 1, heads, seq, qpk, dev(scores), out, ws, wsb)
+    B.ecco_attn_values(*args)
+    want = out.clone()
+    for _ in range(3):
+        B.ecco_test_attn_values_give_up(*args)
+        torch.cuda.synchronize()
+        assert B.ecco_device_status() == B.ERR_DEVICE_TIMEOUT
+        assert not counts_left(ws, (heads * 20 + heads) * (128 * 8 + 16), 1, heads).any()
+        B.ecco_attn_values(*args)
+        assert torch.equal(out, want) and B.ecco_device_status() == 0
+
+
 # ------------------------------------------------------------------ fused attention scores
 @pytest.mark.parametrize("batch,heads,seq,qpk", [(2, 4, 256, 1), (2, 4, 256, 2), (2, 4, 256, 8), (1, 3, 77, 4), (1, 1, 1, 1),
                                                  (2, 2, 513, 3)])
