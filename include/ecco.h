@@ -120,7 +120,8 @@ int ecco_encode_host(ecco_meta* meta, const uint16_t* src_fp16, uint64_t n_group
 
 /* Device image of the metadata (Sec. 4.2: loaded once before the compressed loads): header,
  * patterns, and the prebuilt decode tables.  The caller copies `bytes` bytes from host_staging to
- * 16-byte aligned device memory and passes that pointer as d_meta. */
+ * 16-byte aligned device memory and passes that pointer as d_meta.  The image is not checked again on the device: its
+ * header has to be whole; damaged table bytes give unspecified values. */
 size_t ecco_meta_device_bytes(const ecco_meta* meta);
 int ecco_meta_serialize_device(const ecco_meta* meta, void* host_staging, size_t bytes);
 

@@ -28,9 +28,12 @@ constexpr uint32_t kSmemPairMin = kSmemRec + kCbRecBytes;            // 7168
 constexpr uint32_t kCentBytes = kMaxPatterns * kCodebooks * 32;      // centroids in rank order, fp16 [256][16]
 constexpr uint32_t kBitRows = 19;                                    // 16 words of a block and three zero rows
 constexpr uint32_t kBitBytes = kBitRows * 128;
-// A lane whose stream has ended goes on reading rows after its own: the next warp's or, behind the last warp, this slack.  What it
-// decodes there is cut to zero, and no row lies further than 128 codewords of 8 bits behind the header: 22 + 1024 bits, rows 32..34.
-constexpr uint32_t kSlackBytes = (35 - kBitRows) * 128;              // 2048
+// A lane whose stream has ended goes on reading rows after its own: the next warp's or, behind the last warp, what lies there.  What it
+// decodes is cut to zero.  Whatever bytes the tables hold, an ID_KP entry moves the position by 255 bits at most, a step by 127 (the
+// sum of four entries' lengths is taken modulo 128; one symbol at a time 8 x 15) and the second window of the last step lies 63 bits
+// on: the third word of it is the furthest.  So the last part of a CTA's shared memory belongs to a table that is longer than that.
+constexpr uint32_t kFurthestRow = (kHeaderBits + 255 + 15 * 127 + 63) / 32 + 2;
+static_assert((kFurthestRow + 1 - kBitRows) * 128 <= kKpLutBytes, "a lane that runs on stays in the CTA's shared memory");
 
 struct DecodeTables {
     uint32_t base;          // misc area (barrier word at +0)
@@ -51,8 +54,8 @@ __device__ __forceinline__ DecodeTables plan_decode_tables(uint32_t smem_base, c
     const uint32_t align = min(max(__ldg(&hd->pair_align), 512u), 2u << kPairMaxBits);
     tb.pair = smem_base + kSmemPairMin;
     if (tb.pair_bytes) tb.pair = (tb.pair + align - 1u) & ~(align - 1u);
-    tb.kp = tb.pair + tb.pair_bytes;
-    tb.cent = tb.kp + kKpLutBytes;
+    tb.kp = smem_base + kSmemCtaBytes - kKpLutBytes;      // see kFurthestRow
+    tb.cent = tb.pair + tb.pair_bytes;
     tb.shape = (tb.cent + kCentBytes + 255u) & ~255u;
     tb.warp_base = (tb.shape + tb.shape_bytes + 127u) & ~127u;
     tb.pairs = tb.pair_bytes != 0;
@@ -64,7 +67,7 @@ __device__ __forceinline__ DecodeTables plan_decode_tables(uint32_t smem_base, c
 // warps of this CTA that have room for warp_bytes each (the others sit the launch out)
 __device__ __forceinline__ uint32_t decode_warps(const DecodeTables& tb, uint32_t warp_bytes, uint32_t tail_bytes = 0)
 {
-    const uint32_t used = tb.warp_base - tb.base + kSlackBytes + tail_bytes;
+    const uint32_t used = tb.warp_base - tb.base + kKpLutBytes + tail_bytes;
     const uint32_t room = used < kSmemCtaBytes ? kSmemCtaBytes - used : 0u;
     return min(room / warp_bytes, blockDim.x >> 5);
 }
@@ -144,7 +147,7 @@ __device__ __forceinline__ LaneGroup open_lane_group(uint32_t hdr, uint32_t firs
     LaneGroup g;
     const uint32_t kpe = lds_u16(tb.kp + ((hdr >> (kHeaderBits - 1)) & 0x1ffeu));
     g.p = first_bit + kHeaderBits - 1u + (kpe >> 8);
-    const uint32_t cb = (kpe & 0xffu) * kCodebooks + ((hdr >> 8) & 3u);
+    const uint32_t cb = (kpe & (kMaxPatterns - 1u)) * kCodebooks + ((hdr >> 8) & 3u);
     uint32_t top;
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(g.blut), "=r"(g.plut), "=r"(g.mask), "=r"(top) : "r"(tb.base + kSmemRec + cb * 16));
     uint32_t c[8];
@@ -245,7 +248,7 @@ __device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t b
     uint32_t q = g.p + 1u;
     auto step = [&](int i, auto tested) {
         constexpr bool kTest = decltype(tested)::value;
-        const uint32_t row = bits + (q >> 5) * 128;        // past its end a lane reads whatever follows: see kSlackBytes
+        const uint32_t row = bits + (q >> 5) * 128;        // past its end a lane reads whatever follows: see kFurthestRow
         const uint32_t w0 = lds_u32(row), w1 = lds_u32(row + 128), w2 = lds_u32(row + 256);
         const uint32_t lo = __funnelshift_r(w0, w1, q), hi = __funnelshift_r(w1, w2, q);
         uint32_t e[8], x = lo, n = 0;
@@ -308,7 +311,7 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
     };
     auto step = [&](int i, auto tested) {
         constexpr bool kTest = decltype(tested)::value;
-        const uint32_t row = bits + (g.p >> 5) * 128;      // past its end a lane reads whatever follows: see kSlackBytes
+        const uint32_t row = bits + (g.p >> 5) * 128;      // past its end a lane reads whatever follows: see kFurthestRow
         const uint32_t w0 = lds_u32(row), w1 = lds_u32(row + 128), w2 = lds_u32(row + 256);
         const uint32_t lo = __funnelshift_r(w0, w1, g.p), hi = __funnelshift_r(w1, w2, g.p);
         // an entry's low bits are the length of its codewords; funnel shifts take their amount modulo 32

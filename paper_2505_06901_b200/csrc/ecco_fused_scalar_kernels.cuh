@@ -31,7 +31,7 @@ __device__ __forceinline__ void fma_half2(float& acc, uint32_t w, uint32_t x)
 __device__ __forceinline__ float value_of(uint32_t hdr, uint32_t rank, const DecodeTables& tb, float T)
 {
     const uint32_t kpe = lds_u16(tb.kp + ((hdr >> (kHeaderBits - 1)) & 0x1ffeu));
-    const uint32_t cb = (kpe & 0xffu) * kCodebooks + ((hdr >> 8) & 3u);
+    const uint32_t cb = (kpe & (kMaxPatterns - 1u)) * kCodebooks + ((hdr >> 8) & 3u);
     const uint32_t top = lds_u32(tb.base + kSmemRec + cb * 16 + 12);
     const float c = __half2float(__ushort_as_half(static_cast<unsigned short>(lds_u16(cent_row(tb, cb) ^ (rank * 2)))));
     const float v = __half2float(__float2half_rn(c * (fp8_to_float(hdr & 0x7fu) * T)));

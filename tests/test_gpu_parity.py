@@ -245,6 +245,60 @@ def test_decompress_batch_matches_oracle_per_item(B, eo, cfg1_small, kv_small, s
     assert bool((canary == 7.0).all())
 
 
+@pytest.mark.parametrize("fill", ["ones", "random"])
+@pytest.mark.parametrize("which", ["weights", "cache", "many shapes"])
+def test_damaged_tables_give_unspecified_values_only(B, eo, cfg1_small, kv_small, synth, which, fill):
+    """Any bytes in the tables that the decoders look up (ID_KP codes, shape and pair tables; the header and the records whole): lengths
+    of up to 15 bits a symbol, so that lanes run on far behind their streams.  Every call still ends, writes its own output and nothing
+    else, and the same call with the whole image is right afterwards.  The last warp's reads stay inside the CTA's shared memory: the
+    static_assert at kFurthestRow."""
+    from test_gpu_random import code_shapes
+
+    all_shapes = code_shapes()                             # one to a codebook: an image without pair tables
+    any_lens = lambda k, h, rng: list(rng.permutation(np.repeat(np.arange(2, 9), all_shapes[(4 * k + h) % len(all_shapes)])))
+    meta = {"weights": cfg1_small["meta"], "cache": kv_small["meta"], "many shapes": make_meta(eo, any_lens, S=64, seed=6)}[which]
+    whole = B.ecco_meta_serialize_device(lib_meta_from_oracle(B, meta))
+    rng = np.random.Generator(np.random.PCG64(4))
+    hdr = whole[:64].view(np.uint32)
+    kp, rec, shape, pair = 64 + 64 * 32, 64 + 64 * 32 + 8192, 64 + 64 * 32 + 8192 + 4096 + 8320, int(hdr[11])     # csrc/ecco_format.h
+    assert pair >= shape + int(hdr[8]) and pair + int(hdr[9]) == whole.size and (hdr[9] == 0) == (which == "many shapes")
+    damaged = whole.copy()
+    for lo, hi in ((kp, rec), (shape, shape + int(hdr[8])), (pair, whole.size)):
+        damaged[lo:hi] = 0xFF if fill == "ones" else rng.integers(0, 256, hi - lo, dtype=np.uint8)
+    n_out, k, heads, seq, qpk = 256, 1024, 4, 512, 8
+    blocks, n = synth.random_blocks(2048, 11), 2048
+    lm = lib_meta_from_oracle(B, meta)
+    x16 = synth.weight_matrix(256, 1024, 1001)
+    stream, index, _ = B.ecco_var_encode_host(lm, x16, B.SELECT_MSE | B.KEEP_EXPONENT)
+    d_blocks, d_stream, d_index = dev(blocks), dev(stream), dev(index)
+    d_x, d_q, d_s = dev(synth.activations(8, k, 3)), dev(synth.queries(1, heads * qpk, 4)), torch.zeros((1, heads * qpk, seq), device="cuda")
+    ws = torch.empty(max(B.ecco_gemv_workspace_bytes(n_out, k, 8), B.ecco_attn_values_workspace_bytes(1, heads, seq, qpk)), dtype=torch.uint8, device="cuda")
+
+    def calls(image):
+        d_meta, outs = dev(image), []
+
+        def out(count, dtype):                             # with a margin that nobody may write
+            t = torch.full((count + 4096,), 7.0, dtype=dtype, device="cuda")
+            outs.append((t, count))
+            return t
+        B.ecco_decompress(d_meta, d_blocks, n, out(n * 128, torch.float16))
+        B.ecco_decompress(d_meta, d_blocks, 31, out(31 * 128, torch.float16))
+        B.ecco_var_decompress(d_meta, d_stream, d_index, n, out(n * 128, torch.float16))
+        for batch in (1, 4, 8):
+            B.ecco_gemv(d_meta, d_blocks, n_out, k, d_x, batch, out(batch * n_out, torch.float32), ws, ws.numel())
+        for q in (1, 8):
+            B.ecco_attn_scores(d_meta, d_blocks, 1, heads, seq, q, d_q, 0.5, out(heads * q * seq, torch.float32))
+            B.ecco_attn_values(d_meta, d_blocks, 1, heads, seq, q, d_s, out(heads * q * 128, torch.float32), ws, ws.numel())
+        assert B.ecco_device_status() == 0
+        assert all(bool((t[c:] == 7.0).all()) for t, c in outs)
+        return outs
+
+    want = calls(whole)
+    assert_bit_exact(want[0][0][: n * 128].cpu().numpy().reshape(n, 128), eo.decode(meta, blocks))
+    calls(damaged)
+    assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for (a, _), (b, _) in zip(calls(whole), want))
+
+
 @pytest.mark.parametrize("n_groups", [32, 33, 700])
 def test_decompress_batch_of_short_tensors_with_tables_of_their_own(B, eo, cfg1_small, kv_small, synth, n_groups):
     """Eight runs in one launch, each with other tables than the one before and its arrays elsewhere: most warps
