@@ -8,6 +8,8 @@
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
 
+#include <sys/random.h>
+
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -16,7 +18,6 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <random>
 
 #include "../../include/ecco.h"
 #include "ecco_format.h"

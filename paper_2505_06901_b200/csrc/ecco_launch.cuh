@@ -52,11 +52,14 @@ int launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, 
 }
 
 // the tag of a call's ticket words (see take_ticket): 48 bits, never zero, another one for every call of the process
-inline Ticket next_ticket_tag()
+inline Ticket next_ticket_tag() noexcept
 {
     static std::atomic<uint64_t> next{[] {
-        std::random_device rd;
-        return (static_cast<uint64_t>(rd()) << 32 | rd()) ^ static_cast<uint64_t>(std::chrono::steady_clock::now().time_since_epoch().count());
+        // without exceptions: none may leave a C entry (std::random_device throws where it finds no source)
+        uint64_t start = 0;
+        if (getrandom(&start, sizeof start, GRND_NONBLOCK) != static_cast<ssize_t>(sizeof start))
+            start = static_cast<uint64_t>(std::chrono::steady_clock::now().time_since_epoch().count()) * 0x9e3779b97f4a7c15ull ^ reinterpret_cast<uintptr_t>(&start);
+        return start;
     }()};
     for (;;) {
         const Ticket tag = next.fetch_add(1, std::memory_order_relaxed) & ((1ull << 48) - 1);
