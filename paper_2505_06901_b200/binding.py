@@ -263,8 +263,11 @@ def _stream(stream) -> int:
             import torch
 
             torch.cuda.init()
-            raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-            _current_raw_stream = lambda: raw(device())  # noqa: E731
+            raw, device = (getattr(torch._C, name, None) for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+            if raw and device:
+                _current_raw_stream = lambda: raw(device())  # noqa: E731
+            else:
+                _current_raw_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
         return _current_raw_stream()
     return stream if isinstance(stream, int) else stream.cuda_stream
 

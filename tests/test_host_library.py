@@ -32,6 +32,21 @@ def test_library_exports_every_declared_symbol(binding):
     assert binding.lib().ecco_error_string(-3) == b"non-finite input value"
 
 
+def test_current_stream_without_the_short_cut(binding, monkeypatch):
+    """The current stream's handle comes from two functions that torch does not document; without them, from torch.cuda.current_stream()."""
+    import types
+
+    import torch
+
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1234))
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        with monkeypatch.context() as m:
+            m.setattr(binding, "_current_raw_stream", None)
+            m.delattr(torch._C, name, raising=False)
+            assert binding._stream(None) == 0x1234
+
+
 def test_argument_errors_without_a_gpu(binding, cfg1_small, eo):
     L = binding.lib()
     lm = lib_meta_from_oracle(binding, cfg1_small["meta"])
