@@ -26,7 +26,7 @@ constexpr uint32_t kSmemPat = kMisc;                                 // [64][16]
 constexpr uint32_t kSmemRec = kSmemPat + kPatternBytes;              // [256] x 16 B codebook records, see build_rank_tables
 constexpr uint32_t kSmemPairMin = kSmemRec + kCbRecBytes;            // 7168
 constexpr uint32_t kCentBytes = kMaxPatterns * kCodebooks * 32;      // centroids in rank order, fp16 [256][16]
-constexpr uint32_t kBitRows = 19;                                    // 16 words of a block and three zero rows
+constexpr uint32_t kBitRows = 19;                                    // 16 words of a block, three rows of scratch for the outliers
 constexpr uint32_t kBitBytes = kBitRows * 128;
 // A lane whose stream has ended goes on reading rows after its own: the next warp's or, behind the last warp, what lies there.  What it
 // decodes is cut to zero.  Whatever bytes the tables hold, an ID_KP entry moves the position by 255 bits at most, a step by 127 (the
@@ -76,10 +76,7 @@ __device__ __forceinline__ void issue_decode_tables(const DecodeTables& tb, cons
 {
     const uint32_t bar = tb.base;
     if (threadIdx.x == 0) {
-        if (first) {
-            mbar_init(bar, 1);
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
+        if (first) mbar_init(bar, 1);
         const DevHeader* hd = reinterpret_cast<const DevHeader*>(d_meta);
         mbar_expect_tx(bar, kFixedTableBytes + tb.shape_bytes + tb.pair_bytes);
         bulk_g2s(tb.base + kSmemPat, d_meta + kOffPattern, kPatternBytes, bar);
@@ -190,12 +187,6 @@ __device__ __forceinline__ LaneGroup open_block(const Block& blk, uint32_t bits,
     for (int i = 0; i < 16; ++i) sts_u32(bits + i * 128, blk.w[i]);
     return open_lane_group(blk.w[0], 0u, tb, T);
 }
-__device__ __forceinline__ void clear_tail_rows(uint32_t bits)
-{
-    sts_u32(bits + 16 * 128, 0u);
-    sts_u32(bits + 17 * 128, 0u);
-    sts_u32(bits + 18 * 128, 0u);
-}
 
 // Eight ranks (nibbles, first symbol lowest) -> eight fp16 values, two to a word.  A byte permute selects among eight
 // bytes with three bits of a nibble, so both halves of a plane are read and the ranks' top bits choose between them.
@@ -242,9 +233,9 @@ __device__ __forceinline__ void cut_values(uint32_t (&v)[4], int n_ok)
 // them: twice the lookups (3.4 wavefronts per symbol of a warp instead of 1.7).
 struct NoRefill {};
 template <uint32_t kEndBit, int kFreeSteps, class Sink, class Refill = NoRefill>
-__device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t bits, Sink&& sink, int* n_valid = nullptr, Refill&& refill = {})
+__device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t bits, Sink&& sink, Refill&& refill = {})
 {
-    int fit = kGroup;
+    bool complete = true;
     uint32_t q = g.p + 1u;
     auto step = [&](int i, auto tested) {
         constexpr bool kTest = decltype(tested)::value;
@@ -272,7 +263,7 @@ __device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t b
                 if (at > kEndBit) n_ok = j;                // positions only grow
                 at -= e[j] >> 4;
             }
-            if (n_ok < 8) fit = min(fit, 8 * i + n_ok);
+            complete = complete && n_ok == 8;
         }
         sink(i, ranks, cutting, n_ok);
         if constexpr (!cuda::std::is_same_v<cuda::std::remove_reference_t<Refill>, NoRefill>) {
@@ -286,24 +277,25 @@ __device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t b
 #pragma unroll 1
     for (int i = kFreeSteps; i < 16; i += 2) { step(i, cuda::std::true_type{}); step(i + 1, cuda::std::true_type{}); }
     g.p = q - 1u;
-    if (n_valid) *n_valid = fit;
-    return fit == kGroup ? q : 0u;
+    return complete ? q : 0u;
 }
 
 // Decodes the 128 symbols of the lane's group, eight per step (Sec. 4.2, Huffman decode), and hands every step's ranks (nibbles,
 // first symbol lowest) to sink(step, ranks, cutting, n_ok).  A codeword that would cross the end bit ends the group: that and
 // all later positions are clipped.  cutting (uniform over the warp) says that some lane may have clipped positions in this step, n_ok how
-// many of the lane's eight are there (8 if not cutting).  Returns the end bit if all 128 fitted, else 0; *n_valid = number of positions that
-// fitted.  Must be called by all 32 lanes of the warp.
-// kLastRow / kEndBit: last data row of the lane's staged stream (two more rows follow, which read as zero) and the bit at which
-// the stream ends.  kFreeSteps: that many leading steps carry no end test; the caller guarantees that the stream cannot end in them.
+// many of the lane's eight are there (8 if not cutting).  Returns the end bit if all 128 fitted, else 0.  Must be called by all 32 lanes of
+// the warp.
+// What lies behind the end bit is arbitrary: a codeword that ends by then does not depend on it, and one that does not ends behind it
+// whatever it looks like there.
+// kLastRow / kEndBit: the row of that bit, and the bit, counted from the lane's staged stream.  kFreeSteps: that many leading steps
+// carry no end test; the caller guarantees that the stream cannot end in them.
 // pairs = false (uniform): decode_group_by_one.
 // refill(p): called after every step, for a lane that holds a part of its stream only; it may move p, which is LaneGroup::p.
 template <uint32_t kLastRow, uint32_t kEndBit, int kFreeSteps, class Sink, class Refill = NoRefill>
-__device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink, int* n_valid = nullptr, Refill&& refill = {})
+__device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink, Refill&& refill = {})
 {
-    if (!pairs) return decode_group_by_one<kEndBit, kFreeSteps>(g, bits, sink, n_valid, refill);
-    int fit = kGroup;
+    if (!pairs) return decode_group_by_one<kEndBit, kFreeSteps>(g, bits, sink, refill);
+    bool complete = true;
     // second symbol of an escape entry: its codeword starts 1 + (length of the first) bits into win
     auto resolve = [&](uint32_t e, uint32_t win) {
         const uint32_t b = lds_u8(g.blut ^ ((win >> (1u + (e & 15u))) & 0xffu));
@@ -361,7 +353,7 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
             const int first = lds_u8(g.blut ^ (__funnelshift_r(lds_u32(r), lds_u32(r + 128), q) & 0xffu)) >> 4;
             n_ok = (start + first <= room ? 1 : 0) + (c0 <= room ? 2 : 0) + (c1 <= room ? 2 : 0) + (c2 <= room ? 2 : 0);
             if (c3 <= room) n_ok = 8;
-            else fit = min(fit, 8 * i + n_ok);
+            else complete = false;
         }
         g.p += n;
         sink(i, ranks, cutting, n_ok);
@@ -371,8 +363,7 @@ __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bo
     for (int i = 0; i < kFreeSteps; i += 2) { step(i, cuda::std::false_type{}); step(i + 1, cuda::std::false_type{}); }
 #pragma unroll 1
     for (int i = kFreeSteps; i < 16; i += 2) { step(i, cuda::std::true_type{}); step(i + 1, cuda::std::true_type{}); }
-    if (n_valid) *n_valid = fit;
-    return fit == kGroup ? g.p + 1u : 0u;
+    return complete ? g.p + 1u : 0u;
 }
 constexpr int kBlockFreeSteps = 6;     // the indices of a block start at bit 22 at the latest: 6 steps end by bit 22 + 6 * 64 = 406
 

@@ -28,7 +28,6 @@ ecco_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __rest
     const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, true);
     const uint32_t nw = decode_warps(tb, kSmallWarpBytes);
     const uint32_t bits = tb.warp_base + warp * kSmallWarpBytes + lane * 4;
-    if (warp < nw) clear_tail_rows(bits);
     const uint64_t n_tiles = (n_groups + 31) / 32;
     // every working warp gets the same number of tiles (+-1 over the whole grid); warp ids interleave over
     // the CTAs, so every SM keeps the same number busy
@@ -133,7 +132,6 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
         const uint32_t stage = tiles_base + warp * 1024;                       // this warp's staging tile
         const uint32_t bits = tiles_base + nw * 1024 + warp * kBitBytes + lane * 4;
         const uint32_t my_row = stage + lane * 32;
-        if (warp < nw) clear_tail_rows(bits);
         const uint32_t tile_stride = balanced_warps(run_tiles, gridDim.x * nw);
         uint32_t gt = warp * gridDim.x + blockIdx.x;                           // tile in the run's tile space
         if (warp >= nw || gt >= tile_stride) gt = run_tiles;
@@ -335,7 +333,7 @@ ecco_var_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint4* __re
                 __syncwarp();
                 if (lane == 0) { tma_store_2d(&out_map, stage, i * 8 - 8, row0); bulk_commit(); }
             }
-        }, nullptr, [&](uint32_t& p) {
+        }, [&](uint32_t& p) {
             if (p > limit) {
                 sp.at += p >> 6;
                 sp.end -= min(sp.end, p & ~63u);

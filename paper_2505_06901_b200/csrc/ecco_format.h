@@ -20,10 +20,10 @@ constexpr int kHeaderBits = 10;    // scale byte + ID_HF
 constexpr int kExpMin = -32, kExpMax = 16;
 
 // Device image of the per-tensor metadata: a 64-byte header, fixed-size tables, then two sections whose size
-// depends on the codebooks (DevHeader says how large they are).  What the decoders stage into shared memory is
-//   [pattern | ID_KP table | codebook records]   one bulk copy, kFixedTableBytes
-//   [shape tables]                                 one bulk copy, n_shapes * 256 bytes
-//   [pair tables]                                  one bulk copy, pair_bytes, to an address aligned to pair_align
+// depends on the codebooks (DevHeader says how large they are).  The decoders stage into shared memory, with a bulk copy each,
+//   pattern, codebook records, ID_KP table         kFixedTableBytes together
+//   shape tables                                   n_shapes * 256 bytes
+//   pair tables                                    pair_bytes, to an address aligned to pair_align (kernels that use them)
 //
 // Code shapes.  A canonical code is fixed by how many of its 16 codewords have each length; the 256 codebooks of a
 // tensor share a few dozen such shapes.  The decode tables are stored per shape and work on the symbol's RANK, its
@@ -34,8 +34,8 @@ constexpr int kExpMin = -32, kExpMax = 16;
 // Shape table [256] u8, indexed by the next 8 stream bits (first stream bit in bit 0): length << 4 | rank.
 // Pair table [2^W] u16 (W = 8..12 per shape), indexed by the next W stream bits: two symbols per lookup,
 //   bits 0..3   length of both codewords together           (escape: length of the first)
-//   bits 4..6   zero (room for the sum of two entries)
-//   bits 7..10  rank of the first symbol, i.e. rank << 7 = its byte offset in a [16][32] u32 value table
+//   bits 4..6   zero
+//   bits 7..10  rank of the first symbol, which leaves room below for the sum of four entries' lengths
 //   bits 11..14 rank of the second symbol                   (escape: zero)
 //   bit  15     escape: the W bits end before the second codeword does; the decoder fetches it on its own
 // Shapes get table widths by expected use (from the ID_KP code lengths) and by how much a wider table lowers the

@@ -260,7 +260,6 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     const int lane = static_cast<int>(threadIdx.x & 31u), warp = static_cast<int>(threadIdx.x >> 5);
     const uint32_t xs = tb.warp_base + warp * scalar_warp_bytes(kV);             // this warp's slice [kV][128] fp16
     const uint32_t bits = xs + kV * kGroup * 2 + kRankRows * 128 + lane * 4;
-    if (warp < nw) clear_tail_rows(bits);
 
     // W working warps (chosen so that they all get the same number of units, and never more than there are
     // units); warp ids interleave over the CTAs; the other warps idle
@@ -392,7 +391,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
     flush(cur_j, cur_tile);
 }
 
-// K3: scores[b][hq][t] = scale * q[b][hq] . K~[b][hq / q_per_kv][t] for one or two query heads per KV head.
+// K3: scores[b][hq][t] = scale * q[b][hq] . K~[b][hq / kV][t] for one or two (kV) query heads per KV head.
 // Built like K2: a work unit is (one (batch, kv head) pair, 32 consecutive tokens), a lane owns one token, every
 // working warp owns a contiguous run of units and keeps its own query slice (restaged
 // when the head changes), so warps never meet at a barrier and a ragged sequence length costs at most one
@@ -400,7 +399,7 @@ ecco_gemv_warp_kernel(const __grid_constant__ GemvBatch batch, float* __restrict
 template <int kV, int kMaxWarps>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __restrict__ d_kblocks, int heads, int seq,
-                        int q_per_kv, const __half* d_q, float scale, float* __restrict__ d_scores)
+                        const __half* d_q, float scale, float* __restrict__ d_scores)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     release_dependents();
@@ -409,7 +408,6 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     const int lane = static_cast<int>(threadIdx.x & 31u), warp = static_cast<int>(threadIdx.x >> 5);
     const uint32_t xs = tb.warp_base + warp * scalar_warp_bytes(kV);             // this warp's slice [kV][128] fp16
     const uint32_t bits = xs + kV * kGroup * 2 + kRankRows * 128 + lane * 4;
-    if (warp < nw) clear_tail_rows(bits);
 
     const int wg = warp < nw ? warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x) : INT_MAX;
     const int tiles = (seq + 31) / 32;
@@ -433,12 +431,11 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     for (int64_t u = u0; u < u1; ++u) {
         const int t = tile * 32 + lane;
         if (bh != cur_bh) {
-            // lane l stages q[b][h*q_per_kv + r][4l .. 4l+3]; heads beyond q_per_kv are zero
+            // lane l stages q[b][h * kV + r][4l .. 4l+3]
             __syncwarp();                                  // every lane is done with the previous head's slice
 #pragma unroll
             for (int r = 0; r < kV; ++r) {
-                uint2 raw = make_uint2(0u, 0u);
-                if (r < q_per_kv) raw = __ldcg(reinterpret_cast<const uint2*>(d_q + (static_cast<size_t>(bh) * q_per_kv + r) * kGroup) + lane);
+                const uint2 raw = __ldcg(reinterpret_cast<const uint2*>(d_q + (static_cast<size_t>(bh) * kV + r) * kGroup) + lane);
                 sts_v2(xs + r * (kGroup * 2) + lane * 8, raw.x, raw.y);
             }
             __syncwarp();
@@ -458,7 +455,7 @@ ecco_attn_scores_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         if (t < seq) {
 #pragma unroll
             for (int r = 0; r < kV; ++r)
-                if (r < q_per_kv) d_scores[(static_cast<size_t>(out_bh) * q_per_kv + r) * seq + t] = scale * sum_of(acc[r]);
+                d_scores[(static_cast<size_t>(out_bh) * kV + r) * seq + t] = scale * sum_of(acc[r]);
         }
     }
 }

@@ -11,8 +11,8 @@
 //            [256][16] fp16 | shape tables [n_shapes][256] u8; all but the centroids are brought in by bulk copies (cp.async.bulk + mbarrier)
 //   per warp bits[19][32] u32   the warp's 32 blocks, word-transposed: lane L's word w at
 //                               [w][L] -> bank L whatever w is (conflict-free refills);
-//                               rows 16 to 18 stay zero (stream bits past 512 read as 0).  The scalar fused kernels keep the decoded
-//                               ranks over its consumed rows, for the outlier fix-up
+//                               rows 16 to 18 are scratch: what a lane reads past stream bit 512 does not matter (decode_group).  The
+//                               scalar fused kernels keep the decoded ranks over its consumed rows, for the outlier fix-up
 //            tiles              ecco_decompress: one [32 groups][16 values] fp16 staging tile for the tensor stores;
 //                               tensor-core kernels: eight of them, the whole decoded group, as MMA operands
 //
@@ -464,7 +464,7 @@ extern "C" int ecco_gemv_static_ws(const void* d_meta, const uint8_t* d_blocks, 
 
 template <int kV>
 static int launch_attn(const DeviceInfo& di, const void* d_meta, const uint8_t* d_kblocks, int batch, int n_kv_heads,
-                       int seq, int q_per_kv, const void* d_q, float scale, float* d_scores, cudaStream_t stream)
+                       int seq, const void* d_q, float scale, float* d_scores, cudaStream_t stream)
 {
     constexpr int kFusedWarps = fused_warps(kV);
     auto kernel = ecco_attn_scores_kernel<kV, kFusedWarps>;
@@ -476,7 +476,7 @@ static int launch_attn(const DeviceInfo& di, const void* d_meta, const uint8_t* 
     const int64_t units = static_cast<int64_t>(heads) * ((seq + 31) / 32);
     const unsigned grid = static_cast<unsigned>(spread_ctas(units, di.sms));
     return launch_overlapped(kernel, grid, spread_threads(units, static_cast<int>(grid), kFusedWarps), kSmemCtaBytes, stream, static_cast<const uint8_t*>(d_meta),
-                             d_kblocks, heads, seq, q_per_kv, static_cast<const __half*>(d_q), scale, d_scores);
+                             d_kblocks, heads, seq, static_cast<const __half*>(d_q), scale, d_scores);
 }
 
 extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, int32_t batch, int32_t n_kv_heads, int32_t seq,
@@ -492,8 +492,8 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     switch (pad_v(q_per_kv)) {
-        case 1: return launch_attn<1>(di, d_meta, d_kblocks, batch, n_kv_heads, seq, q_per_kv, d_q, scale, d_scores, s);
-        case 2: return launch_attn<2>(di, d_meta, d_kblocks, batch, n_kv_heads, seq, q_per_kv, d_q, scale, d_scores, s);
+        case 1: return launch_attn<1>(di, d_meta, d_kblocks, batch, n_kv_heads, seq, d_q, scale, d_scores, s);
+        case 2: return launch_attn<2>(di, d_meta, d_kblocks, batch, n_kv_heads, seq, d_q, scale, d_scores, s);
         default: {
             auto kernel = ecco_attn_scores_mma_kernel<kMmaWarps>;
             static thread_local bool configured[64] = {};
@@ -519,7 +519,7 @@ struct AvPlan { int grid, unit_warps, teams; size_t partial_bytes, ticket_bytes;
 // How a CTA's warps share the work.  A unit is unit_warps tiles (of 32 tokens) of one head.
 // One team: the units of all heads are split evenly over the CTAs, and all SMs should be busy for the same number of turns.  A turn
 // costs about the time of six tiles' decoding however few tiles it has (6, 16 and 40 measured alike), so long rows take the
-// largest units (16 x 8 x 32768 tokens: 16 warps) and short ones are cut until every SM has some.  Against 16 warps throughout:
+// largest units (16 x 8 x 32768 tokens: 19 warps) and short ones are cut until every SM has some.  Against 16 warps throughout:
 // 8 x 32 x 64 tokens 27.1 -> 22.2 us, 2 x 8 x 777 17.4 -> 15.9, 1 x 1 x 32768 39.9 -> 25.5.
 // Several teams of warps, each with heads of its own, for many short rows: one team spends 5 us on every head's reduction, most of it
 // waiting, and the warps beyond the row's few tiles have nothing to do.  Against one team: 32 x 32 x 40 tokens 69.7 -> 17.6 us, 8 x 32 x 64
