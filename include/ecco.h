@@ -151,7 +151,9 @@ int ecco_decompress_batch(const ecco_decompress_item* items, int32_t n_items, vo
 /* Decode-phase GEMV on compressed weights (Sec. 2.1: M = 1 matrix-vector products; Sec. 4.2
  * decode): y[b][n] = sum_k W~[n][k] * x[b][k], fp32 accumulation.  W is row-major [n_out][k],
  * groups along k, block of (n, kblock) at byte 64*(n*(k/128) + kblock).  x is fp16 [batch][k],
- * y is fp32 [batch][n_out], batch in 1..8, k a multiple of 128.  d_workspace: device scratch of
+ * y is fp32 [batch][n_out], batch in 1..8, k a multiple of 128.  A product with a number in x or a
+ * decoded value that is not finite makes the sums it enters not finite; whether infinite or NaN is not
+ * specified.  d_workspace: device scratch of
  * at least ecco_gemv_workspace_bytes(n_out, k, batch) bytes, 16-byte aligned, contents
  * irrelevant before and undefined after; calls sharing a workspace must not overlap. */
 size_t ecco_gemv_workspace_bytes(int32_t n_out, int32_t k, int32_t batch);

@@ -457,6 +457,24 @@ def test_gemv_error_does_not_grow_with_the_rows_of_x(B, eo, cfg1_small, synth, b
     assert rel <= 0.43 * 2.0 ** -24 * np.sqrt((96 + k // 128) / 2), rel
 
 
+@pytest.mark.parametrize("batch", [1, 3, 5, 8])
+def test_gemv_numbers_that_are_not_finite_stay_in_their_sums(B, eo, cfg1_small, synth, batch):
+    """An infinity or a NaN in one row of x, under mapped values and under outliers: that row's outputs are not finite, the others are
+    what they are without it, bit for bit."""
+    lm = lib_meta_from_oracle(B, cfg1_small["meta"])
+    n_out, k = 256, 1024
+    x = synth.activations(batch, k, 9)
+    clean, _ = gpu_gemv(B, lm, cfg1_small["blocks"], n_out, k, x, batch)
+    for bad in (np.inf, -np.inf, np.nan):
+        for at in (0, 517, 1023):
+            y = x.copy()
+            y[batch // 2, at] = bad
+            got, _ = gpu_gemv(B, lm, cfg1_small["blocks"], n_out, k, y, batch)
+            assert not np.isfinite(got[batch // 2]).any()
+            rest = np.arange(batch) != batch // 2
+            assert np.array_equal(got[rest], clean[rest])
+
+
 @pytest.mark.parametrize("batch", [1, 2, 3, 8])
 def test_gemv_batch_gives_every_item_what_gemv_gives(B, eo, cfg1_small, synth, batch):
     """Several matrices in one call (shapes that differ in rows and in k, a ragged row count, a one-row matrix, a shared
