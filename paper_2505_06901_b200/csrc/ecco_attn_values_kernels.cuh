@@ -35,9 +35,6 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     release_dependents();
     const DecodeTables tb = plan_decode_tables(smem_u32(smem), d_meta, false);       // one symbol per lookup: the tiles need the room
-    // More than sixteen warps leave 96 registers to a thread: then the weights are formed behind the decode, not held through it
-    // (19 warps, [16][8][32768][128] cache, eight heads: 535 -> 526 us; 16 warps 551 -> 565).
-    constexpr bool kLate = kMaxWarps > 16;
     constexpr uint32_t kFull = 0xffffffffu, kSlotFloats = kGroup * 8 + 8;       // sums, sums of weights
     // A team of nw warps takes a head at a time.  One team: all CTAs share the units, and the CTA's other warps help with the
     // reductions.  Several: every team has whole heads of its own and meets at a barrier of its own.
@@ -225,7 +222,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
         if ((token += kTokens) >= seq) { token = 0; ++bh; }
         if (working) {                                     // warps without room for their arrays only help with the reductions
             uint32_t p_hi[4], p_lo[4];                     // P^T fragments (B operand): head = lane / 4, tokens (lane % 4) * 2 + {0, 1} + 8 j
-            auto weigh = [&]() {
+            {                                              // (behind the decode, not held through it: 518 -> 541 us with 19 warps, 534 -> 562 with 16)
                 const int r = static_cast<int>(lane >> 2);
                 const float* srow = d_scores + (static_cast<size_t>(head) * q_per_kv + min(r, q_per_kv - 1)) * seq;
                 float s[8], top = m;
@@ -252,8 +249,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
                     p_hi[j] = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);
                     p_lo[j] = static_cast<uint32_t>(__half_as_ushort(l0)) | (static_cast<uint32_t>(__half_as_ushort(l1)) << 16);
                 }
-            };
-            if (!kLate) weigh();
+            }
             Block cur;                                     // fetched now, prefetched into L2 one unit earlier
             ldg_block(cur, block_ptr(head, first_token));
             if (n > 1) {
@@ -264,10 +260,9 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(d_scores + (static_cast<size_t>(bh) * q_per_kv + lane) * seq + nt));
             }
             decode_to_tiles<false, true>(cur, tb, tiles, T, valid);             // past the end of the row: zeros
-            if (kLate) weigh();
             // Per 16-dim tile: (V tile)^T x P^T on the tensor cores.  They cut their sums off instead of rounding them, so only a tile's 32
             // tokens are summed there: error of 16 x 32 x 300 tokens (five tiles to a warp) 2.5e-7 -> 1.6e-7 of the result, of 16 x 8 x
-            // 32768 2.3e-6 -> 2.0e-7, for 54.1 -> 54.4 and 957 -> 976 us with the scores.
+            // 32768 2.3e-6 -> 2.0e-7; [8][32][4096][128] 141.6 -> 142.6 us.
             const uint32_t a_at = tiles + tile_byte((lane >> 4) * 8 + (lane & 7u), ((lane >> 3) & 1u) * 8);
 #pragma unroll
             for (int ch = 0; ch < 8; ++ch) {

@@ -513,7 +513,7 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
 namespace {
 // Warps of a CTA of ecco_attn_values that decode.  19 find room (9.4 KB of shared memory per warp), but with more than 16 a thread has 96
 // registers and the kernel spills a little and takes a few percent more per tile: two kernels, and units of 17 to 19 tiles only where
-// they save turns (a [16][8][32768][128] cache, eight heads, 551 us with 16 and 526 with 19; [8][32][4096][128] 162 and 166).
+// they save turns (a [16][8][32768][128] cache, eight heads, 534 us with 16 and 518 with 19; [8][32][4096][128], before, 162 and 166).
 constexpr int kAvWarps = 16, kAvManyWarps = 19;
 struct AvPlan { int grid, unit_warps, teams; size_t partial_bytes, ticket_bytes; };
 // How a CTA's warps share the work.  A unit is unit_warps tiles (of 32 tokens) of one head.

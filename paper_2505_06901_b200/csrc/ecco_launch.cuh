@@ -93,7 +93,8 @@ constexpr int gemv_warp_warps(int v) { return v == 1 ? 32 : v <= 3 ? 28 : v == 4
 
 // CTAs for `units` warp-sized pieces of work: one per SM as soon as there are that many.  The kernels number their warps
 // across the CTAs first, so a call with fewer pieces than the machine has warp slots puts a few on every SM instead of
-// filling some SMs and leaving the others idle (decode attention over 2 x 8 x 777 tokens, 400 pieces: 37.6 -> 30.4 us).
+// filling some SMs and leaving the others idle (decode attention over 2 x 8 x 777 tokens, 400 pieces: 37.6 -> 30.4 us).  The price is paid by
+// small calls on several streams at once, which find no SM free: eight such calls side by side 20.4 us each, 6.5 with SMs filled first.
 inline int spread_ctas(int64_t units, int ctas_max) { return static_cast<int>(units < ctas_max ? units : ctas_max); }
 
 // Threads of such a CTA: a warp per piece it can get, but no more than the kernel is made for, and at least eight (they share the
