@@ -226,25 +226,28 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
 //  * min / max of the normalised values = normalised min / max (division by the scale is monotone): packed fp16 extremes,
 //    two divisions per group.
 //  * the pattern with the least fp32 fitness wins unless another comes within 2^-20 of it; only then are the fp64 scores formed.
-//  * nearest centroid = number of midpoints below the value.  A table per pattern says for 256 cells of [-1, 1) how many
-//    midpoints lie below the cell and how many inside, so a value is compared with one midpoint or none; the value is x times the
-//    scale's reciprocal, and where that comes within 2^-21 of a midpoint the exact division and fp64 distances decide.
+//  * nearest centroid = number of midpoints below the value.  A table per pattern holds for 256 cells of [-1, 1) how many
+//    midpoints lie below the cell and, in the same word, the next one, so a value costs one lookup and one comparison; the value is x times
+//    the scale's reciprocal, and where that comes within 2.4e-6 of a midpoint the exact division and fp64 distances decide.
+//    (Count and midpoint in tables of their own: two calls of 131 072 groups 106.9 us, in one word 102.3.)
 //  * the four codebooks' lengths are bytes of one word, summed together.
 //  * a lane joins its sixteen codewords into one string of at most 128 bits in registers and ORs five words into the block.
-// Bound by the issue slots (80 % busy, ncu): 310 warp instructions per group against 735 of the kernel above; two calls of
-// 131 072 groups take 106 us against 218.5.  Making the tables costs a call 3 us, which is what the smaller instruction count
+// Bound by the issue slots (80 % busy, ncu): some 300 warp instructions per group against 735 of the kernel above; two calls of
+// 131 072 groups take 102 us against 218.5.  Making the tables costs a call 3 us, which is what the smaller instruction count
 // saves at about 16 000 groups (two calls of 8192: 26.5 against 19.5 us, of 16 384: 30.6 against 31.3): fewer go to the kernel above.
 // ---------------------------------------------------------------------------------------------
 constexpr int kKvManyWarps = 32;
 constexpr int kKvCells = 256;
 constexpr float kCellWidth = 1.0f / 127.5f;
+constexpr float kBeyond = 1.0e30f;                         // no value is above it
 struct KvManySmem {
-    uint8_t cell[kMaxPatterns * kKvCells];                 // midpoints below the cell, | 0x80 if it holds several; rows of 256 bytes
+    // per cell the first midpoint not below it, as a float whose low five bits hold the number of those below, | 16 if the cell holds several
+    uint32_t cell[kMaxPatterns * kKvCells];
     uint16_t pat[kMaxPatterns * 16];
     uint16_t enc[kMaxPatterns * kCodebooks * kSymbols];    // length | codeword in stream order << 8
     uint16_t kp[kMaxPatterns];
     uint32_t len4[kMaxPatterns * kSymbols];                // code lengths of a symbol in the four codebooks, one per byte
-    float mid[kMaxPatterns * 16];                          // midpoints of neighbouring centroids (14 per pattern)
+    float mid[kMaxPatterns * 16];                          // midpoints of neighbouring centroids (14 per pattern), then a large number
     float2 ends[kMaxPatterns];                             // first and last centroid
     uint4 x[kKvManyWarps][64];                             // the warp's four groups, fp16 [4][128]
     uint32_t blk[kKvManyWarps][64];                        // their blocks
@@ -290,7 +293,7 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
             }
         }
         sm.len4[i] = v;
-        sm.mid[i] = s < kCentroids - 1 ? 0.5f * (centroid(k, s) + centroid(k, s + 1)) : INFINITY;
+        sm.mid[i] = s < kCentroids - 1 ? 0.5f * (centroid(k, s) + centroid(k, s + 1)) : kBeyond;
         if (s == 0) sm.ends[k] = make_float2(centroid(k, 0), centroid(k, kCentroids - 1));
     }
     __syncthreads();
@@ -299,14 +302,17 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
     for (int i = tid; i < kMaxPatterns * kKvCells / 16; i += kKvManyWarps * 32) {
         const float* const m = sm.mid + (i / (kKvCells / 16)) * 16;
         int c = (i % (kKvCells / 16)) * 16, below = 0, upto = 0;
-        uint32_t out[4] = {0, 0, 0, 0};
+        uint32_t out[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q, ++c) {
             if (c > 0) while (below < kCentroids - 1 && m[below] < (static_cast<float>(c) - 0.51f) * kCellWidth - 1.0f) ++below;
             while (upto < kCentroids - 1 && (c == kKvCells - 1 || m[upto] <= (static_cast<float>(c) + 0.51f) * kCellWidth - 1.0f)) ++upto;
-            out[q >> 2] |= static_cast<uint32_t>(below | (upto - below > 1 ? 0x80 : 0)) << (8 * (q & 3));
+            // the nearest float that ends in those five bits: at most sixteen places off
+            const uint32_t low = static_cast<uint32_t>(below) | (upto - below > 1 ? 16u : 0u);
+            out[q] = ((__float_as_uint(m[below]) + 16u - low) & ~31u) | low;
         }
-        reinterpret_cast<uint4*>(sm.cell)[i] = make_uint4(out[0], out[1], out[2], out[3]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) reinterpret_cast<uint4*>(sm.cell)[i * 4 + q] = make_uint4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
     }
     __syncthreads();
     dependency_wait();                                     // x and the blocks: after the previous kernel of the stream
@@ -403,16 +409,13 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
         }
         // value mappers
         const float inv = scale == 0.0f ? 0.0f : __fdiv_rn(1.0f, scale);
-        const uint32_t cells = smem_u32(sm.cell) + kp * kKvCells, mids = smem_u32(sm.mid) + kp * 64, lens = smem_u32(sm.len4) + kp * 64;
-        auto cell_of = [&](float u) {                      // NaN: cell 0
-            const uint32_t at = __float_as_uint(fmaf(__saturatef(fmaf(u, 0.5f, 0.5f)), 255.0f, 12582912.0f)) & (kKvCells - 1);
-            uint32_t e;
-            asm("ld.shared.u8 %0, [%1];" : "=r"(e) : "r"(cells | at));
-            return e;
-        };
-        auto shared_float = [](uint32_t a) { float v; asm("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a)); return v; };
+        const uint32_t cells = smem_u32(sm.cell) + kp * (kKvCells * 4) - (0x4b400000u << 2), lens = smem_u32(sm.len4) + kp * 64;
         auto shared_word = [](uint32_t a) { uint32_t v; asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a)); return v; };
-        constexpr float kBand = 4.76837158203125e-7f;      // 2^-21: more than x * (1 / scale) is off by for values up to 1.5
+        auto cell_of = [&](float u) {                      // NaN: cell 0.  The sum's bits are those of 1.5 * 2^23 plus the cell's number
+            return shared_word(__float_as_uint(fmaf(__saturatef(fmaf(u, 0.5f, 0.5f)), 255.0f, 12582912.0f)) * 4u + cells);
+        };
+        // more than x * (1 / scale) is off by for values up to 1.5 (2^-21) and a midpoint up to there by the bits in its last places (2^-19)
+        constexpr float kBand = 2.4e-6f;
         uint32_t syms[2] = {0, 0}, l4 = 0, flags = 0;      // nibbles of values 0..7 and 8..15, the first one highest
         bool near = lo < -1.5f || hi > 1.5f;
 #pragma unroll
@@ -421,19 +424,19 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
             const uint32_t e = cell_of(u);
             flags |= e;
             uint32_t s = e & 15u;
-            const float d = u - shared_float(mids + s * 4);   // without a midpoint in the cell this is the next one above: no step
+            const float d = u - __uint_as_float(e);        // without a midpoint in the cell this is the next one above: no step
             near = near || fabsf(d) <= kBand;
             if (d > 0.0f) ++s;
             syms[j >> 3] = syms[j >> 3] * 16u + s;
             l4 += shared_word(lens + s * 4);
         }
-        if (warp_any(near || (flags & 0x80u))) {
+        if (warp_any(near || (flags & 16u))) {
             // the values in question as defined: exact quotient, fp64 distances, ties to the first centroid
             for (int j = 0; j < 16; ++j) {
                 const float x = __half2float(__ushort_as_half(xs[sub * 16 + j]));
                 const uint32_t e = cell_of(x * inv);
                 if (!(fabsf(x) <= 65504.0f)) continue;     // the abs-max itself
-                if (!(e & 0x80u) && fabsf(x * inv) <= 1.5f && !(fabsf(x * inv - shared_float(mids + (e & 15u) * 4)) <= kBand)) continue;
+                if (!(e & 16u) && fabsf(x * inv) <= 1.5f && !(fabsf(x * inv - __uint_as_float(e)) <= kBand)) continue;
                 const float u = scale == 0.0f ? 0.0f : __fdiv_rn(x, scale);
                 int below = 0;
                 for (int i = 0; i < kCentroids; ++i) below += centroid(kp, i) <= u;
@@ -517,7 +520,7 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
             for (int p = 0; p < n_max; ++p) {
                 uint32_t next = 0;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) next = max(next, key[i] - top);
+                for (int i = 0; i < 16; ++i) next = __viaddmax_u32(key[i], 0u - top, next);
                 top += group_max(next);
                 if (p < n_pad && sub == 0) {
                     const uint32_t loc = 127u - (top & 127u);
