@@ -14,14 +14,18 @@ namespace {
 // bit 7 of the four bytes of w, gathered into bits 0..3
 __device__ __forceinline__ uint32_t top_bits(uint32_t w) { return ((w & 0x80808080u) * 0x00204081u) >> 28; }
 
-// Both kernels are bound by HBM at large sizes.  A thread takes two chunks at a time, both loads in flight before either is
+// Both kernels are bound by HBM at large sizes.  A thread takes kLoads chunks at a time, their loads in flight before any is
 // used: 2048 threads of one 16-byte load each are less than an SM has to have in flight to draw its share of the bandwidth.
+// One or two, as long as the CTAs get by with one turn each, then four.  There and back, one pass among others, us with one / two / four: 1000
+// groups 2.8 / 3.6 / 4.5, 65 536 6.1 / 6.5 / 10.6, 98 304 10.4 / 9.3 / 11.4, 131 072 11.6 / 11.5 / 13.1, 196 608 15.9 / 17.6 / 15.2,
+// 262 144 20.3 / 20.0 / 18.2, 1 000 003 69.0 / 68.4 / 66.5, 2 000 000 135.6 / 138.0 / 131.9.
 // No conversion instruction between integers and floats is used (they issue at a quarter of the rate): a byte becomes a float by its place
 // below the exponent of 2^23, and a float is rounded to an integer by adding 1.5 * 2^23.  262 144 groups there and back, the
-// second kernel becoming resident while the first drains: 26.7 -> 20.4 us (100 MB: 4.9 TB/s).
+// second kernel becoming resident while the first drains: 26.7 -> 20.4 us, and 18.7 with four loads (100 MB: 5.4 TB/s).
 constexpr int kActThreads = 256;
-constexpr uint64_t kActChunks = 2 * kActThreads;           // chunks a CTA takes at a time
+__host__ __device__ constexpr int act_chunks(int loads) { return loads * kActThreads; }        // a CTA takes at a time
 
+template <int kLoads>
 __global__ void __launch_bounds__(kActThreads)
 ecco_act_decompress_kernel(const uint4* __restrict__ d_blocks, uint64_t n_chunks, uint4* __restrict__ d_out)
 {
@@ -29,16 +33,16 @@ ecco_act_decompress_kernel(const uint4* __restrict__ d_blocks, uint64_t n_chunks
     release_dependents();
     dependency_wait();                                     // the blocks may come from the previous kernel of the stream
     const uint32_t lane = threadIdx.x & 31u;
-    for (uint64_t base = blockIdx.x * kActChunks; base < n_chunks; base += gridDim.x * kActChunks) {
-        uint4 in[2];
+    for (uint64_t base = static_cast<uint64_t>(blockIdx.x) * act_chunks(kLoads); base < n_chunks; base += static_cast<uint64_t>(gridDim.x) * act_chunks(kLoads)) {
+        uint4 in[kLoads];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < kLoads; ++k) {
             const uint64_t c = base + k * kActThreads + threadIdx.x;
             in[k] = make_uint4(0, 0, 0, 0);
             if (c < n_chunks) asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(in[k].x), "=r"(in[k].y), "=r"(in[k].z), "=r"(in[k].w) : "l"(d_blocks + c));
         }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < kLoads; ++k) {
             const uint64_t c = base + k * kActThreads + threadIdx.x;
             const uint4 b = in[k];
             const uint32_t bits16 = top_bits(b.x) | (top_bits(b.y) << 4) | (top_bits(b.z) << 8) | (top_bits(b.w) << 12);
@@ -63,15 +67,16 @@ ecco_act_decompress_kernel(const uint4* __restrict__ d_blocks, uint64_t n_chunks
     }
 }
 
+template <int kLoads>
 __global__ void __launch_bounds__(kActThreads)
 ecco_act_compress_kernel(const uint4* __restrict__ d_x, uint64_t n_chunks, uint4* __restrict__ d_blocks)
 {
     release_dependents();
     dependency_wait();                                     // x may come from the previous kernel of the stream
-    for (uint64_t base = blockIdx.x * kActChunks; base < n_chunks; base += gridDim.x * kActChunks) {
-        uint32_t in[2][8];
+    for (uint64_t base = static_cast<uint64_t>(blockIdx.x) * act_chunks(kLoads); base < n_chunks; base += static_cast<uint64_t>(gridDim.x) * act_chunks(kLoads)) {
+        uint32_t in[kLoads][8];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < kLoads; ++k) {
             const uint64_t c = base + k * kActThreads + threadIdx.x;
 #pragma unroll
             for (int i = 0; i < 8; ++i) in[k][i] = 0;
@@ -81,7 +86,7 @@ ecco_act_compress_kernel(const uint4* __restrict__ d_x, uint64_t n_chunks, uint4
                              : "l"(d_x + c * 2));
         }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < kLoads; ++k) {
             const uint64_t c = base + k * kActThreads + threadIdx.x;
             const __half2* h = reinterpret_cast<const __half2*>(in[k]);
             // min / max over the four lanes of the group (the compressor's sorter stage, Sec. 4.3), as (min, -max) in one number
@@ -122,12 +127,14 @@ ecco_act_compress_kernel(const uint4* __restrict__ d_x, uint64_t n_chunks, uint4
     }
 }
 
-// eight CTAs per SM, and no more than it takes for every CTA to get the same number of turns
-int act_grid(uint64_t n_chunks, const DeviceInfo& di)
+// Loads per thread, and CTAs: eight per SM, and no more than it takes for every CTA to get the same number of turns.
+struct ActPlan { int loads; unsigned grid; };
+ActPlan act_plan(uint64_t n_chunks, const DeviceInfo& di)
 {
-    const uint64_t turns = (n_chunks + kActChunks - 1) / kActChunks, cap = static_cast<uint64_t>(di.sms) * 8;
-    const uint64_t rounds = (turns + cap - 1) / cap;
-    return static_cast<int>((turns + rounds - 1) / rounds);
+    const uint64_t cap = static_cast<uint64_t>(di.sms) * 8;
+    const int loads = n_chunks <= cap * act_chunks(1) ? 1 : n_chunks <= cap * act_chunks(2) ? 2 : 4;
+    const uint64_t turns = (n_chunks + act_chunks(loads) - 1) / act_chunks(loads), rounds = (turns + cap - 1) / cap;
+    return {loads, static_cast<unsigned>((turns + rounds - 1) / rounds)};
 }
 
 }  // namespace

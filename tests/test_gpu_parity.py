@@ -922,6 +922,14 @@ def test_act2x_compress_and_decompress_match_oracle(B, eo, synth, n_groups):
     assert np.array_equal(got[finite], want[finite])
 
 
+@pytest.mark.parametrize("loads,past", [(1, 0), (1, 1), (2, 0), (2, 1), (4, 0), (4, 1)])
+def test_act2x_at_the_change_of_loads_per_thread(B, eo, synth, loads, past):
+    """The largest call with one and with two loads per thread (eight CTAs of 256 threads per SM, four threads to a group) and the next
+    one, which has twice as many; the largest with four whose CTAs get one turn, and the next one."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    test_act2x_compress_and_decompress_match_oracle(B, eo, synth, sms * 8 * 256 * loads // 4 + past)
+
+
 # ------------------------------------------------------------------ fused attention output (softmax . V)
 def gpu_attn_values(B, lmeta, blocks, batch, heads, seq, qpk, scores):
     d_meta, d_blocks, d_s = B.meta_to_device(lmeta), dev(blocks), dev(scores)
