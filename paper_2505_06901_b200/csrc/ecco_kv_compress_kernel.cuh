@@ -234,7 +234,7 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
 //  * a lane joins its sixteen codewords into one string of at most 128 bits in registers and ORs five words into the block.
 // Bound by the issue slots (80 % busy, ncu): some 300 warp instructions per group against 735 of the kernel above; two calls of
 // 131 072 groups take 102 us against 218.5.  Making the tables costs a call 3 us, which is what the smaller instruction count
-// saves at about 16 000 groups (two calls of 8192: 26.5 against 19.5 us, of 16 384: 30.6 against 31.3): fewer go to the kernel above.
+// saves at about 16 000 groups (two calls of 8192: 26.5 against 19.5 us, of 16 384: 28.9, where the kernel above takes 29.2 for 16 000): fewer go to the kernel above.
 // ---------------------------------------------------------------------------------------------
 constexpr int kKvManyWarps = 32;
 constexpr int kKvCells = 256;
