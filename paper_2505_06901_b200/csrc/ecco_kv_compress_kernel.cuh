@@ -239,7 +239,6 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
 constexpr int kKvManyWarps = 32;
 constexpr int kKvCells = 256;
 constexpr float kCellWidth = 1.0f / 127.5f;
-constexpr float kBeyond = 1.0e30f;                         // no value is above it
 struct KvManySmem {
     // per cell the first midpoint not below it, as a float whose low five bits hold the number of those below, | 16 if the cell holds several
     uint32_t cell[kMaxPatterns * kKvCells];
@@ -247,7 +246,7 @@ struct KvManySmem {
     uint16_t enc[kMaxPatterns * kCodebooks * kSymbols];    // length | codeword in stream order << 8
     uint16_t kp[kMaxPatterns];
     uint32_t len4[kMaxPatterns * kSymbols];                // code lengths of a symbol in the four codebooks, one per byte
-    float mid[kMaxPatterns * 16];                          // midpoints of neighbouring centroids (14 per pattern), then a large number
+    float mid[kMaxPatterns * 16];                          // midpoints of neighbouring centroids (14 per pattern), then infinity
     float2 ends[kMaxPatterns];                             // first and last centroid
     uint4 x[kKvManyWarps][64];                             // the warp's four groups, fp16 [4][128]
     uint32_t blk[kKvManyWarps][64];                        // their blocks
@@ -293,7 +292,7 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
             }
         }
         sm.len4[i] = v;
-        sm.mid[i] = s < kCentroids - 1 ? 0.5f * (centroid(k, s) + centroid(k, s + 1)) : kBeyond;
+        sm.mid[i] = s < kCentroids - 1 ? 0.5f * (centroid(k, s) + centroid(k, s + 1)) : INFINITY;
         if (s == 0) sm.ends[k] = make_float2(centroid(k, 0), centroid(k, kCentroids - 1));
     }
     __syncthreads();
@@ -307,7 +306,7 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
         for (int q = 0; q < 16; ++q, ++c) {
             if (c > 0) while (below < kCentroids - 1 && m[below] < (static_cast<float>(c) - 0.51f) * kCellWidth - 1.0f) ++below;
             while (upto < kCentroids - 1 && (c == kKvCells - 1 || m[upto] <= (static_cast<float>(c) + 0.51f) * kCellWidth - 1.0f)) ++upto;
-            // the nearest float that ends in those five bits: at most sixteen places off
+            // the nearest float that ends in those five bits: at most sixteen places off.  Infinity becomes a NaN, which nothing is above
             const uint32_t low = static_cast<uint32_t>(below) | (upto - below > 1 ? 16u : 0u);
             out[q] = ((__float_as_uint(m[below]) + 16u - low) & ~31u) | low;
         }

@@ -1185,6 +1185,19 @@ def test_kv_compress_of_many_groups_matches_the_host_encoder(B, eo, kv_small, sy
     assert_blocks_equal(gpu_kv_compress(B, lm, x), want)
 
 
+def test_kv_compress_of_many_groups_maps_a_second_infinity_to_an_end_centroid(B, eo):
+    """Blocks of groups with infinities are unspecified, but only the abs-max itself carries the abs-max's symbol: a value above all midpoints
+    takes the last centroid, one below all of them the first.  Codewords of four bits, so that every group is cut off and no outlier hides the symbol."""
+    om = make_meta(eo, lambda k, h, rng: [4] * 16, S=5, e=-3, seed=6)
+    x = np.zeros((16384, 128), dtype=np.float16)
+    x[::3, :3] = np.inf, np.inf, -np.inf
+    x[1::3, 5:8] = -np.inf, -np.inf, np.inf
+    dec = eo.decode(om, gpu_kv_compress(B, lib_meta_from_oracle(B, om), x)).astype(np.float64)
+    scale, ends = 448.0 * 2.0 ** om.e, om.patterns()[0].astype(np.float64)[[0, 14]]      # no pattern fits: the first one
+    first, last = np.float16(scale * ends)
+    assert (dec[::3, :3] == [scale, last, first]).all() and (dec[1::3, 5:8] == [-scale, first, last]).all()
+
+
 def test_kv_compress_full_size_round_trip(B, eo, W, synth):
     """cfg 3 K cache: GPU-compressed blocks equal the host encoder's, and decompress to the same fp16."""
     (t,) = W.config3(which=("K",), keep_source=True)
