@@ -630,9 +630,8 @@ extern "C" int ecco_act_decompress(const uint8_t* d_blocks, uint64_t n_groups, v
     int rc = device_info(&di);
     if (rc) return rc;
     const uint64_t n_chunks = n_groups * 4;
-    const ActPlan p = act_plan(n_chunks, di);
-    return launch_overlapped(p.loads == 1 ? ecco_act_decompress_kernel<1> : p.loads == 2 ? ecco_act_decompress_kernel<2> : ecco_act_decompress_kernel<4>, p.grid, static_cast<unsigned>(kActThreads), 0,
-                             static_cast<cudaStream_t>(stream), reinterpret_cast<const uint4*>(d_blocks), n_chunks, static_cast<uint4*>(d_out_fp16));
+    return launch_overlapped(ecco_act_decompress_kernel, act_ctas(n_chunks, 1), static_cast<unsigned>(kActThreads), 0, static_cast<cudaStream_t>(stream),
+                             reinterpret_cast<const uint4*>(d_blocks), n_chunks, static_cast<uint4*>(d_out_fp16));
 }
 
 extern "C" int ecco_act_compress(const void* d_x_fp16, uint64_t n_groups, uint8_t* d_blocks, void* stream)
@@ -645,8 +644,8 @@ extern "C" int ecco_act_compress(const void* d_x_fp16, uint64_t n_groups, uint8_
     int rc = device_info(&di);
     if (rc) return rc;
     const uint64_t n_chunks = n_groups * 4;
-    const ActPlan p = act_plan(n_chunks, di);
-    return launch_overlapped(p.loads == 1 ? ecco_act_compress_kernel<1> : p.loads == 2 ? ecco_act_compress_kernel<2> : ecco_act_compress_kernel<4>, p.grid, static_cast<unsigned>(kActThreads), 0,
+    const int loads = act_compress_loads(n_chunks, di);
+    return launch_overlapped(loads == 1 ? ecco_act_compress_kernel<1> : ecco_act_compress_kernel<2>, act_ctas(n_chunks, loads), static_cast<unsigned>(kActThreads), 0,
                              static_cast<cudaStream_t>(stream), static_cast<const uint4*>(d_x_fp16), n_chunks, reinterpret_cast<uint4*>(d_blocks));
 }
 

@@ -924,8 +924,8 @@ def test_act2x_compress_and_decompress_match_oracle(B, eo, synth, n_groups):
 
 @pytest.mark.parametrize("loads,past", [(1, 0), (1, 1), (2, 0), (2, 1), (4, 0), (4, 1)])
 def test_act2x_at_the_change_of_loads_per_thread(B, eo, synth, loads, past):
-    """The largest call with one and with two loads per thread (eight CTAs of 256 threads per SM, four threads to a group) and the next
-    one, which has twice as many; the largest with four whose CTAs get one turn, and the next one."""
+    """Multiples of eight CTAs of 256 threads per SM, four threads to a group, whose last CTA is full, and the next call, whose last CTA
+    has one group.  The first multiple is the largest call with one load per thread in the compressor, the next call the smallest with two."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     test_act2x_compress_and_decompress_match_oracle(B, eo, synth, sms * 8 * 256 * loads // 4 + past)
 
