@@ -240,7 +240,8 @@ constexpr int kKvManyWarps = 32;
 constexpr int kKvCells = 256;
 constexpr float kCellWidth = 1.0f / 127.5f;
 struct KvManySmem {
-    // per cell the first midpoint not below it, as a float whose low five bits hold the number of those below, | 16 if the cell holds several
+    // per cell the first midpoint not below it, as a float whose low five bits hold the number of those below; if the cell holds several,
+    // that number | 16 and no midpoint: its values are decided exactly
     uint32_t cell[kMaxPatterns * kKvCells];
     uint16_t pat[kMaxPatterns * 16];
     uint16_t enc[kMaxPatterns * kCodebooks * kSymbols];    // length | codeword in stream order << 8
@@ -307,8 +308,8 @@ ecco_kv_compress_many_kernel(const uint8_t* __restrict__ d_meta, const __half* _
             if (c > 0) while (below < kCentroids - 1 && m[below] < (static_cast<float>(c) - 0.51f) * kCellWidth - 1.0f) ++below;
             while (upto < kCentroids - 1 && (c == kKvCells - 1 || m[upto] <= (static_cast<float>(c) + 0.51f) * kCellWidth - 1.0f)) ++upto;
             // the nearest float that ends in those five bits: at most sixteen places off.  Infinity becomes a NaN, which nothing is above
-            const uint32_t low = static_cast<uint32_t>(below) | (upto - below > 1 ? 16u : 0u);
-            out[q] = ((__float_as_uint(m[below]) + 16u - low) & ~31u) | low;
+            const uint32_t low = static_cast<uint32_t>(below);
+            out[q] = upto - below > 1 ? low | 16u : ((__float_as_uint(m[below]) + 16u - low) & ~31u) | low;
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) reinterpret_cast<uint4*>(sm.cell)[i * 4 + q] = make_uint4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);

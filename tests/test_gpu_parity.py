@@ -1147,11 +1147,12 @@ def test_kv_compress_edge_groups_and_s16(B, eo, kv_small, synth):
 
 
 @pytest.mark.parametrize("kind,n_groups", [("calibrated", 16383), ("calibrated", 16384), ("s16", 16385), ("equal centroids", 16386),
-                                           ("dense centroids", 16387), ("wide centroids", 16384), ("skewed codes", 16385)])
+                                           ("dense centroids", 16387), ("wide centroids", 16384), ("skewed codes", 16385),
+                                           ("midpoint at zero", 16386)])
 def test_kv_compress_of_many_groups_matches_the_host_encoder(B, eo, kv_small, synth, kind, n_groups):
     """Calls on both sides of the size from which eight lanes share a group, ragged in the last four groups, on groups that
     decide at the edges: values at midpoints of centroids, ties, zeros, one value only, saturating and subnormal scales,
-    patterns with equal centroids, with several midpoints per table cell and with centroids far outside [-1, 1]."""
+    patterns with equal centroids, with several midpoints per table cell (a zero the first of them, too) and with centroids far outside [-1, 1]."""
     rng = np.random.Generator(np.random.PCG64(n_groups))
     if kind == "calibrated":
         om = kv_small["meta"]
@@ -1167,6 +1168,8 @@ def test_kv_compress_of_many_groups_matches_the_host_encoder(B, eo, kv_small, sy
                 p[2:12] = p[2] + np.arange(10) * 0.0007
             elif kind == "wide centroids":
                 p *= 4.0
+            elif kind == "midpoint at zero":
+                p = np.concatenate([np.linspace(-0.9, -0.1, 7), [-0.0003, 0.0003, 0.0011], np.linspace(0.2, 0.9, 5)])
             for j, c in enumerate(np.sort(p.astype(np.float16)).view(np.uint16)):
                 om.pattern[k][j] = int(c)
     lm = lib_meta_from_oracle(B, om)
