@@ -1010,7 +1010,7 @@ def values_floor(eo, meta, blocks, batch, heads, seq, qpk):
 
 @pytest.mark.parametrize("batch,heads,seq,qpk", [(1, 1, 31, 8), (1, 1, 6000, 5), (3, 50, 65, 1), (2, 8, 777, 2), (1, 3, 40000, 1), (1, 4, 22000, 8), (2, 70, 590, 3)])
 def test_attn_values_of_every_unit_size(B, eo, kv_small, batch, heads, seq, qpk):
-    """Units of one warp to nineteen; one head in a piece per SM; more short heads than SMs."""
+    """Units of one warp to nineteen, one or two of them to a CTA; one head in a piece per SM; more short heads than SMs."""
     meta = kv_small["meta"]
     n = batch * heads * seq
     blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
@@ -1028,9 +1028,9 @@ def test_attn_values_of_many_short_rows(B, eo, kv_small, batch, heads, seq, qpk)
 
 @pytest.mark.parametrize("batch,heads,seq,qpk", [(16, 32, 300, 2), (4, 32, 1500, 1)])
 def test_attn_values_error_does_not_grow_with_the_tiles_of_a_warp(B, eo, kv_small, batch, heads, seq, qpk):
-    """2-norm of the error over that of the result, rows of which a warp takes several tiles.  An addition is off by 0.43 * 2^-24 of its
-    result (rms), a chain of n terms of random sign by that times sqrt(n / 2): 47 tiles one after the other make 1.2e-7.  A weight
-    is off by a last place or two (2^-24..2^-22), at random over some hundred tokens that count: 1e-7.  Together 1.6e-7; sums
+    """2-norm of the error over that of the result, rows of which a warp takes three tiles.  An addition is off by 0.43 * 2^-24 of its
+    result (rms), a chain of n terms of random sign by that times sqrt(n / 2), 47 tiles one after the other by 1.2e-7.  A weight
+    is off by a last place or two (2^-24..2^-22), at random over some hundred tokens that count: 1e-7.  Together 1.6e-7 at most; sums
     that grow inside the tensor cores, which cut off, are off by 2.5e-7 here.  Limit 2e-7."""
     n = batch * heads * seq
     blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
@@ -1043,10 +1043,56 @@ def test_attn_values_error_does_not_grow_with_the_tiles_of_a_warp(B, eo, kv_smal
     assert rel <= 2e-7, rel
 
 
+def values_plan(heads, seq):
+    """(warps of a unit, teams) that ecco_attn_values takes: the rule of av_teams (ecco_kernels.cu) restated, to see what a shape exercises."""
+    tiles, ctas = (seq + 31) // 32, torch.cuda.get_device_properties(0).multi_processor_count
+    ctas = min(ctas, 256, heads * tiles)
+    best = None
+    for w in range(19, 0, -1):
+        cost = -(-heads * -(-tiles // w) // ctas) * (6 + w) + max(1, -(-heads // ctas) - 1) * 10
+        cost += cost // 32 + 1 if w > 16 else 0
+        if best is None or cost < best[0]:
+            best = (cost, w, 1)
+    for t in range(2, 17):
+        for w in range(1, 16 // t + 1):
+            cost = -(-heads // (ctas * t)) * (-(-tiles // w) * (6 + w * min(t, -(-heads // ctas))) + 10)
+            if cost < best[0]:
+                best = (cost, w, t)
+    return best[1:]
+
+
+@pytest.mark.parametrize("heads,seq,qpk,plan", [(296, 4096, 3, (16, 1)), (160, 7777, 2, (19, 1)), (300, 512, 8, (4, 3))])
+def test_attn_values_with_many_tiles_of_a_row_to_a_warp(B, eo, kv_small, heads, seq, qpk, plan):
+    """Rows of which a warp takes four to thirteen tiles one after the other, in both kernels and in teams: random scores, held to
+    the 2-norm limit above, too; scores that grow or fall along the row, so that every tile or only the first raises the maximum; rows whose first
+    half is masked, so that warps go from tiles without any weight to others."""
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert values_plan(heads, seq) == plan and -(-seq // (32 * plan[0])) >= 4
+    meta, n = kv_small["meta"], heads * seq
+    blocks = np.tile(kv_small["blocks"], (-(-n // 2048), 1))[:n]
+    dec = eo.decode(meta, kv_small["blocks"]).astype(np.float64)
+    s = np.random.Generator(np.random.PCG64(seq)).standard_normal((heads, qpk, seq)).astype(np.float32)
+    ramp = np.linspace(-60, 60, seq, dtype=np.float32)
+    s[1::4] += ramp
+    s[2::4] -= ramp
+    s[3::4, :, : seq // 2] = -np.inf
+    got = gpu_attn_values(B, lib_meta_from_oracle(B, meta), blocks, 1, heads, seq, qpk, s.reshape(1, heads * qpk, seq)).reshape(heads, qpk, 128)
+    p = np.exp(s.astype(np.float64) - s.max(axis=2, keepdims=True))
+    p /= p.sum(axis=2, keepdims=True)
+    # blocks repeat after 2048 groups: weights of the same block are added first
+    at = (np.arange(n).reshape(heads, seq)) % 2048
+    folded = np.stack([np.stack([np.bincount(at[h], p[h, q], 2048) for q in range(qpk)]) for h in range(heads)])
+    ref, refabs = folded @ dec, folded @ np.abs(dec)
+    floor = 2.0 ** -38 * np.stack([np.bincount(at[h], minlength=2048) @ np.abs(dec) for h in range(heads)])[:, None]
+    check_fused(got, ref, refabs, "values many tiles", VALUES_TOL, floor)
+    rel = float(np.linalg.norm(got[::4] - ref[::4]) / np.linalg.norm(ref[::4]))
+    assert rel <= 2e-7, rel
+
+
 @pytest.mark.parametrize("seq", [33, 700, 3000])
 def test_attn_values_with_rising_scores_and_any_workspace(B, eo, kv_small, seq):
-    """Scores that grow along the row (every tile raises the running maximum), fall, or hold their largest value in the last token, over
-    heads split between several blocks; the same bits whatever the workspace held."""
+    """Scores that grow along the row, fall, or hold their largest value in the last token, over heads split between several blocks, each of
+    which has one unit of its head (several: the test above); the same bits whatever the workspace held."""
     meta, heads, qpk = kv_small["meta"], 3, 4
     rng = np.random.Generator(np.random.PCG64(seq))
     n = heads * seq
