@@ -287,14 +287,15 @@ __device__ __forceinline__ uint32_t decode_group_by_one(LaneGroup& g, uint32_t b
 // the warp.
 // What lies behind the end bit is arbitrary: a codeword that ends by then does not depend on it, and one that does not ends behind it
 // whatever it looks like there.
-// kLastRow / kEndBit: the row of that bit, and the bit, counted from the lane's staged stream.  kFreeSteps: that many leading steps
-// carry no end test; the caller guarantees that the stream cannot end in them.
+// kEndBit: that bit, counted from the lane's staged stream.  kFreeSteps: that many leading steps carry no end test; the caller
+// guarantees that the stream cannot end in them.
 // pairs = false (uniform): decode_group_by_one.
 // refill(p): called after every step, for a lane that holds a part of its stream only; it may move p, which is LaneGroup::p.
-template <uint32_t kLastRow, uint32_t kEndBit, int kFreeSteps, class Sink, class Refill = NoRefill>
+template <uint32_t kEndBit, int kFreeSteps, class Sink, class Refill = NoRefill>
 __device__ __forceinline__ uint32_t decode_group(LaneGroup& g, uint32_t bits, bool pairs, Sink&& sink, Refill&& refill = {})
 {
     if (!pairs) return decode_group_by_one<kEndBit, kFreeSteps>(g, bits, sink, refill);
+    constexpr uint32_t kLastRow = kEndBit / 32;
     bool complete = true;
     // second symbol of an escape entry: its codeword starts 1 + (length of the first) bits into win
     auto resolve = [&](uint32_t e, uint32_t win) {

@@ -45,7 +45,7 @@ ecco_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __rest
         ldg_block(blk, d_blocks + min(g, n_groups - 1) * kBlockBytes);
         LaneGroup lg = open_block(blk, bits, tb, T);
         uint16_t* out = d_out + min(g, n_groups - 1) * kGroup;
-        const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
+        const uint32_t end = decode_group<kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
             uint32_t v[4];
             map_ranks(lg, ranks, v);
             if (cutting) cut_values(v, n_ok);
@@ -168,7 +168,7 @@ ecco_decompress_tma_kernel(const __grid_constant__ DecompressBatch batch)
                 __syncwarp();
                 if (lane == 0) { tma_store_2d(out_map, stage, x, static_cast<int>(row0)); bulk_commit(); }
             };
-            const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
+            const uint32_t end = decode_group<kBlockBits, kBlockFreeSteps>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
                 uint32_t v[4];
                 map_ranks(lg, ranks, v);
                 if (cutting) cut_values(v, n_ok);
@@ -320,7 +320,7 @@ ecco_var_decompress_kernel(const uint8_t* __restrict__ d_meta, const uint4* __re
         const uint32_t hdr = __funnelshift_r(lds_u32(bits + (first >> 5) * 128), lds_u32(bits + (first >> 5) * 128 + 128), first);
         LaneGroup lg = open_lane_group(hdr, first, tb, T);
         const int row0 = static_cast<int>(tile * 32);
-        decode_group<kVarRows - 3, kVarRows * 32, 16>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool, int) {
+        decode_group<kVarRows * 32, 16>(lg, bits, tb.pairs, [&](int i, uint32_t ranks, bool, int) {
             uint32_t v[4];
             map_ranks(lg, ranks, v);
             if (!(i & 1)) {

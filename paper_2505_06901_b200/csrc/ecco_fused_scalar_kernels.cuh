@@ -63,7 +63,7 @@ __device__ __forceinline__ void fused_group(const Block& blk, const DecodeTables
     LaneGroup g = open_block(blk, bits, tb, T);
     if (kDeal) sts_u32(bits + 18 * 128, blk.w[0]);                    // the ranks will lie over the block's first words
     const uint32_t ranks_at = bits - kRankRows * 128;
-    const uint32_t end = decode_group<16, kBlockBits, kBlockFreeSteps>(g, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
+    const uint32_t end = decode_group<kBlockBits, kBlockFreeSteps>(g, bits, tb.pairs, [&](int i, uint32_t ranks, bool cutting, int n_ok) {
         uint32_t v[4];
         map_ranks(g, ranks, v);
         if (cutting) cut_values(v, n_ok);
