@@ -125,7 +125,9 @@ int ecco_encode_host(ecco_meta* meta, const uint16_t* src_fp16, uint64_t n_group
 size_t ecco_meta_device_bytes(const ecco_meta* meta);
 int ecco_meta_serialize_device(const ecco_meta* meta, void* host_staging, size_t bytes);
 
-/* ---------------------------------------------------------------- device, asynchronous */
+/* ---------------------------------------------------------------- device, asynchronous
+ * A call takes a share of every SM as soon as it has a piece of work for each, so small calls on several streams
+ * largely wait for one another; independent ones are faster together in one ecco_decompress_batch or ecco_gemv_batch. */
 
 /* Sec. 4.2 (pattern retriever, Huffman decode, outlier handling, mapper): n_groups blocks at
  * d_blocks -> n_groups*128 fp16 at d_out_fp16.  Value = fp16_rn(fp32(centroid) * fp32(scale));

@@ -261,7 +261,7 @@ ecco_attn_values_kernel(const uint8_t* __restrict__ d_meta, const uint8_t* __res
             }
             decode_to_tiles<false, true>(cur, tb, tiles, T, valid);             // past the end of the row: zeros
             // Per 16-dim tile: (V tile)^T x P^T on the tensor cores.  They cut their sums off instead of rounding them, so only a tile's 32
-            // tokens are summed there: error of 16 x 32 x 300 tokens (five tiles to a warp) 2.5e-7 -> 1.6e-7 of the result, of 16 x 8 x
+            // tokens are summed there: error of 16 x 32 x 300 tokens (three tiles to a warp) 2.5e-7 -> 1.6e-7 of the result, of 16 x 8 x
             // 32768 2.3e-6 -> 2.0e-7; [8][32][4096][128] 141.6 -> 142.6 us.
             const uint32_t a_at = tiles + tile_byte((lane >> 4) * 8 + (lane & 7u), ((lane >> 3) & 1u) * 8);
 #pragma unroll

@@ -18,8 +18,8 @@
 namespace {
 
 // Shared memory of a CTA, from its 1 KB-aligned base: misc words (the barrier word first: images come and go, the barrier stays), patterns
-// and codebook records, then the tables of the decode and the arrays of as many warps as find room behind them.  The first three fill
-// the gap in front of the pair tables, which are aligned to the widest.  The sizes come from the image's header, so the kernels are
+// and codebook records, then the tables of the decode and the arrays of as many warps as find room behind them, and the ID_KP table as the
+// last part.  The first three fill the gap in front of the pair tables, which are aligned to the widest.  The sizes come from the image's header, so the kernels are
 // launched with all the shared memory an SM has and lay themselves out once they have read it.
 constexpr uint32_t kMisc = 1024;
 constexpr uint32_t kSmemPat = kMisc;                                 // [64][16] fp16

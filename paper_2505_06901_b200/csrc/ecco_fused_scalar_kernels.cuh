@@ -49,7 +49,8 @@ __device__ __forceinline__ float rank_value(const LaneGroup& g, uint32_t rank)
 
 // Partial sums per product.  One chain over a group's 128 products is less exact than the tensor cores' shorter ones where a warp has
 // a single unit: 513 x 512 by three rows, error 2.06e-7 of the result against 1.97e-7, and 1.38e-7 with two chains.  At three to
-// five rows the second chain costs 1.5 to 4 % (two 11008 x 4096 matrices 65.7 -> 66.8, 71.5 -> 74.4 and 79.4 -> 81.0 us).
+// five rows the second chain costs 1.5 to 4 % (two 11008 x 4096 matrices 65.7 -> 66.8, 71.5 -> 74.4 and 79.4 -> 81.0 us), some of it by
+// spills: 12 bytes per thread at four rows (none with one chain), 28 at five (16).
 constexpr int kChains = 2;
 __device__ __forceinline__ float sum_of(const float (&a)[kChains]) { return a[0] + a[1]; }
 

@@ -7,8 +7,9 @@
 // keeps every per-symbol index (output position, activation element) uniform across the warp.
 //
 // Shared memory per CTA (sizes from the image's header, see ecco_decode_core.cuh):
-//   tables   pattern[64][16] fp16 | codebook records [256] x 16 B | pair tables | ID_KP table [4096] u16 | centroids in rank order
-//            [256][16] fp16 | shape tables [n_shapes][256] u8; all but the centroids are brought in by bulk copies (cp.async.bulk + mbarrier)
+//   tables   pattern[64][16] fp16 | codebook records [256] x 16 B | pair tables | centroids in rank order [256][16] fp16 | shape tables
+//            [n_shapes][256] u8, and behind the warps' arrays, at the end of shared memory, ID_KP table [4096] u16; all but the centroids
+//            are brought in by bulk copies (cp.async.bulk + mbarrier)
 //   per warp bits[19][32] u32   the warp's 32 blocks, word-transposed: lane L's word w at
 //                               [w][L] -> bank L whatever w is (conflict-free refills);
 //                               rows 16 to 18 are scratch: what a lane reads past stream bit 512 does not matter (decode_group).  The
@@ -511,9 +512,10 @@ extern "C" int ecco_attn_scores(const void* d_meta, const uint8_t* d_kblocks, in
 // ecco_attn_values
 // ---------------------------------------------------------------------------------------------
 namespace {
-// Warps of a CTA of ecco_attn_values that decode.  19 find room (9.4 KB of shared memory per warp), but with more than 16 a thread has 96
+// Warps of a CTA of ecco_attn_values that decode.  20 find room (9.4 KB of shared memory per warp), but with more than 16 a thread has 96
 // registers and the kernel spills a little and takes a few percent more per tile: two kernels, and units of 17 to 19 tiles only where
-// they save turns (a [16][8][32768][128] cache, eight heads, 534 us with 16 and 518 with 19; [8][32][4096][128], before, 162 and 166).
+// they save turns (a [16][8][32768][128] cache, eight heads, 534 us with 16 and 518 with 19; [8][32][4096][128] 162 and 166, by an earlier
+// state of the kernel).  20, which takes the same registers, has not been measured.
 constexpr int kAvWarps = 16, kAvManyWarps = 19;
 struct AvPlan { int grid, unit_warps, teams; size_t partial_bytes, ticket_bytes; };
 // How a CTA's warps share the work.  A unit is unit_warps tiles (of 32 tokens) of one head.

@@ -229,12 +229,13 @@ ecco_kv_compress_kernel(const uint8_t* __restrict__ d_meta, const __half* __rest
 //  * nearest centroid = number of midpoints below the value.  A table per pattern holds for 256 cells of [-1, 1) how many
 //    midpoints lie below the cell and, in the same word, the next one, so a value costs one lookup and one comparison; the value is x times
 //    the scale's reciprocal, and where that comes within 2.4e-6 of a midpoint the exact division and fp64 distances decide.
-//    (Count and midpoint in tables of their own: two calls of 131 072 groups 106.9 us, in one word 102.3.)
+//    (Count and midpoint in tables of their own: two calls of 131 072 groups 106.3 us, in one word 102.2.)
 //  * the four codebooks' lengths are bytes of one word, summed together.
 //  * a lane joins its sixteen codewords into one string of at most 128 bits in registers and ORs five words into the block.
-// Bound by the issue slots (80 % busy, ncu): some 300 warp instructions per group against 735 of the kernel above; two calls of
-// 131 072 groups take 102 us against 218.5.  Making the tables costs a call 3 us, which is what the smaller instruction count
-// saves at about 16 000 groups (two calls of 8192: 26.5 against 19.5 us, of 16 384: 28.9, where the kernel above takes 29.2 for 16 000): fewer go to the kernel above.
+// Bound by the issue slots (82 % busy, ncu): 304 warp instructions per group against 735 of the kernel above; two calls of
+// 131 072 groups take 102 us against 213.6.  Making the tables costs a call 3 us, which is what the smaller instruction count
+// saves at about 14 500 groups (two calls of 8192 24.4 against 17.8 us, of 12 288 26.4 / 24.3, of 14 336 27.6 / 27.7, of 16 383 28.9 / 29.6):
+// fewer than 16 384, where it is 2 % faster, go to the kernel above.
 // ---------------------------------------------------------------------------------------------
 constexpr int kKvManyWarps = 32;
 constexpr int kKvCells = 256;

@@ -122,7 +122,7 @@ inline GemvPlan gemv_plan(int64_t units, int row_tiles, int warps, int cols, int
     return p;
 }
 
-constexpr int kMmaWarps = 20;      // 19 find room beside the tables of a typical image (9.4 KB of shared memory per warp)
+constexpr int kMmaWarps = 20;      // all find room beside the tables of an image of up to 66 code shapes (9.4 KB of shared memory per warp)
 
 // the per-warp kernel (one to five rows of x: vpad columns) or the tensor-core kernel (6..8 rows: eight columns)
 // Per-warp against tensor-core kernel, two 11008 x 4096 matrices in a call: 67 against 81 us at three rows, 81 against 81 at five,
